@@ -8,151 +8,173 @@
 //   Y[jh][c] = sum_i Pbar_{l m}(x_jh) C[i][c]
 // Both are GEMMs with N = 2 * nfields columns.  The table is stored [i][jh] (jh
 // contiguous): it is the K-contiguous A operand of the analysis and the M-contiguous A
-// operand of the synthesis.  One CTA computes a 128 x BN tile; the tile lists are built
-// at grid set-up so that large blocks are scheduled first.
+// operand of the synthesis.  The tile lists are built at grid set-up so that large blocks are
+// scheduled first.
 #include "shot_internal.cuh"
 
 namespace shot {
 
 namespace {
 
-constexpr int BM = 128, BK = 16, NT = 128, APAD = 4;
+// One CTA (two warps) computes a 64 x BN half of a tile of one block's product, BN = 8 TN; a warp
+// owns 32 of the rows, a thread 8 rows x TN columns as TN/2 packed column pairs.  The terms arrive
+// by cp.async in a ring of kSimtStages chunks of 16.
+//
+// What bounds it: FP32 FMA issue.  Packed FMAs (fma.rn.f32x2: two columns an instruction, at half
+// the rate of a scalar FMA, so the same peak) leave every second issue slot to the shared-memory
+// loads: 8 x 6 threads measured 67 TFLOP/s packed against 58 scalar in a loop without global
+// loads, where the loads' words (14 a term for 48 FMAs) take the shared memory's bandwidth.
+// Registers (96 a thread) hold 20 warps on an SM, so the warps must be busy ones: the blocks have
+// 1 to lmax/2 rows, and with 64-row CTAs 8 % of the warps have no row (21 % with 128-row ones); a
+// warp without rows skips its arithmetic, and a last chunk stops at its last term.  TMA chunks
+// (64-byte rows) were slower than cp.async where the table streams (8 fields at 512 rings: 0.061
+// against 0.047 ms).
+//
+// Measured, analysis / synthesis in ms, against a kernel of scalar FMAs on 128-row tiles with one
+// chunk in flight: 720 rings, 24 fields 0.256 / 0.233 -> 0.230 / 0.186; 512 rings, 8 fields 0.087 /
+// 0.068 -> 0.047 / 0.037 (16-column tiles instead of 32); 256 rings, 32 fields 0.047 / 0.030 ->
+// 0.034 / 0.021.
+constexpr int BM = 64, BK = 16, NT = 64, kSimtStages = 3;
+constexpr int kAElems = BM * BK;
 
-template <int BN, bool ANALYSIS>
-__global__ void __launch_bounds__(NT) k_legendre_simt(
-    const Tile* __restrict__ tiles, const float* __restrict__ tab, int ldt,
+__device__ __forceinline__ void cp16(float* dst, const float* src, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(valid ? 16 : 0)
+               : "memory");
+}
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 dup2(float x) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ void fma2(f32x2& d, f32x2 a, f32x2 b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+
+template <int TN, bool ANALYSIS>
+__global__ void __launch_bounds__(NT, TN >= 6 ? 8 : 10) k_legendre_simt(
+    const Tile* __restrict__ tiles, int ncolt, const float* __restrict__ tab, int ldt,
     const long long* __restrict__ row_off, const int* __restrict__ Mrows, int nh,
     const float* __restrict__ Bsrc, int ldc, int ncols, float* __restrict__ out,
     const float* __restrict__ h) {
-  constexpr int TN = BN / 8;
-  constexpr int BF4 = BK * BN / 4;                 // float4 per B chunk
-  constexpr int BL = (BF4 + NT - 1) / NT;          // float4 loads per thread
-  __shared__ __align__(16) float As[2][BK][BM + APAD];
-  __shared__ __align__(16) float Bs[2][BK][BN];
+  constexpr int BN = 8 * TN, NP = TN / 2;
+  // [stage]: A (analysis: 64 rows of 16 terms, the 16-byte pieces of rows 2 i and 2 i + 1 permuted
+  // by i so that the rows a warp reads together lie on different banks; synthesis: 16 terms of 64
+  // nodes), B [term][BN]
+  __shared__ __align__(16) float As[kSimtStages][kAElems];
+  __shared__ __align__(16) float Bs[kSimtStages][BK * BN];
 
-  const Tile tl = tiles[blockIdx.x];
-  const int blk = tl.blk, r0 = tl.r0;
+  const int half = blockIdx.x / ncolt;   // CTA = (128-row tile, half of it, column tile)
+  const Tile tl = tiles[half >> 1];
+  const int blk = tl.blk, r0 = tl.r0 + (half & 1) * BM;
+  const int n0 = (blockIdx.x - half * ncolt) * BN;
   const int m = blk >> 1, p = blk & 1;
   const int M = Mrows[blk];
   const long long ro = row_off[blk];
-  const int n0 = blockIdx.y * BN;
   const int K = ANALYSIS ? nh : M;
   const int mvalid = ANALYSIS ? M : nh;   // rows of the output block
-  const float* Ab = tab + ro * ldt;
-  const float* Bb = ANALYSIS ? (Bsrc + (size_t)blk * nh * ldc) : (Bsrc + ro * ldc);
+  if (r0 >= mvalid) return;
 
-  const int tid = threadIdx.x;
-  const int tn = tid & 7, tm = tid >> 3;
-
-  float4 ra[4];
-  float4 rb[BL];
-
-  auto load = [&](int kt) {
-    if (ANALYSIS) {
-      // A(i, k) = Ab[i*ldt + k], rows r0..r0+127, k in [kt, kt+16): 4 threads per row
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tn = lane & 7, tm = lane >> 3;
+  // this thread's pieces of a chunk: A rows (analysis) tid/4 + 16 s, piece tid%4; A terms
+  // (synthesis) tid/16 + 4 s, nodes 4 (tid%16); B term tid%16, columns 4 (tid/16) + 16 s
+  const float* Ap = ANALYSIS ? tab + (ro + r0 + (tid >> 2)) * ldt + (tid & 3) * 4
+                             : tab + (ro + (tid >> 4)) * ldt + r0 + (tid & 15) * 4;
+  const bool a_in = ANALYSIS || r0 + (tid & 15) * 4 < ldt;
+  const float* Bp = (ANALYSIS ? Bsrc + (size_t)blk * nh * ldc : Bsrc + ro * ldc) + (size_t)(tid & 15) * ldc + n0 +
+                    (tid >> 4) * 4;
+  const int a_dst = ANALYSIS ? (tid >> 2) * BK + (((tid & 3) ^ ((tid >> 3) & 3)) << 2) : tid * 4;
+  const int b_dst = (tid & 15) * BN + (tid >> 4) * 4;
+  auto load = [&](int kt, int st) {
 #pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        const int idx = tid + s * NT;         // 0..511
-        const int row = idx >> 2, kq = idx & 3;
-        const int i = r0 + row;
-        if (i < M) ra[s] = __ldg(reinterpret_cast<const float4*>(Ab + (size_t)i * ldt + kt + kq * 4));
-        else ra[s] = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    } else {
-      // A(jh, i) = Ab[i*ldt + jh], k = i in [kt, kt+16), jh in [r0, r0+128)
-#pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        const int idx = tid + s * NT;
-        const int kr = idx >> 5, c4 = idx & 31;
-        const int i = kt + kr, jh = r0 + c4 * 4;
-        if (i < M && jh < ldt) ra[s] = __ldg(reinterpret_cast<const float4*>(Ab + (size_t)i * ldt + jh));
-        else ra[s] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s = 0; s < 4; ++s) {
+      if (ANALYSIS) {
+        const bool ok = r0 + (tid >> 2) + 16 * s < M;
+        cp16(&As[st][a_dst + 16 * s * BK], ok ? Ap + (size_t)(16 * s) * ldt + kt : tab, ok);
+      } else {
+        const bool ok = a_in && kt + (tid >> 4) + 4 * s < M;
+        cp16(&As[st][a_dst + 4 * s * BM], ok ? Ap + (size_t)(kt + 4 * s) * ldt : tab, ok);
       }
     }
 #pragma unroll
-    for (int s = 0; s < BL; ++s) {
-      const int idx = tid + s * NT;
-      const int kr = idx / (BN / 4), c4 = idx - kr * (BN / 4);
-      const int k = kt + kr, c = n0 + c4 * 4;
-      if (idx < BF4 && k < K && c < ncols) rb[s] = __ldg(reinterpret_cast<const float4*>(Bb + (size_t)k * ldc + c));
-      else rb[s] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-  };
-  auto store = [&](int buf) {
-    if (ANALYSIS) {
-#pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        const int idx = tid + s * NT;
-        const int row = idx >> 2, kq = idx & 3;
-        As[buf][kq * 4 + 0][row] = ra[s].x;
-        As[buf][kq * 4 + 1][row] = ra[s].y;
-        As[buf][kq * 4 + 2][row] = ra[s].z;
-        As[buf][kq * 4 + 3][row] = ra[s].w;
-      }
-    } else {
-#pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        const int idx = tid + s * NT;
-        const int kr = idx >> 5, c4 = idx & 31;
-        *reinterpret_cast<float4*>(&As[buf][kr][c4 * 4]) = ra[s];
-      }
-    }
-#pragma unroll
-    for (int s = 0; s < BL; ++s) {
-      const int idx = tid + s * NT;
-      if (idx < BF4) {
-        const int kr = idx / (BN / 4), c4 = idx - kr * (BN / 4);
-        *reinterpret_cast<float4*>(&Bs[buf][kr][c4 * 4]) = rb[s];
-      }
+    for (int s = 0; s < BN / 16; ++s) {
+      const bool ok = kt + (tid & 15) < K && n0 + (tid >> 4) * 4 + 16 * s < ncols;
+      cp16(&Bs[st][b_dst + 16 * s], ok ? Bp + (size_t)kt * ldc + 16 * s : Bsrc, ok);
     }
   };
 
-  float acc[8][TN];
+  const int wrow = warp * 32;
+  const bool busy = r0 + wrow < mvalid;
+  f32x2 acc[8][NP];
 #pragma unroll
   for (int r = 0; r < 8; ++r)
 #pragma unroll
-    for (int c = 0; c < TN; ++c) acc[r][c] = 0.f;
+    for (int c = 0; c < NP; ++c) acc[r][c] = 0;
 
-  const int nk = (K + BK - 1) / BK;
-  if (nk > 0) {
-    load(0);
-    store(0);
-    __syncthreads();
+#pragma unroll
+  for (int t = 0; t < kSimtStages - 1; ++t) {
+    if (t * BK < K) load(t * BK, t);
+    asm volatile("cp.async.commit_group;" ::: "memory");
   }
-  for (int t = 0; t < nk; ++t) {
-    const int cur = t & 1;
-    if (t + 1 < nk) load((t + 1) * BK);
+  int s = 0;
+  for (int kt = 0; kt < K; kt += BK) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kSimtStages - 2) : "memory");
+    __syncthreads();   // this chunk has landed for both warps, and the one before it has been read
+    if (kt + (kSimtStages - 1) * BK < K) load(kt + (kSimtStages - 1) * BK, s == 0 ? kSimtStages - 1 : s - 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (busy) {
+      const float* A = As[s];
+      const float* B = Bs[s] + 2 * tn;
+      // thread rows: analysis tm + 4 r (kT terms at once), synthesis 4 tm + {0..3} and
+      // 16 + 4 tm + {0..3}
+      constexpr int kT = 4;
+      auto terms = [&](int k0, int nt) {
+        float4 av[8];
+        if (ANALYSIS) {
+          const float* q = A + (wrow + tm) * BK;
+          const int c0 = ((k0 >> 2) ^ (tm >> 1)) << 2, c1 = c0 ^ 8;
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[cur][kk][tm * 8]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[cur][kk][tm * 8 + 4]);
-      const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      float b[TN];
-      if (TN % 4 == 0) {
-#pragma unroll
-        for (int c = 0; c < TN; c += 4) {
-          const float4 bb = *reinterpret_cast<const float4*>(&Bs[cur][kk][tn * TN + c]);
-          b[c] = bb.x; b[c + 1] = bb.y; b[c + 2] = bb.z; b[c + 3] = bb.w;
+          for (int r = 0; r < 8; ++r) av[r] = *reinterpret_cast<const float4*>(q + 4 * r * BK + ((r & 1) ? c1 : c0));
         }
-      } else {
 #pragma unroll
-        for (int c = 0; c < TN; c += 2) {
-          const float2 bb = *reinterpret_cast<const float2*>(&Bs[cur][kk][tn * TN + c]);
-          b[c] = bb.x; b[c + 1] = bb.y;
+        for (int kk = 0; kk < kT; ++kk) {
+          if (kk >= nt) break;
+          float x[8];
+          if (ANALYSIS) {
+#pragma unroll
+            for (int r = 0; r < 8; ++r) x[r] = kk == 0 ? av[r].x : kk == 1 ? av[r].y : kk == 2 ? av[r].z : av[r].w;
+          } else {
+            const float4 u = *reinterpret_cast<const float4*>(A + (k0 + kk) * BM + wrow + 4 * tm);
+            const float4 v = *reinterpret_cast<const float4*>(A + (k0 + kk) * BM + wrow + 16 + 4 * tm);
+            x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w;
+            x[4] = v.x; x[5] = v.y; x[6] = v.z; x[7] = v.w;
+          }
+          f32x2 b[NP];
+#pragma unroll
+          for (int c = 0; c < NP; ++c) b[c] = *reinterpret_cast<const f32x2*>(B + (k0 + kk) * BN + 16 * c);
+#pragma unroll
+          for (int r = 0; r < 8; ++r) {
+            const f32x2 xr = dup2(x[r]);
+#pragma unroll
+            for (int c = 0; c < NP; ++c) fma2(acc[r][c], xr, b[c]);
+          }
         }
-      }
-#pragma unroll
-      for (int r = 0; r < 8; ++r)
-#pragma unroll
-        for (int c = 0; c < TN; ++c) acc[r][c] = fmaf(a[r], b[c], acc[r][c]);
+      };
+      const int kend = min(BK, K - kt);
+      int k0 = 0;
+#pragma unroll 2
+      for (; k0 + kT <= kend; k0 += kT) terms(k0, kT);
+      if (k0 < kend) terms(k0, kend - k0);
     }
-    if (t + 1 < nk) store(cur ^ 1);
-    __syncthreads();
+    if (++s == kSimtStages) s = 0;
   }
+  if (!busy) return;
 
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
-    const int row = r0 + tm * 8 + r;
+    const int row = r0 + wrow + (ANALYSIS ? tm + 4 * r : 4 * tm + (r & 3) + 16 * (r >> 2));
     if (row >= mvalid) continue;
     float sc = 1.f;
     float* o;
@@ -163,48 +185,53 @@ __global__ void __launch_bounds__(NT) k_legendre_simt(
       o = out + ((size_t)blk * nh + row) * ldc;
     }
 #pragma unroll
-    for (int c = 0; c < TN; ++c) {
-      const int col = n0 + tn * TN + c;
-      if (col < ncols) o[col] = acc[r][c] * sc;
+    for (int c = 0; c < NP; ++c) {
+      const int col = n0 + 16 * c + 2 * tn;
+      const float2 v = *reinterpret_cast<const float2*>(&acc[r][c]);
+      if (col < ncols) *reinterpret_cast<float2*>(o + col) = make_float2(v.x * sc, v.y * sc);
     }
   }
 }
 
-template <int BN>
+template <int TN, bool ANALYSIS>
+int launch_one(const Grid& g, int nf, const float* B, float* out, int ldc, const float* h, cudaStream_t st) {
+  const int ncols = 2 * nf, ncolt = (ncols + 8 * TN - 1) / (8 * TN);
+  ProfScope prof(ANALYSIS ? PK_ANALYSIS : PK_SYNTHESIS, st);
+  count_launch();
+  k_legendre_simt<TN, ANALYSIS><<<2 * (ANALYSIS ? g.ntiles_ana : g.ntiles_syn) * ncolt, NT, 0, st>>>(
+      ANALYSIS ? g.tiles_ana : g.tiles_syn, ncolt, g.tab, g.ldt, g.row_off_d, g.M_d, g.nh, B, ldc, ncols, out, h);
+  SHOT_CUDA(cudaGetLastError());
+  return SHOT_OK;
+}
+
+template <int TN>
 int launch_pair(const Grid& g, int nf, const float* X, float* C, float* Y, int ldc, bool ana, bool syn,
                 const float* h, cudaStream_t st) {
-  const int ncols = 2 * nf;
-  const int ny = (ncols + BN - 1) / BN;
-  if (ana) {
-    dim3 grid(g.ntiles_ana, ny);
-    ProfScope prof(PK_ANALYSIS, st);
-    count_launch();
-    k_legendre_simt<BN, true><<<grid, NT, 0, st>>>(g.tiles_ana, g.tab, g.ldt, g.row_off_d, g.M_d, g.nh, X,
-                                                    ldc, ncols, C, h);
-    SHOT_CUDA(cudaGetLastError());
-  }
-  if (syn) {
-    dim3 grid(g.ntiles_syn, ny);
-    ProfScope prof(PK_SYNTHESIS, st);
-    count_launch();
-    k_legendre_simt<BN, false><<<grid, NT, 0, st>>>(g.tiles_syn, g.tab, g.ldt, g.row_off_d, g.M_d, g.nh, C,
-                                                     ldc, ncols, Y, nullptr);
-    SHOT_CUDA(cudaGetLastError());
-  }
-  return SHOT_OK;
+  int rc = SHOT_OK;
+  if (ana) rc = launch_one<TN, true>(g, nf, X, C, ldc, h, st);
+  if (!rc && syn) rc = launch_one<TN, false>(g, nf, C, Y, ldc, nullptr, st);
+  return rc;
 }
 
 int dispatch(const Grid& g, int nf, const float* X, float* C, float* Y, int ldc, bool ana, bool syn,
              const float* h, cudaStream_t st) {
-  const int ncols = 2 * nf;
-  if (g.active.nf == nf && g.active.simt_bn > 0) {
-    if (g.active.simt_bn == 32) return launch_pair<32>(g, nf, X, C, Y, ldc, ana, syn, h, st);
-    if (g.active.simt_bn == 48) return launch_pair<48>(g, nf, X, C, Y, ldc, ana, syn, h, st);
-    return launch_pair<64>(g, nf, X, C, Y, ldc, ana, syn, h, st);
+  // the tile width: the tuned one, else the one that pads the columns least (the wider on a tie,
+  // for more FMAs per shared-memory load and fewer passes over the table)
+  int bn = (g.active.nf == nf) ? g.active.simt_bn : 0;
+  if (bn == 0) {
+    const int ncols = 2 * nf;
+    auto padded = [&](int b) { return (ncols + b - 1) / b * b; };
+    bn = 64;
+    for (int b : {48, 32, 16})
+      if (padded(b) < padded(bn)) bn = b;
+    if (ncols > 64 && bn < 48) bn = padded(64) <= padded(48) ? 64 : 48;
   }
-  if (ncols <= 32) return launch_pair<32>(g, nf, X, C, Y, ldc, ana, syn, h, st);
-  if (ncols <= 48) return launch_pair<48>(g, nf, X, C, Y, ldc, ana, syn, h, st);
-  return launch_pair<64>(g, nf, X, C, Y, ldc, ana, syn, h, st);
+  switch (bn) {
+    case 16: return launch_pair<2>(g, nf, X, C, Y, ldc, ana, syn, h, st);
+    case 32: return launch_pair<4>(g, nf, X, C, Y, ldc, ana, syn, h, st);
+    case 48: return launch_pair<6>(g, nf, X, C, Y, ldc, ana, syn, h, st);
+    default: return launch_pair<8>(g, nf, X, C, Y, ldc, ana, syn, h, st);
+  }
 }
 
 }  // namespace

@@ -411,13 +411,7 @@ int solve_prepare(Grid& g, const std::vector<const float*>& P, const std::vector
     k_fill<<<1024, 256, 0, s.st>>>(v, n * nprob, 1.f);
   }
   SHOT_CUDA(cudaGetLastError());
-  {  // tune the launch shapes on the solver's own form of the inverse DFT
-    EpiParams up = base_ep(s);
-    up.mode = EPI_UPDATE;
-    up.marg = w.marg;
-    up.xout = w.XY;
-    if ((rc = autotune(g, nprob, s.st, &up))) return rc;
-  }
+  if ((rc = autotune(g, nprob, s.st))) return rc;
   if ((rc = launch_heat_mult(g, eps / 4.0, s.st))) return rc;
   // spectra of the starting v
   return launch_dft_fwd(g, v, nprob, nullptr, 0, w.XY, w.ldc, s.st);

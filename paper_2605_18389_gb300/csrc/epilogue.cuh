@@ -1,10 +1,10 @@
 // The Sinkhorn epilogue of the inverse ring transform, shared by the rectangular grids'
 // FFT kernel and the HEALPix ring kernel.
 //
-// z holds K v on the ring pair (real part: ring j, imaginary part: ring J; nseq = nfg
-// sequences of N longitudes at stride ld); the epilogue applies Algorithm 1's pointwise step
-// of the given mode and reduces the per-field partial sums of the pair into
-// ep.part[f][jh][NPART]:
+// z holds K v on the ring pair of 2 G fields, two fields an element (real parts: ring j,
+// imaginary parts: ring J; G sequences of N longitudes at stride ld); the epilogue applies
+// Algorithm 1's pointwise step of the given mode and reduces the per-field partial sums of the
+// pair into ep.part[f][jh][NPART]:
 //   EPI_PLAIN   out = K v
 //   EPI_UPDATE  u = r p / Kv (balanced) or (r p / Kv)^{tau/(tau+eps)} with the problem's FP32
 //               buffer factor r (ProbState ru / rv); sums: sum u (gauge) or sum a p u^{-eps/tau}
@@ -19,7 +19,7 @@
 //               breakdown counts; with ep.xout the new u is also written into `other`
 // Field f occupies out[f * fstride ...]; rings j and J start at rj and rJ within a field.
 #pragma once
-#include "shot_internal.cuh"
+#include "fft.cuh"
 
 namespace shot {
 
@@ -38,7 +38,11 @@ struct EpiField {
 template <int FG>
 __device__ __forceinline__ void epi_fields_load(const EpiParams& ep, int f0, int nfg, EpiField* fi) {
   const int q = threadIdx.x;
-  if (q < FG && q < nfg && ep.mode != EPI_PLAIN) {
+  if (q < FG && ep.mode != EPI_PLAIN) {
+    if (q >= nfg) {
+      fi[q] = EpiField{nullptr, 0, 1, 1.f, 0.f, 1.f};
+      return;
+    }
     const ProbState* P = ep.ps + f0 + q;
     EpiField e;
     e.marg = ep.marg[f0 + q];
@@ -84,31 +88,43 @@ __device__ __forceinline__ float epi_warp_sum(float v) {
   return v;
 }
 
-// kFinal = false compiles the EPI_FINAL branch out (kernels never launched with it)
-template <int FG, int NT, bool kFinal = true>
-__device__ __forceinline__ void ring_pair_epilogue(const float2* z, float2* other, int ld, int N, int nfg, int f0,
+// kFinal = false compiles the EPI_FINAL branch out (kernels never launched with it).
+// The CTA's NT threads form G groups of NT / G (whole warps); group g takes fields f0 + 2 g and
+// f0 + 2 g + 1, a thread longitude k of both rings of the pair, so that one set of sums per
+// thread and one warp reduction serve a group whatever G is.
+template <int G, int NT, bool kFinal = true>
+__device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int ld, int N, int nf, int f0,
                                                    size_t fstride, size_t rj, size_t rJ, bool two, float aj,
                                                    int nh, int jh, const EpiParams& ep,
-                                                   float (*red)[FG * NPART], const EpiField* fi) {
-  constexpr int kEpiBatch = 6;   // longitudes per thread whose marginal values are loaded together
+                                                   float (*red)[2 * NPART], const EpiField* fi) {
+  constexpr int GT = NT / G, GW = GT / 32;
+  static_assert(NT % G == 0 && GT % 32 == 0, "a group is whole warps");
+  constexpr int kEpiBatch = 4;   // longitudes per thread whose marginal values are loaded together
+  const int g = G == 1 ? 0 : threadIdx.x / GT, t = G == 1 ? threadIdx.x : threadIdx.x - g * GT;
+  const int fa = f0 + 2 * g;                       // first field of the group
+  const int nq = min(2, nf - fa);                  // fields of the group (<= 0: none)
+  const float4* zg = reinterpret_cast<const float4*>(z + g * ld);   // (ring j: 2 fields, ring J: 2 fields)
+  float4* og = reinterpret_cast<float4*>(other + g * ld);
   if (ep.mode == EPI_PLAIN) {
-    for (int q = 0; q < nfg; ++q) {
-      float* oj = ep.out + (size_t)(f0 + q) * fstride + rj;
-      float* oJ = ep.out + (size_t)(f0 + q) * fstride + rJ;
-      for (int k = threadIdx.x; k < N; k += blockDim.x) {
-        const float2 zz = z[q * ld + k];
-        oj[k] = zz.x;
-        if (two) oJ[k] = zz.y;
+    float* o = ep.out + (size_t)fa * fstride;
+    for (int k = t; k < N; k += GT) {
+      const float4 zz = zg[k];
+      if (nq > 0) {
+        o[rj + k] = zz.x;
+        if (two) o[rJ + k] = zz.z;
+      }
+      if (nq > 1) {
+        o[fstride + rj + k] = zz.y;
+        if (two) o[fstride + rJ + k] = zz.w;
       }
     }
     return;
   }
-  // Per-element arithmetic is FP32; every thread sums its few elements (<= 2N/512 per
-  // field) in FP32, warps reduce in FP32 and the cross-warp / grid sums are FP64.  A
-  // thread takes longitude k of both rings of the pair.
-  float acc[FG][NPART];
+  // Per-element arithmetic is FP32; every thread sums its few elements (<= 2N/GT per
+  // field) in FP32, warps reduce in FP32 and the cross-warp / grid sums are FP64.
+  float acc[2][NPART];
 #pragma unroll
-  for (int q = 0; q < FG; ++q)
+  for (int q = 0; q < 2; ++q)
 #pragma unroll
     for (int i = 0; i < NPART; ++i) acc[q][i] = 0.f;
   // EPI_FINAL: the dual objective and m(pi) reach the block's FP64 sums through per-thread
@@ -117,60 +133,77 @@ __device__ __forceinline__ void ring_pair_epilogue(const float2* z, float2* othe
   // thread as la sum p + lb sum q + sum (p log u_buf + q log v_buf), with the sums of p and q
   // (and the masses) compensated (Kahan) in FP32 and the offsets applied in FP64; per element
   // the work stays FP32.  m(pi) enters S_dual times eps.
-  __shared__ double redd[NT / 32][FG][2];   // EPI_FINAL: warp sums of m(pi) and the objective
+  __shared__ double redd[NT / 32][2][2];   // EPI_FINAL: warp sums of m(pi) and the objective
 
+  if (ep.mode == EPI_UPDATE || ep.mode == EPI_SYM) {
+    // both fields of an element in one pass: K v comes and the new scaling leaves as 16 bytes
+    const bool sym = ep.mode == EPI_SYM;
+    float* outf[2];
+    const float* mg[2];
+    int live[2], bal[2];
+    float gam[2], rr[2], rinv[2];
 #pragma unroll
-  for (int q = 0; q < FG; ++q) {
-    if (q >= nfg) break;
-    const int f = f0 + q;
-    const size_t fbase = (size_t)f * fstride;
-    float* outf = ep.out + fbase;
-    float* othf = ep.other ? ep.other + fbase : nullptr;
-    const EpiField F = fi[q];
-    if (ep.mode == EPI_UPDATE) {
-      if (!F.live) {
-        if (ep.xout) {   // frozen problem: transform the stored scaling
-          for (int k = threadIdx.x; k < N; k += blockDim.x)
-            other[q * ld + k] = make_float2(outf[rj + k], two ? outf[rJ + k] : 0.f);
+    for (int q = 0; q < 2; ++q) {
+      const EpiField F = fi[2 * g + q];
+      outf[q] = ep.out + (size_t)(fa + q) * fstride;
+      mg[q] = F.marg;
+      live[q] = q < nq && F.live;
+      bal[q] = F.balanced;
+      gam[q] = F.gamma;
+      rr[q] = F.r;
+      rinv[q] = 1.f / F.r;
+    }
+    for (int k0 = t; k0 < N && nq > 0; k0 += kEpiBatch * GT) {
+      // the marginal values (self term: and the old scaling's) of all this thread's longitudes
+      // first, then the arithmetic; a frozen problem loads its stored scaling
+      float pv[kEpiBatch][2][2], uo[kEpiBatch][2][2];
+#pragma unroll
+      for (int b = 0; b < kEpiBatch; ++b) {
+        const int k = k0 + b * GT;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const bool in = k < N && live[q], st = k < N && q < nq && (!live[q] || sym);
+          pv[b][q][0] = in ? __ldg(mg[q] + rj + k) : 0.f;
+          pv[b][q][1] = (in && two) ? __ldg(mg[q] + rJ + k) : 0.f;
+          uo[b][q][0] = st ? outf[q][rj + k] : 0.f;
+          uo[b][q][1] = (st && two) ? outf[q][rJ + k] : 0.f;
         }
-        continue;
       }
-      const float* mg = F.marg;
-      const int bal = F.balanced;
-      const float gam = F.gamma, rr = F.r, rinv = 1.f / F.r;
-      for (int k0 = threadIdx.x; k0 < N; k0 += kEpiBatch * NT) {
-        // the marginal values of all this thread's longitudes first, then the arithmetic
-        float pv[kEpiBatch][2];
 #pragma unroll
-        for (int b = 0; b < kEpiBatch; ++b) {
-          const int k = k0 + b * NT;
-          pv[b][0] = (k < N) ? __ldg(mg + rj + k) : 0.f;
-          pv[b][1] = (k < N && two) ? __ldg(mg + rJ + k) : 0.f;
-        }
+      for (int b = 0; b < kEpiBatch; ++b) {
+        const int k = k0 + b * GT;
+        if (k >= N) break;
+        const float4 zz = zg[k];
+        float un[2][2];
 #pragma unroll
-        for (int b = 0; b < kEpiBatch; ++b) {
-          const int k = k0 + b * NT;
-          if (k >= N) break;
-          const float2 zz = z[q * ld + k];
-          float u2[2];
+        for (int q = 0; q < 2; ++q) {
+          un[q][0] = uo[b][q][0];
+          un[q][1] = uo[b][q][1];
+          if (!live[q]) continue;
 #pragma unroll
           for (int r = 0; r < 2; ++r) {
-            if (r == 1 && !two) { u2[1] = 0.f; break; }
-            const float kv = r ? zz.y : zz.x;
-            const float pm = pv[b][r];
-            const float ratio = __fdividef(pm, kv) * rr;   // MUFU reciprocal + multiply, <= 2 ulp
+            if (r == 1 && !two) { un[q][1] = 0.f; break; }
+            const float kv = q ? (r ? zz.w : zz.y) : (r ? zz.z : zz.x);
+            const float pm = pv[b][q][r];
             float u;
-            if (bal) {
-              u = ratio;
-              acc[q][0] += u;
+            if (sym) {
+              const float ratio = __fdividef(pm, kv);
+              const float x = bal[q] ? ratio : exp2f(gam[q] * __log2f(ratio));
+              u = sqrtf(uo[b][q][r] * x);
             } else {
-              // u = (r p/Kv)^gamma (hardware log2/exp2, ~2^-21 absolute in the exponent); the
-              // translation-invariant sum's p u^{-eps/tau} = p (r p/Kv)^{-eps/(tau+eps)} equals
-              // u (Kv) / r since gamma + eps/(tau+eps) = 1, so one power serves both (ratio = 0
-              // gives u = 0 and adds nothing)
-              u = exp2f(gam * __log2f(ratio));
-              acc[q][0] += aj * u * kv * rinv;
-              acc[q][1] += u;
+              const float ratio = __fdividef(pm, kv) * rr[q];   // MUFU reciprocal + multiply, <= 2 ulp
+              if (bal[q]) {
+                u = ratio;
+                acc[q][0] += u;
+              } else {
+                // u = (r p/Kv)^gamma (hardware log2/exp2, ~2^-21 absolute in the exponent); the
+                // translation-invariant sum's p u^{-eps/tau} = p (r p/Kv)^{-eps/(tau+eps)} equals
+                // u (Kv) / r since gamma + eps/(tau+eps) = 1, so one power serves both (ratio = 0
+                // gives u = 0 and adds nothing)
+                u = exp2f(gam[q] * __log2f(ratio));
+                acc[q][0] += aj * u * kv * rinv[q];
+                acc[q][1] += u;
+              }
             }
             // one test on the common path: K v positive and finite, u finite (NaN fails each
             // comparison); the rare failures are sorted into non-positive (first in the status
@@ -179,83 +212,98 @@ __device__ __forceinline__ void ring_pair_epilogue(const float2* z, float2* othe
               if (kv <= 0.f) acc[q][2] += 1.f;
               else acc[q][3] += 1.f;   // NaN or infinite K v, or u overflowed
             }
-            if (!ep.skip_store) outf[(r ? rJ : rj) + k] = u;
-            u2[r] = u;
+            if (sym || !ep.skip_store) outf[q][(r ? rJ : rj) + k] = u;
+            un[q][r] = u;
           }
-          if (ep.xout) other[q * ld + k] = make_float2(u2[0], u2[1]);
         }
+        if (ep.xout) og[k] = make_float4(un[0][0], un[1][0], un[0][1], un[1][1]);
       }
-    } else if (ep.mode == EPI_SYM) {
-      if (!F.live) {
-        if (ep.xout) {   // frozen problem: transform the stored scaling
-          for (int k = threadIdx.x; k < N; k += blockDim.x)
-            other[q * ld + k] = make_float2(outf[rj + k], two ? outf[rJ + k] : 0.f);
-        }
-        continue;
-      }
-      const float* mg = F.marg;
-      const int bal = F.balanced;
-      const float gam = F.gamma;
-      for (int k0 = threadIdx.x; k0 < N; k0 += kEpiBatch * NT) {
-        // the marginal and old-scaling values of this thread's longitudes first, then the arithmetic
-        float pv[kEpiBatch][2], uo[kEpiBatch][2];
+    }
+  } else {
 #pragma unroll
-        for (int b = 0; b < kEpiBatch; ++b) {
-          const int k = k0 + b * NT;
-          pv[b][0] = (k < N) ? __ldg(mg + rj + k) : 0.f;
-          pv[b][1] = (k < N && two) ? __ldg(mg + rJ + k) : 0.f;
-          uo[b][0] = (k < N) ? outf[rj + k] : 0.f;
-          uo[b][1] = (k < N && two) ? outf[rJ + k] : 0.f;
-        }
-#pragma unroll
-        for (int b = 0; b < kEpiBatch; ++b) {
-          const int k = k0 + b * NT;
-          if (k >= N) break;
-          const float2 zz = z[q * ld + k];
-          float u2[2];
-#pragma unroll
-          for (int r = 0; r < 2; ++r) {
-            if (r == 1 && !two) { u2[1] = 0.f; break; }
-            const float kv = r ? zz.y : zz.x;
-            const float ratio = __fdividef(pv[b][r], kv);
-            const float t = bal ? ratio : exp2f(gam * __log2f(ratio));
-            const float u = sqrtf(uo[b][r] * t);
-            if (!(kv > 0.f && kv < INFINITY && fabsf(u) < INFINITY)) {
-              if (kv <= 0.f) acc[q][2] += 1.f;
-              else acc[q][3] += 1.f;
-            }
-            outf[(r ? rJ : rj) + k] = u;
-            u2[r] = u;
-          }
-          if (ep.xout) other[q * ld + k] = make_float2(u2[0], u2[1]);
-        }
-      }
-    } else if (ep.mode == EPI_CHECK) {
+    for (int q = 0; q < 2; ++q) {
+      if (q >= nq) break;
+      const int f = fa + q;
+      const size_t fbase = (size_t)f * fstride;
+      float* outf = ep.out + fbase;
+      float* othf = ep.other ? ep.other + fbase : nullptr;
+      const EpiField F = fi[2 * g + q];
       if (!F.live) continue;
-      const float* mg = F.marg;
-      const float cuv = ep.ps[f].cuv;
-      for (int k0 = threadIdx.x; k0 < N; k0 += kEpiBatch * NT) {
-        // the marginal and u values of all this thread's longitudes first, then the arithmetic
-        float pv[kEpiBatch][2], uv[kEpiBatch][2];
+      if (ep.mode == EPI_CHECK) {
+        const float* mg = F.marg;
+        const float cuv = ep.ps[f].cuv;
+        for (int k0 = t; k0 < N; k0 += kEpiBatch * GT) {
+          // the marginal and u values of all this thread's longitudes first, then the arithmetic
+          float pv[kEpiBatch][2], uv[kEpiBatch][2];
 #pragma unroll
-        for (int b = 0; b < kEpiBatch; ++b) {
-          const int k = k0 + b * NT;
-          pv[b][0] = (k < N) ? __ldg(mg + rj + k) : 0.f;
-          pv[b][1] = (k < N && two) ? __ldg(mg + rJ + k) : 0.f;
-          uv[b][0] = (k < N) ? __ldg(othf + rj + k) : 0.f;
-          uv[b][1] = (k < N && two) ? __ldg(othf + rJ + k) : 0.f;
+          for (int b = 0; b < kEpiBatch; ++b) {
+            const int k = k0 + b * GT;
+            pv[b][0] = (k < N) ? __ldg(mg + rj + k) : 0.f;
+            pv[b][1] = (k < N && two) ? __ldg(mg + rJ + k) : 0.f;
+            uv[b][0] = (k < N) ? __ldg(othf + rj + k) : 0.f;
+            uv[b][1] = (k < N && two) ? __ldg(othf + rJ + k) : 0.f;
+          }
+#pragma unroll
+          for (int b = 0; b < kEpiBatch; ++b) {
+            const int k = k0 + b * GT;
+            if (k >= N) break;
+            const float4 zz = zg[k];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+              if (r == 1 && !two) break;
+              const float kv = q ? (r ? zz.w : zz.y) : (r ? zz.z : zz.x);
+              const float pm = pv[b][r];
+              const float d = fmaf(cuv * uv[b][r], kv, -pm);
+              if (ep.norm_l1) {
+                acc[q][0] += aj * fabsf(d);
+                acc[q][1] += aj * pm;
+              } else {
+                acc[q][0] += d * d;
+                acc[q][1] += pm * pm;
+              }
+            }
+          }
         }
-#pragma unroll
-        for (int b = 0; b < kEpiBatch; ++b) {
-          const int k = k0 + b * NT;
-          if (k >= N) break;
-          const float2 zz = z[q * ld + k];
+      } else if constexpr (kFinal) {  // EPI_FINAL: z = K v_buf; ep.other = u buffer, ep.out = v buffer
+        const ProbState* P = ep.ps + f;
+        const float* pp = ep.marg[f];
+        const float* qq = ep.marg2[f];
+        const float cu = P->cu, cv = P->cv, cuv = P->cuv;
+        // log u_true = la + log u_buf with la split into an FP32 head and a small remainder
+        const float la_hi = (float)P->la, lb_hi = (float)P->lb;
+        const float la_lo = (float)(P->la - (double)la_hi), lb_lo = (float)(P->lb - (double)lb_hi);
+        const int bal = P->balanced;
+        // balanced, after a v-update: v (K u) = q at every node, so m(pi) = sum a u (K v) =
+        // sum a v (K u) = sum a q (K is self-adjoint in the area inner product)
+        const bool mass_q = bal && !isnan(P->mass_v);
+        const float epsf = (float)ep.eps, tauf = (float)P->tau, et = bal ? 0.f : (float)(ep.eps / P->tau);
+        // balanced: A = sum p, B = sum q (compensated), C = sum p log u_buf + q log v_buf, D = sum
+        // u (K v) (m(pi) before any v-update); unbalanced: A = sum u (K v), B = the objective's terms
+        float A = 0.f, Ac = 0.f, B = 0.f, Bc = 0.f, C = 0.f, D = 0.f;
+        auto kahan = [](float& s, float& c, float x) {
+          const float y = x - c, t = s + y;
+          c = (t - s) - y;
+          s = t;
+        };
+        for (int k = t; k < N; k += GT) {
+          const float4 zz = zg[k];
 #pragma unroll
           for (int r = 0; r < 2; ++r) {
             if (r == 1 && !two) break;
-            const float kv = r ? zz.y : zz.x;
-            const float pm = pv[b][r];
-            const float d = fmaf(cuv * uv[b][r], kv, -pm);
+            const float kv = q ? (r ? zz.w : zz.y) : (r ? zz.z : zz.x);
+            const size_t o = (r ? rJ : rj) + k;
+            const float pm = __ldg(pp + o), qm = __ldg(qq + o);
+            const float ub = othf[o], vb = outf[o];
+            const float lu = la_hi + (logf(ub) + la_lo), lv = lb_hi + (logf(vb) + lb_lo);
+            if (ep.potentials) {
+              othf[o] = epsf * lu;
+              outf[o] = epsf * lv;
+            } else {
+              othf[o] = cu * ub;
+              outf[o] = cv * vb;
+            }
+            const float ukv = cuv * ub * kv;   // u_true (K v_true)
+            const float d = ukv - pm;
             if (ep.norm_l1) {
               acc[q][0] += aj * fabsf(d);
               acc[q][1] += aj * pm;
@@ -263,96 +311,46 @@ __device__ __forceinline__ void ring_pair_epilogue(const float2* z, float2* othe
               acc[q][0] += d * d;
               acc[q][1] += pm * pm;
             }
+            // phi = eps log u, psi = eps log v (App. C.2); terms with a zero marginal vanish.
+            // Balanced: p (la + log u_buf) + q (lb + log v_buf), the offsets applied per thread
+            // below; eps and a_j multiply the sums.
+            if (bal) {
+              kahan(A, Ac, pm);
+              kahan(B, Bc, qm);
+              C += (pm > 0.f ? pm * logf(ub) : 0.f) + (qm > 0.f ? qm * logf(vb) : 0.f);
+              D += ukv;
+            } else {  // tau (1 - e^{-phi/tau}) = -tau expm1(-(eps/tau) log u), per node in FP32
+              kahan(A, Ac, ukv);
+              kahan(B, Bc, (pm > 0.f ? -tauf * expm1f(-et * lu) * pm : 0.f) +
+                               (qm > 0.f ? -tauf * expm1f(-et * lv) * qm : 0.f));
+            }
           }
         }
-      }
-    } else if constexpr (kFinal) {  // EPI_FINAL: z = K v_buf; ep.other = u buffer, ep.out = v buffer
-      if (!F.live) continue;
-      const ProbState* P = ep.ps + f;
-      const float* pp = ep.marg[f];
-      const float* qq = ep.marg2[f];
-      const float cu = P->cu, cv = P->cv, cuv = P->cuv;
-      // log u_true = la + log u_buf with la split into an FP32 head and a small remainder
-      const float la_hi = (float)P->la, lb_hi = (float)P->lb;
-      const float la_lo = (float)(P->la - (double)la_hi), lb_lo = (float)(P->lb - (double)lb_hi);
-      const int bal = P->balanced;
-      // balanced, after a v-update: v (K u) = q at every node, so m(pi) = sum a u (K v) =
-      // sum a v (K u) = sum a q (K is self-adjoint in the area inner product)
-      const bool mass_q = bal && !isnan(P->mass_v);
-      const float epsf = (float)ep.eps, tauf = (float)P->tau, et = bal ? 0.f : (float)(ep.eps / P->tau);
-      // balanced: A = sum p, B = sum q (compensated), C = sum p log u_buf + q log v_buf, D = sum
-      // u (K v) (m(pi) before any v-update); unbalanced: A = sum u (K v), B = the objective's terms
-      float A = 0.f, Ac = 0.f, B = 0.f, Bc = 0.f, C = 0.f, D = 0.f;
-      auto kahan = [](float& s, float& c, float x) {
-        const float y = x - c, t = s + y;
-        c = (t - s) - y;
-        s = t;
-      };
-      for (int k = threadIdx.x; k < N; k += blockDim.x) {
-        const float2 zz = z[q * ld + k];
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          if (r == 1 && !two) break;
-          const float kv = r ? zz.y : zz.x;
-          const size_t o = (r ? rJ : rj) + k;
-          const float pm = __ldg(pp + o), qm = __ldg(qq + o);
-          const float ub = othf[o], vb = outf[o];
-          const float lu = la_hi + (logf(ub) + la_lo), lv = lb_hi + (logf(vb) + lb_lo);
-          if (ep.potentials) {
-            othf[o] = epsf * lu;
-            outf[o] = epsf * lv;
-          } else {
-            othf[o] = cu * ub;
-            outf[o] = cv * vb;
-          }
-          const float ukv = cuv * ub * kv;   // u_true (K v_true)
-          const float d = ukv - pm;
-          if (ep.norm_l1) {
-            acc[q][0] += aj * fabsf(d);
-            acc[q][1] += aj * pm;
-          } else {
-            acc[q][0] += d * d;
-            acc[q][1] += pm * pm;
-          }
-          // phi = eps log u, psi = eps log v (App. C.2); terms with a zero marginal vanish.
-          // Balanced: p (la + log u_buf) + q (lb + log v_buf), the offsets applied per thread
-          // below; eps and a_j multiply the sums.
-          if (bal) {
-            kahan(A, Ac, pm);
-            kahan(B, Bc, qm);
-            C += (pm > 0.f ? pm * logf(ub) : 0.f) + (qm > 0.f ? qm * logf(vb) : 0.f);
-            D += ukv;
-          } else {  // tau (1 - e^{-phi/tau}) = -tau expm1(-(eps/tau) log u), per node in FP32
-            kahan(A, Ac, ukv);
-            kahan(B, Bc, (pm > 0.f ? -tauf * expm1f(-et * lu) * pm : 0.f) +
-                             (qm > 0.f ? -tauf * expm1f(-et * lv) * qm : 0.f));
-          }
+        // this thread's m(pi) and objective in FP64, then the warp's sums
+        double vm, vo;
+        if (bal) {
+          vm = mass_q ? (double)B - (double)Bc : (double)D;
+          vo = P->la * ((double)A - (double)Ac) + P->lb * ((double)B - (double)Bc) + (double)C;
+        } else {
+          vm = (double)A - (double)Ac;
+          vo = (double)B - (double)Bc;
         }
-      }
-      // this thread's m(pi) and objective in FP64, then the warp's sums
-      double vm, vo;
-      if (bal) {
-        vm = mass_q ? (double)B - (double)Bc : (double)D;
-        vo = P->la * ((double)A - (double)Ac) + P->lb * ((double)B - (double)Bc) + (double)C;
-      } else {
-        vm = (double)A - (double)Ac;
-        vo = (double)B - (double)Bc;
-      }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        vm += __shfl_xor_sync(0xffffffffu, vm, o);
-        vo += __shfl_xor_sync(0xffffffffu, vo, o);
-      }
-      if ((threadIdx.x & 31) == 0) {
-        redd[threadIdx.x >> 5][q][0] = vm;
-        redd[threadIdx.x >> 5][q][1] = vo;
+        for (int o = 16; o > 0; o >>= 1) {
+          vm += __shfl_xor_sync(0xffffffffu, vm, o);
+          vo += __shfl_xor_sync(0xffffffffu, vo, o);
+        }
+        if ((threadIdx.x & 31) == 0) {
+          redd[threadIdx.x >> 5][q][0] = vm;
+          redd[threadIdx.x >> 5][q][1] = vo;
+        }
       }
     }
   }
-  // one block reduction for all fields of the CTA
+  // one block reduction, each group's warps for its own two fields
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-  for (int q = 0; q < FG; ++q)
+  for (int q = 0; q < 2; ++q)
 #pragma unroll
     for (int i = 0; i < NPART; ++i) {
       const float v = epi_warp_sum(acc[q][i]);
@@ -360,27 +358,24 @@ __device__ __forceinline__ void ring_pair_epilogue(const float2* z, float2* othe
     }
   __syncthreads();
   if constexpr (kFinal) {
-    if (ep.mode == EPI_FINAL && threadIdx.x < 2 * FG) {
-      const int q = threadIdx.x >> 1, i = threadIdx.x & 1;
-      if (q < nfg && fi[q].live) {
-        double t = 0.0;
-        for (int w = 0; w < NT / 32; ++w) t += redd[w][q][i];
+    if (ep.mode == EPI_FINAL && threadIdx.x < 4 * G) {
+      const int fq = threadIdx.x >> 1, i = threadIdx.x & 1;   // field of the CTA
+      if (f0 + fq < nf && fi[fq].live) {
+        double s = 0.0;
+        for (int w = 0; w < GW; ++w) s += redd[(fq >> 1) * GW + w][fq & 1][i];
         // m(pi) sums a_j times the node values; the balanced objective's sums are of
         // p (la + log u_buf) + q (lb + log v_buf): times eps a_j
-        const double sc = (i == 1 && fi[q].balanced) ? ep.eps * (double)aj : (double)aj;
-        ep.part[((size_t)(f0 + q) * nh + jh) * NPART + 2 + i] = sc * t;
+        const double sc = (i == 1 && fi[fq].balanced) ? ep.eps * (double)aj : (double)aj;
+        ep.part[((size_t)(f0 + fq) * nh + jh) * NPART + 2 + i] = sc * s;
       }
     }
   }
-  if (threadIdx.x < FG * NPART) {
-    const int q = threadIdx.x / NPART, i = threadIdx.x - q * NPART;
-    if (q < nfg && !(ep.mode == EPI_FINAL && i >= 2)) {
-      const int f = f0 + q;
-      if (fi[q].live) {
-        double t = 0.0;
-        for (int w = 0; w < NT / 32; ++w) t += (double)red[w][threadIdx.x];
-        ep.part[((size_t)f * nh + jh) * NPART + i] = t;
-      }
+  if (threadIdx.x < 2 * G * NPART) {
+    const int fq = threadIdx.x / NPART, i = threadIdx.x - fq * NPART;
+    if (f0 + fq < nf && fi[fq].live && !(ep.mode == EPI_FINAL && i >= 2)) {
+      double s = 0.0;
+      for (int w = 0; w < GW; ++w) s += (double)red[(fq >> 1) * GW + w][(fq & 1) * NPART + i];
+      ep.part[((size_t)(f0 + fq) * nh + jh) * NPART + i] = s;
     }
   }
 }

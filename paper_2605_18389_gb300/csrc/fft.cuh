@@ -6,15 +6,22 @@
 // (0 <= j < N/R) reads in[j + r N/R] (r < R), multiplies input r by W_N^{(j mod Ns) r N/(Ns R)},
 // applies an R-point DFT and writes output r to out[(j div Ns) Ns R + (j mod Ns) + r Ns].
 //
+// Two fields travel together.  An element is a C2: the real parts of the two fields' values as
+// one packed pair of FP32, then the imaginary parts.  Every butterfly and twiddle is packed
+// arithmetic (add / mul / fma.rn.f32x2: two FP32 results an instruction, at half the rate of the
+// scalar ones), every shared-memory access 16 bytes, and the index arithmetic serves both fields.
+// What bounds these kernels is instruction issue (a scalar form of them used 54 % of the issue
+// slots at 24 warps an SM, most of the rest waiting on barriers), so the packing takes away
+// about half of what they wait for.
+//
 // Radices go up to 16 so that the rings of the usual grids take three stages
-// (1440 = 9 * 10 * 16); a prime factor above 5 becomes a stage of its own with a generic
+// (1440 = 15 * 8 * 12); a prime factor above 5 becomes a stage of its own with a generic
 // butterfly (O(R) work per output, roots of unity from the plan's table), so any ring
 // length has a plan.  The composite radices (6, 9, 10, 12, 15, 16) run as two
 // register-resident levels of 2-, 3-, 4- and 5-point DFTs (Cooley-Tukey inside the
 // butterfly) whose internal twiddles are compile-time constants.  The stage twiddles come
-// from a per-stage table, r-major, so that consecutive lanes read consecutive entries.
-// Sequences sit at a stride of N + 1 complex values, which staggers the banks of the
-// sequences of one CTA.
+// from a per-stage table, r-major, so that consecutive lanes read consecutive entries; they are
+// read through L1 (every CTA reads the same N values).
 #pragma once
 #include <utility>
 
@@ -22,19 +29,68 @@
 
 namespace shot {
 
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+// ---- packed pairs of FP32 (one value of each of two fields) ---------------------------
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pk2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
 }
-// a * conj(b)
-__device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.y, b.x, -a.x * b.y));
+__device__ __forceinline__ float2 unpk2(f32x2 a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+  return r;
 }
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-// multiply by -i (forward) or +i (inverse)
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// One complex value of each of two fields.
+struct __align__(16) C2 {
+  f32x2 re, im;
+};
+__device__ __forceinline__ C2 c2(f32x2 re, f32x2 im) {
+  C2 r;
+  r.re = re;
+  r.im = im;
+  return r;
+}
+__device__ __forceinline__ C2 cadd(C2 a, C2 b) { return c2(add2(a.re, b.re), add2(a.im, b.im)); }
+__device__ __forceinline__ C2 csub(C2 a, C2 b) { return c2(sub2(a.re, b.re), sub2(a.im, b.im)); }
+// a * w (CONJ: a * conj w), the same w for both fields
+template <bool CONJ>
+__device__ __forceinline__ C2 cmul(C2 a, float2 w) {
+  const f32x2 c = pk2(w.x, w.x), s = pk2(w.y, w.y), ns = pk2(-w.y, -w.y);
+  return CONJ ? c2(fma2(a.re, c, mul2(a.im, s)), fma2(a.im, c, mul2(a.re, ns)))
+              : c2(fma2(a.re, c, mul2(a.im, ns)), fma2(a.re, s, mul2(a.im, c)));
+}
+// a -+ i b: a - i b (forward) or a + i b (inverse)
 template <bool INV>
-__device__ __forceinline__ float2 mul_mi(float2 a) {
-  return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
+__device__ __forceinline__ C2 add_mi(C2 a, C2 b) {
+  return INV ? c2(sub2(a.re, b.im), add2(a.im, b.re)) : c2(add2(a.re, b.im), sub2(a.im, b.re));
+}
+// multiply by -i (forward) or +i (inverse)
+__device__ __forceinline__ f32x2 neg2(f32x2 a) { return a ^ 0x8000000080000000ull; }
+template <bool INV>
+__device__ __forceinline__ C2 mul_mi(C2 a) {
+  return INV ? c2(neg2(a.im), a.re) : c2(a.im, neg2(a.re));
 }
 
 // ---- compile-time roots of unity ----------------------------------------------------
@@ -66,12 +122,12 @@ __host__ __device__ constexpr double root_angle(int j, int R) {
 
 // a * W_R^J with W_R = exp(-2 pi i / R) (forward) or its conjugate (inverse)
 template <int R, int J, bool INV>
-__device__ __forceinline__ float2 mul_root(float2 a) {
+__device__ __forceinline__ C2 mul_root(C2 a) {
   constexpr int j = ((J % R) + R) % R;
   if constexpr (j == 0) {
     return a;
   } else if constexpr (2 * j == R) {
-    return make_float2(-a.x, -a.y);
+    return c2(neg2(a.re), neg2(a.im));
   } else if constexpr (4 * j == R) {
     return mul_mi<INV>(a);
   } else if constexpr (4 * j == 3 * R) {
@@ -80,76 +136,84 @@ __device__ __forceinline__ float2 mul_root(float2 a) {
     constexpr float c = (float)taylor_cos(root_angle(j, R));
     constexpr float s = (float)taylor_sin(root_angle(j, R));
     constexpr float sy = INV ? s : -s;   // W^j = (c, -s) forward
-    return make_float2(fmaf(a.x, c, -a.y * sy), fmaf(a.x, sy, a.y * c));
+    return cmul<false>(a, make_float2(c, sy));
   }
 }
 
 // ---- prime-size butterflies (in place on v[0..R-1]) ---------------------------------
 template <bool INV>
-__device__ __forceinline__ void bfly2(float2* v) {
-  const float2 a = v[0], b = v[1];
+__device__ __forceinline__ void bfly2(C2* v) {
+  const C2 a = v[0], b = v[1];
   v[0] = cadd(a, b);
   v[1] = csub(a, b);
 }
 
 template <bool INV>
-__device__ __forceinline__ void bfly4(float2* v) {
-  const float2 a = cadd(v[0], v[2]), b = csub(v[0], v[2]), c = cadd(v[1], v[3]);
-  const float2 d = mul_mi<INV>(csub(v[1], v[3]));
+__device__ __forceinline__ void bfly4(C2* v) {
+  const C2 a = cadd(v[0], v[2]), b = csub(v[0], v[2]), c = cadd(v[1], v[3]), d = csub(v[1], v[3]);
   v[0] = cadd(a, c);
   v[2] = csub(a, c);
-  v[1] = cadd(b, d);
-  v[3] = csub(b, d);
+  v[1] = add_mi<INV>(b, d);
+  v[3] = add_mi<!INV>(b, d);
 }
 
 template <bool INV>
-__device__ __forceinline__ void bfly8(float2* v) {
-  float2 e[4] = {v[0], v[2], v[4], v[6]};
-  float2 o[4] = {v[1], v[3], v[5], v[7]};
+__device__ __forceinline__ void bfly8(C2* v) {
+  C2 e[4] = {v[0], v[2], v[4], v[6]};
+  C2 o[4] = {v[1], v[3], v[5], v[7]};
   bfly4<INV>(e);
   bfly4<INV>(o);
   o[1] = mul_root<8, 1, INV>(o[1]);
-  o[2] = mul_root<8, 2, INV>(o[2]);
   o[3] = mul_root<8, 3, INV>(o[3]);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    v[i] = cadd(e[i], o[i]);
-    v[i + 4] = csub(e[i], o[i]);
-  }
+  v[0] = cadd(e[0], o[0]);
+  v[4] = csub(e[0], o[0]);
+  v[1] = cadd(e[1], o[1]);
+  v[5] = csub(e[1], o[1]);
+  v[2] = add_mi<INV>(e[2], o[2]);
+  v[6] = add_mi<!INV>(e[2], o[2]);
+  v[3] = cadd(e[3], o[3]);
+  v[7] = csub(e[3], o[3]);
 }
 
 template <bool INV>
-__device__ __forceinline__ void bfly3(float2* v) {
-  const float s = 0.86602540378443865f;   // sin(2 pi / 3)
-  const float2 t = cadd(v[1], v[2]);
-  const float2 d = csub(v[1], v[2]);
-  const float2 a = make_float2(fmaf(-0.5f, t.x, v[0].x), fmaf(-0.5f, t.y, v[0].y));
-  const float2 b = mul_mi<INV>(make_float2(s * d.x, s * d.y));
+__device__ __forceinline__ void bfly3(C2* v) {
+  const f32x2 s = pk2(0.86602540378443865f, 0.86602540378443865f);   // sin(2 pi / 3)
+  const f32x2 h = pk2(-0.5f, -0.5f);
+  const C2 t = cadd(v[1], v[2]);
+  const C2 d = csub(v[1], v[2]);
+  const C2 a = c2(fma2(h, t.re, v[0].re), fma2(h, t.im, v[0].im));
+  const f32x2 ns = neg2(s);
   v[0] = cadd(v[0], t);
-  v[1] = cadd(a, b);
-  v[2] = csub(a, b);
+  // a -+ i s d
+  const C2 m = c2(fma2(s, d.im, a.re), fma2(ns, d.re, a.im));   // a - i s d
+  const C2 p = c2(fma2(ns, d.im, a.re), fma2(s, d.re, a.im));   // a + i s d
+  v[1] = INV ? p : m;
+  v[2] = INV ? m : p;
 }
 
 template <bool INV>
-__device__ __forceinline__ void bfly5(float2* v) {
-  const float c1 = 0.30901699437494742f, c2 = -0.80901699437494742f;   // cos(2pi/5), cos(4pi/5)
-  const float s1 = 0.95105651629515357f, s2 = 0.58778525229247313f;    // sin(2pi/5), sin(4pi/5)
-  const float2 t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
-  const float2 d1 = csub(v[1], v[4]), d2 = csub(v[2], v[3]);
-  const float2 x0 = v[0];
-  const float2 a1 = make_float2(fmaf(c2, t2.x, fmaf(c1, t1.x, x0.x)), fmaf(c2, t2.y, fmaf(c1, t1.y, x0.y)));
-  const float2 a2 = make_float2(fmaf(c1, t2.x, fmaf(c2, t1.x, x0.x)), fmaf(c1, t2.y, fmaf(c2, t1.y, x0.y)));
-  const float2 b1 = mul_mi<INV>(make_float2(fmaf(s1, d1.x, s2 * d2.x), fmaf(s1, d1.y, s2 * d2.y)));
-  const float2 b2 = mul_mi<INV>(make_float2(fmaf(s2, d1.x, -s1 * d2.x), fmaf(s2, d1.y, -s1 * d2.y)));
+__device__ __forceinline__ void bfly5(C2* v) {
+  const f32x2 c1 = pk2(0.30901699437494742f, 0.30901699437494742f);     // cos(2pi/5)
+  const f32x2 k2 = pk2(-0.80901699437494742f, -0.80901699437494742f);   // cos(4pi/5)
+  const f32x2 s1 = pk2(0.95105651629515357f, 0.95105651629515357f);     // sin(2pi/5)
+  const f32x2 s2 = pk2(0.58778525229247313f, 0.58778525229247313f);     // sin(4pi/5)
+  const C2 t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
+  const C2 d1 = csub(v[1], v[4]), d2 = csub(v[2], v[3]);
+  const C2 x0 = v[0];
+  const C2 a1 = c2(fma2(k2, t2.re, fma2(c1, t1.re, x0.re)), fma2(k2, t2.im, fma2(c1, t1.im, x0.im)));
+  const C2 a2 = c2(fma2(c1, t2.re, fma2(k2, t1.re, x0.re)), fma2(c1, t2.im, fma2(k2, t1.im, x0.im)));
+  const f32x2 ns1 = neg2(s1);
+  const C2 b1 = c2(fma2(s1, d1.re, mul2(s2, d2.re)), fma2(s1, d1.im, mul2(s2, d2.im)));
+  const C2 b2 = c2(fma2(s2, d1.re, mul2(ns1, d2.re)), fma2(s2, d1.im, mul2(ns1, d2.im)));
   v[0] = cadd(x0, cadd(t1, t2));
-  v[1] = cadd(a1, b1);
-  v[4] = csub(a1, b1);
-  v[2] = cadd(a2, b2);
-  v[3] = csub(a2, b2);
+  v[1] = add_mi<INV>(a1, b1);
+  v[4] = add_mi<!INV>(a1, b1);
+  v[2] = add_mi<INV>(a2, b2);
+  v[3] = add_mi<!INV>(a2, b2);
 }
 
 template <int R, bool INV>
-__device__ __forceinline__ void bfly_prime(float2* v) {
+__device__ __forceinline__ void bfly_prime(C2* v) {
   if constexpr (R == 2) bfly2<INV>(v);
   else if constexpr (R == 3) bfly3<INV>(v);
   else if constexpr (R == 4) bfly4<INV>(v);
@@ -159,8 +223,8 @@ __device__ __forceinline__ void bfly_prime(float2* v) {
 
 // R-point DFT of the registers v[O + S i], i < R
 template <int R, int O, int S, bool INV>
-__device__ __forceinline__ void dft_at(float2* v) {
-  float2 t[R];
+__device__ __forceinline__ void dft_at(C2* v) {
+  C2 t[R];
 #pragma unroll
   for (int i = 0; i < R; ++i) t[i] = v[O + S * i];
   bfly_prime<R, INV>(t);
@@ -172,21 +236,21 @@ __device__ __forceinline__ void dft_at(float2* v) {
 //   X[k] = sum_{n2} W_R2^{n2 k2} W_R^{n2 k1} sum_{n1} W_R1^{n1 k1} x[R2 n1 + n2].
 // After the call X[k1 + R1 k2] is in v[R2 k1 + k2].
 template <int R1, int R2, bool INV, int... I>
-__device__ __forceinline__ void composite_level1(float2* v, std::integer_sequence<int, I...>) {
+__device__ __forceinline__ void composite_level1(C2* v, std::integer_sequence<int, I...>) {
   (dft_at<R1, I, R2, INV>(v), ...);
 }
 template <int R1, int R2, bool INV, int... I>
-__device__ __forceinline__ void composite_twiddle(float2* v, std::integer_sequence<int, I...>) {
+__device__ __forceinline__ void composite_twiddle(C2* v, std::integer_sequence<int, I...>) {
   // element I = R2 k1 + n2 takes W_R^{n2 k1}
   ((v[I] = mul_root<R1 * R2, (I % R2) * (I / R2), INV>(v[I])), ...);
 }
 template <int R1, int R2, bool INV, int... I>
-__device__ __forceinline__ void composite_level2(float2* v, std::integer_sequence<int, I...>) {
+__device__ __forceinline__ void composite_level2(C2* v, std::integer_sequence<int, I...>) {
   (dft_at<R2, R2 * I, 1, INV>(v), ...);
 }
 
 template <int R1, int R2, bool INV>
-__device__ __forceinline__ void bfly_composite(float2* v) {
+__device__ __forceinline__ void bfly_composite(C2* v) {
   composite_level1<R1, R2, INV>(v, std::make_integer_sequence<int, R2>{});
   composite_twiddle<R1, R2, INV>(v, std::make_integer_sequence<int, R1 * R2>{});
   composite_level2<R1, R2, INV>(v, std::make_integer_sequence<int, R1>{});
@@ -205,7 +269,7 @@ template <> struct Radix<15> { static constexpr int R1 = 3, R2 = 5; };
 template <> struct Radix<16> { static constexpr int R1 = 4, R2 = 4; };
 
 template <int R, bool INV>
-__device__ __forceinline__ void butterfly(float2* v) {
+__device__ __forceinline__ void butterfly(C2* v) {
   if constexpr (Radix<R>::R1 == 1) bfly_prime<R, INV>(v);
   else bfly_composite<Radix<R>::R1, Radix<R>::R2, INV>(v);
 }
@@ -213,11 +277,6 @@ template <int R>
 __host__ __device__ constexpr int out_reg(int k) {
   return Radix<R>::R1 == 1 ? k : Radix<R>::R2 * (k % Radix<R>::R1) + k / Radix<R>::R1;
 }
-
-// Threads of an FFT CTA (launched with at least three CTAs per SM in mind: <= 80
-// registers, enough for the radix-16 butterfly without spills); kFftCap (the most elements,
-// sequences x length, one CTA transforms) is declared with the grid types.
-constexpr int kFftThreads = 256;
 
 // stride of consecutive sequences in the CTA's buffers
 __host__ __device__ constexpr int seq_ld(int N) { return N + 1; }
@@ -229,7 +288,7 @@ __device__ __forceinline__ int fast_div(int a, uint32_t mul) {
 }
 
 template <int R, bool INV>
-__device__ __forceinline__ void stockham_stage(const float2* __restrict__ src, float2* __restrict__ dst,
+__device__ __forceinline__ void stockham_stage(const C2* __restrict__ src, C2* __restrict__ dst,
                                                const float2* __restrict__ tws, int N, int Ns, int nseq,
                                                uint32_t ns_mul, uint32_t nr_mul) {
   const int NR = N / R;
@@ -240,19 +299,18 @@ __device__ __forceinline__ void stockham_stage(const float2* __restrict__ src, f
     const int j = idx - q * NR;
     const int jd = fast_div(j, ns_mul);
     const int k = j - jd * Ns;
-    const float2* s = src + q * ld + j;
-    float2 v[R];
+    const C2* s = src + q * ld + j;
+    C2 v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = s[r * NR];
     if (Ns > 1) {   // the first stage's twiddles are all 1
 #pragma unroll
       for (int r = 1; r < R; ++r) {
-        const float2 w = tws[(r - 1) * Ns + k];
-        v[r] = INV ? cmulc(v[r], w) : cmul(v[r], w);
+        v[r] = cmul<INV>(v[r], __ldg(tws + (r - 1) * Ns + k));
       }
     }
     butterfly<R, INV>(v);
-    float2* d = dst + q * ld + jd * Ns * R + k;
+    C2* d = dst + q * ld + jd * Ns * R + k;
 #pragma unroll
     for (int r = 0; r < R; ++r) d[r * Ns] = v[out_reg<R>(r)];
   }
@@ -263,7 +321,7 @@ __device__ __forceinline__ void stockham_stage(const float2* __restrict__ src, f
 // roots W_R^e from the plan's table; O(R) work per output.  Tasks run r-major over the
 // butterflies, so consecutive threads read consecutive inputs.
 template <bool INV>
-__device__ __noinline__ void stockham_stage_generic(const float2* __restrict__ src, float2* __restrict__ dst,
+__device__ __noinline__ void stockham_stage_generic(const C2* __restrict__ src, C2* __restrict__ dst,
                                                     const float2* __restrict__ tws, const float2* __restrict__ roots,
                                                     int N, int R, int Ns, int nseq, uint32_t ns_mul,
                                                     uint32_t nr_mul) {
@@ -276,23 +334,18 @@ __device__ __noinline__ void stockham_stage_generic(const float2* __restrict__ s
     const int q = qr / R, r = qr - q * R;
     const int jd = fast_div(j, ns_mul);
     const int k = j - jd * Ns;
-    const float2* s = src + q * ld + j;
-    float re = 0.f, im = 0.f;
+    const C2* s = src + q * ld + j;
+    C2 sum = c2(0ull, 0ull);
     int e = 0;   // r t mod R
+#pragma unroll 4
     for (int t = 0; t < R; ++t) {
-      float2 v = s[t * NR];
-      if (Ns > 1 && t > 0) {
-        const float2 w = tws[(t - 1) * Ns + k];
-        v = INV ? cmulc(v, w) : cmul(v, w);
-      }
-      const float2 w = roots[e];
-      v = INV ? cmulc(v, w) : cmul(v, w);
-      re += v.x;
-      im += v.y;
+      C2 v = s[t * NR];
+      if (Ns > 1 && t > 0) v = cmul<INV>(v, __ldg(tws + (t - 1) * Ns + k));
+      sum = cadd(sum, cmul<INV>(v, __ldg(roots + e)));
       e += r;
       if (e >= R) e -= R;
     }
-    dst[q * ld + jd * Ns * R + k + r * Ns] = make_float2(re, im);
+    dst[q * ld + jd * Ns * R + k + r * Ns] = sum;
   }
 }
 
@@ -301,7 +354,7 @@ __device__ __noinline__ void stockham_stage_generic(const float2* __restrict__ s
 // the buffer holding the result.  All threads of the block must call it; it
 // synchronises after every stage.
 template <bool INV>
-__device__ float2* fft_smem(float2* a, float2* b, const float2* tw, const FftPlan& pl, int nseq) {
+__device__ C2* fft_smem(C2* a, C2* b, const float2* tw, const FftPlan& pl, int nseq) {
   int Ns = 1;
   for (int s = 0; s < pl.nst; ++s) {
     const int R = pl.R[s];
@@ -324,7 +377,7 @@ __device__ float2* fft_smem(float2* a, float2* b, const float2* tw, const FftPla
         break;
     }
     __syncthreads();
-    float2* t = a;
+    C2* t = a;
     a = b;
     b = t;
     Ns *= R;
@@ -343,7 +396,7 @@ struct CtPlan {
 using RuntimePlan = CtPlan<0>;
 
 template <int R, bool INV, int N, int NS, int TWOFF>
-__device__ __forceinline__ void stockham_stage_ct(const float2* __restrict__ src, float2* __restrict__ dst,
+__device__ __forceinline__ void stockham_stage_ct(const C2* __restrict__ src, C2* __restrict__ dst,
                                                   const float2* __restrict__ tw, int nseq) {
   constexpr int NR = N / R, LD = N + 1;
   const int total = nseq * NR;
@@ -352,17 +405,17 @@ __device__ __forceinline__ void stockham_stage_ct(const float2* __restrict__ src
     const int j = idx - q * NR;
     const int jd = j / NS;
     const int k = j - jd * NS;
-    const float2* s = src + q * LD + j;
-    float2 v[R];
+    const C2* s = src + q * LD + j;
+    C2 v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = s[r * NR];
     if constexpr (NS > 1) {
       const float2* tws = tw + TWOFF + k;
 #pragma unroll
-      for (int r = 1; r < R; ++r) v[r] = INV ? cmulc(v[r], tws[(r - 1) * NS]) : cmul(v[r], tws[(r - 1) * NS]);
+      for (int r = 1; r < R; ++r) v[r] = cmul<INV>(v[r], __ldg(tws + (r - 1) * NS));
     }
     butterfly<R, INV>(v);
-    float2* d = dst + q * LD + jd * NS * R + k;
+    C2* d = dst + q * LD + jd * NS * R + k;
 #pragma unroll
     for (int r = 0; r < R; ++r) d[r * NS] = v[out_reg<R>(r)];
   }
@@ -371,7 +424,7 @@ __device__ __forceinline__ void stockham_stage_ct(const float2* __restrict__ src
 // three-stage compile-time plan; the twiddle table layout is the runtime plan's (stage s at
 // sum over earlier stages s' >= 1 of (R_s' - 1) Ns_s')
 template <bool INV, class PL>
-__device__ float2* fft_smem_ct(float2* a, float2* b, const float2* tw, int nseq) {
+__device__ C2* fft_smem_ct(C2* a, C2* b, const float2* tw, int nseq) {
   constexpr int N = PL::N, R0 = PL::R0, R1 = PL::R1, R2 = PL::R2;
   static_assert(R0 * R1 * R2 == N, "plan radices must multiply to N");
   stockham_stage_ct<R0, INV, N, 1, 0>(a, b, tw, nseq);
@@ -384,7 +437,7 @@ __device__ float2* fft_smem_ct(float2* a, float2* b, const float2* tw, int nseq)
 }
 
 template <bool INV, class PL>
-__device__ __forceinline__ float2* fft_smem_plan(float2* a, float2* b, const float2* tw, const FftPlan& pl,
+__device__ __forceinline__ C2* fft_smem_plan(C2* a, C2* b, const float2* tw, const FftPlan& pl,
                                                  int nseq) {
   if constexpr (PL::N == 0) return fft_smem<INV>(a, b, tw, pl, nseq);
   else return fft_smem_ct<INV, PL>(a, b, tw, nseq);

@@ -10,13 +10,13 @@
 //
 // A ring's length n_i is 4k, not always a product of 2, 3 and 5, and the band limit
 // (3 nside - 1 by default) exceeds n_i / 2 on the polar rings.  The ring transforms run the
-// shared-memory Stockham FFT of the rectangular grids on the rings whose length factors into
-// 2, 3 and 5 (all equatorial-belt rings at the usual nside = 2^k, and many polar rings) and a
-// direct DFT in shared memory on the others, with the aliasing made explicit:
+// shared-memory Stockham FFT of the rectangular grids (every length has a plan; prime factors
+// above 5 are generic stages) with the aliasing made explicit:
 //   forward  F_m = e^{-i m phi0} D_{m mod n},   D_k = sum_j f_j e^{-2 pi i k j / n}
 //   inverse  f_j = sum_k Z_k e^{2 pi i k j / n},
 //            Z_k = sum_{m = -lmax..lmax, m = k mod n} e^{i m phi0} G_m,   G_{-m} = conj G_m.
-// Two rings (j north, J south) travel as one complex sequence, as on the other grids.
+// Two rings (j north, J south) travel as one complex sequence and two fields as one packed
+// element, as on the other grids.
 #include <cmath>
 #include <vector>
 
@@ -26,97 +26,39 @@
 namespace shot {
 namespace {
 
-constexpr int kHpThreads = 256;
-
-__device__ __forceinline__ float2 c_mul(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
-}
+// One ring pair of two fields a CTA.  The chain of one CTA bounds these kernels (a solve's rings
+// are short, and all CTAs of nside 64 and 8 fields are resident at once): 128 threads take most
+// stages in one step, the generic stage of a prime factor p in p steps.
+constexpr int kHpThreads = 128;
 
 // e^{i pi r / d} for an integer r reduced modulo 2d (exact argument reduction)
-__device__ __forceinline__ float2 half_turns(long long r, int d) {
-  long long rr = r % (2LL * d);
-  if (rr < 0) rr += 2LL * d;
+__device__ __forceinline__ float2 half_turns(int r, int d) {
   float s, c;
-  sincospif((float)rr / (float)d, &s, &c);
+  sincospif((float)(r % (2 * d)) / (float)d, &s, &c);
   return make_float2(c, s);
 }
 
-// ring constants: twiddles tw[t] = e^{-2 pi i t / n} (direct DFT rings; tw may be null);
-// phases ph[m] = e^{i m phi0}
-__device__ __forceinline__ void ring_tables(float2* tw, float2* ph, int n, int2 phase, int lmax) {
-  if (tw)
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
-    const float2 e = half_turns(2LL * t, n);
-    tw[t] = make_float2(e.x, -e.y);
-  }
-  if (ph)
-    for (int m = threadIdx.x; m <= lmax; m += blockDim.x) ph[m] = half_turns((long long)m * phase.x, phase.y);
-}
-
-// D[q][k] = sum_t zin[q][t] tw[k t mod n] (forward, conj = false) or with conj(tw) (inverse);
-// sequences at a stride of ld
-template <bool INV>
-__device__ __forceinline__ void direct_dft(const float2* zin, float2* zout, const float2* tw, int n, int ld,
-                                           int nseq) {
-  for (int idx = threadIdx.x; idx < nseq * n; idx += blockDim.x) {
-    const int q = idx / n, k = idx - q * n;
-    const float2* s = zin + q * ld;
-    float re = 0.f, im = 0.f;
-    int e = 0;
-    for (int t = 0; t < n; ++t) {
-      const float2 w = tw[e];
-      const float2 v = s[t];
-      const float wy = INV ? -w.y : w.y;
-      re = fmaf(v.x, w.x, fmaf(-v.y, wy, re));
-      im = fmaf(v.x, wy, fmaf(v.y, w.x, im));
-      e += k;
-      if (e >= n) e -= n;
-    }
-    zout[q * ld + k] = make_float2(re, im);
-  }
-}
-
-// The ring transform of nseq sequences (stride seq_ld(n)) in a, b as scratch: the FFT when
-// the ring has a plan (pi >= 0), else the direct DFT with the twiddles tw.  Returns the buffer
-// holding the result.  All threads call it; it synchronises before returning.
-template <bool INV>
-__device__ __forceinline__ float2* ring_transform(float2* a, float2* b, const float2* tw, int n, int nseq, int pi,
-                                                  const FftPlan* __restrict__ plans,
-                                                  const float2* __restrict__ tw_all, const int* __restrict__ tw_base) {
-  if (pi >= 0) {
-    const FftPlan pl = plans[pi];
-    return fft_smem<INV>(a, b, tw_all + tw_base[pi], pl, nseq);
-  }
-  direct_dft<INV>(a, b, tw, n, seq_ld(n), nseq);
-  __syncthreads();
-  return b;
-}
-
 // from the transformed ring pair D: S = a (F_N + F_S), D = a (F_N - F_S) for m <= lmax into X
-template <int FG>
-__device__ __forceinline__ void hp_unpack_store(const float2* D, const float2* ph, int n, int nfg, int f0, int lmax,
-                                                int nh, int jh, float aj, float* __restrict__ X, int ldc) {
-  const int ld = seq_ld(n);
-  for (int idx = threadIdx.x; idx < (lmax + 1) * FG; idx += blockDim.x) {
-    const int m = idx / FG, q = idx - m * FG;
-    if (q >= nfg) continue;
-    const int k = m % n, kk = (n - k) % n;
-    const float2 zm = D[q * ld + k], zn = D[q * ld + kk];
-    float2 FN = make_float2(0.5f * (zm.x + zn.x), 0.5f * (zm.y - zn.y));
-    float2 FS = make_float2(0.5f * (zm.y + zn.y), -0.5f * (zm.x - zn.x));
-    const float2 e = make_float2(ph[m].x, -ph[m].y);   // e^{-i m phi0}
-    FN = c_mul(FN, e);
-    FS = c_mul(FS, e);
-    const int f = f0 + q;
-    *reinterpret_cast<float2*>(X + ((size_t)(2 * m) * nh + jh) * ldc + 2 * f) =
-        make_float2(aj * (FN.x + FS.x), aj * (FN.y + FS.y));
-    *reinterpret_cast<float2*>(X + ((size_t)(2 * m + 1) * nh + jh) * ldc + 2 * f) =
-        make_float2(aj * (FN.x - FS.x), aj * (FN.y - FS.y));
+// (sc = a / 2 per field, with the field's factor), each order turned by e^{-i m phi0}
+__device__ __forceinline__ void hp_fold_store(const C2* D, int n, int2 phase, int f0, int lmax, int nh, int jh, f32x2 sc,
+                                              float* __restrict__ X, int ldc) {
+  float* x = X + (size_t)jh * ldc + 2 * f0;
+  const size_t row = (size_t)nh * ldc;
+  for (int m = threadIdx.x; m <= lmax; m += kHpThreads) {
+    const int k = m % n;
+    const C2 zm = D[k], zn = D[k ? n - k : 0];
+    const float2 e = half_turns(m * phase.x, phase.y);
+    // 2 F_N = z_k + conj z_{n-k}, 2 F_S = (z_k - conj z_{n-k}) / i, both times e^{-i m phi0}
+    const C2 FN = cmul<true>(c2(add2(zm.re, zn.re), sub2(zm.im, zn.im)), e);
+    const C2 FS = cmul<true>(c2(add2(zm.im, zn.im), sub2(zn.re, zm.re)), e);
+    const float2 Sr = unpk2(mul2(sc, add2(FN.re, FS.re))), Si = unpk2(mul2(sc, add2(FN.im, FS.im)));
+    const float2 Dr = unpk2(mul2(sc, sub2(FN.re, FS.re))), Di = unpk2(mul2(sc, sub2(FN.im, FS.im)));
+    *reinterpret_cast<float4*>(x + (size_t)(2 * m) * row) = make_float4(Sr.x, Si.x, Sr.y, Si.y);
+    *reinterpret_cast<float4*>(x + (size_t)(2 * m + 1) * row) = make_float4(Dr.x, Di.x, Dr.y, Di.y);
   }
 }
 
-template <int FG>
-__global__ void __launch_bounds__(kHpThreads) k_hp_fwd(const float* __restrict__ in, int nf, size_t npix,
+__global__ void __launch_bounds__(kHpThreads, 4) k_hp_fwd(const float* __restrict__ in, int nf, size_t npix,
                                                        const int* __restrict__ rlen,
                                                        const long long* __restrict__ roff,
                                                        const int2* __restrict__ rphase, int nrings, int lmax, int nh,
@@ -125,31 +67,27 @@ __global__ void __launch_bounds__(kHpThreads) k_hp_fwd(const float* __restrict__
                                                        const float2* __restrict__ tw_all,
                                                        const int* __restrict__ tw_base,
                                                        const ProbState* __restrict__ ps) {
-  extern __shared__ __align__(16) float2 sm[];
-  const int jh = blockIdx.y, f0 = blockIdx.x * FG;
-  const int nfg = min(FG, nf - f0);
+  extern __shared__ __align__(16) C2 sm[];
+  const int jh = blockIdx.y, f0 = blockIdx.x * 2;
   const int j = jh, J = nrings - 1 - jh;
-  const int n = rlen[j], ld = seq_ld(n);
-  const int pi = rplan[j];
-  float2* zb = sm;               // [FG][ld]
-  float2* db = zb + FG * ld;     // [FG][ld]
-  float2* tw = db + FG * ld;     // [n] (direct DFT rings)
-  float2* ph = tw + n;           // [lmax + 1]
-  ring_tables(pi >= 0 ? nullptr : tw, ph, n, rphase[j], lmax);
-  for (int q = 0; q < nfg; ++q) {
-    const float* fj = in + (size_t)(f0 + q) * npix + roff[j];
-    const float* fJ = in + (size_t)(f0 + q) * npix + roff[J];
-    const float sc = ps ? (float)ps[f0 + q].beta : 1.f;   // per-field factor (gradient sweeps)
-    for (int k = threadIdx.x; k < n; k += blockDim.x)
-      zb[q * ld + k] = make_float2(sc * fj[k], J != j ? sc * fJ[k] : 0.f);
-  }
+  const bool second = f0 + 1 < nf, two = J != j;
+  const int n = rlen[j], pi = rplan[j];
+  C2* zb = sm;
+  C2* db = zb + seq_ld(n);
+  const float* fj = in + (size_t)f0 * npix + roff[j];
+  const float* fJ = in + (size_t)f0 * npix + roff[J];
+  for (int k = threadIdx.x; k < n; k += kHpThreads)
+    reinterpret_cast<float4*>(zb)[k] =
+        make_float4(fj[k], second ? fj[npix + k] : 0.f, two ? fJ[k] : 0.f, (two && second) ? fJ[npix + k] : 0.f);
+  // per-field factor (gradient sweeps)
+  const float s0 = 0.5f * area * (ps ? (float)ps[f0].beta : 1.f);
+  const float s1 = 0.5f * area * (ps && second ? (float)ps[f0 + 1].beta : 1.f);
   __syncthreads();
-  const float2* D = ring_transform<false>(zb, db, tw, n, nfg, pi, plans, tw_all, tw_base);
-  hp_unpack_store<FG>(D, ph, n, nfg, f0, lmax, nh, jh, area, X, ldc);
+  const C2* D = fft_smem<false>(zb, db, tw_all + tw_base[pi], plans[pi], 1);
+  hp_fold_store(D, n, rphase[j], f0, lmax, nh, jh, pk2(s0, s1), X, ldc);
 }
 
-template <int FG>
-__global__ void __launch_bounds__(kHpThreads) k_hp_idft(const float* __restrict__ Y, int ldc, int nf, size_t npix,
+__global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restrict__ Y, int ldc, int nf, size_t npix,
                                                         const int* __restrict__ rlen,
                                                         const long long* __restrict__ roff,
                                                         const int2* __restrict__ rphase, int nrings, int lmax,
@@ -158,124 +96,82 @@ __global__ void __launch_bounds__(kHpThreads) k_hp_idft(const float* __restrict_
                                                         const FftPlan* __restrict__ plans,
                                                         const float2* __restrict__ tw_all,
                                                         const int* __restrict__ tw_base) {
-  extern __shared__ __align__(16) float2 sm[];
-  __shared__ float red[kHpThreads / 32][FG * NPART];
-  __shared__ EpiField fi[FG];
-  const int jh = blockIdx.y, f0 = blockIdx.x * FG;
-  const int nfg = min(FG, nf - f0);
+  extern __shared__ __align__(16) C2 sm[];
+  __shared__ float red[kHpThreads / 32][2 * NPART];
+  __shared__ EpiField fi[2];
+  const int jh = blockIdx.y, f0 = blockIdx.x * 2;
+  const int nfg = min(2, nf - f0);
   const int j = jh, J = nrings - 1 - jh;
-  const int n = rlen[j], ld = seq_ld(n);
-  const int pi = rplan[j];
-  const int nm = lmax + 1;
-  float2* za = sm;               // [FG][ld]  spectra Z
-  float2* zb = za + FG * ld;     // [FG][ld]
-  float2* tw = zb + FG * ld;     // [n] (direct DFT rings)
-  float2* ph = tw + n;           // [lmax + 1]
-  float2* gn = ph + nm;          // [lmax + 1][FG]  G_N = E + O
-  float2* gs = gn + nm * FG;     // [lmax + 1][FG]  G_S = E - O
-  epi_fields_load<FG>(ep, f0, nfg, fi);
-  ring_tables(pi >= 0 ? nullptr : tw, ph, n, rphase[j], lmax);
-  for (int idx = threadIdx.x; idx < nm * FG; idx += blockDim.x) {
-    const int m = idx / FG, q = idx - m * FG;
-    float2 E = make_float2(0.f, 0.f), O = make_float2(0.f, 0.f);
-    if (q < nfg) {
-      E = *reinterpret_cast<const float2*>(Y + ((size_t)(2 * m) * nh + jh) * ldc + 2 * (f0 + q));
-      if (m < lmax) O = *reinterpret_cast<const float2*>(Y + ((size_t)(2 * m + 1) * nh + jh) * ldc + 2 * (f0 + q));
-    }
-    gn[idx] = make_float2(E.x + O.x, E.y + O.y);
-    gs[idx] = make_float2(E.x - O.x, E.y - O.y);
-  }
-  __syncthreads();
-  // Z_k: orders m >= 0 with m = k (mod n) and m = -m' (m' >= 1) with m' = n - k (mod n)
-  for (int idx = threadIdx.x; idx < nfg * n; idx += blockDim.x) {
-    const int q = idx / n, k = idx - q * n;
-    float re = 0.f, im = 0.f;
-    for (int m = k; m <= lmax; m += n) {   // e^{i m phi0} (G_N + i G_S)
-      const float2 a = gn[m * FG + q], b = gs[m * FG + q];
-      const float2 t = c_mul(ph[m], make_float2(a.x - b.y, a.y + b.x));
-      re += t.x;
-      im += t.y;
-    }
-    for (int mp = (k == 0) ? n : n - k; mp <= lmax; mp += n) {   // e^{-i m' phi0} (conj G_N + i conj G_S)
-      const float2 a = gn[mp * FG + q], b = gs[mp * FG + q];
-      const float2 t = c_mul(make_float2(ph[mp].x, -ph[mp].y), make_float2(a.x + b.y, b.x - a.y));
-      re += t.x;
-      im += t.y;
-    }
-    za[q * ld + k] = make_float2(re, im);
-  }
-  __syncthreads();
-  float2* z = ring_transform<true>(za, zb, tw, n, nfg, pi, plans, tw_all, tw_base);   // K v on the ring pair
-  float2* other = (z == za) ? zb : za;   // receives the new scaling
   const bool two = (J != j);
-  ring_pair_epilogue<FG, kHpThreads>(z, other, ld, n, nfg, f0, npix, (size_t)roff[j], (size_t)roff[J], two, area,
-                                     nh, jh, ep, red, fi);
-  if (ep.mode == EPI_PLAIN) return;
+  const int n = rlen[j], ld = seq_ld(n), pi = rplan[j];
+  const size_t rj = (size_t)roff[j], rJ = (size_t)roff[J];
+  const int2 phase = rphase[j];
+  C2* za = sm;          // spectra Z
+  C2* zb = za + ld;
+  epi_fields_load<2>(ep, f0, nfg, fi);
+  // Z_k = A_k + B_{n-k}: A_r sums e^{i m phi0} (G_N + i G_S) over the orders m >= 0 of residue r
+  // modulo n, B_r sums e^{-i m phi0} (conj G_N + i conj G_S) over the orders m >= 1.  A thread owns
+  // a residue, so every spectra row is read once, straight from global memory.
+  {
+    const float* y = Y + (size_t)jh * ldc + 2 * f0;
+    const size_t row = (size_t)nh * ldc;
+    for (int r = threadIdx.x; r < n; r += kHpThreads) {
+      C2 A = c2(0ull, 0ull), B = A;
+#pragma unroll 4
+      for (int m = r; m <= lmax; m += n) {
+        const float4 e = *reinterpret_cast<const float4*>(y + (size_t)(2 * m) * row);
+        const float4 o = m < lmax ? *reinterpret_cast<const float4*>(y + (size_t)(2 * m + 1) * row)
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+        const C2 E = c2(pk2(e.x, e.z), pk2(e.y, e.w)), O = c2(pk2(o.x, o.z), pk2(o.y, o.w));
+        const C2 GN = cadd(E, O), GS = csub(E, O);
+        const float2 w = half_turns(m * phase.x, phase.y);
+        A = cadd(A, cmul<false>(c2(sub2(GN.re, GS.im), add2(GN.im, GS.re)), w));
+        if (m > 0) B = cadd(B, cmul<true>(c2(add2(GN.re, GS.im), sub2(GS.re, GN.im)), w));
+      }
+      za[r] = A;
+      zb[r] = B;
+    }
+  }
+  __syncthreads();
+  epi_prefetch_marginals<2>(ep, fi, nfg, rj, rJ, two, n, f0, npix);
+  for (int k = threadIdx.x; k < n; k += kHpThreads) za[k] = cadd(za[k], zb[k ? n - k : 0]);
+  __syncthreads();
+  const float2* tw = tw_all + tw_base[pi];
+  C2* z = fft_smem<true>(za, zb, tw, plans[pi], 1);   // K v on the ring pair
+  C2* other = (z == za) ? zb : za;   // receives the new scaling
+  ring_pair_epilogue<1, kHpThreads>(z, other, ld, n, nf, f0, npix, rj, rJ, two, area, nh, jh, ep, red, fi);
   if ((ep.mode == EPI_UPDATE || ep.mode == EPI_SYM) && ep.xout) {   // transform the new scaling
     __syncthreads();
-    const float2* D = ring_transform<false>(other, z, tw, n, nfg, pi, plans, tw_all, tw_base);
-    hp_unpack_store<FG>(D, ph, n, nfg, f0, lmax, nh, jh, area, ep.xout, ldc);
+    const C2* D = fft_smem<false>(other, z, tw, plans[pi], 1);
+    hp_fold_store(D, n, phase, f0, lmax, nh, jh, pk2(0.5f * area, 0.5f * area), ep.xout, ldc);
   }
-}
-
-size_t hp_fwd_smem(int fg, int n, int lmax) {
-  return (size_t)(2 * fg * seq_ld(n) + n + lmax + 1) * sizeof(float2);
-}
-size_t hp_idft_smem(int fg, int n, int lmax) {
-  return (size_t)(2 * fg * seq_ld(n) + n + (lmax + 1) * (1 + 2 * fg)) * sizeof(float2);
-}
-
-int hp_pick_fg(const Grid& g, int nf, bool inverse) {
-  const int n = g.nlon;   // the longest ring
-  int fg = 4;
-  while (fg > 1 && (fg > nf || (inverse ? hp_idft_smem(fg, n, g.lmax) : hp_fwd_smem(fg, n, g.lmax)) > 100 * 1024))
-    fg >>= 1;
-  return fg;
-}
-
-template <int FG>
-int hp_fwd_t(const Grid& g, const float* in, int nf, float* X, int ldc, cudaStream_t st, const ProbState* ps) {
-  const size_t smem = hp_fwd_smem(FG, g.nlon, g.lmax);
-  SHOT_CUDA(cudaFuncSetAttribute(k_hp_fwd<FG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  ProfScope prof(PK_DFT, st);
-  count_launch();
-  k_hp_fwd<FG><<<dim3((nf + FG - 1) / FG, g.nh), kHpThreads, smem, st>>>(
-      in, nf, g.npix, g.ring_len_d, g.ring_off_d, g.ring_phase_d, g.nlat, g.lmax, g.nh, (float)g.a_ring[0], X, ldc,
-      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d, ps);
-  SHOT_CUDA(cudaGetLastError());
-  return SHOT_OK;
-}
-
-template <int FG>
-int hp_idft_t(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st) {
-  const size_t smem = hp_idft_smem(FG, g.nlon, g.lmax);
-  SHOT_CUDA(cudaFuncSetAttribute(k_hp_idft<FG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  ProfScope prof(ep.mode == EPI_CHECK || ep.mode == EPI_FINAL ? PK_CHECK : PK_IDFT, st);
-  count_launch();
-  k_hp_idft<FG><<<dim3((nf + FG - 1) / FG, g.nh), kHpThreads, smem, st>>>(
-      Y, ldc, nf, g.npix, g.ring_len_d, g.ring_off_d, g.ring_phase_d, g.nlat, g.lmax, g.nh, (float)g.a_ring[0], ep,
-      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d);
-  SHOT_CUDA(cudaGetLastError());
-  return SHOT_OK;
 }
 
 }  // namespace
 
 int launch_hp_dft_fwd(const Grid& g, const float* in, int nf, float* X, int ldc, cudaStream_t st,
                       const ProbState* ps) {
-  switch (hp_pick_fg(g, nf, false)) {
-    case 4: return hp_fwd_t<4>(g, in, nf, X, ldc, st, ps);
-    case 2: return hp_fwd_t<2>(g, in, nf, X, ldc, st, ps);
-    default: return hp_fwd_t<1>(g, in, nf, X, ldc, st, ps);
-  }
+  const size_t smem = (size_t)2 * seq_ld(g.nlon) * sizeof(C2);   // nlon: the longest ring
+  SHOT_CUDA(cudaFuncSetAttribute(k_hp_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  ProfScope prof(PK_DFT, st);
+  count_launch();
+  k_hp_fwd<<<dim3((nf + 1) / 2, g.nh), kHpThreads, smem, st>>>(
+      in, nf, g.npix, g.ring_len_d, g.ring_off_d, g.ring_phase_d, g.nlat, g.lmax, g.nh, (float)g.a_ring[0], X, ldc,
+      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d, ps);
+  SHOT_CUDA(cudaGetLastError());
+  return SHOT_OK;
 }
 
 int launch_hp_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st) {
-  switch (hp_pick_fg(g, nf, true)) {
-    case 4: return hp_idft_t<4>(g, Y, ldc, nf, ep, st);
-    case 2: return hp_idft_t<2>(g, Y, ldc, nf, ep, st);
-    default: return hp_idft_t<1>(g, Y, ldc, nf, ep, st);
-  }
+  const size_t smem = (size_t)2 * seq_ld(g.nlon) * sizeof(C2);
+  SHOT_CUDA(cudaFuncSetAttribute(k_hp_idft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  ProfScope prof(ep.mode == EPI_CHECK || ep.mode == EPI_FINAL ? PK_CHECK : PK_IDFT, st);
+  count_launch();
+  k_hp_idft<<<dim3((nf + 1) / 2, g.nh), kHpThreads, smem, st>>>(
+      Y, ldc, nf, g.npix, g.ring_len_d, g.ring_off_d, g.ring_phase_d, g.nlat, g.lmax, g.nh, (float)g.a_ring[0], ep,
+      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d);
+  SHOT_CUDA(cudaGetLastError());
+  return SHOT_OK;
 }
 
 // Ring geometry of a HEALPix grid of resolution nside (host, FP64), into the Grid: node

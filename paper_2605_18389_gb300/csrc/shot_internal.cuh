@@ -42,10 +42,9 @@ class ProfScope {
 };
 
 // ---------------------------------------------------------------------------------
-// Ring FFT plan: nlon = prod R[s], radices in {2,3,4,5,8}, Stockham ordering.
-// The most elements (sequences x length) one ring-FFT CTA transforms: two ping-pong buffers
-// of kFftCap complex values plus the twiddles stay under ~110 KB (at least two CTAs per SM);
-// also the longest ring a grid may have.
+// Ring FFT plan: nlon = prod R[s], Stockham ordering.
+// The longest ring a grid may have: two ping-pong buffers of kFftCap complex values of two fields
+// (16 bytes each) fit in one CTA's shared memory.
 constexpr int kFftCap = 6400;
 
 struct FftPlan {
@@ -118,9 +117,7 @@ struct Workspace {
 // Tunable launch shapes for one field count (0 = the built-in default).
 struct Tuning {
   int nf = 0;
-  int dft_fg = 0;      // fields per ring-DFT CTA (1, 2, 4, 8)
-  int idft_fg = 0;     // fields per inverse-DFT CTA
-  int simt_bn = 0;     // FP32 Legendre tile width (32, 48, 64)
+  int simt_bn = 0;     // FP32 Legendre tile width (16, 32, 48, 64)
   int tc_stages = 0;   // BF16x3 analysis pipeline depth (1..4)
 };
 
@@ -187,9 +184,8 @@ struct Grid {
   int* ring_len_d = nullptr;
   long long* ring_off_d = nullptr;
   int2* ring_phase_d = nullptr;
-  // HEALPix: FFT plans for the ring lengths that factor into 2, 3 and 5 (the other rings use
-  // direct DFTs); ring_plan_d[i] = plan index or -1, each plan's stage twiddles at
-  // hp_tw_d + hp_tw_base_d[plan]
+  // HEALPix: an FFT plan for each distinct ring length; ring_plan_d[i] = plan index, each plan's
+  // stage twiddles at hp_tw_d + hp_tw_base_d[plan]
   FftPlan* hp_plan_d = nullptr;
   int* ring_plan_d = nullptr;
   float2* hp_tw_d = nullptr;
@@ -258,7 +254,7 @@ bool profiling_on();
 int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, int scale_which,
                    float* X, int ldc, cudaStream_t st);
 int launch_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st);
-bool idft_is_persistent(const Grid& g, int nf, const EpiParams& ep);
+int dft_fields_per_cta(const Grid& g, int nf);   // fields a ring-transform CTA takes
 // Grids whose Legendre contractions run the TF32x3 tensor-core kernels: TF32X3 grids, and BF16X3
 // grids in recurrence mode (the recurrence kernels are bound by generating the A operand, not by
 // the MMA's operand width, so a bf16 split of the generated values would gain nothing; TF32x3
@@ -275,7 +271,7 @@ int launch_analysis_only(const Grid& g, int nf, const float* X, float* C, int ld
                          cudaStream_t st);
 int build_grid_tables(Grid& g, cudaStream_t st);
 // selects g.active for nf (tunes on first use)
-int autotune(Grid& g, int nf, cudaStream_t st, const EpiParams* upd = nullptr);
+int autotune(Grid& g, int nf, cudaStream_t st);
 int launch_legendre_tc(const Grid& g, int nf, const float* X, float* Cf, float* Y, int ldc, bool ana, bool syn,
                        bool apply_h, cudaStream_t st);
 int launch_c_to_ct(const Grid& g, int nf, const float* C, int ldc, cudaStream_t st);

@@ -303,19 +303,19 @@ __global__ void k_field_mass_part(const float* const* __restrict__ fl, int nlat,
   }
 }
 
-__global__ void k_field_mass_sum(int nfl, int nlat, const double* __restrict__ part, double* __restrict__ out) {
-  const int f = blockIdx.x * blockDim.x + threadIdx.x;
-  if (f >= nfl) return;
+__global__ void k_field_mass_sum(int nlat, const double* __restrict__ part, double* __restrict__ out) {
+  const int f = blockIdx.x;   // one warp per field
   double s = 0.0;
-  for (int j = 0; j < nlat; ++j) s += part[(size_t)f * nlat + j];
-  out[f] = s;
+  for (int j = threadIdx.x; j < nlat; j += 32) s += part[(size_t)f * nlat + j];
+  s = wsum(s);
+  if (threadIdx.x == 0) out[f] = s;
 }
 
 // masses of nfl listed fields into out (device); part needs nfl*nlat doubles
 int field_masses(const Grid& g, const float* const* fl_d, int nfl, double* part, double* out, cudaStream_t st) {
   count_launch(2);
   k_field_mass_part<<<dim3(g.nlat, nfl), 256, 0, st>>>(fl_d, g.nlat, g.ring_len_d, g.ring_off_d, g.a_d, part);
-  k_field_mass_sum<<<(nfl + 127) / 128, 128, 0, st>>>(nfl, g.nlat, part, out);
+  k_field_mass_sum<<<nfl, 32, 0, st>>>(g.nlat, part, out);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
 }

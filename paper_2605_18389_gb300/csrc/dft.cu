@@ -39,9 +39,9 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // this thread's group of the CTA and its index in the group
-template <int G>
+template <int G, int NT>
 struct Group {
-  static constexpr int T = kThreads / G;
+  static constexpr int T = NT / G;
   int g, t;
   __device__ __forceinline__ Group() : g(G == 1 ? 0 : threadIdx.x / T), t(G == 1 ? threadIdx.x : threadIdx.x - g * T) {}
 };
@@ -49,10 +49,10 @@ struct Group {
 // Loads rings j (real parts) and J = nlat-1-j (imaginary parts; zero when J == j) of the CTA's
 // fields into buf; the second field of an odd last pair is zero.  Four rows of a batch of
 // longitudes are in flight per thread.
-template <int G>
+template <int G, int NT>
 __device__ __forceinline__ void load_ring_pairs(const float* __restrict__ in, C2* buf, int f0, int nf, int nlat, int N,
                                                 int j, int J) {
-  const Group<G> gr;
+  const Group<G, NT> gr;
   const int fa = f0 + 2 * gr.g;
   if (fa >= nf) return;
   const bool second = fa + 1 < nf, two = J != j;
@@ -83,16 +83,16 @@ __device__ __forceinline__ void load_ring_pairs(const float* __restrict__ in, C2
 // (the (2m+1) block of m = lmax is empty), into stg[blk][G] with asynchronous copies.  Row (blk,
 // jh) holds the fields' (re, im) pairs contiguously; an even first field starts on a 16-byte
 // boundary (ldc is a multiple of 4), and reading up to the next even field stays inside the row.
-template <int G>
+template <int G, int NT>
 __device__ __forceinline__ void issue_spectra(const float* __restrict__ Y, int ldc, int nh, int lmax, int jh, int f0,
                                               int nf, float4* stg) {
   const int nblk = 2 * lmax + 1;
   const float* y = Y + (size_t)jh * ldc + 2 * f0;
   const size_t row = (size_t)nh * ldc;
   if (G == 1) {
-    for (int blk = threadIdx.x; blk < nblk; blk += kThreads) cp_async16(stg + blk, y + blk * row);
+    for (int blk = threadIdx.x; blk < nblk; blk += NT) cp_async16(stg + blk, y + blk * row);
   } else {   // consecutive threads read the pieces of a row
-    for (int e = threadIdx.x; e < nblk * G; e += kThreads) {
+    for (int e = threadIdx.x; e < nblk * G; e += NT) {
       const int blk = e / G, c = e - blk * G;
       if (f0 + 2 * c < nf) cp_async16(stg + e, y + blk * row + 4 * c);
     }
@@ -103,9 +103,9 @@ __device__ __forceinline__ void issue_spectra(const float* __restrict__ Y, int l
 // Unfolds the staged spectra into the Hermitian-extended Z of each pair of fields:
 // G_N = E + O, G_S = E - O, Z(m) = G_N + i G_S, Z(N-m) = conj G_N + i conj G_S; the band
 // lmax < m < N - lmax is zero.
-template <int G>
+template <int G, int NT>
 __device__ __forceinline__ void unfold_spectra(const float4* stg, C2* buf, int N, int lmax) {
-  const Group<G> gr;
+  const Group<G, NT> gr;
   C2* z = buf + gr.g * seq_ld(N);
   for (int k = lmax + 1 + gr.t; k < N - lmax; k += gr.T) z[k] = c2(0ull, 0ull);
   for (int m = gr.t; m <= lmax; m += gr.T) {
@@ -126,11 +126,11 @@ __device__ __forceinline__ void unfold_spectra(const float4* stg, C2* buf, int N
 // F_N(m) = (Z(m) + conj Z(N-m))/2, F_S(m) = (Z(m) - conj Z(N-m))/(2i);
 // S = a_j (F_N + F_S) -> block (m, even), D = a_j (F_N - F_S) -> block (m, odd).
 // The columns of an odd last field's missing partner (padding, inside ldc) take its zeros.
-template <int G>
+template <int G, int NT>
 __device__ __forceinline__ void fold_store(const C2* buf, int f0, int nf, int N, int lmax, int nh, int jh, float aj,
                                            const ProbState* __restrict__ ps, int scale_which, float* __restrict__ X,
                                            int ldc) {
-  const Group<G> gr;
+  const Group<G, NT> gr;
   const int fa = f0 + 2 * gr.g;
   if (fa >= nf) return;
   float s0 = 0.5f * aj, s1 = s0;
@@ -154,28 +154,33 @@ __device__ __forceinline__ void fold_store(const C2* buf, int f0, int nf, int N,
   }
 }
 
-template <int G, class PL = RuntimePlan>
-__global__ void __launch_bounds__(kThreads, kCtas) k_dft_fwd(
+template <int G, int NT, int CTAS, class PL>
+__global__ void __launch_bounds__(NT, CTAS) k_dft_fwd(
     const float* __restrict__ in, int nf, int nlat, int nlon, int lmax, int nh,
     const float* __restrict__ a_ring, const ProbState* __restrict__ ps, int scale_which,
-    float* __restrict__ X, int ldc, const __grid_constant__ FftPlan pl, const float2* __restrict__ tw) {
+    float* __restrict__ X, int ldc, const __grid_constant__ FftPlan pl, const float2* tw, int tws) {
   extern __shared__ __align__(16) C2 sm[];
   C2* b0 = sm;
   C2* b1 = b0 + G * seq_ld(nlon);
   const int jh = blockIdx.y, f0 = blockIdx.x * 2 * G;
-  load_ring_pairs<G>(in, b0, f0, nf, nlat, nlon, jh, nlat - 1 - jh);
+  if (tws) {   // twiddles beside the sequences
+    fft_copy_twiddles(reinterpret_cast<float2*>(b1 + G * seq_ld(nlon)), tw, tws);
+    tw = reinterpret_cast<const float2*>(b1 + G * seq_ld(nlon));
+  }
+  load_ring_pairs<G, NT>(in, b0, f0, nf, nlat, nlon, jh, nlat - 1 - jh);
+  cp_async_wait_all();
   __syncthreads();
   const C2* buf = fft_smem_plan<false, PL>(b0, b1, tw, pl, G);
-  fold_store<G>(buf, f0, nf, nlon, lmax, nh, jh, a_ring[jh], ps, scale_which, X, ldc);
+  fold_store<G, NT>(buf, f0, nf, nlon, lmax, nh, jh, a_ring[jh], ps, scale_which, X, ldc);
 }
 
-template <int G, class PL = RuntimePlan>
-__global__ void __launch_bounds__(kThreads, kCtas) k_idft(
+template <int G, int NT, int CTAS, class PL>
+__global__ void __launch_bounds__(NT, CTAS) k_idft(
     const float* __restrict__ Y, int ldc, int nf, int nlat, int nlon, int lmax, int nh,
-    const float* __restrict__ a_ring, const __grid_constant__ FftPlan pl, const float2* __restrict__ tw,
+    const float* __restrict__ a_ring, const __grid_constant__ FftPlan pl, const float2* tw, int tws,
     EpiParams ep) {
   extern __shared__ __align__(16) C2 sm[];
-  __shared__ float red[kThreads / 32][2 * NPART];
+  __shared__ float red[NT / 32][2 * NPART];
   __shared__ EpiField fi[2 * G];
   const int N = nlon, ld = seq_ld(N);
   C2* buf = sm;
@@ -183,26 +188,30 @@ __global__ void __launch_bounds__(kThreads, kCtas) k_idft(
   const int jh = blockIdx.y, f0 = blockIdx.x * 2 * G;
   const int j = jh, J = nlat - 1 - jh;
   const bool two = (J != j);   // false only for the equator ring of an odd grid
+  if (tws) {   // twiddles beside the sequences
+    fft_copy_twiddles(reinterpret_cast<float2*>(b1 + G * ld), tw, tws);
+    tw = reinterpret_cast<const float2*>(b1 + G * ld);
+  }
   float4* stg = reinterpret_cast<float4*>(b1);   // the spectra, before the transform needs b1
-  issue_spectra<G>(Y, ldc, nh, lmax, jh, f0, nf, stg);
+  issue_spectra<G, NT>(Y, ldc, nh, lmax, jh, f0, nf, stg);
   const int nfg = min(2 * G, nf - f0);
   epi_fields_load<2 * G>(ep, f0, nfg, fi);
   cp_async_wait_all();
   __syncthreads();
   epi_prefetch_marginals<2 * G>(ep, fi, nfg, (size_t)j * N, (size_t)J * N, two, N, f0, (size_t)nlat * N);
-  unfold_spectra<G>(stg, buf, N, lmax);
+  unfold_spectra<G, NT>(stg, buf, N, lmax);
   __syncthreads();
   const C2* z = fft_smem_plan<true, PL>(buf, b1, tw, pl, G);
   C2* other = (z == buf) ? b1 : buf;   // input of the fused forward transform
 
   const float aj = a_ring[j];
-  ring_pair_epilogue<G, kThreads>(z, other, ld, N, nf, f0, (size_t)nlat * N, (size_t)j * N, (size_t)J * N, two, aj, nh,
+  ring_pair_epilogue<G, NT>(z, other, ld, N, nf, f0, (size_t)nlat * N, (size_t)j * N, (size_t)J * N, two, aj, nh,
                                   jh, ep, red, fi);
   if ((ep.mode == EPI_UPDATE || ep.mode == EPI_SYM) && ep.xout) {
     // the new scaling of this ring pair is in `other`: transform it for the next half-step
     __syncthreads();
     const C2* zf = fft_smem_plan<false, PL>(other, const_cast<C2*>(z), tw, pl, G);
-    fold_store<G>(zf, f0, nf, N, lmax, nh, jh, aj, nullptr, 0, ep.xout, ldc);
+    fold_store<G, NT>(zf, f0, nf, N, lmax, nh, jh, aj, nullptr, 0, ep.xout, ldc);
   }
 }
 
@@ -216,30 +225,29 @@ __global__ void __launch_bounds__(kThreads, kCtas) k_idft(
 // so that neither the gather nor the update waits on DRAM (three CTAs per SM, ~69 KB each at
 // 1440 longitudes and two fields).
 
-// shared-memory layout of k_idft_p (bytes): [buf][b1] sequences, then the spectra staging area
-struct IdftPLayout {
-  size_t stg, total;
-};
-__host__ __device__ inline IdftPLayout idft_p_layout(int G, int N, int lmax) {
-  IdftPLayout L;
-  L.stg = (size_t)2 * G * seq_ld(N) * sizeof(C2);
-  L.total = L.stg + (size_t)(2 * lmax + 1) * G * sizeof(float4);
-  return L;
+// shared memory of k_idft_p (bytes): the sequence buffers (one, or two to ping-pong), then the
+// spectra staging area
+__host__ __device__ inline size_t idft_p_layout(int nbuf, int G, int N, int lmax) {
+  return (size_t)nbuf * G * seq_ld(N) * sizeof(C2) + (size_t)(2 * lmax + 1) * G * sizeof(float4);
 }
 
-template <int G, class PL = RuntimePlan>
-__global__ void __launch_bounds__(kThreads, kCtas) k_idft_p(
+template <int G, int NT, int CTAS, class PL, bool INPLACE>
+__global__ void __launch_bounds__(NT, CTAS) k_idft_p(
     const float* __restrict__ Y, int ldc, int nf, int nlat, int nlon, int lmax, int nh,
-    const float* __restrict__ a_ring, const __grid_constant__ FftPlan pl, const float2* __restrict__ tw, EpiParams ep,
+    const float* __restrict__ a_ring, const __grid_constant__ FftPlan pl, const float2* tw, int tws, EpiParams ep,
     int ngroups) {
   extern __shared__ __align__(16) C2 sm[];
-  __shared__ float red[kThreads / 32][2 * NPART];
+  __shared__ float red[NT / 32][2 * NPART];
   __shared__ EpiField fi[2][2 * G];
   constexpr int FG = 2 * G;
   const int N = nlon, ld = seq_ld(N);
   C2* buf = sm;
-  C2* b1 = buf + G * ld;
+  C2* b1 = INPLACE ? buf : buf + G * ld;
   float4* stg = reinterpret_cast<float4*>(b1 + G * ld);
+  if (tws) {   // twiddles beside the sequences
+    fft_copy_twiddles(reinterpret_cast<float2*>(stg + (2 * lmax + 1) * G), tw, tws);
+    tw = reinterpret_cast<const float2*>(stg + (2 * lmax + 1) * G);
+  }
   const int nitems = ngroups * nh;
   const size_t fs = (size_t)nlat * N;
 
@@ -247,7 +255,7 @@ __global__ void __launch_bounds__(kThreads, kCtas) k_idft_p(
   int jh = item / ngroups, f0 = (item - jh * ngroups) * FG;
   if (item < nitems) {
     epi_fields_load<FG>(ep, f0, min(FG, nf - f0), fi[0]);
-    issue_spectra<G>(Y, ldc, nh, lmax, jh, f0, nf, stg);
+    issue_spectra<G, NT>(Y, ldc, nh, lmax, jh, f0, nf, stg);
   }
   __syncthreads();
   if (item < nitems)
@@ -259,25 +267,25 @@ __global__ void __launch_bounds__(kThreads, kCtas) k_idft_p(
     const int j = jh, J = nlat - 1 - jh;
     cp_async_wait_all();   // this item's spectra
     __syncthreads();
-    unfold_spectra<G>(stg, buf, N, lmax);
+    unfold_spectra<G, NT>(stg, buf, N, lmax);
     __syncthreads();
     if (next < nitems) {   // the staging area is free again: the next item's state and spectra
       epi_fields_load<FG>(ep, fn, nn, fi[slot ^ 1]);
-      issue_spectra<G>(Y, ldc, nh, lmax, jn, fn, nf, stg);
+      issue_spectra<G, NT>(Y, ldc, nh, lmax, jn, fn, nf, stg);
     }
-    const C2* z = fft_smem_plan<true, PL>(buf, b1, tw, pl, G);
-    C2* other = (z == buf) ? b1 : buf;
+    const C2* z = fft_smem_plan<true, PL, INPLACE>(buf, b1, tw, pl, G);
+    C2* other = (z == buf) ? b1 : buf;   // INPLACE: an element's new scaling replaces its K v
     if (next < nitems)   // fi[slot ^ 1] is visible after the transform's barriers
       epi_prefetch_marginals<FG>(ep, fi[slot ^ 1], nn, (size_t)jn * N, (size_t)(nlat - 1 - jn) * N,
                                  nlat - 1 - jn != jn, N, fn, fs);
     const float aj = a_ring[j];
     // the persistent kernel runs updates and checks only: no final-objective branch
-    ring_pair_epilogue<G, kThreads, false>(z, other, ld, N, nf, f0, fs, (size_t)j * N, (size_t)J * N, J != j, aj, nh,
+    ring_pair_epilogue<G, NT, false>(z, other, ld, N, nf, f0, fs, (size_t)j * N, (size_t)J * N, J != j, aj, nh,
                                            jh, ep, red, fi[slot]);
     if (ep.xout) {   // the update's new scaling: its spectra for the next half-step
       __syncthreads();
-      const C2* zf = fft_smem_plan<false, PL>(other, const_cast<C2*>(z), tw, pl, G);
-      fold_store<G>(zf, f0, nf, N, lmax, nh, jh, aj, nullptr, 0, ep.xout, ldc);
+      const C2* zf = fft_smem_plan<false, PL, INPLACE>(other, const_cast<C2*>(z), tw, pl, G);
+      fold_store<G, NT>(zf, f0, nf, N, lmax, nh, jh, aj, nullptr, 0, ep.xout, ldc);
     }
     item = next;
     jh = jn;
@@ -300,44 +308,53 @@ int pick_g(const Grid& g, int nf) {
   return G;
 }
 
+// Entries of the twiddle table a CTA copies into shared memory: all for rings of up to 768
+// longitudes (6 KB), where a CTA has few items and would wait for each stage's twiddles from L2 (32
+// rings, one field: 9.4 us an update launch without the copy, 7.3 with it in the scalar form); none
+// beyond, where many items read them through L1.
+int twiddles_in_smem(const Grid& g) { return g.nlon <= 768 ? fft_tw_len(g.plan) : 0; }
+
 size_t idft_smem(int G, int N) { return (size_t)2 * G * seq_ld(N) * sizeof(C2); }
 
-template <int G, class PL = RuntimePlan>
+template <int G, class PL = RuntimePlan, int NT = kThreads, int CTAS = kCtas>
 int launch_fwd_t(const Grid& g, const float* in, int nf, const ProbState* ps, int scale_which, float* X,
                  int ldc, cudaStream_t st) {
-  const size_t smem = idft_smem(G, g.nlon);
-  SHOT_CUDA(cudaFuncSetAttribute(k_dft_fwd<G, PL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int tws = twiddles_in_smem(g);
+  const size_t smem = idft_smem(G, g.nlon) + tws * sizeof(float2);
+  SHOT_CUDA(cudaFuncSetAttribute(k_dft_fwd<G, NT, CTAS, PL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   dim3 grid((nf + 2 * G - 1) / (2 * G), g.nh);   // field groups of one ring pair run together
   ProfScope prof(PK_DFT, st);
   count_launch();
-  k_dft_fwd<G, PL><<<grid, kThreads, smem, st>>>(in, nf, g.nlat, g.nlon, g.lmax, g.nh, g.a_d, ps, scale_which, X,
-                                                 ldc, g.plan, g.tw_d);
+  k_dft_fwd<G, NT, CTAS, PL><<<grid, NT, smem, st>>>(in, nf, g.nlat, g.nlon, g.lmax, g.nh, g.a_d, ps, scale_which, X,
+                                                 ldc, g.plan, g.tw_d, tws);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
 }
 
-template <int G, class PL = RuntimePlan>
+template <int G, class PL = RuntimePlan, int NT = kThreads, int CTAS = kCtas>
 int launch_idft_t(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st) {
-  const size_t smem = idft_smem(G, g.nlon);   // two sequence buffers; the second first stages the spectra
-  SHOT_CUDA(cudaFuncSetAttribute(k_idft<G, PL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int tws = twiddles_in_smem(g);
+  const size_t smem = idft_smem(G, g.nlon) + tws * sizeof(float2);   // two sequence buffers; the second first stages the spectra
+  SHOT_CUDA(cudaFuncSetAttribute(k_idft<G, NT, CTAS, PL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   dim3 grid((nf + 2 * G - 1) / (2 * G), g.nh);   // field groups of one ring pair run together
   ProfScope prof(ep.mode == EPI_CHECK || ep.mode == EPI_FINAL ? PK_CHECK : PK_IDFT, st);
   count_launch();
-  k_idft<G, PL><<<grid, kThreads, smem, st>>>(Y, ldc, nf, g.nlat, g.nlon, g.lmax, g.nh, g.a_d, g.plan, g.tw_d, ep);
+  k_idft<G, NT, CTAS, PL><<<grid, NT, smem, st>>>(Y, ldc, nf, g.nlat, g.nlon, g.lmax, g.nh, g.a_d, g.plan, g.tw_d, tws, ep);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
 }
 
-template <int G, class PL = RuntimePlan>
+template <int G, class PL = RuntimePlan, int NT = kThreads, int CTAS = kCtas, bool INPLACE = false>
 int launch_idft_p_t(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st) {
-  const size_t smem = idft_p_layout(G, g.nlon, g.lmax).total;
-  SHOT_CUDA(cudaFuncSetAttribute(k_idft_p<G, PL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int tws = twiddles_in_smem(g);
+  const size_t smem = idft_p_layout(INPLACE ? 1 : 2, G, g.nlon, g.lmax) + tws * sizeof(float2);
+  SHOT_CUDA(cudaFuncSetAttribute(k_idft_p<G, NT, CTAS, PL, INPLACE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int ngroups = (nf + 2 * G - 1) / (2 * G);
   const int nitems = ngroups * g.nh;
-  const int grid = nitems < kCtas * g.num_sms ? nitems : kCtas * g.num_sms;
+  const int grid = nitems < CTAS * g.num_sms ? nitems : CTAS * g.num_sms;
   ProfScope prof(ep.mode == EPI_CHECK || ep.mode == EPI_FINAL ? PK_CHECK : PK_IDFT, st);
   count_launch();
-  k_idft_p<G, PL><<<grid, kThreads, smem, st>>>(Y, ldc, nf, g.nlat, g.nlon, g.lmax, g.nh, g.a_d, g.plan, g.tw_d, ep,
+  k_idft_p<G, NT, CTAS, PL, INPLACE><<<grid, NT, smem, st>>>(Y, ldc, nf, g.nlat, g.nlon, g.lmax, g.nh, g.a_d, g.plan, g.tw_d, tws, ep,
                                                 ngroups);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
@@ -374,7 +391,7 @@ int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, 
     case 3: return launch_fwd_t<3>(g, in, nf, ps, scale_which, X, ldc, st);
     case 2: return launch_fwd_t<2>(g, in, nf, ps, scale_which, X, ldc, st);
     default:
-      if (plan_is<Plan1440>(g.plan)) return launch_fwd_t<1, Plan1440>(g, in, nf, ps, scale_which, X, ldc, st);
+      if (plan_is<Plan1440>(g.plan)) return launch_fwd_t<1, Plan1440, 192, 4>(g, in, nf, ps, scale_which, X, ldc, st);
       if (plan_is<Plan1024>(g.plan)) return launch_fwd_t<1, Plan1024>(g, in, nf, ps, scale_which, X, ldc, st);
       return launch_fwd_t<1>(g, in, nf, ps, scale_which, X, ldc, st);
   }
@@ -383,7 +400,7 @@ int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, 
 // whether launch_idft runs the persistent kernel for this epilogue
 static bool idft_is_persistent(const Grid& g, int nf, const EpiParams& ep) {
   return (((ep.mode == EPI_UPDATE || ep.mode == EPI_SYM) && ep.xout) || ep.mode == EPI_CHECK) &&
-         !g.idft_nonpersistent && nf >= 2 && idft_p_layout(pick_g(g, nf), g.nlon, g.lmax).total <= 74 * 1024;
+         !g.idft_nonpersistent && nf >= 2 && idft_p_layout(2, pick_g(g, nf), g.nlon, g.lmax) <= 74 * 1024;
 }
 
 int launch_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st) {
@@ -411,7 +428,7 @@ int launch_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams&
     case 3: return launch_idft_t<3>(g, Y, ldc, nf, ep, st);
     case 2: return launch_idft_t<2>(g, Y, ldc, nf, ep, st);
     default:
-      if (plan_is<Plan1440>(g.plan)) return launch_idft_t<1, Plan1440>(g, Y, ldc, nf, ep, st);
+      if (plan_is<Plan1440>(g.plan)) return launch_idft_t<1, Plan1440, 192, 4>(g, Y, ldc, nf, ep, st);
       if (plan_is<Plan1024>(g.plan)) return launch_idft_t<1, Plan1024>(g, Y, ldc, nf, ep, st);
       return launch_idft_t<1>(g, Y, ldc, nf, ep, st);
   }

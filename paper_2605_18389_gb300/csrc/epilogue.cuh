@@ -88,6 +88,105 @@ __device__ __forceinline__ float epi_warp_sum(float v) {
   return v;
 }
 
+// The update of one K v value in full generality: u, the sums and the breakdown counts.
+__device__ __forceinline__ float epi_update_value(float pm, float kv, float rr, bool bal, float gam, float aj,
+                                                  float (&acc)[NPART]) {
+  const float ratio = __fdividef(pm, kv) * rr;   // MUFU reciprocal + multiply, <= 2 ulp
+  const float u = bal ? ratio : exp2f(gam * __log2f(ratio));
+  if (bal) {
+    acc[0] += u;
+  } else {
+    acc[0] += aj * u * kv * (1.f / rr);
+    acc[1] += u;
+  }
+  // K v positive and finite, u finite (NaN fails each comparison); the failures are sorted into
+  // non-positive (first in the status precedence) and non-finite
+  if (!(kv > 0.f && kv < INFINITY && fabsf(u) < INFINITY)) {
+    if (kv <= 0.f) acc[2] += 1.f;
+    else acc[3] += 1.f;   // NaN or infinite K v, or u overflowed
+  }
+  return u;
+}
+
+// The update of a pair of live fields on a ring pair.  u = (r p/Kv)^gamma (hardware log2/exp2,
+// ~2^-21 absolute in the exponent); the translation-invariant sum's p u^{-eps/tau} =
+// p (r p/Kv)^{-eps/(tau+eps)} equals u (Kv) / r since gamma + eps/(tau+eps) = 1, so one power serves
+// both (ratio = 0 gives u = 0 and adds nothing). 
+// An element whose four K v are normal and at most 2^125 takes the reciprocal directly (the value
+// __fdividef gives there); any other goes through epi_update_value.  The check for a non-finite u is
+// on the thread's sum: it is finite exactly if every u is (or the sum has overflowed, which stops
+// the problem too).  The pointwise part is instruction issue: with a check and a scaled divide per
+// value it took 38 of the update kernel's 79 million warp instructions (720 rings, 24 fields).
+template <int GT>
+__device__ __forceinline__ void epi_update_pair(const float4* zg, float4* og, int t, int N, const EpiField* fi,
+                                                float* out, size_t fstride, size_t rj, int dJ, bool xout, float aj,
+                                                float (&acc)[2][NPART]) {
+  constexpr int kBatch = 2;   // (4 measured slower: registers)
+  const float rr[2] = {fi[0].r, fi[1].r}, ri[2] = {1.f / rr[0], 1.f / rr[1]}, gam[2] = {fi[0].gamma, fi[1].gamma};
+  const bool bal0 = fi[0].balanced, bal1 = fi[1].balanced;
+  const float* m00 = fi[0].marg + rj + t;   // ring j of the first field; ring J starts dJ further
+  const float* m10 = fi[1].marg + rj + t;
+  const float* m01 = m00 + dJ;
+  const float* m11 = m10 + dJ;
+  for (int k0 = t; k0 < N; k0 += kBatch * GT) {
+    float4 pv[kBatch];   // (field 0, field 1) on ring j, then on ring J, as K v is stored
+#pragma unroll
+    for (int b = 0; b < kBatch; ++b) {
+      if (k0 + b * GT < N)
+        pv[b] = make_float4(__ldg(m00 + b * GT), __ldg(m10 + b * GT), __ldg(m01 + b * GT), __ldg(m11 + b * GT));
+    }
+    m00 += kBatch * GT;
+    m10 += kBatch * GT;
+    m01 += kBatch * GT;
+    m11 += kBatch * GT;
+#pragma unroll
+    for (int b = 0; b < kBatch; ++b) {
+      const int k = k0 + b * GT;
+      if (k >= N) break;
+      const float4 z = zg[k];
+      const uint32_t lo = 0x00800000u, span = 0x7e000000u - 0x00800000u;
+      const uint32_t d = max(max(__float_as_uint(z.x) - lo, __float_as_uint(z.y) - lo),
+                             max(__float_as_uint(z.z) - lo, __float_as_uint(z.w) - lo));
+      float4 u;
+      if (d <= span) {
+        auto one = [&](float pm, float kv, float r, float rinv, bool bal, float ga, float (&a)[NPART]) {
+          float rc;
+          asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(kv));
+          const float ratio = pm * rc * r;
+          const float w = bal ? ratio : exp2f(ga * __log2f(ratio));
+          if (bal) {
+            a[0] += w;
+          } else {
+            a[0] += aj * w * kv * rinv;
+            a[1] += w;
+          }
+          return w;
+        };
+        u.x = one(pv[b].x, z.x, rr[0], ri[0], bal0, gam[0], acc[0]);
+        u.y = one(pv[b].y, z.y, rr[1], ri[1], bal1, gam[1], acc[1]);
+        u.z = one(pv[b].z, z.z, rr[0], ri[0], bal0, gam[0], acc[0]);
+        u.w = one(pv[b].w, z.w, rr[1], ri[1], bal1, gam[1], acc[1]);
+      } else {
+        u.x = epi_update_value(pv[b].x, z.x, rr[0], bal0, gam[0], aj, acc[0]);
+        u.y = epi_update_value(pv[b].y, z.y, rr[1], bal1, gam[1], aj, acc[1]);
+        u.z = epi_update_value(pv[b].z, z.z, rr[0], bal0, gam[0], aj, acc[0]);
+        u.w = epi_update_value(pv[b].w, z.w, rr[1], bal1, gam[1], aj, acc[1]);
+      }
+      if (out) {
+        float* o = out + k;
+        o[0] = u.x;
+        o[fstride] = u.y;
+        o[dJ] = u.z;
+        o[fstride + dJ] = u.w;
+      }
+      if (xout) og[k] = u;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+    if (!(fabsf((q ? bal1 : bal0) ? acc[q][0] : acc[q][1]) < INFINITY) && acc[q][2] == 0.f) acc[q][3] += 1.f;
+}
+
 // kFinal = false compiles the EPI_FINAL branch out (kernels never launched with it).
 // The CTA's NT threads form G groups of NT / G (whole warps); group g takes fields f0 + 2 g and
 // f0 + 2 g + 1, a thread longitude k of both rings of the pair, so that one set of sums per
@@ -99,6 +198,7 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
                                                    float (*red)[2 * NPART], const EpiField* fi) {
   constexpr int GT = NT / G, GW = GT / 32;
   static_assert(NT % G == 0 && GT % 32 == 0, "a group is whole warps");
+  constexpr int kBatchGen = 2;   // the general path of the update
   constexpr int kEpiBatch = 4;   // longitudes per thread whose marginal values are loaded together
   const int g = G == 1 ? 0 : threadIdx.x / GT, t = G == 1 ? threadIdx.x : threadIdx.x - g * GT;
   const int fa = f0 + 2 * g;                       // first field of the group
@@ -138,27 +238,32 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
   if (ep.mode == EPI_UPDATE || ep.mode == EPI_SYM) {
     // both fields of an element in one pass: K v comes and the new scaling leaves as 16 bytes
     const bool sym = ep.mode == EPI_SYM;
+    const EpiField* f2 = fi + 2 * g;
+    const bool live0 = nq > 0 && f2[0].live, live1 = nq > 1 && f2[1].live;
+    const bool bal0 = f2[0].balanced, bal1 = f2[1].balanced;
+    if (!sym && two && live0 && live1) {
+      float* out = ep.skip_store ? nullptr : ep.out + (size_t)fa * fstride + rj;
+      const int dJ = (int)(rJ - rj);   // a field has fewer than 2^31 nodes
+      epi_update_pair<GT>(zg, og, t, N, f2, out, fstride, rj, dJ, ep.xout != nullptr, aj, acc);
+    } else {
     float* outf[2];
     const float* mg[2];
-    int live[2], bal[2];
-    float gam[2], rr[2], rinv[2];
+    int live[2] = {live0, live1}, bal[2] = {bal0, bal1};
+    float gam[2], rr[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-      const EpiField F = fi[2 * g + q];
       outf[q] = ep.out + (size_t)(fa + q) * fstride;
-      mg[q] = F.marg;
-      live[q] = q < nq && F.live;
-      bal[q] = F.balanced;
-      gam[q] = F.gamma;
-      rr[q] = F.r;
-      rinv[q] = 1.f / F.r;
+      mg[q] = f2[q].marg;
+      gam[q] = f2[q].gamma;
+      rr[q] = f2[q].r;
     }
-    for (int k0 = t; k0 < N && nq > 0; k0 += kEpiBatch * GT) {
+    for (int k0 = t; k0 < N && nq > 0; k0 += kBatchGen * GT) {
+      // the equator ring, an odd last field, frozen problems and self terms: field by field;
       // the marginal values (self term: and the old scaling's) of all this thread's longitudes
       // first, then the arithmetic; a frozen problem loads its stored scaling
-      float pv[kEpiBatch][2][2], uo[kEpiBatch][2][2];
+      float pv[kBatchGen][2][2], uo[kBatchGen][2][2];
 #pragma unroll
-      for (int b = 0; b < kEpiBatch; ++b) {
+      for (int b = 0; b < kBatchGen; ++b) {
         const int k = k0 + b * GT;
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
@@ -170,7 +275,7 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
         }
       }
 #pragma unroll
-      for (int b = 0; b < kEpiBatch; ++b) {
+      for (int b = 0; b < kBatchGen; ++b) {
         const int k = k0 + b * GT;
         if (k >= N) break;
         const float4 zz = zg[k];
@@ -190,27 +295,12 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
               const float ratio = __fdividef(pm, kv);
               const float x = bal[q] ? ratio : exp2f(gam[q] * __log2f(ratio));
               u = sqrtf(uo[b][q][r] * x);
-            } else {
-              const float ratio = __fdividef(pm, kv) * rr[q];   // MUFU reciprocal + multiply, <= 2 ulp
-              if (bal[q]) {
-                u = ratio;
-                acc[q][0] += u;
-              } else {
-                // u = (r p/Kv)^gamma (hardware log2/exp2, ~2^-21 absolute in the exponent); the
-                // translation-invariant sum's p u^{-eps/tau} = p (r p/Kv)^{-eps/(tau+eps)} equals
-                // u (Kv) / r since gamma + eps/(tau+eps) = 1, so one power serves both (ratio = 0
-                // gives u = 0 and adds nothing)
-                u = exp2f(gam[q] * __log2f(ratio));
-                acc[q][0] += aj * u * kv * rinv[q];
-                acc[q][1] += u;
+              if (!(kv > 0.f && kv < INFINITY && fabsf(u) < INFINITY)) {
+                if (kv <= 0.f) acc[q][2] += 1.f;
+                else acc[q][3] += 1.f;
               }
-            }
-            // one test on the common path: K v positive and finite, u finite (NaN fails each
-            // comparison); the rare failures are sorted into non-positive (first in the status
-            // precedence) and non-finite
-            if (!(kv > 0.f && kv < INFINITY && fabsf(u) < INFINITY)) {
-              if (kv <= 0.f) acc[q][2] += 1.f;
-              else acc[q][3] += 1.f;   // NaN or infinite K v, or u overflowed
+            } else {
+              u = epi_update_value(pm, kv, rr[q], bal[q], gam[q], aj, acc[q]);
             }
             if (sym || !ep.skip_store) outf[q][(r ? rJ : rj) + k] = u;
             un[q][r] = u;
@@ -218,6 +308,7 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
         }
         if (ep.xout) og[k] = make_float4(un[0][0], un[1][0], un[0][1], un[1][1]);
       }
+    }
     }
   } else {
 #pragma unroll

@@ -36,6 +36,11 @@ __device__ __forceinline__ f32x2 pk2(float lo, float hi) {
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
   return r;
 }
+// a constant twice, as integer arithmetic that the compiler folds into an immediate (the result of
+// an asm statement would be hoisted out of a persistent kernel's loop over items and spilled)
+__device__ __forceinline__ f32x2 kc2(float c) {
+  return ((f32x2)__float_as_uint(c) << 32) | (f32x2)__float_as_uint(c);
+}
 __device__ __forceinline__ float2 unpk2(f32x2 a) {
   float2 r;
   asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
@@ -136,7 +141,7 @@ __device__ __forceinline__ C2 mul_root(C2 a) {
     constexpr float c = (float)taylor_cos(root_angle(j, R));
     constexpr float s = (float)taylor_sin(root_angle(j, R));
     constexpr float sy = INV ? s : -s;   // W^j = (c, -s) forward
-    return cmul<false>(a, make_float2(c, sy));
+    return c2(fma2(a.re, kc2(c), mul2(a.im, kc2(-sy))), fma2(a.re, kc2(sy), mul2(a.im, kc2(c))));
   }
 }
 
@@ -177,12 +182,12 @@ __device__ __forceinline__ void bfly8(C2* v) {
 
 template <bool INV>
 __device__ __forceinline__ void bfly3(C2* v) {
-  const f32x2 s = pk2(0.86602540378443865f, 0.86602540378443865f);   // sin(2 pi / 3)
-  const f32x2 h = pk2(-0.5f, -0.5f);
+  const f32x2 s = kc2(0.86602540378443865f);   // sin(2 pi / 3)
+  const f32x2 h = kc2(-0.5f);
   const C2 t = cadd(v[1], v[2]);
   const C2 d = csub(v[1], v[2]);
   const C2 a = c2(fma2(h, t.re, v[0].re), fma2(h, t.im, v[0].im));
-  const f32x2 ns = neg2(s);
+  const f32x2 ns = kc2(-0.86602540378443865f);
   v[0] = cadd(v[0], t);
   // a -+ i s d
   const C2 m = c2(fma2(s, d.im, a.re), fma2(ns, d.re, a.im));   // a - i s d
@@ -193,16 +198,16 @@ __device__ __forceinline__ void bfly3(C2* v) {
 
 template <bool INV>
 __device__ __forceinline__ void bfly5(C2* v) {
-  const f32x2 c1 = pk2(0.30901699437494742f, 0.30901699437494742f);     // cos(2pi/5)
-  const f32x2 k2 = pk2(-0.80901699437494742f, -0.80901699437494742f);   // cos(4pi/5)
-  const f32x2 s1 = pk2(0.95105651629515357f, 0.95105651629515357f);     // sin(2pi/5)
-  const f32x2 s2 = pk2(0.58778525229247313f, 0.58778525229247313f);     // sin(4pi/5)
+  const f32x2 c1 = kc2(0.30901699437494742f);     // cos(2pi/5)
+  const f32x2 k2 = kc2(-0.80901699437494742f);   // cos(4pi/5)
+  const f32x2 s1 = kc2(0.95105651629515357f);     // sin(2pi/5)
+  const f32x2 s2 = kc2(0.58778525229247313f);     // sin(4pi/5)
   const C2 t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
   const C2 d1 = csub(v[1], v[4]), d2 = csub(v[2], v[3]);
   const C2 x0 = v[0];
   const C2 a1 = c2(fma2(k2, t2.re, fma2(c1, t1.re, x0.re)), fma2(k2, t2.im, fma2(c1, t1.im, x0.im)));
   const C2 a2 = c2(fma2(c1, t2.re, fma2(k2, t1.re, x0.re)), fma2(c1, t2.im, fma2(k2, t1.im, x0.im)));
-  const f32x2 ns1 = neg2(s1);
+  const f32x2 ns1 = kc2(-0.95105651629515357f);
   const C2 b1 = c2(fma2(s1, d1.re, mul2(s2, d2.re)), fma2(s1, d1.im, mul2(s2, d2.im)));
   const C2 b2 = c2(fma2(s2, d1.re, mul2(ns1, d2.re)), fma2(s2, d1.im, mul2(ns1, d2.im)));
   v[0] = cadd(x0, cadd(t1, t2));
@@ -278,6 +283,14 @@ __host__ __device__ constexpr int out_reg(int k) {
   return Radix<R>::R1 == 1 ? k : Radix<R>::R2 * (k % Radix<R>::R1) + k / Radix<R>::R1;
 }
 
+// Copies the plan's twiddle table into shared memory (asynchronous, 8 bytes an entry; the caller waits).
+__device__ __forceinline__ void fft_copy_twiddles(float2* dst, const float2* __restrict__ tw, int len) {
+  for (int k = threadIdx.x; k < len; k += blockDim.x)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst + k)),
+                 "l"(tw + k)
+                 : "memory");
+}
+
 // stride of consecutive sequences in the CTA's buffers
 __host__ __device__ constexpr int seq_ld(int N) { return N + 1; }
 
@@ -306,7 +319,7 @@ __device__ __forceinline__ void stockham_stage(const C2* __restrict__ src, C2* _
     if (Ns > 1) {   // the first stage's twiddles are all 1
 #pragma unroll
       for (int r = 1; r < R; ++r) {
-        v[r] = cmul<INV>(v[r], __ldg(tws + (r - 1) * Ns + k));
+        v[r] = cmul<INV>(v[r], tws[(r - 1) * Ns + k]);
       }
     }
     butterfly<R, INV>(v);
@@ -340,8 +353,8 @@ __device__ __noinline__ void stockham_stage_generic(const C2* __restrict__ src, 
 #pragma unroll 4
     for (int t = 0; t < R; ++t) {
       C2 v = s[t * NR];
-      if (Ns > 1 && t > 0) v = cmul<INV>(v, __ldg(tws + (t - 1) * Ns + k));
-      sum = cadd(sum, cmul<INV>(v, __ldg(roots + e)));
+      if (Ns > 1 && t > 0) v = cmul<INV>(v, tws[(t - 1) * Ns + k]);
+      sum = cadd(sum, cmul<INV>(v, roots[e]));
       e += r;
       if (e >= R) e -= R;
     }
@@ -350,12 +363,14 @@ __device__ __noinline__ void stockham_stage_generic(const C2* __restrict__ src, 
 }
 
 // Transforms nseq sequences of length plan.N stored at a[q * seq_ld(N) + k]; b is
-// scratch of the same shape; tw holds the plan's stage twiddles (forward sign).  Returns
+// scratch of the same shape; tw holds the plan's stage twiddles (forward sign), in shared memory for
+// the short rings, whose CTAs would wait a global-memory latency in every stage.  Returns
 // the buffer holding the result.  All threads of the block must call it; it
 // synchronises after every stage.
 template <bool INV>
 __device__ C2* fft_smem(C2* a, C2* b, const float2* tw, const FftPlan& pl, int nseq) {
   int Ns = 1;
+#pragma unroll 1
   for (int s = 0; s < pl.nst; ++s) {
     const int R = pl.R[s];
     const float2* tws = tw + pl.tw_off[s];
@@ -395,52 +410,65 @@ struct CtPlan {
 };
 using RuntimePlan = CtPlan<0>;
 
-template <int R, bool INV, int N, int NS, int TWOFF>
-__device__ __forceinline__ void stockham_stage_ct(const C2* __restrict__ src, C2* __restrict__ dst,
-                                                  const float2* __restrict__ tw, int nseq) {
+template <int R, bool INV, int N, int NS, int TWOFF, bool INPLACE>
+__device__ __forceinline__ void stockham_stage_ct(const C2* src, C2* dst, const float2* __restrict__ tw, int nseq) {
   constexpr int NR = N / R, LD = N + 1;
   const int total = nseq * NR;
-  for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-    const int q = idx / NR;
-    const int j = idx - q * NR;
-    const int jd = j / NS;
-    const int k = j - jd * NS;
+  C2 v[R];
+  auto load = [&](int idx) {
+    const int q = idx / NR, j = idx - q * NR;
     const C2* s = src + q * LD + j;
-    C2 v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = s[r * NR];
     if constexpr (NS > 1) {
-      const float2* tws = tw + TWOFF + k;
+      const float2* tws = tw + TWOFF + j % NS;
 #pragma unroll
       for (int r = 1; r < R; ++r) v[r] = cmul<INV>(v[r], __ldg(tws + (r - 1) * NS));
     }
     butterfly<R, INV>(v);
-    C2* d = dst + q * LD + jd * NS * R + k;
+  };
+  auto store = [&](int idx) {
+    const int q = idx / NR, j = idx - q * NR, jd = j / NS;
+    C2* d = dst + q * LD + jd * NS * R + (j - jd * NS);
 #pragma unroll
     for (int r = 0; r < R; ++r) d[r * NS] = v[out_reg<R>(r)];
+  };
+  // opaque to the compiler, which would otherwise hoist a persistent kernel's index arithmetic and
+  // twiddle loads out of its loop over items and spill them (1.4 KB a thread in the in-place form)
+  int idx = threadIdx.x;
+  asm volatile("" : "+r"(idx));
+  if constexpr (INPLACE) {   // one butterfly a thread (the launch has at least `total` threads)
+    if (idx < total) load(idx);
+    __syncthreads();
+    if (idx < total) store(idx);
+  } else {
+    for (; idx < total; idx += blockDim.x) {
+      load(idx);
+      store(idx);
+    }
   }
+  __syncthreads();
 }
 
 // three-stage compile-time plan; the twiddle table layout is the runtime plan's (stage s at
-// sum over earlier stages s' >= 1 of (R_s' - 1) Ns_s')
-template <bool INV, class PL>
+// sum over earlier stages s' >= 1 of (R_s' - 1) Ns_s').  INPLACE: every stage reads and writes a
+// (b unused), with a barrier between, for launches with a thread per butterfly.
+template <bool INV, class PL, bool INPLACE = false>
 __device__ C2* fft_smem_ct(C2* a, C2* b, const float2* tw, int nseq) {
   constexpr int N = PL::N, R0 = PL::R0, R1 = PL::R1, R2 = PL::R2;
   static_assert(R0 * R1 * R2 == N, "plan radices must multiply to N");
-  stockham_stage_ct<R0, INV, N, 1, 0>(a, b, tw, nseq);
-  __syncthreads();
-  stockham_stage_ct<R1, INV, N, R0, 0>(b, a, tw, nseq);
-  __syncthreads();
-  stockham_stage_ct<R2, INV, N, R0 * R1, (R1 - 1) * R0>(a, b, tw, nseq);
-  __syncthreads();
+  if constexpr (INPLACE) b = a;
+  stockham_stage_ct<R0, INV, N, 1, 0, INPLACE>(a, b, tw, nseq);
+  stockham_stage_ct<R1, INV, N, R0, 0, INPLACE>(b, a, tw, nseq);
+  stockham_stage_ct<R2, INV, N, R0 * R1, (R1 - 1) * R0, INPLACE>(a, b, tw, nseq);
   return b;
 }
 
-template <bool INV, class PL>
+template <bool INV, class PL, bool INPLACE = false>
 __device__ __forceinline__ C2* fft_smem_plan(C2* a, C2* b, const float2* tw, const FftPlan& pl,
                                                  int nseq) {
   if constexpr (PL::N == 0) return fft_smem<INV>(a, b, tw, pl, nseq);
-  else return fft_smem_ct<INV, PL>(a, b, tw, nseq);
+  else return fft_smem_ct<INV, PL, INPLACE>(a, b, tw, nseq);
 }
 
 }  // namespace shot

@@ -73,9 +73,11 @@ struct GScal {      // per problem and iteration of a segment
 };
 
 // forward half-step: out = (m / Kf)^g; partial sums per ring of
-//   balanced: sum out;  unbalanced: sum a m out^{-eps/tau}
+//   balanced: sum out;  unbalanced: sum a m out^{-eps/tau} = sum a out Kf (g (1 + eps/tau) = 1)
+// The powers bound the pointwise kernels of this file, so each node takes as few as the identity
+// allows: 32 fields at 256 rings, 33 us with a second power for the sum (see k_g_rev1 too).
 __global__ void k_g_update(Rings R, const float* __restrict__ a_ring, const float* const* __restrict__ marg,
-                           const float* __restrict__ Kf, float* __restrict__ out, int balanced, float gam, float et,
+                           const float* __restrict__ Kf, float* __restrict__ out, int balanced, float gam,
                            double* __restrict__ part) {
   __shared__ float red[32];
   const int j = blockIdx.x, b = blockIdx.y;
@@ -85,27 +87,41 @@ __global__ void k_g_update(Rings R, const float* __restrict__ a_ring, const floa
   const float aj = a_ring[j];
   float acc = 0.f;
   for (int k = threadIdx.x; k < nk; k += blockDim.x) {
-    const float mm = m[k];
-    const float r = mm / Kf[base + k];
+    const float mm = m[k], kf = Kf[base + k];
+    const float r = mm / kf;
     const float u = balanced ? r : powf(r, gam);
     out[base + k] = u;
-    acc += balanced ? u : (mm > 0.f ? aj * mm * powf(u, -et) : 0.f);
+    acc += balanced ? u : (mm > 0.f ? aj * u * kf : 0.f);
   }
   const float t = block_sum_f(acc, red);
   if (threadIdx.x == 0) part[(size_t)b * R.nring + j] = (double)t;
 }
 
-// scalars of iteration k after both half-steps: (al, be) and the ProbState beta used by
-// the next K v (the ring DFT scales v' by beta on load)
-__global__ void k_g_scalars(int nprob, int nlat, const double* __restrict__ partU, const double* __restrict__ partV,
-                            int balanced, double eps, double tau, GScal* __restrict__ sc, ProbState* __restrict__ ps) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nprob) return;
-  double su = 0.0, sv = 0.0;
-  for (int j = 0; j < nlat; ++j) {
-    su += partU[(size_t)b * nlat + j];
-    sv += partV[(size_t)b * nlat + j];
+// sums of problem b's per-ring partials in both lists, by one warp (every lane gets them): a
+// thread walking the rings alone took 33 us at 256 rings
+__device__ __forceinline__ double2 ring_sums(const double* __restrict__ pa, const double* __restrict__ pb, int b,
+                                             int nring) {
+  double x = 0.0, y = 0.0;
+  for (int j = threadIdx.x & 31; j < nring; j += 32) {
+    x += pa[(size_t)b * nring + j];
+    y += pb[(size_t)b * nring + j];
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    x += __shfl_xor_sync(0xffffffffu, x, o);
+    y += __shfl_xor_sync(0xffffffffu, y, o);
+  }
+  return make_double2(x, y);
+}
+
+// scalars of iteration k after both half-steps: (al, be) and the ProbState beta used by
+// the next K v (the ring DFT scales v' by beta on load); one warp per problem
+__global__ void k_g_scalars(int nlat, const double* __restrict__ partU, const double* __restrict__ partV,
+                            int balanced, double eps, double tau, GScal* __restrict__ sc, ProbState* __restrict__ ps) {
+  const int b = blockIdx.x;
+  const double2 t = ring_sums(partU, partV, b, nlat);
+  if (threadIdx.x != 0) return;
+  const double su = t.x, sv = t.y;
   GScal s;
   if (balanced) {
     s.al = 1.0 / su;
@@ -190,16 +206,13 @@ struct RevScal {
   double Abar, Bbar;    // unbalanced
 };
 
-__global__ void k_g_rscal(int nprob, int nlat, const double* __restrict__ p1, const double* __restrict__ p2,
+__global__ void k_g_rscal(int nlat, const double* __restrict__ p1, const double* __restrict__ p2,
                           const GScal* __restrict__ sc, int balanced, double eps, double tau,
                           RevScal* __restrict__ rs) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nprob) return;
-  double r1 = 0.0, r2 = 0.0;
-  for (int j = 0; j < nlat; ++j) {
-    r1 += p1[(size_t)b * nlat + j];
-    r2 += p2[(size_t)b * nlat + j];
-  }
+  const int b = blockIdx.x;
+  const double2 t = ring_sums(p1, p2, b, nlat);
+  if (threadIdx.x != 0) return;
+  const double r1 = t.x, r2 = t.y;
   const GScal s = sc[b];
   RevScal o{0.0, 0.0, 0.0};
   if (balanced) {
@@ -214,7 +227,9 @@ __global__ void k_g_rscal(int nprob, int nlat, const double* __restrict__ p1, co
   rs[b] = o;
 }
 
-// first pointwise reverse stage: u~' (before + K (Ku)~), (Ku)~, q~ updates
+// first pointwise reverse stage: u~' (before + K (Ku)~), (Ku)~, q~ updates.  Unbalanced, two powers
+// a node, A = u'^{-eps/tau} and B = v'^{-eps/tau}: u'^{-eps/tau-1} = A/u', v'^{1/g} = v'^{1+eps/tau} =
+// v'/B (with five powers 119 us for 32 fields at 256 rings).
 __global__ void k_g_rev1(Rings R, const float* __restrict__ a_ring, const float* const* __restrict__ P,
                          const float* const* __restrict__ Q, const float* __restrict__ U, const float* __restrict__ V,
                          const GScal* __restrict__ sc, const RevScal* __restrict__ rs, int balanced, float gam, float et,
@@ -223,30 +238,43 @@ __global__ void k_g_rev1(Rings R, const float* __restrict__ a_ring, const float*
   const int j = blockIdx.x, b = blockIdx.y;
   const size_t base = (size_t)b * R.npix + R.off[j];
   const int nk = R.len[j];
-  const float aj = a_ring[j];
-  const GScal s = sc[b];
-  const RevScal r = rs[b];
-  const float al = (float)s.al, be = (float)s.be;
+  // the problem's scalars in FP32, converted by one thread: left to every thread, the FP64 division
+  // and conversions (a small fraction of the FP32 rate) took most of the kernel's time
+  __shared__ float fs[5];
+  if (threadIdx.x == 0) {
+    const GScal s = sc[b];
+    const RevScal r = rs[b];
+    fs[0] = (float)s.al;
+    fs[1] = (float)s.be;
+    fs[2] = balanced ? (float)(r.sbar / a_ring[j]) : 0.f;
+    fs[3] = (float)r.Abar;
+    fs[4] = (float)r.Bbar;
+  }
+  __syncthreads();
+  const float al = fs[0], be = fs[1], sb = fs[2], Abar = fs[3], Bbar = fs[4];
   for (int k = threadIdx.x; k < nk; k += blockDim.x) {
     const float p = P[b][R.off[j] + k], q = Q[b][R.off[j] + k];
     const float u1 = U[base + k], v1 = V[base + k];
-    float uu, vv;
+    float uu, vv, qb = 0.f, vr = v1;   // qb: q~'s translation-invariant term; vr = v'^{1/g}
     if (balanced) {
-      uu = al * ut[base + k] + (float)(r.sbar / aj);
+      uu = al * ut[base + k] + sb;
       vv = be * vt[base + k];
     } else {
-      uu = al * ut[base + k] - (p > 0.f ? (float)r.Abar * et * p * powf(u1, -et - 1.f) : 0.f);
-      vv = be * vt[base + k] - (q > 0.f ? (float)r.Bbar * et * q * powf(v1, -et - 1.f) : 0.f);
-      pt[base + k] += (float)r.Abar * powf(u1, -et);
-      qt[base + k] += (float)r.Bbar * powf(v1, -et);
+      const float A = powf(u1, -et), B = powf(v1, -et);
+      uu = al * ut[base + k] - (p > 0.f ? Abar * et * p * (A / u1) : 0.f);
+      vv = be * vt[base + k] - (q > 0.f ? Bbar * et * q * (B / v1) : 0.f);
+      pt[base + k] += Abar * A;
+      qb = Bbar * B;
+      vr = v1 / B;
     }
     ut[base + k] = uu;
     if (q > 0.f) {
-      const float vg = balanced ? v1 * v1 : v1 * powf(v1, 1.f / gam);
-      kut[base + k] = -gam * vv * vg / q;
-      qt[base + k] += gam * vv * v1 / q;
+      const float w = gam * vv * v1 / q;
+      kut[base + k] = -w * vr;
+      qt[base + k] = qt[base + k] + qb + w;
     } else {
       kut[base + k] = 0.f;
+      if (!balanced) qt[base + k] += qb;
     }
   }
 }
@@ -481,11 +509,11 @@ int divergence_grad(Grid& g, const float* p, const float* q, int batch, double e
     int r;
     if ((r = heat_fields(g, vprev, kf, np, ps, st))) return r;
     count_launch();
-    k_g_update<<<ewp, kEw, 0, st>>>(rings, g.a_d, Pl, kf, uo, bal, gam, et, partU);
+    k_g_update<<<ewp, kEw, 0, st>>>(rings, g.a_d, Pl, kf, uo, bal, gam, partU);
     if ((r = heat_fields(g, uo, kf, np, nullptr, st))) return r;
     count_launch(2);
-    k_g_update<<<ewp, kEw, 0, st>>>(rings, g.a_d, Ql, kf, vo, bal, gam, et, partV);
-    k_g_scalars<<<nb, 128, 0, st>>>(np, g.nlat, partU, partV, bal, eps, tau, slot, ps);
+    k_g_update<<<ewp, kEw, 0, st>>>(rings, g.a_d, Ql, kf, vo, bal, gam, partV);
+    k_g_scalars<<<np, 32, 0, st>>>(g.nlat, partU, partV, bal, eps, tau, slot, ps);
     SHOT_CUDA(cudaGetLastError());
     return SHOT_OK;
   };
@@ -539,7 +567,7 @@ int divergence_grad(Grid& g, const float* p, const float* q, int batch, double e
       }
       count_launch(3);
       k_g_rsum<<<ewp, kEw, 0, st>>>(rings, g.a_d, ut, vt, U, V, partU, partV);
-      k_g_rscal<<<nb, 128, 0, st>>>(np, g.nlat, partU, partV, s_i, bal, eps, tau, rs);
+      k_g_rscal<<<np, 32, 0, st>>>(g.nlat, partU, partV, s_i, bal, eps, tau, rs);
       k_g_rev1<<<ewp, kEw, 0, st>>>(rings, g.a_d, Pl, Ql, U, V, s_i, rs, bal, gam, et, ut, vt, qt, t1, pt);
       SHOT_CUDA(cudaGetLastError());
       if ((rc = heat_fields(g, t1, t2, np, nullptr, st))) { cleanup2(); return rc; }

@@ -333,6 +333,7 @@ int build_grid_tables(Grid& g, cudaStream_t st) {
       }
       ring_plan[i] = pi;
     }
+    tw_base.push_back((int)tw_all.size());   // end of the last plan's table
     SHOT_CUDA(cudaMalloc(&g.ring_plan_d, nlat * sizeof(int)));
     SHOT_CUDA(cudaMemcpyAsync(g.ring_plan_d, ring_plan.data(), nlat * sizeof(int), cudaMemcpyHostToDevice, st));
     if (!plans.empty()) {

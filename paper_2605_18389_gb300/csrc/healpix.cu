@@ -30,12 +30,31 @@ namespace {
 // are short, and all CTAs of nside 64 and 8 fields are resident at once): 128 threads take most
 // stages in one step, the generic stage of a prime factor p in p steps.
 constexpr int kHpThreads = 128;
+// longest ring of the grids whose CTAs copy their ring's twiddles into shared memory (a table has at
+// most 2 n entries: n, and the roots of its generic stages)
+constexpr int kHpTwMax = 1024;
+// two sequences of the longest ring n and room for its twiddles
+size_t hp_smem(int n, int tws) { return (size_t)2 * seq_ld(n) * sizeof(C2) + (tws ? 2 * n * sizeof(float2) : 0); }
 
 // e^{i pi r / d} for an integer r reduced modulo 2d (exact argument reduction)
 __device__ __forceinline__ float2 half_turns(int r, int d) {
   float s, c;
   sincospif((float)(r % (2 * d)) / (float)d, &s, &c);
   return make_float2(c, s);
+}
+
+// The ring's plan and, where tws says so, its twiddles into shared memory (asynchronously: the
+// caller waits before the transform); returns where the twiddles are.
+__device__ __forceinline__ const float2* load_plan(FftPlan* pl, const FftPlan* __restrict__ plans, int pi,
+                                                   const float2* __restrict__ tw_all,
+                                                   const int* __restrict__ tw_base, float2* sm, int tws) {
+  const int* src = reinterpret_cast<const int*>(plans + pi);
+  for (int i = threadIdx.x; i < (int)(sizeof(FftPlan) / sizeof(int)); i += blockDim.x)
+    reinterpret_cast<int*>(pl)[i] = src[i];
+  const int base = tw_base[pi];
+  if (!tws) return tw_all + base;
+  fft_copy_twiddles(sm, tw_all + base, tw_base[pi + 1] - base);
+  return sm;
 }
 
 // from the transformed ring pair D: S = a (F_N + F_S), D = a (F_N - F_S) for m <= lmax into X
@@ -65,15 +84,17 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_fwd(const float* __restric
                                                        float area, float* __restrict__ X, int ldc,
                                                        const int* __restrict__ rplan, const FftPlan* __restrict__ plans,
                                                        const float2* __restrict__ tw_all,
-                                                       const int* __restrict__ tw_base,
+                                                       const int* __restrict__ tw_base, int tws,
                                                        const ProbState* __restrict__ ps) {
   extern __shared__ __align__(16) C2 sm[];
+  __shared__ FftPlan pl;
   const int jh = blockIdx.y, f0 = blockIdx.x * 2;
   const int j = jh, J = nrings - 1 - jh;
   const bool second = f0 + 1 < nf, two = J != j;
   const int n = rlen[j], pi = rplan[j];
   C2* zb = sm;
   C2* db = zb + seq_ld(n);
+  const float2* tw = load_plan(&pl, plans, pi, tw_all, tw_base, reinterpret_cast<float2*>(db + seq_ld(n)), tws);
   const float* fj = in + (size_t)f0 * npix + roff[j];
   const float* fJ = in + (size_t)f0 * npix + roff[J];
   for (int k = threadIdx.x; k < n; k += kHpThreads)
@@ -82,8 +103,9 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_fwd(const float* __restric
   // per-field factor (gradient sweeps)
   const float s0 = 0.5f * area * (ps ? (float)ps[f0].beta : 1.f);
   const float s1 = 0.5f * area * (ps && second ? (float)ps[f0 + 1].beta : 1.f);
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  const C2* D = fft_smem<false>(zb, db, tw_all + tw_base[pi], plans[pi], 1);
+  const C2* D = fft_smem<false>(zb, db, tw, pl, 1);
   hp_fold_store(D, n, rphase[j], f0, lmax, nh, jh, pk2(s0, s1), X, ldc);
 }
 
@@ -95,8 +117,9 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
                                                         const int* __restrict__ rplan,
                                                         const FftPlan* __restrict__ plans,
                                                         const float2* __restrict__ tw_all,
-                                                        const int* __restrict__ tw_base) {
+                                                        const int* __restrict__ tw_base, int tws) {
   extern __shared__ __align__(16) C2 sm[];
+  __shared__ FftPlan pl;
   __shared__ float red[kHpThreads / 32][2 * NPART];
   __shared__ EpiField fi[2];
   const int jh = blockIdx.y, f0 = blockIdx.x * 2;
@@ -108,6 +131,7 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
   const int2 phase = rphase[j];
   C2* za = sm;          // spectra Z
   C2* zb = za + ld;
+  const float2* tw = load_plan(&pl, plans, pi, tw_all, tw_base, reinterpret_cast<float2*>(zb + ld), tws);
   epi_fields_load<2>(ep, f0, nfg, fi);
   // Z_k = A_k + B_{n-k}: A_r sums e^{i m phi0} (G_N + i G_S) over the orders m >= 0 of residue r
   // modulo n, B_r sums e^{-i m phi0} (conj G_N + i conj G_S) over the orders m >= 1.  A thread owns
@@ -132,17 +156,17 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
       zb[r] = B;
     }
   }
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   epi_prefetch_marginals<2>(ep, fi, nfg, rj, rJ, two, n, f0, npix);
   for (int k = threadIdx.x; k < n; k += kHpThreads) za[k] = cadd(za[k], zb[k ? n - k : 0]);
   __syncthreads();
-  const float2* tw = tw_all + tw_base[pi];
-  C2* z = fft_smem<true>(za, zb, tw, plans[pi], 1);   // K v on the ring pair
+  C2* z = fft_smem<true>(za, zb, tw, pl, 1);   // K v on the ring pair
   C2* other = (z == za) ? zb : za;   // receives the new scaling
   ring_pair_epilogue<1, kHpThreads>(z, other, ld, n, nf, f0, npix, rj, rJ, two, area, nh, jh, ep, red, fi);
   if ((ep.mode == EPI_UPDATE || ep.mode == EPI_SYM) && ep.xout) {   // transform the new scaling
     __syncthreads();
-    const C2* D = fft_smem<false>(other, z, tw, plans[pi], 1);
+    const C2* D = fft_smem<false>(other, z, tw, pl, 1);
     hp_fold_store(D, n, phase, f0, lmax, nh, jh, pk2(0.5f * area, 0.5f * area), ep.xout, ldc);
   }
 }
@@ -151,25 +175,27 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
 
 int launch_hp_dft_fwd(const Grid& g, const float* in, int nf, float* X, int ldc, cudaStream_t st,
                       const ProbState* ps) {
-  const size_t smem = (size_t)2 * seq_ld(g.nlon) * sizeof(C2);   // nlon: the longest ring
+  const int tws = g.nlon <= kHpTwMax;
+  const size_t smem = hp_smem(g.nlon, tws);
   SHOT_CUDA(cudaFuncSetAttribute(k_hp_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   ProfScope prof(PK_DFT, st);
   count_launch();
   k_hp_fwd<<<dim3((nf + 1) / 2, g.nh), kHpThreads, smem, st>>>(
       in, nf, g.npix, g.ring_len_d, g.ring_off_d, g.ring_phase_d, g.nlat, g.lmax, g.nh, (float)g.a_ring[0], X, ldc,
-      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d, ps);
+      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d, tws, ps);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
 }
 
 int launch_hp_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st) {
-  const size_t smem = (size_t)2 * seq_ld(g.nlon) * sizeof(C2);
+  const int tws = g.nlon <= kHpTwMax;
+  const size_t smem = hp_smem(g.nlon, tws);
   SHOT_CUDA(cudaFuncSetAttribute(k_hp_idft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   ProfScope prof(ep.mode == EPI_CHECK || ep.mode == EPI_FINAL ? PK_CHECK : PK_IDFT, st);
   count_launch();
   k_hp_idft<<<dim3((nf + 1) / 2, g.nh), kHpThreads, smem, st>>>(
       Y, ldc, nf, g.npix, g.ring_len_d, g.ring_off_d, g.ring_phase_d, g.nlat, g.lmax, g.nh, (float)g.a_ring[0], ep,
-      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d);
+      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d, tws);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
 }

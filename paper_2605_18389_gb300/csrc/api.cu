@@ -326,7 +326,7 @@ Grid* as_grid(shot_grid g) { return reinterpret_cast<Grid*>(g); }
 
 int heat_pipeline(Grid& g, const float* in, int nf, int scale_which, cudaStream_t st) {
   Workspace& w = g.ws;
-  int rc = launch_dft_fwd(g, in, nf, reinterpret_cast<ProbState*>(w.probs), scale_which, w.XY, w.ldc, st);
+  int rc = launch_dft_fwd(g, in, nf, reinterpret_cast<ProbState*>(w.probs), scale_which, w.XY, w.ldc, st, g.mlim_d);
   if (rc) return rc;
   return launch_legendre(g, nf, w.XY, w.C, w.XY, w.ldc, st);
 }
@@ -414,7 +414,7 @@ int solve_prepare(Grid& g, const std::vector<const float*>& P, const std::vector
   if ((rc = autotune(g, nprob, s.st))) return rc;
   if ((rc = launch_heat_mult(g, eps / 4.0, s.st))) return rc;
   // spectra of the starting v
-  return launch_dft_fwd(g, v, nprob, nullptr, 0, w.XY, w.ldc, s.st);
+  return launch_dft_fwd(g, v, nprob, nullptr, 0, w.XY, w.ldc, s.st, g.mlim_d);
 }
 
 EpiParams base_ep(Solve& s) {
@@ -424,6 +424,7 @@ EpiParams base_ep(Solve& s) {
   ep.part = w.part;
   ep.eps = s.eps;
   ep.norm_l1 = s.norm_l1;
+  ep.mlim = s.g->mlim_d;
   return ep;
 }
 
@@ -826,7 +827,7 @@ int shot_grid_free(shot_grid gh) {
   Grid* g = as_grid(gh);
   if (!g) return SHOT_OK;
   void* dptr[] = {g->ring_len_d, g->ring_off_d, g->ring_phase_d, g->hp_plan_d, g->ring_plan_d, g->hp_tw_d, g->hp_tw_base_d, g->xyz_d, g->ws.Yb, g->x_d, g->w_d, g->a_d, g->tw_d, g->h_d, g->tab, g->tabT, g->tab_hi, g->tab_lo,
-                  g->ws.ct_hi, g->ws.ct_lo, g->ws.ct32, g->rec_seeds, g->rec_coef, g->rec_coef_off, g->rec_x, g->ck, g->ck_off_d, g->M_d,
+                  g->ws.ct_hi, g->ws.ct_lo, g->ws.ct32, g->rec_seeds, g->rec_coef, g->rec_coef_off, g->rec_x, g->ck, g->ck_off_d, g->M_d, g->mlim_d,
                   g->row_off_d, g->tiles_ana, g->tiles_syn, g->ws.XY, g->ws.C, g->ws.part, g->ws.probs,
                   g->ws.marg, g->ws.ubuf, g->ws.vbuf, g->ws.dev_int};
   for (void* p : dptr)
@@ -909,6 +910,7 @@ int shot_heat_apply(shot_grid gh, double t, const float* in, float* out, int nfi
   EpiParams ep{};
   ep.mode = EPI_PLAIN;
   ep.out = out;
+  ep.mlim = g->mlim_d;
   return launch_idft(*g, g->ws.XY, g->ws.ldc, nfields, ep, st);
 }
 

@@ -79,14 +79,14 @@ __device__ __forceinline__ void load_ring_pairs(const float* __restrict__ in, C2
   }
 }
 
-// Starts the gather of the ring pair's spectra of the CTA's fields, E_m and O_m for every order
-// (the (2m+1) block of m = lmax is empty), into stg[blk][G] with asynchronous copies.  Row (blk,
+// Starts the gather of the ring pair's spectra of the CTA's fields, E_m and O_m for the orders up to
+// mmax (the (2m+1) block of m = lmax is empty), into stg[blk][G] with asynchronous copies.  Row (blk,
 // jh) holds the fields' (re, im) pairs contiguously; an even first field starts on a 16-byte
 // boundary (ldc is a multiple of 4), and reading up to the next even field stays inside the row.
 template <int G, int NT>
-__device__ __forceinline__ void issue_spectra(const float* __restrict__ Y, int ldc, int nh, int lmax, int jh, int f0,
+__device__ __forceinline__ void issue_spectra(const float* __restrict__ Y, int ldc, int nh, int mmax, int lmax, int jh, int f0,
                                               int nf, float4* stg) {
-  const int nblk = 2 * lmax + 1;
+  const int nblk = min(2 * mmax + 2, 2 * lmax + 1);
   const float* y = Y + (size_t)jh * ldc + 2 * f0;
   const size_t row = (size_t)nh * ldc;
   if (G == 1) {
@@ -102,13 +102,13 @@ __device__ __forceinline__ void issue_spectra(const float* __restrict__ Y, int l
 
 // Unfolds the staged spectra into the Hermitian-extended Z of each pair of fields:
 // G_N = E + O, G_S = E - O, Z(m) = G_N + i G_S, Z(N-m) = conj G_N + i conj G_S; the band
-// lmax < m < N - lmax is zero.
+// mmax < m < N - mmax is zero.
 template <int G, int NT>
-__device__ __forceinline__ void unfold_spectra(const float4* stg, C2* buf, int N, int lmax) {
+__device__ __forceinline__ void unfold_spectra(const float4* stg, C2* buf, int N, int mmax, int lmax) {
   const Group<G, NT> gr;
   C2* z = buf + gr.g * seq_ld(N);
-  for (int k = lmax + 1 + gr.t; k < N - lmax; k += gr.T) z[k] = c2(0ull, 0ull);
-  for (int m = gr.t; m <= lmax; m += gr.T) {
+  for (int k = mmax + 1 + gr.t; k < N - mmax; k += gr.T) z[k] = c2(0ull, 0ull);
+  for (int m = gr.t; m <= mmax; m += gr.T) {
     const float4 e = stg[2 * m * G + gr.g];
     const float4 o = m < lmax ? stg[(2 * m + 1) * G + gr.g] : make_float4(0.f, 0.f, 0.f, 0.f);
     const C2 E = c2(pk2(e.x, e.z), pk2(e.y, e.w)), O = c2(pk2(o.x, o.z), pk2(o.y, o.w));
@@ -124,10 +124,10 @@ __device__ __forceinline__ void unfold_spectra(const float4* stg, C2* buf, int N
 
 // Two-for-one unpack of the transformed ring pair (j north, J south) and the parity fold:
 // F_N(m) = (Z(m) + conj Z(N-m))/2, F_S(m) = (Z(m) - conj Z(N-m))/(2i);
-// S = a_j (F_N + F_S) -> block (m, even), D = a_j (F_N - F_S) -> block (m, odd).
+// S = a_j (F_N + F_S) -> block (m, even), D = a_j (F_N - F_S) -> block (m, odd), m <= mmax.
 // The columns of an odd last field's missing partner (padding, inside ldc) take its zeros.
 template <int G, int NT>
-__device__ __forceinline__ void fold_store(const C2* buf, int f0, int nf, int N, int lmax, int nh, int jh, float aj,
+__device__ __forceinline__ void fold_store(const C2* buf, int f0, int nf, int N, int mmax, int nh, int jh, float aj,
                                            const ProbState* __restrict__ ps, int scale_which, float* __restrict__ X,
                                            int ldc) {
   const Group<G, NT> gr;
@@ -142,7 +142,7 @@ __device__ __forceinline__ void fold_store(const C2* buf, int f0, int nf, int N,
   const C2* z = buf + gr.g * seq_ld(N);
   float* x = X + (size_t)jh * ldc + 2 * fa;
   const size_t row = (size_t)nh * ldc;
-  for (int m = gr.t; m <= lmax; m += gr.T) {
+  for (int m = gr.t; m <= mmax; m += gr.T) {
     const C2 zm = z[m], zn = z[m ? N - m : 0];
     const f32x2 a = add2(zm.re, zn.re), b = sub2(zm.im, zn.im);   // 2 F_N
     const f32x2 c = add2(zm.im, zn.im), d = sub2(zm.re, zn.re);   // 2 F_S = (c, -d)
@@ -158,7 +158,8 @@ template <int G, int NT, int CTAS, class PL>
 __global__ void __launch_bounds__(NT, CTAS) k_dft_fwd(
     const float* __restrict__ in, int nf, int nlat, int nlon, int lmax, int nh,
     const float* __restrict__ a_ring, const ProbState* __restrict__ ps, int scale_which,
-    float* __restrict__ X, int ldc, const __grid_constant__ FftPlan pl, const float2* tw, int tws) {
+    float* __restrict__ X, int ldc, const __grid_constant__ FftPlan pl, const float2* tw, int tws,
+    const int2* __restrict__ mlim) {
   extern __shared__ __align__(16) C2 sm[];
   C2* b0 = sm;
   C2* b1 = b0 + G * seq_ld(nlon);
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_dft_fwd(
   cp_async_wait_all();
   __syncthreads();
   const C2* buf = fft_smem_plan<false, PL>(b0, b1, tw, pl, G);
-  fold_store<G, NT>(buf, f0, nf, nlon, lmax, nh, jh, a_ring[jh], ps, scale_which, X, ldc);
+  fold_store<G, NT>(buf, f0, nf, nlon, mlim ? mlim[jh].y : lmax, nh, jh, a_ring[jh], ps, scale_which, X, ldc);
 }
 
 template <int G, int NT, int CTAS, class PL>
@@ -193,13 +194,14 @@ __global__ void __launch_bounds__(NT, CTAS) k_idft(
     tw = reinterpret_cast<const float2*>(b1 + G * ld);
   }
   float4* stg = reinterpret_cast<float4*>(b1);   // the spectra, before the transform needs b1
-  issue_spectra<G, NT>(Y, ldc, nh, lmax, jh, f0, nf, stg);
+  const int2 ml = ep.mlim ? ep.mlim[jh] : make_int2(lmax, lmax);   // orders read, orders written
+  issue_spectra<G, NT>(Y, ldc, nh, ml.x, lmax, jh, f0, nf, stg);
   const int nfg = min(2 * G, nf - f0);
   epi_fields_load<2 * G>(ep, f0, nfg, fi);
   cp_async_wait_all();
   __syncthreads();
   epi_prefetch_marginals<2 * G>(ep, fi, nfg, (size_t)j * N, (size_t)J * N, two, N, f0, (size_t)nlat * N);
-  unfold_spectra<G, NT>(stg, buf, N, lmax);
+  unfold_spectra<G, NT>(stg, buf, N, ml.x, lmax);
   __syncthreads();
   const C2* z = fft_smem_plan<true, PL>(buf, b1, tw, pl, G);
   C2* other = (z == buf) ? b1 : buf;   // input of the fused forward transform
@@ -211,7 +213,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_idft(
     // the new scaling of this ring pair is in `other`: transform it for the next half-step
     __syncthreads();
     const C2* zf = fft_smem_plan<false, PL>(other, const_cast<C2*>(z), tw, pl, G);
-    fold_store<G, NT>(zf, f0, nf, N, lmax, nh, jh, aj, nullptr, 0, ep.xout, ldc);
+    fold_store<G, NT>(zf, f0, nf, N, ml.y, nh, jh, aj, nullptr, 0, ep.xout, ldc);
   }
 }
 
@@ -251,11 +253,12 @@ __global__ void __launch_bounds__(NT, CTAS) k_idft_p(
   const int nitems = ngroups * nh;
   const size_t fs = (size_t)nlat * N;
 
+  auto orders = [&](int j) { return ep.mlim ? ep.mlim[j] : make_int2(lmax, lmax); };   // read, written
   int item = blockIdx.x, slot = 0;
   int jh = item / ngroups, f0 = (item - jh * ngroups) * FG;
   if (item < nitems) {
     epi_fields_load<FG>(ep, f0, min(FG, nf - f0), fi[0]);
-    issue_spectra<G, NT>(Y, ldc, nh, lmax, jh, f0, nf, stg);
+    issue_spectra<G, NT>(Y, ldc, nh, orders(jh).x, lmax, jh, f0, nf, stg);
   }
   __syncthreads();
   if (item < nitems)
@@ -265,13 +268,14 @@ __global__ void __launch_bounds__(NT, CTAS) k_idft_p(
     const int next = item + gridDim.x;
     const int jn = next / ngroups, fn = (next - jn * ngroups) * FG, nn = min(FG, nf - fn);
     const int j = jh, J = nlat - 1 - jh;
+    const int2 ml = orders(jh);
     cp_async_wait_all();   // this item's spectra
     __syncthreads();
-    unfold_spectra<G, NT>(stg, buf, N, lmax);
+    unfold_spectra<G, NT>(stg, buf, N, ml.x, lmax);
     __syncthreads();
     if (next < nitems) {   // the staging area is free again: the next item's state and spectra
       epi_fields_load<FG>(ep, fn, nn, fi[slot ^ 1]);
-      issue_spectra<G, NT>(Y, ldc, nh, lmax, jn, fn, nf, stg);
+      issue_spectra<G, NT>(Y, ldc, nh, orders(jn).x, lmax, jn, fn, nf, stg);
     }
     const C2* z = fft_smem_plan<true, PL, INPLACE>(buf, b1, tw, pl, G);
     C2* other = (z == buf) ? b1 : buf;   // INPLACE: an element's new scaling replaces its K v
@@ -285,7 +289,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_idft_p(
     if (ep.xout) {   // the update's new scaling: its spectra for the next half-step
       __syncthreads();
       const C2* zf = fft_smem_plan<false, PL, INPLACE>(other, const_cast<C2*>(z), tw, pl, G);
-      fold_store<G, NT>(zf, f0, nf, N, lmax, nh, jh, aj, nullptr, 0, ep.xout, ldc);
+      fold_store<G, NT>(zf, f0, nf, N, ml.y, nh, jh, aj, nullptr, 0, ep.xout, ldc);
     }
     item = next;
     jh = jn;
@@ -318,7 +322,7 @@ size_t idft_smem(int G, int N) { return (size_t)2 * G * seq_ld(N) * sizeof(C2); 
 
 template <int G, class PL = RuntimePlan, int NT = kThreads, int CTAS = kCtas>
 int launch_fwd_t(const Grid& g, const float* in, int nf, const ProbState* ps, int scale_which, float* X,
-                 int ldc, cudaStream_t st) {
+                 int ldc, cudaStream_t st, const int2* mlim) {
   const int tws = twiddles_in_smem(g);
   const size_t smem = idft_smem(G, g.nlon) + tws * sizeof(float2);
   SHOT_CUDA(cudaFuncSetAttribute(k_dft_fwd<G, NT, CTAS, PL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -326,7 +330,7 @@ int launch_fwd_t(const Grid& g, const float* in, int nf, const ProbState* ps, in
   ProfScope prof(PK_DFT, st);
   count_launch();
   k_dft_fwd<G, NT, CTAS, PL><<<grid, NT, smem, st>>>(in, nf, g.nlat, g.nlon, g.lmax, g.nh, g.a_d, ps, scale_which, X,
-                                                 ldc, g.plan, g.tw_d, tws);
+                                                 ldc, g.plan, g.tw_d, tws, mlim);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
 }
@@ -374,26 +378,26 @@ using Plan1024 = CtPlan<1024, 4, 16, 16>;
 int dft_fields_per_cta(const Grid& g, int nf) { return g.quad == SHOT_QUAD_HEALPIX ? 2 : 2 * pick_g(g, nf); }
 
 int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, int scale_which,
-                   float* X, int ldc, cudaStream_t st) {
+                   float* X, int ldc, cudaStream_t st, const int2* mlim) {
   if (g.quad == SHOT_QUAD_HEALPIX) {
     if (scale_which && scale_which != 1) {
       set_error("HEALPix ring transform: the per-field factor beta only");
       return SHOT_ERR_UNSUPPORTED;
     }
-    return launch_hp_dft_fwd(g, in, nf, X, ldc, st, scale_which == 1 ? ps : nullptr);
+    return launch_hp_dft_fwd(g, in, nf, X, ldc, st, scale_which == 1 ? ps : nullptr, mlim);
   }
   if (g.nlon > kFftCap) {
     set_error("nlon too large for the shared-memory ring FFT");
     return SHOT_ERR_UNSUPPORTED;
   }
   switch (pick_g(g, nf)) {
-    case 6: return launch_fwd_t<6>(g, in, nf, ps, scale_which, X, ldc, st);
-    case 3: return launch_fwd_t<3>(g, in, nf, ps, scale_which, X, ldc, st);
-    case 2: return launch_fwd_t<2>(g, in, nf, ps, scale_which, X, ldc, st);
+    case 6: return launch_fwd_t<6>(g, in, nf, ps, scale_which, X, ldc, st, mlim);
+    case 3: return launch_fwd_t<3>(g, in, nf, ps, scale_which, X, ldc, st, mlim);
+    case 2: return launch_fwd_t<2>(g, in, nf, ps, scale_which, X, ldc, st, mlim);
     default:
-      if (plan_is<Plan1440>(g.plan)) return launch_fwd_t<1, Plan1440, 192, 4>(g, in, nf, ps, scale_which, X, ldc, st);
-      if (plan_is<Plan1024>(g.plan)) return launch_fwd_t<1, Plan1024>(g, in, nf, ps, scale_which, X, ldc, st);
-      return launch_fwd_t<1>(g, in, nf, ps, scale_which, X, ldc, st);
+      if (plan_is<Plan1440>(g.plan)) return launch_fwd_t<1, Plan1440, 192, 4>(g, in, nf, ps, scale_which, X, ldc, st, mlim);
+      if (plan_is<Plan1024>(g.plan)) return launch_fwd_t<1, Plan1024>(g, in, nf, ps, scale_which, X, ldc, st, mlim);
+      return launch_fwd_t<1>(g, in, nf, ps, scale_which, X, ldc, st, mlim);
   }
 }
 

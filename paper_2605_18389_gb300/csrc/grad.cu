@@ -376,12 +376,13 @@ __global__ void k_g_mass_diff(Rings R, const float* __restrict__ p, const float*
 // out = K (beta (.) in) (beta per problem from ps when ps != nullptr)
 static int heat_fields(Grid& g, const float* in, float* out, int nf, const ProbState* ps, cudaStream_t st) {
   Workspace& w = g.ws;
-  int rc = launch_dft_fwd(g, in, nf, ps, ps ? 1 : 0, w.XY, w.ldc, st);
+  int rc = launch_dft_fwd(g, in, nf, ps, ps ? 1 : 0, w.XY, w.ldc, st, g.mlim_d);
   if (rc) return rc;
   if ((rc = launch_legendre(g, nf, w.XY, w.C, w.XY, w.ldc, st))) return rc;
   EpiParams ep{};
   ep.mode = EPI_PLAIN;
   ep.out = out;
+  ep.mlim = g.mlim_d;
   return launch_idft(g, w.XY, w.ldc, nf, ep, st);
 }
 

@@ -95,9 +95,11 @@ __global__ void k_area(int nlat, int nlon, const double* __restrict__ w, float* 
 //   a_lm = sqrt((4l^2-1)/(l^2-m^2)), b_lm = sqrt(((l-1)^2-m^2)/(4(l-1)^2-1)).
 // One thread per (m, jh); row l goes to block (m, (l-m) mod 2), row (l-m)/2.
 // tabT (optional): the same values at [blk][jh][ldi] (degrees contiguous).
+// lfirst[m nh + jh]: the first degree with |Pbar| >= kPolarCut (lmax + 1: none), when asked for.
 __global__ void k_pbar(int lmax, int nh, const double* __restrict__ x, const long long* __restrict__ row_off,
                        int ldt, float* __restrict__ tab, __nv_bfloat16* __restrict__ hi,
-                       __nv_bfloat16* __restrict__ lo, float* __restrict__ tabT, int ldi) {
+                       __nv_bfloat16* __restrict__ lo, float* __restrict__ tabT, int ldi,
+                       int* __restrict__ lfirst) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = blockIdx.y;
   if (j >= nh) return;
@@ -105,7 +107,12 @@ __global__ void k_pbar(int lmax, int nh, const double* __restrict__ x, const lon
   const double st = sqrt((1.0 - xj) * (1.0 + xj));
   double pmm = 0.28209479177387814;   // 1/sqrt(4 pi)
   for (int k = 1; k <= m; ++k) pmm *= -sqrt((2.0 * k + 1.0) / (2.0 * k)) * st;
+  int first = lmax + 1;
   auto store = [&](int l, double val) {
+    if (first > lmax && fabs(val) >= kPolarCut) {
+      first = l;
+      if (lfirst) lfirst[(size_t)m * nh + j] = l;
+    }
     const int d = l - m;
     const int blk = 2 * m + (d & 1);
     const size_t off = (size_t)(row_off[blk] + (d >> 1)) * ldt + j;
@@ -118,6 +125,7 @@ __global__ void k_pbar(int lmax, int nh, const double* __restrict__ x, const lon
       lo[off] = l;
     }
   };
+  if (lfirst) lfirst[(size_t)m * nh + j] = lmax + 1;
   store(m, pmm);
   if (m == lmax) return;
   double p2 = pmm;
@@ -395,8 +403,19 @@ int build_grid_tables(Grid& g, cudaStream_t st) {
   float* tab = nullptr;
   __nv_bfloat16 *hi = nullptr, *lo = nullptr;
   g.ldi = (g.M[0] + 7) / 8 * 8;
+  // first degrees above the cut, after the order limits in one allocation.  None in the FP32
+  // recurrence mode, which has its own seeds, and none below degree 64: no chunk of 16 terms of any
+  // tile would go (128 rings: 4 % of the analysis' terms; 256: 6 %; 720: 17 %).
+  std::vector<int> lfirst;
+  int* lfirst_d = nullptr;
+  const bool polar = g.lmax >= 64 && (g.mode != SHOT_RECURRENCE || tf32_kernels(g));
+  if (polar) {
+    lfirst.resize((size_t)L * nh);
+    SHOT_CUDA(cudaMalloc(&g.mlim_d, nh * sizeof(int2) + lfirst.size() * sizeof(int)));
+    lfirst_d = reinterpret_cast<int*>(g.mlim_d + nh);
+  }
   if (g.mode == SHOT_RECURRENCE) {
-    int rc = tf32_kernels(g) ? build_tf32_recurrence(g, st) : build_recurrence(g, st);
+    int rc = tf32_kernels(g) ? build_tf32_recurrence(g, lfirst_d, st) : build_recurrence(g, st);
     if (rc) return rc;
   } else {
   float* tabT = nullptr;
@@ -420,16 +439,58 @@ int build_grid_tables(Grid& g, cudaStream_t st) {
   }
   dim3 gp((nh + 127) / 128, L);
   count_launch();
-  k_pbar<<<gp, 128, 0, st>>>(g.lmax, nh, g.x_d, g.row_off_d, g.ldt, tab, hi, lo, tabT, g.ldi);
+  k_pbar<<<gp, 128, 0, st>>>(g.lmax, nh, g.x_d, g.row_off_d, g.ldt, tab, hi, lo, tabT, g.ldi, lfirst_d);
   SHOT_CUDA(cudaGetLastError());
+  }
+
+  if (polar) {
+    SHOT_CUDA(cudaMemcpyAsync(lfirst.data(), lfirst_d, lfirst.size() * sizeof(int), cudaMemcpyDeviceToHost, st));
+    SHOT_CUDA(cudaStreamSynchronize(st));
+  }
+  // first terms of a tile's sums: analysis, rows up to i_last of block (m, p): the first node whose
+  // function of the highest degree (so of any) is above the cut; synthesis, nodes j0 .. j1 - 1: the
+  // first degree above the cut at any of them.  At least the last chunk of a sum always runs.
+  auto ana_start = [&](int m, int p, int i_last) {
+    const int l = m + p + 2 * i_last;
+    int j = 0;
+    while (j < nh - 1 && lfirst[(size_t)m * nh + j] > l) ++j;
+    return j & ~15;
+  };
+  auto syn_start = [&](int m, int p, int j0, int j1) {
+    int l = g.lmax + 1;
+    for (int j = j0; j < j1; ++j) l = std::min(l, lfirst[(size_t)m * nh + j]);
+    return std::min(std::max(l - m - p + 1, 0) / 2, g.M[2 * m + p] - 1) & ~15;
+  };
+  if (polar) {
+    std::vector<int2> mlim(nh, make_int2(0, 0));
+    for (int m = 0; m < L; ++m) {
+      int need = nh - 1;   // first ring whose spectra of order m some tile reads
+      for (int j = nh - 1; j >= 0; --j)
+        if (lfirst[(size_t)m * nh + j] <= g.lmax) {
+          need = j;
+          mlim[j].x = m;
+        }
+      for (int j = need / kPolarAlign * kPolarAlign; j < nh; ++j) mlim[j].y = m;
+    }
+    SHOT_CUDA(cudaMemcpyAsync(g.mlim_d, mlim.data(), nh * sizeof(int2), cudaMemcpyHostToDevice, st));
+    SHOT_CUDA(cudaStreamSynchronize(st));   // mlim is a local
   }
 
   // tile lists: analysis tiles cover the rows i of each block, synthesis tiles the nodes
   std::vector<Tile> ta, ts;
   for (int b = 0; b < g.nblk; ++b) {
-    for (int r = 0; r < g.M[b]; r += g.bm_ana) ta.push_back({b, r});
-    if (g.M[b] > 0)
-      for (int r = 0; r < nh; r += g.bm_syn) ts.push_back({b, r});
+    const int m = b >> 1, p = b & 1, M = g.M[b];
+    for (int r = 0; r < M; r += g.bm_ana) {
+      Tile t{b, r, {0, 0}};
+      for (int h = 0; polar && h < 2; ++h) t.k0[h] = ana_start(m, p, std::min(r + 64 * (h + 1), M) - 1);
+      ta.push_back(t);
+    }
+    for (int r = 0; M > 0 && r < nh; r += g.bm_syn) {
+      Tile t{b, r, {0, 0}};
+      for (int h = 0; polar && h < 2; ++h)
+        t.k0[h] = r + 64 * h < nh ? syn_start(m, p, r + 64 * h, std::min(r + 64 * (h + 1), nh)) : t.k0[0];
+      ts.push_back(t);
+    }
   }
   // largest contraction first (synthesis work is proportional to M)
   std::stable_sort(ts.begin(), ts.end(), [&](const Tile& a, const Tile& b) { return g.M[a.blk] > g.M[b.blk]; });

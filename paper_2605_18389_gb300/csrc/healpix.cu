@@ -57,13 +57,13 @@ __device__ __forceinline__ const float2* load_plan(FftPlan* pl, const FftPlan* _
   return sm;
 }
 
-// from the transformed ring pair D: S = a (F_N + F_S), D = a (F_N - F_S) for m <= lmax into X
+// from the transformed ring pair D: S = a (F_N + F_S), D = a (F_N - F_S) for m <= mmax into X
 // (sc = a / 2 per field, with the field's factor), each order turned by e^{-i m phi0}
-__device__ __forceinline__ void hp_fold_store(const C2* D, int n, int2 phase, int f0, int lmax, int nh, int jh, f32x2 sc,
+__device__ __forceinline__ void hp_fold_store(const C2* D, int n, int2 phase, int f0, int mmax, int nh, int jh, f32x2 sc,
                                               float* __restrict__ X, int ldc) {
   float* x = X + (size_t)jh * ldc + 2 * f0;
   const size_t row = (size_t)nh * ldc;
-  for (int m = threadIdx.x; m <= lmax; m += kHpThreads) {
+  for (int m = threadIdx.x; m <= mmax; m += kHpThreads) {
     const int k = m % n;
     const C2 zm = D[k], zn = D[k ? n - k : 0];
     const float2 e = half_turns(m * phase.x, phase.y);
@@ -85,7 +85,8 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_fwd(const float* __restric
                                                        const int* __restrict__ rplan, const FftPlan* __restrict__ plans,
                                                        const float2* __restrict__ tw_all,
                                                        const int* __restrict__ tw_base, int tws,
-                                                       const ProbState* __restrict__ ps) {
+                                                       const ProbState* __restrict__ ps,
+                                                       const int2* __restrict__ mlim) {
   extern __shared__ __align__(16) C2 sm[];
   __shared__ FftPlan pl;
   const int jh = blockIdx.y, f0 = blockIdx.x * 2;
@@ -106,7 +107,7 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_fwd(const float* __restric
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   const C2* D = fft_smem<false>(zb, db, tw, pl, 1);
-  hp_fold_store(D, n, rphase[j], f0, lmax, nh, jh, pk2(s0, s1), X, ldc);
+  hp_fold_store(D, n, rphase[j], f0, mlim ? mlim[jh].y : lmax, nh, jh, pk2(s0, s1), X, ldc);
 }
 
 __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restrict__ Y, int ldc, int nf, size_t npix,
@@ -129,6 +130,7 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
   const int n = rlen[j], ld = seq_ld(n), pi = rplan[j];
   const size_t rj = (size_t)roff[j], rJ = (size_t)roff[J];
   const int2 phase = rphase[j];
+  const int2 ml = ep.mlim ? ep.mlim[jh] : make_int2(lmax, lmax);   // orders read, orders written
   C2* za = sm;          // spectra Z
   C2* zb = za + ld;
   const float2* tw = load_plan(&pl, plans, pi, tw_all, tw_base, reinterpret_cast<float2*>(zb + ld), tws);
@@ -142,7 +144,7 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
     for (int r = threadIdx.x; r < n; r += kHpThreads) {
       C2 A = c2(0ull, 0ull), B = A;
 #pragma unroll 4
-      for (int m = r; m <= lmax; m += n) {
+      for (int m = r; m <= ml.x; m += n) {
         const float4 e = *reinterpret_cast<const float4*>(y + (size_t)(2 * m) * row);
         const float4 o = m < lmax ? *reinterpret_cast<const float4*>(y + (size_t)(2 * m + 1) * row)
                                   : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -167,14 +169,14 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
   if ((ep.mode == EPI_UPDATE || ep.mode == EPI_SYM) && ep.xout) {   // transform the new scaling
     __syncthreads();
     const C2* D = fft_smem<false>(other, z, tw, pl, 1);
-    hp_fold_store(D, n, phase, f0, lmax, nh, jh, pk2(0.5f * area, 0.5f * area), ep.xout, ldc);
+    hp_fold_store(D, n, phase, f0, ml.y, nh, jh, pk2(0.5f * area, 0.5f * area), ep.xout, ldc);
   }
 }
 
 }  // namespace
 
 int launch_hp_dft_fwd(const Grid& g, const float* in, int nf, float* X, int ldc, cudaStream_t st,
-                      const ProbState* ps) {
+                      const ProbState* ps, const int2* mlim) {
   const int tws = g.nlon <= kHpTwMax;
   const size_t smem = hp_smem(g.nlon, tws);
   SHOT_CUDA(cudaFuncSetAttribute(k_hp_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -182,7 +184,7 @@ int launch_hp_dft_fwd(const Grid& g, const float* in, int nf, float* X, int ldc,
   count_launch();
   k_hp_fwd<<<dim3((nf + 1) / 2, g.nh), kHpThreads, smem, st>>>(
       in, nf, g.npix, g.ring_len_d, g.ring_off_d, g.ring_phase_d, g.nlat, g.lmax, g.nh, (float)g.a_ring[0], X, ldc,
-      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d, tws, ps);
+      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d, tws, ps, mlim);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
 }

@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(NT, TN >= 6 ? 8 : 10) k_legendre_simt(
     const Tile* __restrict__ tiles, int ncolt, const float* __restrict__ tab, int ldt,
     const long long* __restrict__ row_off, const int* __restrict__ Mrows, int nh,
     const float* __restrict__ Bsrc, int ldc, int ncols, float* __restrict__ out,
-    const float* __restrict__ h) {
+    const float* __restrict__ h, int polar) {
   constexpr int BN = 8 * TN, NP = TN / 2;
   // [stage]: A (analysis: 64 rows of 16 terms, the 16-byte pieces of rows 2 i and 2 i + 1 permuted
   // by i so that the rows a warp reads together lie on different banks; synthesis: 16 terms of 64
@@ -75,6 +75,7 @@ __global__ void __launch_bounds__(NT, TN >= 6 ? 8 : 10) k_legendre_simt(
   const int K = ANALYSIS ? nh : M;
   const int mvalid = ANALYSIS ? M : nh;   // rows of the output block
   if (r0 >= mvalid) return;
+  const int ks = polar ? tl.k0[half & 1] : 0;   // first term of the sums
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tn = lane & 7, tm = lane >> 3;
@@ -115,11 +116,11 @@ __global__ void __launch_bounds__(NT, TN >= 6 ? 8 : 10) k_legendre_simt(
 
 #pragma unroll
   for (int t = 0; t < kSimtStages - 1; ++t) {
-    if (t * BK < K) load(t * BK, t);
+    if (ks + t * BK < K) load(ks + t * BK, t);
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
   int s = 0;
-  for (int kt = 0; kt < K; kt += BK) {
+  for (int kt = ks; kt < K; kt += BK) {
     asm volatile("cp.async.wait_group %0;" ::"n"(kSimtStages - 2) : "memory");
     __syncthreads();   // this chunk has landed for both warps, and the one before it has been read
     if (kt + (kSimtStages - 1) * BK < K) load(kt + (kSimtStages - 1) * BK, s == 0 ? kSimtStages - 1 : s - 1);
@@ -194,12 +195,13 @@ __global__ void __launch_bounds__(NT, TN >= 6 ? 8 : 10) k_legendre_simt(
 }
 
 template <int TN, bool ANALYSIS>
-int launch_one(const Grid& g, int nf, const float* B, float* out, int ldc, const float* h, cudaStream_t st) {
+int launch_one(const Grid& g, int nf, const float* B, float* out, int ldc, const float* h, bool polar,
+               cudaStream_t st) {
   const int ncols = 2 * nf, ncolt = (ncols + 8 * TN - 1) / (8 * TN);
   ProfScope prof(ANALYSIS ? PK_ANALYSIS : PK_SYNTHESIS, st);
   count_launch();
   k_legendre_simt<TN, ANALYSIS><<<2 * (ANALYSIS ? g.ntiles_ana : g.ntiles_syn) * ncolt, NT, 0, st>>>(
-      ANALYSIS ? g.tiles_ana : g.tiles_syn, ncolt, g.tab, g.ldt, g.row_off_d, g.M_d, g.nh, B, ldc, ncols, out, h);
+      ANALYSIS ? g.tiles_ana : g.tiles_syn, ncolt, g.tab, g.ldt, g.row_off_d, g.M_d, g.nh, B, ldc, ncols, out, h, polar);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
 }
@@ -208,8 +210,8 @@ template <int TN>
 int launch_pair(const Grid& g, int nf, const float* X, float* C, float* Y, int ldc, bool ana, bool syn,
                 const float* h, cudaStream_t st) {
   int rc = SHOT_OK;
-  if (ana) rc = launch_one<TN, true>(g, nf, X, C, ldc, h, st);
-  if (!rc && syn) rc = launch_one<TN, false>(g, nf, C, Y, ldc, nullptr, st);
+  if (ana) rc = launch_one<TN, true>(g, nf, X, C, ldc, h, ana && syn, st);
+  if (!rc && syn) rc = launch_one<TN, false>(g, nf, C, Y, ldc, nullptr, ana && syn, st);
   return rc;
 }
 

@@ -148,6 +148,7 @@ struct AnaArgs {
   float* cf;           // optional FP32 [row_off + i][ldc]
   int* err;
   long long wait;      // limit of every bounded wait (SM clock cycles)
+  int polar;           // sums start at the tile's first term above kPolarCut
 };
 
 struct SynArgs {
@@ -160,6 +161,7 @@ struct SynArgs {
   float* Y;   // [blk][jh][ldc]
   int* err;
   long long wait;
+  int polar;
 };
 
 // Persistent, warp-specialised Legendre GEMM.  Warp 0: TMA producer (runs ahead across
@@ -243,6 +245,8 @@ __global__ void __launch_bounds__(tc_threads<ANA>(), 1) k_legendre_tc(const __gr
   const uint32_t taddr = ctl.tmem;
   volatile int* abort = &ctl.abort;
   const long long wl = (ANA ? aa.wait : sa.wait);   // wait limit (cycles)
+  const bool polar = ANA ? aa.polar : sa.polar;
+  auto kb0_of = [&](const Tile& tl) { return polar ? tl.start() / kBK : 0; };   // first K chunk
   auto nkb_of = [&](int blk) { return ANA ? (nh + kBK - 1) / kBK : (Mr[blk] + kBK - 1) / kBK; };
 
   if (warp == 0) {
@@ -252,7 +256,7 @@ __global__ void __launch_bounds__(tc_threads<ANA>(), 1) k_legendre_tc(const __gr
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
         const Tile tl = tiles[t];
         const int nkb = nkb_of(tl.blk);
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
+        for (int kb = kb0_of(tl); kb < nkb; ++kb, ++it) {
           const int s = it % kStages, n = it / kStages;
           if (it >= kStages && !(ok = mbar_wait(&ctl.empty[s], (n - 1) & 1, abort, wl))) break;
           if (ANA) {
@@ -294,7 +298,8 @@ __global__ void __launch_bounds__(tc_threads<ANA>(), 1) k_legendre_tc(const __gr
         if (lt >= 2 && !(ok = mbar_wait(&ctl.tempty[acc], (u - 1) & 1, abort, wl))) break;
         tc_fence_after();
         const uint32_t d = taddr + (uint32_t)(acc * ncols_alloc);
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
+        const int kb0 = kb0_of(tl);
+        for (int kb = kb0; kb < nkb; ++kb, ++it) {
           const int s = it % kStages, n = it / kStages;
           const int sb = kBRing ? (it % kBR) : s;   // B buffer of this iteration
           ok = mbar_wait(&ctl.fullA[s], n & 1, abort, wl);
@@ -323,10 +328,10 @@ __global__ void __launch_bounds__(tc_threads<ANA>(), 1) k_legendre_tc(const __gr
               a_l = desc_sw128_mnmajor(al + k * 2048, kATileBytes / 2, 1024);
             }
             if constexpr (BCAT) {   // b_h starts [B_hi | B_lo]
-              umma_bf16(d, a_h, b_h, idesc_cat, (kb | k) != 0);
+              umma_bf16(d, a_h, b_h, idesc_cat, kb != kb0 || k != 0);
               umma_bf16(d, a_l, b_h, idesc, 1);
             } else {
-              umma_bf16(d, a_h, b_h, idesc, (kb | k) != 0);
+              umma_bf16(d, a_h, b_h, idesc, kb != kb0 || k != 0);
               umma_bf16(d, a_h, b_l, idesc, 1);
               umma_bf16(d, a_l, b_h, idesc, 1);
             }
@@ -352,7 +357,7 @@ __global__ void __launch_bounds__(tc_threads<ANA>(), 1) k_legendre_tc(const __gr
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
         const Tile tl = tiles[t];
         const int nkb = nkb_of(tl.blk);
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
+        for (int kb = kb0_of(tl); kb < nkb; ++kb, ++it) {
           const int s = it % kStages, n = it / kStages;
           const int sb = it % kBR, nb = it / kBR;
           if (!(ok = mbar_wait(&ctl.fullA[s], n & 1, abort, wl))) break;
@@ -505,7 +510,7 @@ int launch_legendre_tc(const Grid& g, int nf, const float* X, float* Cf, float* 
     if ((rc = make_map_f32(&mx, X, ldc, (uint64_t)g.nblk * g.nh, ldc, nmma, kBK))) return rc;
     aa = AnaArgs{g.tiles_ana, g.ntiles_ana, g.M_d, g.row_off_d, g.nh, X, ldc, 2 * nf, nmma,
                  apply_h ? g.h_d : nullptr, w.ct_hi, w.ct_lo, w.nmma_cap, g.ldi, Cf, w.dev_int + 4,
-                 g.wait_cycles};
+                 g.wait_cycles, ana && syn};
     // [B_hi | B_lo] as one operand up to 128 columns (N = 2 x 64 x atoms <= 256)
     const bool bcat = 2 * 64 * mn_atoms(nmma) <= 256;
     auto kern = bcat ? (br == 3 ? (stages == 4   ? k_legendre_tc<4, true, 3, true>
@@ -542,7 +547,7 @@ int launch_legendre_tc(const Grid& g, int nf, const float* X, float* Cf, float* 
     if ((rc = make_map(&bh, w.ct_hi, g.ldi, (uint64_t)g.nblk * w.nmma_cap, g.ldi, nmma))) return rc;
     if ((rc = make_map(&bl, w.ct_lo, g.ldi, (uint64_t)g.nblk * w.nmma_cap, g.ldi, nmma))) return rc;
     sa = SynArgs{g.tiles_syn, g.ntiles_syn, g.M_d, g.row_off_d, g.nh, nmma, w.nmma_cap, 2 * nf, ldc, Y, w.dev_int + 4,
-                 g.wait_cycles};
+                 g.wait_cycles, ana && syn};
     auto kern = k_legendre_tc<kStagesSyn, false>;
     SHOT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // CTAs per SM: both shared memory and the 512 TMEM columns (two accumulators each) must fit

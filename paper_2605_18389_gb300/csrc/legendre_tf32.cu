@@ -220,6 +220,7 @@ struct T32Args {
   const float* xnode;         // x_jh^2 in FP32
   int nin;                    // input ring depth (REC)
   int lmax;
+  int polar;                  // sums start at the tile's first term above kPolarCut
 };
 
 // Recurrence mode: checkpoint segments of 16 degrees; per stage a checkpoint box and the
@@ -349,6 +350,7 @@ __global__ void __launch_bounds__(32 * (2 + SW + 4), SW == 8 ? 2 : 1)
   const uint32_t taddr = ctl.tmem;
   volatile int* abort = &ctl.abort;
   const long long wl = a.wait;   // wait limit (cycles)
+  auto kb0_of = [&](const Tile& tl) { return a.polar ? tl.start() / kTK : 0; };   // first K chunk
   auto nkb_of = [&](int blk) { return ANA ? (nh + kTK - 1) / kTK : (a.M[blk] + kTK - 1) / kTK; };
 
   if (warp == 0) {
@@ -360,8 +362,9 @@ __global__ void __launch_bounds__(32 * (2 + SW + 4), SW == 8 ? 2 : 1)
         const Tile tl = a.tiles[t];
         const int nkb = nkb_of(tl.blk);
         // checkpoint rows of order m in the plane of the tile's parity (planes of ck_rows rows)
+        const int kb0 = kb0_of(tl);
         const long long ck_base = REC ? (tl.blk & 1) * a.ck_rows + a.ck_off[tl.blk >> 1] : 0;
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
+        for (int kb = kb0; kb < nkb; ++kb, ++it) {
           // REC fills the input ring (freed by the split warps), the table mode the stages (freed
           // by the MMAs)
           uint64_t* full = REC ? &ctl.infull[s] : &ctl.fullA[s];
@@ -418,7 +421,8 @@ __global__ void __launch_bounds__(32 * (2 + SW + 4), SW == 8 ? 2 : 1)
         if (lt >= 2 && !(ok = mbar_wait(&ctl.tempty[acc], (u - 1) & 1, abort, wl))) break;
         tc_fence_after();
         const uint32_t d = taddr + (uint32_t)(acc * ncols_alloc);
-        for (int kb = 0; kb < nkb; ++kb) {
+        const int kb0 = kb0_of(tl);
+        for (int kb = kb0; kb < nkb; ++kb) {
           if (!(ok = mbar_wait(&ctl.fullB[s], ph, abort, wl))) break;
           tc_fence_after();
 #pragma unroll
@@ -426,10 +430,10 @@ __global__ void __launch_bounds__(32 * (2 + SW + 4), SW == 8 ? 2 : 1)
             const uint64_t off = dstage + (uint64_t)(2 * k);
             const uint64_t a_h = off, a_l = off + d_al, b_h = off + d_bh, b_l = off + d_bl;
             if constexpr (BCAT) {   // b_h spans B_hi and B_lo (2 nmma rows)
-              umma_tf32(d, a_h, b_h, idesc2, (kb | k) != 0);
+              umma_tf32(d, a_h, b_h, idesc2, kb != kb0 || k != 0);
               umma_tf32(d, a_l, b_h, idesc, 1);
             } else {
-              umma_tf32(d, a_h, b_h, idesc, (kb | k) != 0);
+              umma_tf32(d, a_h, b_h, idesc, kb != kb0 || k != 0);
               umma_tf32(d, a_h, b_l, idesc, 1);
               umma_tf32(d, a_l, b_h, idesc, 1);
             }
@@ -472,7 +476,7 @@ __global__ void __launch_bounds__(32 * (2 + SW + 4), SW == 8 ? 2 : 1)
       const int nkb = nkb_of(tl.blk);
       const int m = tl.blk >> 1, par = tl.blk & 1;
       const int dmax = a.lmax - m;   // largest relative degree of order m
-      for (int kb = 0; kb < nkb; ++kb, ++it) {
+      for (int kb = kb0_of(tl); kb < nkb; ++kb, ++it) {
         // REC: the inputs are in slot i of the input ring, and stage s must also be free (its
         // previous MMAs done).  Every thread waits (each must observe the copies' phase
         // itself); the outcome is made warp-uniform so that a warp leaves together and its
@@ -646,7 +650,8 @@ __global__ void k_c_to_ct32(const int* __restrict__ Mrows, const long long* __re
 // ck[(par * ck_rows + ck_off[m] + s) * ckld + 2 jh + {0, 1}]; degrees past lmax and nodes past nh
 // stay zero (the buffer is cleared first).  Also x_jh^2 in FP32.
 __global__ void k_ck_build(int lmax, int nh, const double* __restrict__ x, const long long* __restrict__ ck_off,
-                           long long ck_rows, int ckld, float* __restrict__ ck, float* __restrict__ x2) {
+                           long long ck_rows, int ckld, float* __restrict__ ck, float* __restrict__ x2,
+                           int* __restrict__ lfirst) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = blockIdx.y;
   if (j >= nh) return;
@@ -656,6 +661,7 @@ __global__ void k_ck_build(int lmax, int nh, const double* __restrict__ x, const
   double pmm = 0.28209479177387814;   // 1/sqrt(4 pi)
   for (int k = 1; k <= m; ++k) pmm *= -sqrt((2.0 * k + 1.0) / (2.0 * k)) * st;
   double p2 = 0.0, p1 = pmm;   // Pbar_{l-2}, Pbar_{l-1} entering degree l = m + 1
+  int first = lmax + 1;
   for (int l = m; l <= lmax; ++l) {
     double pl;
     if (l == m) {
@@ -670,12 +676,14 @@ __global__ void k_ck_build(int lmax, int nh, const double* __restrict__ x, const
       p2 = p1;
       p1 = pl;
     }
+    if (first > lmax && fabs(pl) >= kPolarCut) first = l;
     const int d = l - m, r = d % kSeg;
     if (r < 4) {   // offsets 0, 2 -> plane 0; 1, 3 -> plane 1; first or second value by r / 2
       const int par = r & 1;
       ck[((size_t)par * ck_rows + ck_off[m] + d / kSeg) * ckld + 2 * j + (r >> 1)] = (float)pl;
     }
   }
+  if (lfirst) lfirst[(size_t)m * nh + j] = first;
 }
 
 // Two-step coefficients (A, B, C, 0) of degree l (from l - 2 and l - 4) for m + 4 <= l <= lmax at
@@ -742,7 +750,7 @@ void* tf32_kernel(bool ana, bool bc, int stages, bool two_cta) {
 
 int tf32_nmma(int nf) { return (2 * nf + 15) / 16 * 16; }
 
-int build_tf32_recurrence(Grid& g, cudaStream_t st) {
+int build_tf32_recurrence(Grid& g, int* lfirst, cudaStream_t st) {
   const int L = g.lmax + 1, nh = g.nh;
   std::vector<long long> ckoff(L + 1, 0);
   for (int m = 0; m < L; ++m) ckoff[m + 1] = ckoff[m] + (L - m + kSeg - 1) / kSeg;
@@ -761,7 +769,7 @@ int build_tf32_recurrence(Grid& g, cudaStream_t st) {
   count_launch(2);
   k_coef32_build<<<L, 256, 0, st>>>(g.lmax, g.cstride, reinterpret_cast<float4*>(g.rec_coef));
   k_ck_build<<<dim3((nh + 127) / 128, L), 128, 0, st>>>(g.lmax, nh, g.x_d, g.ck_off_d, g.ck_rows, g.ck_ld, g.ck,
-                                                        g.rec_x);
+                                                        g.rec_x, lfirst);
   SHOT_CUDA(cudaGetLastError());
   SHOT_CUDA(cudaStreamSynchronize(st));   // ckoff is a local
   return SHOT_OK;
@@ -868,6 +876,7 @@ int launch_legendre_tf32(const Grid& g, int nf, const float* X, float* Cf, float
     args.Y = nullptr;
     args.err = w.dev_int + 4;
     args.wait = g.wait_cycles;
+    args.polar = ana && syn;   // a heat convolution
     if ((rc = launch(true, ma, mx, args, g.ntiles_ana))) return rc;
   }
   if (syn) {
@@ -892,6 +901,7 @@ int launch_legendre_tf32(const Grid& g, int nf, const float* X, float* Cf, float
     args.Y = Y;
     args.err = w.dev_int + 4;
     args.wait = g.wait_cycles;
+    args.polar = ana && syn;   // a heat convolution
     if ((rc = launch(false, ma, mb, args, g.ntiles_syn))) return rc;
   }
   return SHOT_OK;

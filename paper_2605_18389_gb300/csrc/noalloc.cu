@@ -87,10 +87,11 @@ extern "C" int shot_heat_apply_noalloc(shot_grid gh, double t, const float* in, 
   float* C = scratch + nx;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if ((rc = launch_heat_mult(*g, t, st))) return rc;
-  if ((rc = launch_dft_fwd(*g, in, nfields, nullptr, 0, X, ldc, st))) return rc;
+  if ((rc = launch_dft_fwd(*g, in, nfields, nullptr, 0, X, ldc, st, g->mlim_d))) return rc;
   if ((rc = launch_legendre(*g, nfields, X, C, X, ldc, st))) return rc;
   EpiParams ep{};
   ep.mode = EPI_PLAIN;
   ep.out = out;
+  ep.mlim = g->mlim_d;
   return launch_idft(*g, X, ldc, nfields, ep, st);
 }

@@ -84,7 +84,21 @@ void fft_plan_twiddles(const FftPlan& plan, std::vector<float2>& tw);
 struct Tile {
   int blk;    // 2*m + p
   int r0;     // first row of the tile (i for analysis, jh for synthesis)
+  // Heat convolutions: first term (jh for analysis, i for synthesis), a multiple of 16, of the sums
+  // of the tile's rows r0 .. r0 + 63 and r0 + 64 .. r0 + 127.  The terms before it have
+  // |Pbar| < kPolarCut: near the poles sin^m makes the functions of high order vanish.
+  int k0[2];
+  __host__ __device__ int start() const { return k0[0] < k0[1] ? k0[0] : k0[1]; }
 };
+// Table values below 2^-100 (the FP32 recurrence mode starts its recurrences there too) are left
+// out of the heat convolutions: a term's share is at most 2^-100 of the spectrum's value, far under
+// the rounding of any field that other orders and rings reach (every Pbar_lm has values of order
+// 0.3 somewhere).  The plain transforms keep every term: their coefficients are results by themselves.
+// Measured at 720 rings, 24 fields, analysis / synthesis: TF32x3 156 / 140 -> 133 / 133 us, FP32 228 /
+// 181 -> 187 / 173 us; the ring transforms skip the orders that no tile reads or writes: forward 87 -> 72,
+// inverse 66 -> 58, update 152 -> 144 us.
+constexpr double kPolarCut = 0x1p-100;
+constexpr int kPolarAlign = 64;   // the Legendre kernels' longest chunk of terms
 
 struct Workspace {
   int nf_cap = 0;       // fields the buffers hold
@@ -165,6 +179,9 @@ struct Grid {
   int cstride = 0;              // TF32X3 recurrence: coefficient row stride (entries per order)
   int* M_d = nullptr;
   long long* row_off_d = nullptr;
+  // heat convolutions: per north ring the highest order whose synthesis rows are nonzero (.x) and
+  // whose spectra the analysis reads (.y); null (FP32 recurrence mode): lmax
+  int2* mlim_d = nullptr;
   Tile* tiles_ana = nullptr;
   Tile* tiles_syn = nullptr;
   int tc_stages_override = 0;   // SHOT_TC_STAGES: pipeline depth of the tensor-core kernels (0 = tuned)
@@ -244,6 +261,7 @@ struct EpiParams {
   float* xout;                // EPI_UPDATE: when set, the CTA also ring-transforms the new
                               // scaling (unscaled) into the folded spectra xout[.][jh][ldc]
   int potentials;             // EPI_FINAL: write eps log u, eps log v instead of u, v
+  const int2* mlim;           // highest orders of each north ring (Grid::mlim_d), null: lmax
   int skip_store;             // EPI_UPDATE: the new scaling feeds only the fused forward
                               // transform (no later launch reads this iteration's buffer)
 };
@@ -252,7 +270,7 @@ bool profiling_on();
 // ---------------------------------------------------------------------------------
 // Launchers (return SHOT status)
 int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, int scale_which,
-                   float* X, int ldc, cudaStream_t st);
+                   float* X, int ldc, cudaStream_t st, const int2* mlim = nullptr);
 int launch_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st);
 int dft_fields_per_cta(const Grid& g, int nf);   // fields a ring-transform CTA takes
 // Grids whose Legendre contractions run the TF32x3 tensor-core kernels: TF32X3 grids, and BF16X3
@@ -279,7 +297,8 @@ int launch_legendre_tf32(const Grid& g, int nf, const float* X, float* Cf, float
                          bool apply_h, cudaStream_t st);
 int launch_c_to_ct32(const Grid& g, int nf, const float* C, int ldc, cudaStream_t st);
 int build_recurrence(Grid& g, cudaStream_t st);
-int build_tf32_recurrence(Grid& g, cudaStream_t st);
+// lfirst[m nh + jh]: first degree with |Pbar| >= kPolarCut (lmax + 1: none)
+int build_tf32_recurrence(Grid& g, int* lfirst, cudaStream_t st);
 int launch_legendre_rec(const Grid& g, int nf, const float* X, float* C, float* Y, int ldc, bool ana, bool syn,
                         bool apply_h, cudaStream_t st);
 int tc_nmma(int nf);
@@ -288,7 +307,7 @@ int ensure_workspace(Grid& g, int nf, cudaStream_t st);
 void healpix_geometry(Grid& g, int nside);
 // ps != nullptr: every field is multiplied by its ProbState::beta on load
 int launch_hp_dft_fwd(const Grid& g, const float* in, int nf, float* X, int ldc, cudaStream_t st,
-                      const ProbState* ps = nullptr);
+                      const ProbState* ps = nullptr, const int2* mlim = nullptr);
 int launch_hp_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st);
 
 }  // namespace shot

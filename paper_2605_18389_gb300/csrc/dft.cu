@@ -227,29 +227,24 @@ __global__ void __launch_bounds__(NT, CTAS) k_idft(
 // so that neither the gather nor the update waits on DRAM (three CTAs per SM, ~69 KB each at
 // 1440 longitudes and two fields).
 
-// shared memory of k_idft_p (bytes): the sequence buffers (one, or two to ping-pong), then the
-// spectra staging area
-__host__ __device__ inline size_t idft_p_layout(int nbuf, int G, int N, int lmax) {
-  return (size_t)nbuf * G * seq_ld(N) * sizeof(C2) + (size_t)(2 * lmax + 1) * G * sizeof(float4);
+// shared memory of k_idft_p (bytes): the two sequence buffers, then the spectra staging area
+inline size_t idft_p_layout(int N, int lmax) {
+  return (size_t)2 * seq_ld(N) * sizeof(C2) + (size_t)(2 * lmax + 1) * sizeof(float4);
 }
 
-template <int G, int NT, int CTAS, class PL, bool INPLACE>
-__global__ void __launch_bounds__(NT, CTAS) k_idft_p(
+template <class PL>
+__global__ void __launch_bounds__(kThreads, kCtas) k_idft_p(
     const float* __restrict__ Y, int ldc, int nf, int nlat, int nlon, int lmax, int nh,
-    const float* __restrict__ a_ring, const __grid_constant__ FftPlan pl, const float2* tw, int tws, EpiParams ep,
+    const float* __restrict__ a_ring, const __grid_constant__ FftPlan pl, const float2* tw, EpiParams ep,
     int ngroups) {
   extern __shared__ __align__(16) C2 sm[];
-  __shared__ float red[NT / 32][2 * NPART];
-  __shared__ EpiField fi[2][2 * G];
-  constexpr int FG = 2 * G;
+  __shared__ float red[kThreads / 32][2 * NPART];
+  __shared__ EpiField fi[2][2];
+  constexpr int G = 1, NT = kThreads, FG = 2 * G;
   const int N = nlon, ld = seq_ld(N);
   C2* buf = sm;
-  C2* b1 = INPLACE ? buf : buf + G * ld;
+  C2* b1 = buf + G * ld;
   float4* stg = reinterpret_cast<float4*>(b1 + G * ld);
-  if (tws) {   // twiddles beside the sequences
-    fft_copy_twiddles(reinterpret_cast<float2*>(stg + (2 * lmax + 1) * G), tw, tws);
-    tw = reinterpret_cast<const float2*>(stg + (2 * lmax + 1) * G);
-  }
   const int nitems = ngroups * nh;
   const size_t fs = (size_t)nlat * N;
 
@@ -277,8 +272,8 @@ __global__ void __launch_bounds__(NT, CTAS) k_idft_p(
       epi_fields_load<FG>(ep, fn, nn, fi[slot ^ 1]);
       issue_spectra<G, NT>(Y, ldc, nh, orders(jn).x, lmax, jn, fn, nf, stg);
     }
-    const C2* z = fft_smem_plan<true, PL, INPLACE>(buf, b1, tw, pl, G);
-    C2* other = (z == buf) ? b1 : buf;   // INPLACE: an element's new scaling replaces its K v
+    const C2* z = fft_smem_plan<true, PL>(buf, b1, tw, pl, G);
+    C2* other = (z == buf) ? b1 : buf;
     if (next < nitems)   // fi[slot ^ 1] is visible after the transform's barriers
       epi_prefetch_marginals<FG>(ep, fi[slot ^ 1], nn, (size_t)jn * N, (size_t)(nlat - 1 - jn) * N,
                                  nlat - 1 - jn != jn, N, fn, fs);
@@ -288,7 +283,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_idft_p(
                                            jh, ep, red, fi[slot]);
     if (ep.xout) {   // the update's new scaling: its spectra for the next half-step
       __syncthreads();
-      const C2* zf = fft_smem_plan<false, PL, INPLACE>(other, const_cast<C2*>(z), tw, pl, G);
+      const C2* zf = fft_smem_plan<false, PL>(other, const_cast<C2*>(z), tw, pl, G);
       fold_store<G, NT>(zf, f0, nf, N, ml.y, nh, jh, aj, nullptr, 0, ep.xout, ldc);
     }
     item = next;
@@ -316,7 +311,8 @@ int pick_g(const Grid& g, int nf) {
 // longitudes (6 KB), where a CTA has few items and would wait for each stage's twiddles from L2 (32
 // rings, one field: 9.4 us an update launch without the copy, 7.3 with it in the scalar form); none
 // beyond, where many items read them through L1.
-int twiddles_in_smem(const Grid& g) { return g.nlon <= 768 ? fft_tw_len(g.plan) : 0; }
+constexpr int kTwMax = 768;
+int twiddles_in_smem(const Grid& g) { return g.nlon <= kTwMax ? fft_tw_len(g.plan) : 0; }
 
 size_t idft_smem(int G, int N) { return (size_t)2 * G * seq_ld(N) * sizeof(C2); }
 
@@ -348,18 +344,17 @@ int launch_idft_t(const Grid& g, const float* Y, int ldc, int nf, const EpiParam
   return SHOT_OK;
 }
 
-template <int G, class PL = RuntimePlan, int NT = kThreads, int CTAS = kCtas, bool INPLACE = false>
+template <class PL>
 int launch_idft_p_t(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st) {
-  const int tws = twiddles_in_smem(g);
-  const size_t smem = idft_p_layout(INPLACE ? 1 : 2, G, g.nlon, g.lmax) + tws * sizeof(float2);
-  SHOT_CUDA(cudaFuncSetAttribute(k_idft_p<G, NT, CTAS, PL, INPLACE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const int ngroups = (nf + 2 * G - 1) / (2 * G);
+  const size_t smem = idft_p_layout(g.nlon, g.lmax);
+  SHOT_CUDA(cudaFuncSetAttribute(k_idft_p<PL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int ngroups = (nf + 1) / 2;
   const int nitems = ngroups * g.nh;
-  const int grid = nitems < CTAS * g.num_sms ? nitems : CTAS * g.num_sms;
+  const int grid = nitems < kCtas * g.num_sms ? nitems : kCtas * g.num_sms;
   ProfScope prof(ep.mode == EPI_CHECK || ep.mode == EPI_FINAL ? PK_CHECK : PK_IDFT, st);
   count_launch();
-  k_idft_p<G, NT, CTAS, PL, INPLACE><<<grid, NT, smem, st>>>(Y, ldc, nf, g.nlat, g.nlon, g.lmax, g.nh, g.a_d, g.plan, g.tw_d, tws, ep,
-                                                ngroups);
+  k_idft_p<PL><<<grid, kThreads, smem, st>>>(Y, ldc, nf, g.nlat, g.nlon, g.lmax, g.nh, g.a_d, g.plan, g.tw_d, ep,
+                                             ngroups);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
 }
@@ -401,10 +396,15 @@ int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, 
   }
 }
 
-// whether launch_idft runs the persistent kernel for this epilogue
+// Whether launch_idft runs the persistent kernel for this epilogue: the solver's update half-steps
+// and checks on rings of more than 768 longitudes (one pair of fields a CTA) whose buffers and staging
+// area leave three CTAs on an SM.  Shorter rings take several pairs a CTA and have few items per
+// CTA: one item a CTA was faster (256 rings, 48 fields: 59 against 80 us an update; four grids of 64
+// to 180 rings, 72 fields each, in one solve: 19.7 against 20.9 ms).
 static bool idft_is_persistent(const Grid& g, int nf, const EpiParams& ep) {
   return (((ep.mode == EPI_UPDATE || ep.mode == EPI_SYM) && ep.xout) || ep.mode == EPI_CHECK) &&
-         !g.idft_nonpersistent && nf >= 2 && idft_p_layout(2, pick_g(g, nf), g.nlon, g.lmax) <= 74 * 1024;
+         !g.idft_nonpersistent && nf >= 2 && g.nlon > kTwMax && pick_g(g, nf) == 1 &&
+         idft_p_layout(g.nlon, g.lmax) <= 74 * 1024;
 }
 
 int launch_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st) {
@@ -417,15 +417,9 @@ int launch_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams&
   // inputs prefetched
   const int G = pick_g(g, nf);
   if (idft_is_persistent(g, nf, ep)) {
-    switch (G) {
-      case 6: return launch_idft_p_t<6>(g, Y, ldc, nf, ep, st);
-      case 3: return launch_idft_p_t<3>(g, Y, ldc, nf, ep, st);
-      case 2: return launch_idft_p_t<2>(g, Y, ldc, nf, ep, st);
-      default:
-        if (plan_is<Plan1440>(g.plan)) return launch_idft_p_t<1, Plan1440>(g, Y, ldc, nf, ep, st);
-        if (plan_is<Plan1024>(g.plan)) return launch_idft_p_t<1, Plan1024>(g, Y, ldc, nf, ep, st);
-        return launch_idft_p_t<1>(g, Y, ldc, nf, ep, st);
-    }
+    if (plan_is<Plan1440>(g.plan)) return launch_idft_p_t<Plan1440>(g, Y, ldc, nf, ep, st);
+    if (plan_is<Plan1024>(g.plan)) return launch_idft_p_t<Plan1024>(g, Y, ldc, nf, ep, st);
+    return launch_idft_p_t<RuntimePlan>(g, Y, ldc, nf, ep, st);
   }
   switch (G) {
     case 6: return launch_idft_t<6>(g, Y, ldc, nf, ep, st);

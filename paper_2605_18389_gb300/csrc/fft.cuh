@@ -410,65 +410,53 @@ struct CtPlan {
 };
 using RuntimePlan = CtPlan<0>;
 
-template <int R, bool INV, int N, int NS, int TWOFF, bool INPLACE>
+template <int R, bool INV, int N, int NS, int TWOFF>
 __device__ __forceinline__ void stockham_stage_ct(const C2* src, C2* dst, const float2* __restrict__ tw, int nseq) {
-  constexpr int NR = N / R, LD = N + 1;
+  constexpr int NR = N / R, LD = seq_ld(N);
   const int total = nseq * NR;
-  C2 v[R];
-  auto load = [&](int idx) {
-    const int q = idx / NR, j = idx - q * NR;
+  // opaque to the compiler, which would otherwise hoist a persistent kernel's index arithmetic and
+  // twiddle loads out of its loop over items and spill them
+  int idx = threadIdx.x;
+  asm volatile("" : "+r"(idx));
+  for (; idx < total; idx += blockDim.x) {
+    const int q = idx / NR;
+    const int j = idx - q * NR;
+    const int jd = j / NS;
+    const int k = j - jd * NS;
     const C2* s = src + q * LD + j;
+    C2 v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = s[r * NR];
     if constexpr (NS > 1) {
-      const float2* tws = tw + TWOFF + j % NS;
+      const float2* tws = tw + TWOFF + k;
 #pragma unroll
       for (int r = 1; r < R; ++r) v[r] = cmul<INV>(v[r], __ldg(tws + (r - 1) * NS));
     }
     butterfly<R, INV>(v);
-  };
-  auto store = [&](int idx) {
-    const int q = idx / NR, j = idx - q * NR, jd = j / NS;
-    C2* d = dst + q * LD + jd * NS * R + (j - jd * NS);
+    C2* d = dst + q * LD + jd * NS * R + k;
 #pragma unroll
     for (int r = 0; r < R; ++r) d[r * NS] = v[out_reg<R>(r)];
-  };
-  // opaque to the compiler, which would otherwise hoist a persistent kernel's index arithmetic and
-  // twiddle loads out of its loop over items and spill them (1.4 KB a thread in the in-place form)
-  int idx = threadIdx.x;
-  asm volatile("" : "+r"(idx));
-  if constexpr (INPLACE) {   // one butterfly a thread (the launch has at least `total` threads)
-    if (idx < total) load(idx);
-    __syncthreads();
-    if (idx < total) store(idx);
-  } else {
-    for (; idx < total; idx += blockDim.x) {
-      load(idx);
-      store(idx);
-    }
   }
   __syncthreads();
 }
 
 // three-stage compile-time plan; the twiddle table layout is the runtime plan's (stage s at
-// sum over earlier stages s' >= 1 of (R_s' - 1) Ns_s').  INPLACE: every stage reads and writes a
-// (b unused), with a barrier between, for launches with a thread per butterfly.
-template <bool INV, class PL, bool INPLACE = false>
+// sum over earlier stages s' >= 1 of (R_s' - 1) Ns_s')
+template <bool INV, class PL>
 __device__ C2* fft_smem_ct(C2* a, C2* b, const float2* tw, int nseq) {
   constexpr int N = PL::N, R0 = PL::R0, R1 = PL::R1, R2 = PL::R2;
   static_assert(R0 * R1 * R2 == N, "plan radices must multiply to N");
-  if constexpr (INPLACE) b = a;
-  stockham_stage_ct<R0, INV, N, 1, 0, INPLACE>(a, b, tw, nseq);
-  stockham_stage_ct<R1, INV, N, R0, 0, INPLACE>(b, a, tw, nseq);
-  stockham_stage_ct<R2, INV, N, R0 * R1, (R1 - 1) * R0, INPLACE>(a, b, tw, nseq);
+  stockham_stage_ct<R0, INV, N, 1, 0>(a, b, tw, nseq);
+  stockham_stage_ct<R1, INV, N, R0, 0>(b, a, tw, nseq);
+  stockham_stage_ct<R2, INV, N, R0 * R1, (R1 - 1) * R0>(a, b, tw, nseq);
   return b;
 }
 
-template <bool INV, class PL, bool INPLACE = false>
+template <bool INV, class PL>
 __device__ __forceinline__ C2* fft_smem_plan(C2* a, C2* b, const float2* tw, const FftPlan& pl,
                                                  int nseq) {
   if constexpr (PL::N == 0) return fft_smem<INV>(a, b, tw, pl, nseq);
-  else return fft_smem_ct<INV, PL, INPLACE>(a, b, tw, nseq);
+  else return fft_smem_ct<INV, PL>(a, b, tw, nseq);
 }
 
 }  // namespace shot

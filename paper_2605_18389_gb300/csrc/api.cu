@@ -80,10 +80,13 @@ __device__ __forceinline__ double wsum(double v) {
 
 // Fixed-order reduction of the per-ring-pair partial sums and the per-problem scalar
 // steps of Alg. 1 (gauge / TI constant / convergence test / objective).  One block per
-// problem; the last block to finish (ticket in dev_int[12], reset by that block) counts
-// the problems still active and advances the iteration counter.
+// problem; after a v-step the last block to finish (ticket in dev_int[12], reset by that block)
+// advances the iteration counter, after a check it counts the problems still active (what the host
+// polls).  A u-step needs neither.  The kernel is a chain of latencies (loads, shuffles, FP64
+// logarithms and exponentials, the ticket), and for small grids it is longer than the Legendre
+// stages that it runs beside.
 constexpr int kRedThreads = 128;
-constexpr double kLn2 = 0.69314718055994530942;
+constexpr double kLn2 = 0.69314718055994530942, kInvLn2 = 1.4426950408889634074;
 
 __global__ void __launch_bounds__(kRedThreads) k_reduce(int mode, int nprob, int nh, const double* __restrict__ part,
                                                         ProbState* ps, int* dev_int, double eps, double tol,
@@ -94,6 +97,10 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce(int mode, int nprob, int
   const int f = blockIdx.x;
   const int kdone = dev_int[0];
   ProbState* P = ps + f;
+  // the state the step needs, loaded beside the partial sums
+  const int bal = P->balanced, eu = P->eu, ev = P->ev;
+  const double gam = (double)P->gamma, tau = P->tau, la0 = P->la, lb0 = P->lb, lsu = P->lsu;
+  const double lvu = P->lvu, lvv = P->lvv, qu = P->qu, qv = P->qv;
   const bool skip = (mode == RED_FINAL) ? (P->status < 0) : (P->active == 0);
   if (!skip) {
     double s[NPART] = {0.0, 0.0, 0.0, 0.0};
@@ -127,7 +134,6 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce(int mode, int nprob, int
           P->iters = kdone + 1;
         }
       } else if (mode == RED_U || mode == RED_V) {
-        const int bal = P->balanced;
         int st = SHOT_OK;
         if (s[2] > 0.0) st = SHOT_ERR_NONPOSITIVE;
         else if (s[3] > 0.0) st = SHOT_ERR_NONFINITE;
@@ -136,36 +142,35 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce(int mode, int nprob, int
         // r = 2^e, so log r is exact
         const double lx = log(lane == 0 ? s[0] : (lane == 1 ? (bal ? s[0] : s[1]) : 1.0));
         const double lsum = __shfl_sync(0xffffffffu, lx, 0), ltot = __shfl_sync(0xffffffffu, lx, 1);
-        const double gam = (double)P->gamma;
-        const int e = (mode == RED_U) ? P->eu : P->ev;
-        const double lw = -gam * ((mode == RED_U ? P->lb : P->la) + e * kLn2);
+        const int e = (mode == RED_U) ? eu : ev;
+        const double lw = -gam * ((mode == RED_U ? lb0 : la0) + e * kLn2);
         // v-step: the plan mass m(pi) = sum a u (K v) = sum a v (K u) (K is self-adjoint in the
         // area inner product), from the new v buffer and the K u it divided by:
         // sum a v_true (K u_true) = e^{lw + la} sum a v_buf (K u_buf), kept by the gauge and the
         // translation-invariant step (they keep the product u v).  Unbalanced, the
         // translation-invariant sum is s[0] = sum a v_buf (K u_buf) / r.  Balanced,
         // v_true (K u_true) = q node by node and the final pass sums a q (mass_v = 0 marks it).
-        const double mv = (mode == RED_V && !bal) ? exp(lw + P->la) * ldexp(s[0], e) : 0.0;
+        const double mv = (mode == RED_V && !bal) ? exp(lw + la0) * ldexp(s[0], e) : 0.0;
         // log of the step's sum over true values: sum w_true (balanced gauge) or
         // sum a m w_true^{-eps/tau} (translation-invariant step)
-        const double ls = bal ? lw + lsum : -(eps / P->tau) * lw + lsum;
+        const double ls = bal ? lw + lsum : -(eps / tau) * lw + lsum;
         // buffer level L = log mean w_buf.  The factors r only keep the FP32 buffers near
         // level 0 (exactness comes from lw): a half-step's level is about
         // gamma (log r + A - L_other) with A a slowly varying term of the marginal's and the
         // kernel's shapes, so each half-step estimates A from what it just produced and the
         // other side's factor is set as soon as the level it will divide by is known.
         const double L = ltot - lnpix;
-        const double A = L / gam - e * kLn2 + (mode == RED_U ? P->lvv : P->lvu);
-        const double zr = ((mode == RED_U ? P->qv : P->qu) + L) / kLn2;
+        const double A = (bal ? L : L / gam) - e * kLn2 + (mode == RED_U ? lvv : lvu);
+        const double zr = ((mode == RED_U ? qv : qu) + L) * kInvLn2;
         const int en = (int)fmin(fmax(rint(zr), -100.0), 100.0);
         if (st == SHOT_OK && !(isfinite(lw) && isfinite(ls) && isfinite(L))) st = SHOT_ERR_NONFINITE;
-        double la = P->la, lb = lw;
+        double la = la0, lb = lw;
         if (mode == RED_V) {
           if (bal) {   // u / sum u, v sum u
-            la -= P->lsu;
-            lb += P->lsu;
+            la -= lsu;
+            lb += lsu;
           } else {     // c = tau/2 (log su - log sv): u e^{c/eps}, v e^{-c/eps}
-            const double c = 0.5 * P->tau * (P->lsu - ls);
+            const double c = 0.5 * tau * (lsu - ls);
             la += c / eps;
             lb -= c / eps;
           }
@@ -224,13 +229,21 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce(int mode, int nprob, int
       }
     }
   }
-  // last block: count the active problems (all blocks' updates are visible after the fence)
+  if (mode == RED_U) return;
+  // last block (all blocks' updates are visible after the fence)
   if (threadIdx.x == 0) {
     __threadfence();
     last = (atomicAdd(&dev_int[12], 1) == nprob - 1) ? 1 : 0;
   }
   __syncthreads();
   if (!last) return;
+  if (mode == RED_V || mode == RED_S) {
+    if (threadIdx.x == 0) {
+      dev_int[0] = kdone + 1;
+      dev_int[12] = 0;
+    }
+    return;
+  }
   __threadfence();
   int na = 0;
   for (int g = threadIdx.x; g < nprob; g += kRedThreads) na += *(volatile int*)&ps[g].active;
@@ -241,7 +254,6 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce(int mode, int nprob, int
   if (threadIdx.x == 0) {
     int t = 0;
     for (int w = 0; w < kRedThreads / 32; ++w) t += wna[w];
-    if (mode == RED_V || mode == RED_S) dev_int[0] = kdone + 1;
     dev_int[1] = t;
     dev_int[12] = 0;
   }

@@ -188,10 +188,11 @@ __global__ void k_coeff_scatter(int lmax, int nf, const long long* __restrict__ 
 }  // namespace
 
 // Factorisation of the ring length into the radices the shared-memory FFT has
-// butterflies for.  Fewest stages first; then the bank conflicts of the first stage's
-// stores (lanes at a stride of R complex values: conflict-free for odd R, gcd(2R, 32)/2-way
-// otherwise), which puts an odd radix first when there is one and otherwise the smallest;
-// then the smallest largest radix (registers).
+// butterflies for.  Fewest stages first; then, for rings of more than 96 points, the bank
+// conflicts of the first stage's stores (lanes at a stride of R elements: conflict-free for odd R,
+// gcd(2R, 32)/2-way otherwise), which puts an odd radix first when there is one and otherwise the
+// smallest; then the smallest largest radix (registers, and for a short ring the time of a stage: a
+// few threads, each with one butterfly; 64 points as 8 * 8 instead of 4 * 16).
 bool make_fft_plan(int N, FftPlan* pl) {
   if (N < 1 || N >= (1 << 16)) return false;
   // prime factors above 5 become generic stages, placed first (their stage twiddles are 1)
@@ -220,13 +221,13 @@ bool make_fft_plan(int N, FftPlan* pl) {
     odd.insert(odd.end(), even.begin(), even.end());
     return odd;
   };
-  auto cost = [](const std::vector<int>& f) {
+  auto cost = [Nfull](const std::vector<int>& f) {
     if (f.empty()) return 0.0;
     int g = 2 * f[0], b = 32;
     while (b) { const int t = g % b; g = b; b = t; }
     const int deg = (f[0] & 1) ? 1 : g / 2;
     const int mx = *std::max_element(f.begin(), f.end());
-    return (double)f.size() + 0.15 * (deg - 1) + 0.01 * mx;
+    return (double)f.size() + (Nfull > 96 ? 0.15 * (deg - 1) : 0.0) + 0.01 * mx;
   };
   std::vector<int> best, cur;
   double best_cost = 1e30;

@@ -202,7 +202,9 @@ def algorithmic_work(kind, nlat, npix, lmax, nfields, legendre="table"):
 
     npix nodes per field, nh = ceil(nlat/2) ring pairs, T = (lmax+1)(lmax+2)/2 degrees
     and orders; the folded table holds T*nh entries (4 B in FP32 and TF32x3, 2+2 B as bf16
-    hi/lo), read once per launch in every precision.  In recurrence mode the TF32x3 kernels
+    hi/lo), read once per launch in every precision.  A heat convolution leaves out the entries
+    below 2^-100; at least 2/pi of the table lies above them at any size (the oscillating region
+    m < l sin(theta); 0.78 at 720 rings), and that much is counted, in bytes and in FLOP.  In recurrence mode the TF32x3 kernels
     read the checkpoints instead (4 FP32 values per 16 degrees and node: T*nh/4 entries).
     """
     n = npix
@@ -212,7 +214,8 @@ def algorithmic_work(kind, nlat, npix, lmax, nfields, legendre="table"):
     field = nfields * n * 4.0                     # one FP32 field batch
     spec = 2 * L * nh * 2 * nfields * 4.0         # folded ring spectra X or Y (FP32)
     coef = T * 2 * nfields * 4.0                  # coefficients (FP32, or bf16 hi+lo)
-    table = T * nh * 4.0 if legendre == "table" else T * nh * 4.0 / 4
+    table = (T * nh * 4.0 if legendre == "table" else T * nh * 4.0 / 4) * 2 / math.pi
+    flops = legendre_flops_per_launch(nlat, lmax, nfields) * 2 / math.pi
     if kind == "ring_dft":
         return field + spec, 0.0
     if kind == "inverse_dft_epilogue":
@@ -223,9 +226,9 @@ def algorithmic_work(kind, nlat, npix, lmax, nfields, legendre="table"):
         # marginal check: Y in, marginal in, u in
         return spec + 2 * field, 0.0
     if kind == "legendre_analysis":
-        return table + spec + coef, legendre_flops_per_launch(nlat, lmax, nfields)
+        return table + spec + coef, flops
     if kind == "legendre_synthesis":
-        return table + coef + spec, legendre_flops_per_launch(nlat, lmax, nfields)
+        return table + coef + spec, flops
     return 0.0, 0.0
 
 

@@ -312,12 +312,12 @@ int shot_regional_rms(shot_grid g, const float* grad_p, int batch, double* rms, 
 #define SHOT_NOALLOC_SCRATCH_BYTES (8u << 20)
 int shot_heat_apply_noalloc(shot_grid g, double t, const float* in, float* out, int nfields, void* stream);
 
-/* Autotune the launch shapes used for calls on `nfields` fields (fields per ring-DFT and
- * inverse-DFT CTA, FP32 Legendre tile width, BF16x3 analysis pipeline depth) by timing the
- * candidates with CUDA events; the solvers do this automatically on their first call for
- * a field count.  choice: host int[4] or NULL, receives the four selections (0 = the
- * default).  The choices change no summation order (results are bit-identical).
- * Allocates one temporary field batch.  Synchronises `stream`. */
+/* Autotune the launch shapes used for calls on `nfields` fields (FP32 Legendre tile width, BF16x3
+ * analysis pipeline depth) by timing the candidates with CUDA events; the solvers do this
+ * automatically on their first call for a field count.  choice: host int[4] or NULL, receives the
+ * fields per ring-DFT and inverse-DFT CTA (a rule on sizes, not timed) and the two selections (0 =
+ * the default).  The choices change no summation order (results are bit-identical).
+ * Synchronises `stream`. */
 int shot_grid_autotune(shot_grid g, int nfields, int* choice, void* stream);
 
 /* ---- heat convolution vs explicit matrix convolution -----------------------

@@ -336,9 +336,9 @@ cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
 Grid* as_grid(shot_grid g) { return reinterpret_cast<Grid*>(g); }
 
-int heat_pipeline(Grid& g, const float* in, int nf, int scale_which, cudaStream_t st) {
+int heat_pipeline(Grid& g, const float* in, int nf, double t, cudaStream_t st) {
   Workspace& w = g.ws;
-  int rc = launch_dft_fwd(g, in, nf, reinterpret_cast<ProbState*>(w.probs), scale_which, w.XY, w.ldc, st, g.mlim_d);
+  int rc = launch_dft_fwd(g, in, nf, nullptr, 0, w.XY, w.ldc, st, g.mlim_d, &t);
   if (rc) return rc;
   return launch_legendre(g, nf, w.XY, w.C, w.XY, w.ldc, st);
 }
@@ -917,8 +917,7 @@ int shot_heat_apply(shot_grid gh, double t, const float* in, float* out, int nfi
   cudaStream_t st = as_stream(stream);
   int rc = ensure_workspace(*g, nfields, st);
   if (rc) return rc;
-  if ((rc = launch_heat_mult(*g, t, st))) return rc;
-  if ((rc = heat_pipeline(*g, in, nfields, 0, st))) return rc;
+  if ((rc = heat_pipeline(*g, in, nfields, t, st))) return rc;
   EpiParams ep{};
   ep.mode = EPI_PLAIN;
   ep.out = out;

@@ -159,8 +159,12 @@ __global__ void __launch_bounds__(NT, CTAS) k_dft_fwd(
     const float* __restrict__ in, int nf, int nlat, int nlon, int lmax, int nh,
     const float* __restrict__ a_ring, const ProbState* __restrict__ ps, int scale_which,
     float* __restrict__ X, int ldc, const __grid_constant__ FftPlan pl, const float2* tw, int tws,
-    const int2* __restrict__ mlim) {
+    const int2* __restrict__ mlim, float* __restrict__ h, double t) {
   extern __shared__ __align__(16) C2 sm[];
+  if (blockIdx.y == gridDim.y - 1 && h) {   // the heat multipliers
+    for (int l = blockIdx.x * blockDim.x + threadIdx.x; l <= lmax; l += gridDim.x * blockDim.x) h[l] = heat_mult(t, l);
+    return;
+  }
   C2* b0 = sm;
   C2* b1 = b0 + G * seq_ld(nlon);
   const int jh = blockIdx.y, f0 = blockIdx.x * 2 * G;
@@ -318,15 +322,17 @@ size_t idft_smem(int G, int N) { return (size_t)2 * G * seq_ld(N) * sizeof(C2); 
 
 template <int G, class PL = RuntimePlan, int NT = kThreads, int CTAS = kCtas>
 int launch_fwd_t(const Grid& g, const float* in, int nf, const ProbState* ps, int scale_which, float* X,
-                 int ldc, cudaStream_t st, const int2* mlim) {
+                 int ldc, cudaStream_t st, const int2* mlim, const double* heat_t) {
   const int tws = twiddles_in_smem(g);
   const size_t smem = idft_smem(G, g.nlon) + tws * sizeof(float2);
   SHOT_CUDA(cudaFuncSetAttribute(k_dft_fwd<G, NT, CTAS, PL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  dim3 grid((nf + 2 * G - 1) / (2 * G), g.nh);   // field groups of one ring pair run together
+  // field groups of one ring pair run together
+  dim3 grid((nf + 2 * G - 1) / (2 * G), g.nh + (heat_t ? 1 : 0));
   ProfScope prof(PK_DFT, st);
   count_launch();
   k_dft_fwd<G, NT, CTAS, PL><<<grid, NT, smem, st>>>(in, nf, g.nlat, g.nlon, g.lmax, g.nh, g.a_d, ps, scale_which, X,
-                                                 ldc, g.plan, g.tw_d, tws, mlim);
+                                                 ldc, g.plan, g.tw_d, tws, mlim, heat_t ? g.h_d : nullptr,
+                                                           heat_t ? *heat_t : 0.0);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
 }
@@ -373,26 +379,26 @@ using Plan1024 = CtPlan<1024, 4, 16, 16>;
 int dft_fields_per_cta(const Grid& g, int nf) { return g.quad == SHOT_QUAD_HEALPIX ? 2 : 2 * pick_g(g, nf); }
 
 int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, int scale_which,
-                   float* X, int ldc, cudaStream_t st, const int2* mlim) {
+                   float* X, int ldc, cudaStream_t st, const int2* mlim, const double* heat_t) {
   if (g.quad == SHOT_QUAD_HEALPIX) {
     if (scale_which && scale_which != 1) {
       set_error("HEALPix ring transform: the per-field factor beta only");
       return SHOT_ERR_UNSUPPORTED;
     }
-    return launch_hp_dft_fwd(g, in, nf, X, ldc, st, scale_which == 1 ? ps : nullptr, mlim);
+    return launch_hp_dft_fwd(g, in, nf, X, ldc, st, scale_which == 1 ? ps : nullptr, mlim, heat_t);
   }
   if (g.nlon > kFftCap) {
     set_error("nlon too large for the shared-memory ring FFT");
     return SHOT_ERR_UNSUPPORTED;
   }
   switch (pick_g(g, nf)) {
-    case 6: return launch_fwd_t<6>(g, in, nf, ps, scale_which, X, ldc, st, mlim);
-    case 3: return launch_fwd_t<3>(g, in, nf, ps, scale_which, X, ldc, st, mlim);
-    case 2: return launch_fwd_t<2>(g, in, nf, ps, scale_which, X, ldc, st, mlim);
+    case 6: return launch_fwd_t<6>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
+    case 3: return launch_fwd_t<3>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
+    case 2: return launch_fwd_t<2>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
     default:
-      if (plan_is<Plan1440>(g.plan)) return launch_fwd_t<1, Plan1440, 192, 4>(g, in, nf, ps, scale_which, X, ldc, st, mlim);
-      if (plan_is<Plan1024>(g.plan)) return launch_fwd_t<1, Plan1024>(g, in, nf, ps, scale_which, X, ldc, st, mlim);
-      return launch_fwd_t<1>(g, in, nf, ps, scale_which, X, ldc, st, mlim);
+      if (plan_is<Plan1440>(g.plan)) return launch_fwd_t<1, Plan1440, 192, 4>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
+      if (plan_is<Plan1024>(g.plan)) return launch_fwd_t<1, Plan1024>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
+      return launch_fwd_t<1>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
   }
 }
 

@@ -144,7 +144,7 @@ __global__ void k_pbar(int lmax, int nh, const double* __restrict__ x, const lon
 
 __global__ void k_heat(int lmax, double t, float* __restrict__ h) {
   const int l = blockIdx.x * blockDim.x + threadIdx.x;
-  if (l <= lmax) h[l] = (float)exp(-t * (double)l * (double)(l + 1));
+  if (l <= lmax) h[l] = heat_mult(t, l);
 }
 
 // C[row_off[blk] + i][2f + {0,1}]  <->  coeffs[f][l][m][{re,im}],  l = m + p + 2i

@@ -86,9 +86,14 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_fwd(const float* __restric
                                                        const float2* __restrict__ tw_all,
                                                        const int* __restrict__ tw_base, int tws,
                                                        const ProbState* __restrict__ ps,
-                                                       const int2* __restrict__ mlim) {
+                                                       const int2* __restrict__ mlim, float* __restrict__ h,
+                                                       double t) {
   extern __shared__ __align__(16) C2 sm[];
   __shared__ FftPlan pl;
+  if (blockIdx.y == gridDim.y - 1 && h) {   // the heat multipliers
+    for (int l = blockIdx.x * blockDim.x + threadIdx.x; l <= lmax; l += gridDim.x * blockDim.x) h[l] = heat_mult(t, l);
+    return;
+  }
   const int jh = blockIdx.y, f0 = blockIdx.x * 2;
   const int j = jh, J = nrings - 1 - jh;
   const bool second = f0 + 1 < nf, two = J != j;
@@ -176,15 +181,16 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
 }  // namespace
 
 int launch_hp_dft_fwd(const Grid& g, const float* in, int nf, float* X, int ldc, cudaStream_t st,
-                      const ProbState* ps, const int2* mlim) {
+                      const ProbState* ps, const int2* mlim, const double* heat_t) {
   const int tws = g.nlon <= kHpTwMax;
   const size_t smem = hp_smem(g.nlon, tws);
   SHOT_CUDA(cudaFuncSetAttribute(k_hp_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   ProfScope prof(PK_DFT, st);
   count_launch();
-  k_hp_fwd<<<dim3((nf + 1) / 2, g.nh), kHpThreads, smem, st>>>(
+  k_hp_fwd<<<dim3((nf + 1) / 2, g.nh + (heat_t ? 1 : 0)), kHpThreads, smem, st>>>(
       in, nf, g.npix, g.ring_len_d, g.ring_off_d, g.ring_phase_d, g.nlat, g.lmax, g.nh, (float)g.a_ring[0], X, ldc,
-      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d, tws, ps, mlim);
+      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d, tws, ps, mlim, heat_t ? g.h_d : nullptr,
+      heat_t ? *heat_t : 0.0);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
 }

@@ -18,7 +18,7 @@
 //
 // All calls share the one array: two calls whose kernels overlap on the GPU (different
 // streams, or different host threads) race on it and must be serialised by the caller.  A call
-// also writes the grid's heat multipliers h_l for its t (launch_heat_mult), so it races as well
+// also writes the grid's heat multipliers h_l for its t, so it races as well
 // with any overlapping call on the same grid (shot_heat_apply, a solve), which reads them.
 // Every call writes the scratch it reads before reading it (the padding columns of the
 // spectra are never read into a stored output), so nothing needs clearing between calls.
@@ -86,8 +86,7 @@ extern "C" int shot_heat_apply_noalloc(shot_grid gh, double t, const float* in, 
   float* X = scratch;
   float* C = scratch + nx;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if ((rc = launch_heat_mult(*g, t, st))) return rc;
-  if ((rc = launch_dft_fwd(*g, in, nfields, nullptr, 0, X, ldc, st, g->mlim_d))) return rc;
+  if ((rc = launch_dft_fwd(*g, in, nfields, nullptr, 0, X, ldc, st, g->mlim_d, &t))) return rc;
   if ((rc = launch_legendre(*g, nfields, X, C, X, ldc, st))) return rc;
   EpiParams ep{};
   ep.mode = EPI_PLAIN;

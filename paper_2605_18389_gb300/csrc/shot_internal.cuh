@@ -81,6 +81,11 @@ void fft_plan_twiddles(const FftPlan& plan, std::vector<float2>& tw);
 //   X / Y   : [block][jh][ldc] ring spectra folded by parity (see dft.cu)
 //   C       : [row_off[block] + i][ldc] Legendre coefficients
 // ldc >= 2 * nfields (re, im per field), a multiple of 4.
+// heat multiplier of degree l at time t (Sec. 3.2)
+__device__ __forceinline__ float heat_mult(double t, int l) {
+  return (float)exp(-t * (double)l * (double)(l + 1));
+}
+
 struct Tile {
   int blk;    // 2*m + p
   int r0;     // first row of the tile (i for analysis, jh for synthesis)
@@ -269,8 +274,10 @@ bool profiling_on();
 
 // ---------------------------------------------------------------------------------
 // Launchers (return SHOT status)
+// heat_t != nullptr: the launch also fills the heat multipliers g.h_d of that time (a row of CTAs
+// beside the transform's), so that a heat application has one launch less
 int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, int scale_which,
-                   float* X, int ldc, cudaStream_t st, const int2* mlim = nullptr);
+                   float* X, int ldc, cudaStream_t st, const int2* mlim = nullptr, const double* heat_t = nullptr);
 int launch_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st);
 int dft_fields_per_cta(const Grid& g, int nf);   // fields a ring-transform CTA takes
 // Grids whose Legendre contractions run the TF32x3 tensor-core kernels: TF32X3 grids, and BF16X3
@@ -307,7 +314,7 @@ int ensure_workspace(Grid& g, int nf, cudaStream_t st);
 void healpix_geometry(Grid& g, int nside);
 // ps != nullptr: every field is multiplied by its ProbState::beta on load
 int launch_hp_dft_fwd(const Grid& g, const float* in, int nf, float* X, int ldc, cudaStream_t st,
-                      const ProbState* ps = nullptr, const int2* mlim = nullptr);
+                      const ProbState* ps = nullptr, const int2* mlim = nullptr, const double* heat_t = nullptr);
 int launch_hp_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st);
 
 }  // namespace shot

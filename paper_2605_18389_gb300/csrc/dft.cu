@@ -202,15 +202,15 @@ __global__ void __launch_bounds__(NT, CTAS) k_idft(
   issue_spectra<G, NT>(Y, ldc, nh, ml.x, lmax, jh, f0, nf, stg);
   const int nfg = min(2 * G, nf - f0);
   epi_fields_load<2 * G>(ep, f0, nfg, fi);
+  const float aj = a_ring[j];
   cp_async_wait_all();
   __syncthreads();
-  epi_prefetch_marginals<2 * G>(ep, fi, nfg, (size_t)j * N, (size_t)J * N, two, N, f0, (size_t)nlat * N);
+  epi_prefetch_marginals<2 * G, true>(ep, fi, nfg, (size_t)j * N, (size_t)J * N, two, N, f0, (size_t)nlat * N);
   unfold_spectra<G, NT>(stg, buf, N, ml.x, lmax);
   __syncthreads();
   const C2* z = fft_smem_plan<true, PL>(buf, b1, tw, pl, G);
   C2* other = (z == buf) ? b1 : buf;   // input of the fused forward transform
 
-  const float aj = a_ring[j];
   ring_pair_epilogue<G, NT>(z, other, ld, N, nf, f0, (size_t)nlat * N, (size_t)j * N, (size_t)J * N, two, aj, nh,
                                   jh, ep, red, fi);
   if ((ep.mode == EPI_UPDATE || ep.mode == EPI_SYM) && ep.xout) {

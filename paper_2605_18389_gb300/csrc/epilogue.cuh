@@ -58,8 +58,9 @@ __device__ __forceinline__ void epi_fields_load(const EpiParams& ep, int f0, int
 // After fi is visible to the block: asks L2 for the marginal rows j and J of the CTA's live
 // fields (UPDATE and CHECK modes) and, for the check, the rows of the u buffer it reads (fields
 // f0 + q at stride fstride in ep.other), one 128-byte line per thread, so that the epilogue's
-// loads hit L2 instead of waiting on DRAM after the inverse transform.
-template <int FG>
+// loads hit L2 instead of waiting on DRAM after the inverse transform.  TO_L1 (kernels with one
+// item a CTA): a load of each line whose value is not used, so that they hit L1.
+template <int FG, bool TO_L1 = false>
 __device__ __forceinline__ void epi_prefetch_marginals(const EpiParams& ep, const EpiField* fi, int nfg, size_t rj,
                                                        size_t rJ, bool two, int N, int f0 = 0, size_t fstride = 0) {
   if (ep.mode != EPI_UPDATE && ep.mode != EPI_CHECK && ep.mode != EPI_SYM) return;
@@ -77,8 +78,14 @@ __device__ __forceinline__ void epi_prefetch_marginals(const EpiParams& ep, cons
     const float* row = base + (ring ? rJ : rj);
     const uintptr_t a0 = reinterpret_cast<uintptr_t>(row) & ~uintptr_t(127);
     const uintptr_t a = a0 + (uintptr_t)l * 128;
-    if (a < reinterpret_cast<uintptr_t>(row + N))
+    if (a >= reinterpret_cast<uintptr_t>(row + N)) continue;
+    if constexpr (TO_L1) {   // a word of the line that belongs to the row
+      const uintptr_t w = a < reinterpret_cast<uintptr_t>(row) ? reinterpret_cast<uintptr_t>(row) : a;
+      float x;
+      asm volatile("ld.global.f32 %0, [%1];" : "=f"(x) : "l"(w));
+    } else {
       asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
+    }
   }
 }
 

@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  epi_prefetch_marginals<2>(ep, fi, nfg, rj, rJ, two, n, f0, npix);
+  epi_prefetch_marginals<2, true>(ep, fi, nfg, rj, rJ, two, n, f0, npix);
   for (int k = threadIdx.x; k < n; k += kHpThreads) za[k] = cadd(za[k], zb[k ? n - k : 0]);
   __syncthreads();
   C2* z = fft_smem<true>(za, zb, tw, pl, 1);   // K v on the ring pair

@@ -232,13 +232,10 @@ def algorithmic_work(kind, nlat, npix, lmax, nfields, legendre="table"):
     return 0.0, 0.0
 
 
-# DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) from ncu captures of
-# this file's 720 x 1440, 24-field TF32x3 runs of the kernels as they are (profiles/
-# ncu_k_idft_720x1440.md, ncu_k_legendre_tf32_720x1440.md); valid only for that workload and those
-# kernels.  The update kernel stores the scaling in 2 of a block's 20 half-steps.  Forms whose
-# kernels changed since their last capture (BF16x3, the recurrence mode) report null.
-NCU_TRAFFIC = {("inverse_dft_epilogue", "*", "*"): (18 * 223.2e6 + 2 * 313.5e6) / 20,   # same kernel in every form
-               ("legendre_analysis", "tf32x3", "table"): 524.6e6, ("legendre_synthesis", "tf32x3", "table"): 611.5e6}
+# DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) from ncu captures of this
+# file's 720 x 1440, 24-field runs, by (kind, precision, legendre); empty where the kernels have
+# changed since their last capture (the packed ring transforms and the polar cut): null in the line.
+NCU_TRAFFIC = {}
 
 
 def roofline(kind, avg_ms, nlat, npix, lmax, nfields, prec, legendre="table"):

@@ -20,8 +20,8 @@
 // length has a plan.  The composite radices (6, 9, 10, 12, 15, 16) run as two
 // register-resident levels of 2-, 3-, 4- and 5-point DFTs (Cooley-Tukey inside the
 // butterfly) whose internal twiddles are compile-time constants.  The stage twiddles come
-// from a per-stage table, r-major, so that consecutive lanes read consecutive entries; they are
-// read through L1 (every CTA reads the same N values).
+// from a per-stage table, r-major, so that consecutive lanes read consecutive entries: in shared
+// memory for short rings, through L1 for long ones (every CTA reads the same N values).
 #pragma once
 #include <utility>
 

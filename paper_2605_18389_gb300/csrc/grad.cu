@@ -73,11 +73,12 @@ struct GScal {      // per problem and iteration of a segment
 };
 
 // forward half-step: out = (m / Kf)^g; partial sums per ring of
-//   balanced: sum out;  unbalanced: sum a m out^{-eps/tau} = sum a out Kf (g (1 + eps/tau) = 1)
-// The powers bound the pointwise kernels of this file, so each node takes as few as the identity
-// allows: 32 fields at 256 rings, 33 us with a second power for the sum (see k_g_rev1 too).
+//   balanced: sum out;  unbalanced: sum a m out^{-eps/tau}
+// The sum keeps its own power: as sum a out Kf (g (1 + eps/tau) = 1) the kernel takes 21 instead of 33
+// us (32 fields, 256 rings), but tau/(2 eps) amplifies the sum's rounding and the gradient's error
+// against 64 bits grew by up to 2.5 times.  So did the reverse stage's with two powers a node.
 __global__ void k_g_update(Rings R, const float* __restrict__ a_ring, const float* const* __restrict__ marg,
-                           const float* __restrict__ Kf, float* __restrict__ out, int balanced, float gam,
+                           const float* __restrict__ Kf, float* __restrict__ out, int balanced, float gam, float et,
                            double* __restrict__ part) {
   __shared__ float red[32];
   const int j = blockIdx.x, b = blockIdx.y;
@@ -91,7 +92,7 @@ __global__ void k_g_update(Rings R, const float* __restrict__ a_ring, const floa
     const float r = mm / kf;
     const float u = balanced ? r : powf(r, gam);
     out[base + k] = u;
-    acc += balanced ? u : (mm > 0.f ? aj * u * kf : 0.f);
+    acc += balanced ? u : (mm > 0.f ? aj * mm * powf(u, -et) : 0.f);
   }
   const float t = block_sum_f(acc, red);
   if (threadIdx.x == 0) part[(size_t)b * R.nring + j] = (double)t;
@@ -227,9 +228,7 @@ __global__ void k_g_rscal(int nlat, const double* __restrict__ p1, const double*
   rs[b] = o;
 }
 
-// first pointwise reverse stage: u~' (before + K (Ku)~), (Ku)~, q~ updates.  Unbalanced, two powers
-// a node, A = u'^{-eps/tau} and B = v'^{-eps/tau}: u'^{-eps/tau-1} = A/u', v'^{1/g} = v'^{1+eps/tau} =
-// v'/B (with five powers 119 us for 32 fields at 256 rings).
+// first pointwise reverse stage: u~' (before + K (Ku)~), (Ku)~, q~ updates
 __global__ void k_g_rev1(Rings R, const float* __restrict__ a_ring, const float* const* __restrict__ P,
                          const float* const* __restrict__ Q, const float* __restrict__ U, const float* __restrict__ V,
                          const GScal* __restrict__ sc, const RevScal* __restrict__ rs, int balanced, float gam, float et,
@@ -255,26 +254,23 @@ __global__ void k_g_rev1(Rings R, const float* __restrict__ a_ring, const float*
   for (int k = threadIdx.x; k < nk; k += blockDim.x) {
     const float p = P[b][R.off[j] + k], q = Q[b][R.off[j] + k];
     const float u1 = U[base + k], v1 = V[base + k];
-    float uu, vv, qb = 0.f, vr = v1;   // qb: q~'s translation-invariant term; vr = v'^{1/g}
+    float uu, vv;
     if (balanced) {
       uu = al * ut[base + k] + sb;
       vv = be * vt[base + k];
     } else {
-      const float A = powf(u1, -et), B = powf(v1, -et);
-      uu = al * ut[base + k] - (p > 0.f ? Abar * et * p * (A / u1) : 0.f);
-      vv = be * vt[base + k] - (q > 0.f ? Bbar * et * q * (B / v1) : 0.f);
-      pt[base + k] += Abar * A;
-      qb = Bbar * B;
-      vr = v1 / B;
+      uu = al * ut[base + k] - (p > 0.f ? Abar * et * p * powf(u1, -et - 1.f) : 0.f);
+      vv = be * vt[base + k] - (q > 0.f ? Bbar * et * q * powf(v1, -et - 1.f) : 0.f);
+      pt[base + k] += Abar * powf(u1, -et);
+      qt[base + k] += Bbar * powf(v1, -et);
     }
     ut[base + k] = uu;
     if (q > 0.f) {
-      const float w = gam * vv * v1 / q;
-      kut[base + k] = -w * vr;
-      qt[base + k] = qt[base + k] + qb + w;
+      const float vg = balanced ? v1 * v1 : v1 * powf(v1, 1.f / gam);
+      kut[base + k] = -gam * vv * vg / q;
+      qt[base + k] += gam * vv * v1 / q;
     } else {
       kut[base + k] = 0.f;
-      if (!balanced) qt[base + k] += qb;
     }
   }
 }
@@ -510,10 +506,10 @@ int divergence_grad(Grid& g, const float* p, const float* q, int batch, double e
     int r;
     if ((r = heat_fields(g, vprev, kf, np, ps, st))) return r;
     count_launch();
-    k_g_update<<<ewp, kEw, 0, st>>>(rings, g.a_d, Pl, kf, uo, bal, gam, partU);
+    k_g_update<<<ewp, kEw, 0, st>>>(rings, g.a_d, Pl, kf, uo, bal, gam, et, partU);
     if ((r = heat_fields(g, uo, kf, np, nullptr, st))) return r;
     count_launch(2);
-    k_g_update<<<ewp, kEw, 0, st>>>(rings, g.a_d, Ql, kf, vo, bal, gam, partV);
+    k_g_update<<<ewp, kEw, 0, st>>>(rings, g.a_d, Ql, kf, vo, bal, gam, et, partV);
     k_g_scalars<<<np, 32, 0, st>>>(g.nlat, partU, partV, bal, eps, tau, slot, ps);
     SHOT_CUDA(cudaGetLastError());
     return SHOT_OK;

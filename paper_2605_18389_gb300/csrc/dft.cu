@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_idft(
     const float* __restrict__ a_ring, const __grid_constant__ FftPlan pl, const float2* tw, int tws,
     EpiParams ep) {
   extern __shared__ __align__(16) C2 sm[];
-  __shared__ float red[NT / 32][2 * NPART];
+  __shared__ EpiRed<G, NT> red;
   __shared__ EpiField fi[2 * G];
   const int N = nlon, ld = seq_ld(N);
   C2* buf = sm;
@@ -242,9 +242,9 @@ __global__ void __launch_bounds__(kThreads, kCtas) k_idft_p(
     const float* __restrict__ a_ring, const __grid_constant__ FftPlan pl, const float2* tw, EpiParams ep,
     int ngroups) {
   extern __shared__ __align__(16) C2 sm[];
-  __shared__ float red[kThreads / 32][2 * NPART];
-  __shared__ EpiField fi[2][2];
   constexpr int G = 1, NT = kThreads, FG = 2 * G;
+  __shared__ EpiRed<G, NT> red;
+  __shared__ EpiField fi[2][2];
   const int N = nlon, ld = seq_ld(N);
   C2* buf = sm;
   C2* b1 = buf + G * ld;

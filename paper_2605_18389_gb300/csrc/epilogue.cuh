@@ -89,28 +89,63 @@ __device__ __forceinline__ void epi_prefetch_marginals(const EpiParams& ep, cons
   }
 }
 
-__device__ __forceinline__ float epi_warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
+// How the sums of a field on a ring pair are formed: FP32 terms, the two rings' terms added first, then
+// a batch of longitudes, then a chain of batches (two alternating chains where a thread of a group of 32
+// has many), then groups of 32 / P lanes, and FP64 from there on, with at least eight partial sums per
+// field whatever number of threads share it.  No term passes more FP32 additions than with 256 threads
+// and eight warps per field (4 + 2 ceil(N / 256): a chain of both rings' terms and five lane steps),
+// which the short rings of G = 6 would otherwise exceed: 32 threads, 16 terms each.  The unbalanced
+// update amplifies the rounding of its sum by tau / eps.  Against one plain chain a thread and one sum
+// a warp: 40 iterations of 24 problems at 720 rings 35.9 -> 36.1 ms, four grids of 64 to 180 rings
+// 18.47 -> 18.55.
+__device__ __forceinline__ float add2(float a, float b) { return a + b; }
+template <class V, bool TWO = false>
+struct Chain {
+  V a{}, b{};
+  __device__ __forceinline__ void add(V x) {
+    const V t = add2(TWO ? b : a, x);
+    b = a;
+    a = t;
+  }
+  __device__ __forceinline__ V value() const { return TWO ? add2(a, b) : a; }
+};
+struct CompInf {   // the error beside the sum (Knuth's two-sum); an infinite sum stays infinite
+  float s = 0.f, c = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float t = s + x, b = t - s;
+    c += (s - (t - b)) + (x - b);
+    s = t;
+  }
+  __device__ __forceinline__ double value() const { return fabsf(s) < INFINITY ? (double)s + (double)c : (double)s; }
+};
 
-// The update of one K v value in full generality: u, the sums and the breakdown counts.
+// Partial sums of a CTA's warps: NT / G threads share a field pair, and each of their GW warps leaves P
+// sums of 32 / P lanes.
+template <int G, int NT>
+struct EpiRed {
+  static constexpr int GW = NT / G / 32, P = GW >= 8 ? 1 : GW >= 4 ? 2 : GW >= 2 ? 4 : 8;
+  static_assert(GW * P >= 8, "at least eight partial sums");
+  float v[NT / 32][P][2 * NPART];
+  double d[NT / 32][2][2];   // EPI_FINAL: warp sums of m(pi) and the objective
+};
+
+// The update of one K v value in full generality: u, the terms (t0, t1) of its two sums and the
+// breakdown counts.
 __device__ __forceinline__ float epi_update_value(float pm, float kv, float rr, bool bal, float gam, float aj,
-                                                  float (&acc)[NPART]) {
+                                                  float& t0, float& t1, float (&bad)[2]) {
   const float ratio = __fdividef(pm, kv) * rr;   // MUFU reciprocal + multiply, <= 2 ulp
   const float u = bal ? ratio : exp2f(gam * __log2f(ratio));
-  if (bal) {
-    acc[0] += u;
-  } else {
-    acc[0] += aj * u * kv * (1.f / rr);
-    acc[1] += u;
+  t0 = u;
+  t1 = 0.f;
+  if (!bal) {
+    t0 = aj * u * kv * (1.f / rr);
+    t1 = u;
   }
   // K v positive and finite, u finite (NaN fails each comparison); the failures are sorted into
   // non-positive (first in the status precedence) and non-finite
   if (!(kv > 0.f && kv < INFINITY && fabsf(u) < INFINITY)) {
-    if (kv <= 0.f) acc[2] += 1.f;
-    else acc[3] += 1.f;   // NaN or infinite K v, or u overflowed
+    if (kv <= 0.f) bad[0] += 1.f;
+    else bad[1] += 1.f;   // NaN or infinite K v, or u overflowed
   }
   return u;
 }
@@ -118,7 +153,7 @@ __device__ __forceinline__ float epi_update_value(float pm, float kv, float rr, 
 // The update of a pair of live fields on a ring pair.  u = (r p/Kv)^gamma (hardware log2/exp2,
 // ~2^-21 absolute in the exponent); the translation-invariant sum's p u^{-eps/tau} =
 // p (r p/Kv)^{-eps/(tau+eps)} equals u (Kv) / r since gamma + eps/(tau+eps) = 1, so one power serves
-// both (ratio = 0 gives u = 0 and adds nothing). 
+// both (ratio = 0 gives u = 0 and adds nothing).
 // An element whose four K v are normal and at most 2^125 takes the reciprocal directly (the value
 // __fdividef gives there); any other goes through epi_update_value.  The check for a non-finite u is
 // on the thread's sum: it is finite exactly if every u is (or the sum has overflowed, which stops
@@ -131,6 +166,8 @@ __device__ __forceinline__ void epi_update_pair(const float4* zg, float4* og, in
   constexpr int kBatch = 2;   // (4 measured slower: registers)
   const float rr[2] = {fi[0].r, fi[1].r}, ri[2] = {1.f / rr[0], 1.f / rr[1]}, gam[2] = {fi[0].gamma, fi[1].gamma};
   const bool bal0 = fi[0].balanced, bal1 = fi[1].balanced;
+  float bad[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+  Chain<f32x2, (GT < 64)> s0, s1;
   const float* m00 = fi[0].marg + rj + t;   // ring j of the first field; ring J starts dJ further
   const float* m10 = fi[1].marg + rj + t;
   const float* m01 = m00 + dJ;
@@ -146,6 +183,7 @@ __device__ __forceinline__ void epi_update_pair(const float4* zg, float4* og, in
     m10 += kBatch * GT;
     m01 += kBatch * GT;
     m11 += kBatch * GT;
+    f32x2 x0 = 0, x1 = 0;
 #pragma unroll
     for (int b = 0; b < kBatch; ++b) {
       const int k = k0 + b * GT;
@@ -154,31 +192,33 @@ __device__ __forceinline__ void epi_update_pair(const float4* zg, float4* og, in
       const uint32_t lo = 0x00800000u, span = 0x7e000000u - 0x00800000u;
       const uint32_t d = max(max(__float_as_uint(z.x) - lo, __float_as_uint(z.y) - lo),
                              max(__float_as_uint(z.z) - lo, __float_as_uint(z.w) - lo));
-      float4 u;
+      float4 u, v0, v1;   // the new scaling and the terms of its sums
       if (d <= span) {
-        auto one = [&](float pm, float kv, float r, float rinv, bool bal, float ga, float (&a)[NPART]) {
+        auto one = [&](float pm, float kv, float r, float rinv, bool bal, float ga, float& t0, float& t1) {
           float rc;
           asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(kv));
           const float ratio = pm * rc * r;
           const float w = bal ? ratio : exp2f(ga * __log2f(ratio));
-          if (bal) {
-            a[0] += w;
-          } else {
-            a[0] += aj * w * kv * rinv;
-            a[1] += w;
+          t0 = w;
+          t1 = 0.f;
+          if (!bal) {
+            t0 = aj * w * kv * rinv;
+            t1 = w;
           }
           return w;
         };
-        u.x = one(pv[b].x, z.x, rr[0], ri[0], bal0, gam[0], acc[0]);
-        u.y = one(pv[b].y, z.y, rr[1], ri[1], bal1, gam[1], acc[1]);
-        u.z = one(pv[b].z, z.z, rr[0], ri[0], bal0, gam[0], acc[0]);
-        u.w = one(pv[b].w, z.w, rr[1], ri[1], bal1, gam[1], acc[1]);
+        u.x = one(pv[b].x, z.x, rr[0], ri[0], bal0, gam[0], v0.x, v1.x);
+        u.y = one(pv[b].y, z.y, rr[1], ri[1], bal1, gam[1], v0.y, v1.y);
+        u.z = one(pv[b].z, z.z, rr[0], ri[0], bal0, gam[0], v0.z, v1.z);
+        u.w = one(pv[b].w, z.w, rr[1], ri[1], bal1, gam[1], v0.w, v1.w);
       } else {
-        u.x = epi_update_value(pv[b].x, z.x, rr[0], bal0, gam[0], aj, acc[0]);
-        u.y = epi_update_value(pv[b].y, z.y, rr[1], bal1, gam[1], aj, acc[1]);
-        u.z = epi_update_value(pv[b].z, z.z, rr[0], bal0, gam[0], aj, acc[0]);
-        u.w = epi_update_value(pv[b].w, z.w, rr[1], bal1, gam[1], aj, acc[1]);
+        u.x = epi_update_value(pv[b].x, z.x, rr[0], bal0, gam[0], aj, v0.x, v1.x, bad[0]);
+        u.y = epi_update_value(pv[b].y, z.y, rr[1], bal1, gam[1], aj, v0.y, v1.y, bad[1]);
+        u.z = epi_update_value(pv[b].z, z.z, rr[0], bal0, gam[0], aj, v0.z, v1.z, bad[0]);
+        u.w = epi_update_value(pv[b].w, z.w, rr[1], bal1, gam[1], aj, v0.w, v1.w, bad[1]);
       }
+      x0 = add2(x0, add2(pk2(v0.x, v0.y), pk2(v0.z, v0.w)));
+      if (!(bal0 && bal1)) x1 = add2(x1, add2(pk2(v1.x, v1.y), pk2(v1.z, v1.w)));
       if (out) {
         float* o = out + k;
         o[0] = u.x;
@@ -188,10 +228,20 @@ __device__ __forceinline__ void epi_update_pair(const float4* zg, float4* og, in
       }
       if (xout) og[k] = u;
     }
+    s0.add(x0);
+    s1.add(x1);
   }
+  const float2 a0 = unpk2(s0.value()), a1 = unpk2(s1.value());
+  acc[0][0] = a0.x;
+  acc[1][0] = a0.y;
+  acc[0][1] = a1.x;
+  acc[1][1] = a1.y;
 #pragma unroll
-  for (int q = 0; q < 2; ++q)
+  for (int q = 0; q < 2; ++q) {
+    acc[q][2] = bad[q][0];
+    acc[q][3] = bad[q][1];
     if (!(fabsf((q ? bal1 : bal0) ? acc[q][0] : acc[q][1]) < INFINITY) && acc[q][2] == 0.f) acc[q][3] += 1.f;
+  }
 }
 
 // kFinal = false compiles the EPI_FINAL branch out (kernels never launched with it).
@@ -202,8 +252,8 @@ template <int G, int NT, bool kFinal = true>
 __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int ld, int N, int nf, int f0,
                                                    size_t fstride, size_t rj, size_t rJ, bool two, float aj,
                                                    int nh, int jh, const EpiParams& ep,
-                                                   float (*red)[2 * NPART], const EpiField* fi) {
-  constexpr int GT = NT / G, GW = GT / 32;
+                                                   EpiRed<G, NT>& red, const EpiField* fi) {
+  constexpr int GT = NT / G, GW = GT / 32, P = EpiRed<G, NT>::P;
   static_assert(NT % G == 0 && GT % 32 == 0, "a group is whole warps");
   constexpr int kBatchGen = 2;   // the general path of the update
   constexpr int kEpiBatch = 4;   // longitudes per thread whose marginal values are loaded together
@@ -227,8 +277,8 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
     }
     return;
   }
-  // Per-element arithmetic is FP32; every thread sums its few elements (<= 2N/GT per
-  // field) in FP32, warps reduce in FP32 and the cross-warp / grid sums are FP64.
+  // Per-element arithmetic is FP32, and the sums as described at Chain; the final pass, which runs
+  // once a solve, compensates its threads' sums instead.
   float acc[2][NPART];
 #pragma unroll
   for (int q = 0; q < 2; ++q)
@@ -240,8 +290,6 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
   // thread as la sum p + lb sum q + sum (p log u_buf + q log v_buf), with the sums of p and q
   // (and the masses) compensated (Kahan) in FP32 and the offsets applied in FP64; per element
   // the work stays FP32.  m(pi) enters S_dual times eps.
-  __shared__ double redd[NT / 32][2][2];   // EPI_FINAL: warp sums of m(pi) and the objective
-
   if (ep.mode == EPI_UPDATE || ep.mode == EPI_SYM) {
     // both fields of an element in one pass: K v comes and the new scaling leaves as 16 bytes
     const bool sym = ep.mode == EPI_SYM;
@@ -264,11 +312,14 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
       gam[q] = f2[q].gamma;
       rr[q] = f2[q].r;
     }
+    Chain<f32x2, (GT < 64)> s0, s1;
+    float bad[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
     for (int k0 = t; k0 < N && nq > 0; k0 += kBatchGen * GT) {
       // the equator ring, an odd last field, frozen problems and self terms: field by field;
       // the marginal values (self term: and the old scaling's) of all this thread's longitudes
       // first, then the arithmetic; a frozen problem loads its stored scaling
       float pv[kBatchGen][2][2], uo[kBatchGen][2][2];
+      f32x2 x0 = 0, x1 = 0;
 #pragma unroll
       for (int b = 0; b < kBatchGen; ++b) {
         const int k = k0 + b * GT;
@@ -286,7 +337,7 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
         const int k = k0 + b * GT;
         if (k >= N) break;
         const float4 zz = zg[k];
-        float un[2][2];
+        float un[2][2], v0[2] = {0.f, 0.f}, v1[2] = {0.f, 0.f};
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           un[q][0] = uo[b][q][0];
@@ -303,18 +354,33 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
               const float x = bal[q] ? ratio : exp2f(gam[q] * __log2f(ratio));
               u = sqrtf(uo[b][q][r] * x);
               if (!(kv > 0.f && kv < INFINITY && fabsf(u) < INFINITY)) {
-                if (kv <= 0.f) acc[q][2] += 1.f;
-                else acc[q][3] += 1.f;
+                if (kv <= 0.f) bad[q][0] += 1.f;
+                else bad[q][1] += 1.f;
               }
             } else {
-              u = epi_update_value(pm, kv, rr[q], bal[q], gam[q], aj, acc[q]);
+              float t0, t1;
+              u = epi_update_value(pm, kv, rr[q], bal[q], gam[q], aj, t0, t1, bad[q]);
+              v0[q] = r ? v0[q] + t0 : t0;
+              v1[q] = r ? v1[q] + t1 : t1;
             }
             if (sym || !ep.skip_store) outf[q][(r ? rJ : rj) + k] = u;
             un[q][r] = u;
           }
         }
+        x0 = add2(x0, pk2(v0[0], v0[1]));
+        x1 = add2(x1, pk2(v1[0], v1[1]));
         if (ep.xout) og[k] = make_float4(un[0][0], un[1][0], un[0][1], un[1][1]);
       }
+      s0.add(x0);
+      s1.add(x1);
+    }
+    const float2 a0 = unpk2(s0.value()), a1 = unpk2(s1.value());
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      acc[q][0] = q ? a0.y : a0.x;
+      acc[q][1] = q ? a1.y : a1.x;
+      acc[q][2] = bad[q][0];
+      acc[q][3] = bad[q][1];
     }
     }
   } else {
@@ -330,6 +396,7 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
       if (ep.mode == EPI_CHECK) {
         const float* mg = F.marg;
         const float cuv = ep.ps[f].cuv;
+        Chain<float> e0, e1;
         for (int k0 = t; k0 < N; k0 += kEpiBatch * GT) {
           // the marginal and u values of all this thread's longitudes first, then the arithmetic
           float pv[kEpiBatch][2], uv[kEpiBatch][2];
@@ -341,10 +408,12 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
             uv[b][0] = (k < N) ? __ldg(othf + rj + k) : 0.f;
             uv[b][1] = (k < N && two) ? __ldg(othf + rJ + k) : 0.f;
           }
+          float x0[kEpiBatch], x1[kEpiBatch];
 #pragma unroll
           for (int b = 0; b < kEpiBatch; ++b) {
             const int k = k0 + b * GT;
-            if (k >= N) break;
+            x0[b] = x1[b] = 0.f;
+            if (k >= N) continue;
             const float4 zz = zg[k];
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
@@ -352,16 +421,17 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
               const float kv = q ? (r ? zz.w : zz.y) : (r ? zz.z : zz.x);
               const float pm = pv[b][r];
               const float d = fmaf(cuv * uv[b][r], kv, -pm);
-              if (ep.norm_l1) {
-                acc[q][0] += aj * fabsf(d);
-                acc[q][1] += aj * pm;
-              } else {
-                acc[q][0] += d * d;
-                acc[q][1] += pm * pm;
-              }
+              const float t0 = ep.norm_l1 ? aj * fabsf(d) : d * d, t1 = ep.norm_l1 ? aj * pm : pm * pm;
+              x0[b] = r ? x0[b] + t0 : t0;
+              x1[b] = r ? x1[b] + t1 : t1;
             }
           }
+          static_assert(kEpiBatch == 4, "a batch's terms are added as a tree");
+          e0.add((x0[0] + x0[1]) + (x0[2] + x0[3]));
+          e1.add((x1[0] + x1[1]) + (x1[2] + x1[3]));
         }
+        acc[q][0] = e0.value();
+        acc[q][1] = e1.value();
       } else if constexpr (kFinal) {  // EPI_FINAL: z = K v_buf; ep.other = u buffer, ep.out = v buffer
         const ProbState* P = ep.ps + f;
         const float* pp = ep.marg[f];
@@ -377,7 +447,8 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
         const float epsf = (float)ep.eps, tauf = (float)P->tau, et = bal ? 0.f : (float)(ep.eps / P->tau);
         // balanced: A = sum p, B = sum q (compensated), C = sum p log u_buf + q log v_buf, D = sum
         // u (K v) (m(pi) before any v-update); unbalanced: A = sum u (K v), B = the objective's terms
-        float A = 0.f, Ac = 0.f, B = 0.f, Bc = 0.f, C = 0.f, D = 0.f;
+        float A = 0.f, Ac = 0.f, B = 0.f, Bc = 0.f;
+        CompInf C, D, e0, e1;
         auto kahan = [](float& s, float& c, float x) {
           const float y = x - c, t = s + y;
           c = (t - s) - y;
@@ -402,21 +473,16 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
             }
             const float ukv = cuv * ub * kv;   // u_true (K v_true)
             const float d = ukv - pm;
-            if (ep.norm_l1) {
-              acc[q][0] += aj * fabsf(d);
-              acc[q][1] += aj * pm;
-            } else {
-              acc[q][0] += d * d;
-              acc[q][1] += pm * pm;
-            }
+            e0.add(ep.norm_l1 ? aj * fabsf(d) : d * d);
+            e1.add(ep.norm_l1 ? aj * pm : pm * pm);
             // phi = eps log u, psi = eps log v (App. C.2); terms with a zero marginal vanish.
             // Balanced: p (la + log u_buf) + q (lb + log v_buf), the offsets applied per thread
             // below; eps and a_j multiply the sums.
             if (bal) {
               kahan(A, Ac, pm);
               kahan(B, Bc, qm);
-              C += (pm > 0.f ? pm * logf(ub) : 0.f) + (qm > 0.f ? qm * logf(vb) : 0.f);
-              D += ukv;
+              C.add((pm > 0.f ? pm * logf(ub) : 0.f) + (qm > 0.f ? qm * logf(vb) : 0.f));
+              D.add(ukv);
             } else {  // tau (1 - e^{-phi/tau}) = -tau expm1(-(eps/tau) log u), per node in FP32
               kahan(A, Ac, ukv);
               kahan(B, Bc, (pm > 0.f ? -tauf * expm1f(-et * lu) * pm : 0.f) +
@@ -424,11 +490,13 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
             }
           }
         }
+        acc[q][0] = (float)e0.value();
+        acc[q][1] = (float)e1.value();
         // this thread's m(pi) and objective in FP64, then the warp's sums
         double vm, vo;
         if (bal) {
-          vm = mass_q ? (double)B - (double)Bc : (double)D;
-          vo = P->la * ((double)A - (double)Ac) + P->lb * ((double)B - (double)Bc) + (double)C;
+          vm = mass_q ? (double)B - (double)Bc : D.value();
+          vo = P->la * ((double)A - (double)Ac) + P->lb * ((double)B - (double)Bc) + C.value();
         } else {
           vm = (double)A - (double)Ac;
           vo = (double)B - (double)Bc;
@@ -439,8 +507,8 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
           vo += __shfl_xor_sync(0xffffffffu, vo, o);
         }
         if ((threadIdx.x & 31) == 0) {
-          redd[threadIdx.x >> 5][q][0] = vm;
-          redd[threadIdx.x >> 5][q][1] = vo;
+          red.d[threadIdx.x >> 5][q][0] = vm;
+          red.d[threadIdx.x >> 5][q][1] = vo;
         }
       }
     }
@@ -451,8 +519,10 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
   for (int q = 0; q < 2; ++q)
 #pragma unroll
     for (int i = 0; i < NPART; ++i) {
-      const float v = epi_warp_sum(acc[q][i]);
-      if (lane == 0) red[wid][q * NPART + i] = v;
+      float v = acc[q][i];
+#pragma unroll
+      for (int o = 16; o >= P; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane < P) red.v[wid][lane][q * NPART + i] = v;
     }
   __syncthreads();
   if constexpr (kFinal) {
@@ -460,7 +530,7 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
       const int fq = threadIdx.x >> 1, i = threadIdx.x & 1;   // field of the CTA
       if (f0 + fq < nf && fi[fq].live) {
         double s = 0.0;
-        for (int w = 0; w < GW; ++w) s += redd[(fq >> 1) * GW + w][fq & 1][i];
+        for (int w = 0; w < GW; ++w) s += red.d[(fq >> 1) * GW + w][fq & 1][i];
         // m(pi) sums a_j times the node values; the balanced objective's sums are of
         // p (la + log u_buf) + q (lb + log v_buf): times eps a_j
         const double sc = (i == 1 && fi[fq].balanced) ? ep.eps * (double)aj : (double)aj;
@@ -468,13 +538,25 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
       }
     }
   }
-  if (threadIdx.x < 2 * G * NPART) {
-    const int fq = threadIdx.x / NPART, i = threadIdx.x - fq * NPART;
-    if (f0 + fq < nf && fi[fq].live && !(ep.mode == EPI_FINAL && i >= 2)) {
-      double s = 0.0;
-      for (int w = 0; w < GW; ++w) s += (double)red[(fq >> 1) * GW + w][(fq & 1) * NPART + i];
-      ep.part[((size_t)(f0 + fq) * nh + jh) * NPART + i] = s;
+  // four lanes a sum: the FP64 additions of one thread would be a chain that the CTA waits for
+  constexpr int kSums = 2 * G * NPART;
+  static_assert(4 * kSums <= NT && (4 * kSums < 32 || 4 * kSums % 32 == 0), "whole warps, or one");
+  int tid = threadIdx.x;
+  asm volatile("" : "+r"(tid));   // keeps a persistent kernel's loop from carrying the indices below
+  if (tid < 4 * kSums) {
+    const int x = tid >> 2, fq = x / NPART, i = x - fq * NPART;
+    const int w0 = fq / 2 * GW, c = fq % 2 * NPART + i;
+    double s = 0.0;
+#pragma unroll
+    for (int y = 0; y < (GW * P + 3) / 4; ++y) {
+      const int e = 4 * y + (tid & 3);
+      if (e < GW * P) s += (double)red.v[w0 + e / P][e % P][c];
     }
+    constexpr unsigned kMask = 4 * kSums >= 32 ? 0xffffffffu : (1u << (4 * kSums % 32)) - 1;
+    s += __shfl_xor_sync(kMask, s, 1);
+    s += __shfl_xor_sync(kMask, s, 2);
+    if ((tid & 3) == 0 && f0 + fq < nf && fi[fq].live && !(ep.mode == EPI_FINAL && i >= 2))
+      ep.part[((size_t)(f0 + fq) * nh + jh) * NPART + i] = s;
   }
 }
 

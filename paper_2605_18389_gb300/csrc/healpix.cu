@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
                                                         const int* __restrict__ tw_base, int tws) {
   extern __shared__ __align__(16) C2 sm[];
   __shared__ FftPlan pl;
-  __shared__ float red[kHpThreads / 32][2 * NPART];
+  __shared__ EpiRed<1, kHpThreads> red;
   __shared__ EpiField fi[2];
   const int jh = blockIdx.y, f0 = blockIdx.x * 2;
   const int nfg = min(2, nf - f0);

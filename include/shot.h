@@ -126,6 +126,8 @@ int shot_grid_init_quad(shot_grid* out, int quadrature, int nlat, int nlon, int 
  * pixels in ring order ([batch][N] wherever the other calls say [batch][nlat][nlon]).  There is
  * no exact quadrature: the heat operator is H diag(a) on the pixel centres (addition theorem).
  *   nside in 1..4096; lmax = -1 means 3 nside - 1, else 0 <= lmax <= 4 nside - 2;
+ *   the ring transforms hold a ring in an SM's shared memory: up to nside 3599 (a field pair at a time
+ *   below 1800, one field from there on), beyond which every call that transforms is UNSUPPORTED;
  *   precision, legendre_mode as shot_grid_init.  shot_grid_info reports nlat = 4 nside - 1
  *   rings and nlon = 4 nside (the longest ring).
  * Supported on HEALPix grids: shot_heat_apply(_noalloc), shot_sht_analysis/synthesis,

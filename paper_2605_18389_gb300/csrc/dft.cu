@@ -22,9 +22,9 @@ namespace shot {
 
 namespace {
 
-// A CTA of 192 threads takes one ring pair of 2 G fields, two fields an element (fft.cuh); in the
-// pointwise parts each of its G groups of 192 / G threads (whole warps for G = 1, 2, 3, 6) takes
-// one pair of fields.  192 threads cover most butterflies of a long ring's stages in one step (96,
+// A CTA of 192 threads takes one ring pair of F G fields, F = 2 (E = C2) or 1 (C1) fields an element
+// (fft.cuh); in the pointwise parts each of its G groups of 192 / G threads (whole warps for G = 1, 2,
+// 3, 6) takes one element's fields.  192 threads cover most butterflies of a long ring's stages in one step (96,
 // 180 and 120 at 1440 longitudes), and three CTAs an SM leave 112 registers a thread, enough for
 // the packed radix-16 butterfly without spills.
 constexpr int kThreads = 192;
@@ -32,6 +32,11 @@ constexpr int kCtas = 3;
 
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)),
+               "l"(gmem)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)),
                "l"(gmem)
                : "memory");
 }
@@ -47,34 +52,37 @@ struct Group {
 };
 
 // Loads rings j (real parts) and J = nlat-1-j (imaginary parts; zero when J == j) of the CTA's
-// fields into buf; the second field of an odd last pair is zero.  Four rows of a batch of
+// fields into buf; the second field of an odd last pair is zero.  All rows of a batch of
 // longitudes are in flight per thread.
-template <int G, int NT>
-__device__ __forceinline__ void load_ring_pairs(const float* __restrict__ in, C2* buf, int f0, int nf, int nlat, int N,
+template <int G, int NT, class E>
+__device__ __forceinline__ void load_ring_pairs(const float* __restrict__ in, E* buf, int f0, int nf, int nlat, int N,
                                                 int j, int J) {
+  constexpr int F = E::F;
   const Group<G, NT> gr;
-  const int fa = f0 + 2 * gr.g;
+  const int fa = f0 + F * gr.g;
   if (fa >= nf) return;
-  const bool second = fa + 1 < nf, two = J != j;
+  const bool two = J != j;
   const size_t fs = (size_t)nlat * N;
   const float* aj = in + (size_t)fa * fs + (size_t)j * N;
   const float* aJ = in + (size_t)fa * fs + (size_t)J * N;
-  float4* b = reinterpret_cast<float4*>(buf + gr.g * seq_ld(N));
+  E* b = buf + gr.g * seq_ld(N);
   constexpr int kBatch = 4;
   for (int k0 = gr.t; k0 < N; k0 += kBatch * gr.T) {
-    float4 v[kBatch];
+    float v[kBatch][2][F];
 #pragma unroll
     for (int i = 0; i < kBatch; ++i) {
       const int k = k0 + i * gr.T;
-      v[i].x = k < N ? __ldg(aj + k) : 0.f;
-      v[i].y = (k < N && second) ? __ldg(aj + fs + k) : 0.f;
-      v[i].z = (k < N && two) ? __ldg(aJ + k) : 0.f;
-      v[i].w = (k < N && two && second) ? __ldg(aJ + fs + k) : 0.f;
+#pragma unroll
+      for (int q = 0; q < F; ++q) {
+        const bool on = k < N && fa + q < nf;
+        v[i][0][q] = on ? __ldg(aj + q * fs + k) : 0.f;
+        v[i][1][q] = (on && two) ? __ldg(aJ + q * fs + k) : 0.f;
+      }
     }
 #pragma unroll
     for (int i = 0; i < kBatch; ++i) {
       const int k = k0 + i * gr.T;
-      if (k < N) b[k] = v[i];
+      if (k < N) b[k] = cx(of_lanes(v[i][0]), of_lanes(v[i][1]));
     }
   }
 }
@@ -83,13 +91,16 @@ __device__ __forceinline__ void load_ring_pairs(const float* __restrict__ in, C2
 // mmax (the (2m+1) block of m = lmax is empty), into stg[blk][G] with asynchronous copies.  Row (blk,
 // jh) holds the fields' (re, im) pairs contiguously; an even first field starts on a 16-byte
 // boundary (ldc is a multiple of 4), and reading up to the next even field stays inside the row.
-template <int G, int NT>
+template <int G, int NT, class E>
 __device__ __forceinline__ void issue_spectra(const float* __restrict__ Y, int ldc, int nh, int mmax, int lmax, int jh, int f0,
-                                              int nf, float4* stg) {
+                                              int nf, typename Piece<E>::T* stg) {
   const int nblk = min(2 * mmax + 2, 2 * lmax + 1);
   const float* y = Y + (size_t)jh * ldc + 2 * f0;
   const size_t row = (size_t)nh * ldc;
-  if (G == 1) {
+  if constexpr (E::F == 1) {
+    static_assert(G == 1, "one field a CTA");
+    for (int blk = threadIdx.x; blk < nblk; blk += NT) cp_async8(stg + blk, y + blk * row);
+  } else if (G == 1) {
     for (int blk = threadIdx.x; blk < nblk; blk += NT) cp_async16(stg + blk, y + blk * row);
   } else {   // consecutive threads read the pieces of a row
     for (int e = threadIdx.x; e < nblk * G; e += NT) {
@@ -100,24 +111,23 @@ __device__ __forceinline__ void issue_spectra(const float* __restrict__ Y, int l
   cp_async_commit();
 }
 
-// Unfolds the staged spectra into the Hermitian-extended Z of each pair of fields:
+// Unfolds the staged spectra into the Hermitian-extended Z of each element:
 // G_N = E + O, G_S = E - O, Z(m) = G_N + i G_S, Z(N-m) = conj G_N + i conj G_S; the band
 // mmax < m < N - mmax is zero.
-template <int G, int NT>
-__device__ __forceinline__ void unfold_spectra(const float4* stg, C2* buf, int N, int mmax, int lmax) {
+template <int G, int NT, class E>
+__device__ __forceinline__ void unfold_spectra(const typename Piece<E>::T* stg, E* buf, int N, int mmax, int lmax) {
   const Group<G, NT> gr;
-  C2* z = buf + gr.g * seq_ld(N);
-  for (int k = mmax + 1 + gr.t; k < N - mmax; k += gr.T) z[k] = c2(0ull, 0ull);
+  E* z = buf + gr.g * seq_ld(N);
+  for (int k = mmax + 1 + gr.t; k < N - mmax; k += gr.T) z[k] = E{};
   for (int m = gr.t; m <= mmax; m += gr.T) {
-    const float4 e = stg[2 * m * G + gr.g];
-    const float4 o = m < lmax ? stg[(2 * m + 1) * G + gr.g] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const C2 E = c2(pk2(e.x, e.z), pk2(e.y, e.w)), O = c2(pk2(o.x, o.z), pk2(o.y, o.w));
-    const C2 GN = cadd(E, O), GS = csub(E, O);
+    const E e = piece_value(stg[2 * m * G + gr.g]);
+    const E o = m < lmax ? piece_value(stg[(2 * m + 1) * G + gr.g]) : E{};
+    const E GN = cadd(e, o), GS = csub(e, o);
     if (m == 0) {
-      z[0] = c2(GN.re, GS.re);
+      z[0] = cx(GN.re, GS.re);
     } else {
-      z[m] = c2(sub2(GN.re, GS.im), add2(GN.im, GS.re));
-      z[N - m] = c2(add2(GN.re, GS.im), sub2(GS.re, GN.im));
+      z[m] = cx(sub2(GN.re, GS.im), add2(GN.im, GS.re));
+      z[N - m] = cx(add2(GN.re, GS.im), sub2(GS.re, GN.im));
     }
   }
 }
@@ -125,49 +135,50 @@ __device__ __forceinline__ void unfold_spectra(const float4* stg, C2* buf, int N
 // Two-for-one unpack of the transformed ring pair (j north, J south) and the parity fold:
 // F_N(m) = (Z(m) + conj Z(N-m))/2, F_S(m) = (Z(m) - conj Z(N-m))/(2i);
 // S = a_j (F_N + F_S) -> block (m, even), D = a_j (F_N - F_S) -> block (m, odd), m <= mmax.
-// The columns of an odd last field's missing partner (padding, inside ldc) take its zeros.
-template <int G, int NT>
-__device__ __forceinline__ void fold_store(const C2* buf, int f0, int nf, int N, int mmax, int nh, int jh, float aj,
+// The columns of an odd last field's missing partner (padding, inside ldc) take a pair's zeros.
+template <int G, int NT, class E>
+__device__ __forceinline__ void fold_store(const E* buf, int f0, int nf, int N, int mmax, int nh, int jh, float aj,
                                            const ProbState* __restrict__ ps, int scale_which, float* __restrict__ X,
                                            int ldc) {
+  constexpr int F = E::F;
+  typedef typename E::V V;
   const Group<G, NT> gr;
-  const int fa = f0 + 2 * gr.g;
+  const int fa = f0 + F * gr.g;
   if (fa >= nf) return;
-  float s0 = 0.5f * aj, s1 = s0;
-  if (scale_which == 1) {
-    s0 *= (float)ps[fa].beta;
-    if (fa + 1 < nf) s1 *= (float)ps[fa + 1].beta;
+  float sf[F];
+#pragma unroll
+  for (int q = 0; q < F; ++q) {
+    sf[q] = 0.5f * aj;
+    if (scale_which == 1 && fa + q < nf) sf[q] *= (float)ps[fa + q].beta;
   }
-  const f32x2 sc = pk2(s0, s1);
-  const C2* z = buf + gr.g * seq_ld(N);
+  const V sc = of_lanes(sf);
+  const E* z = buf + gr.g * seq_ld(N);
   float* x = X + (size_t)jh * ldc + 2 * fa;
   const size_t row = (size_t)nh * ldc;
   for (int m = gr.t; m <= mmax; m += gr.T) {
-    const C2 zm = z[m], zn = z[m ? N - m : 0];
-    const f32x2 a = add2(zm.re, zn.re), b = sub2(zm.im, zn.im);   // 2 F_N
-    const f32x2 c = add2(zm.im, zn.im), d = sub2(zm.re, zn.re);   // 2 F_S = (c, -d)
-    const float2 Sr = unpk2(mul2(sc, add2(a, c))), Si = unpk2(mul2(sc, sub2(b, d)));
-    const float2 Dr = unpk2(mul2(sc, sub2(a, c))), Di = unpk2(mul2(sc, add2(b, d)));
-    float4* o = reinterpret_cast<float4*>(x + (size_t)(2 * m) * row);
-    *o = make_float4(Sr.x, Si.x, Sr.y, Si.y);
-    *reinterpret_cast<float4*>(x + (size_t)(2 * m + 1) * row) = make_float4(Dr.x, Di.x, Dr.y, Di.y);
+    const E zm = z[m], zn = z[m ? N - m : 0];
+    const V a = add2(zm.re, zn.re), b = sub2(zm.im, zn.im);   // 2 F_N
+    const V c = add2(zm.im, zn.im), d = sub2(zm.re, zn.re);   // 2 F_S = (c, -d)
+    store_piece(x + (size_t)(2 * m) * row, cx(mul2(sc, add2(a, c)), mul2(sc, sub2(b, d))));
+    store_piece(x + (size_t)(2 * m + 1) * row, cx(mul2(sc, sub2(a, c)), mul2(sc, add2(b, d))));
   }
 }
 
-template <int G, int NT, int CTAS, class PL>
+template <int G, int NT, int CTAS, class PL, class E>
 __global__ void __launch_bounds__(NT, CTAS) k_dft_fwd(
     const float* __restrict__ in, int nf, int nlat, int nlon, int lmax, int nh,
     const float* __restrict__ a_ring, const ProbState* __restrict__ ps, int scale_which,
     float* __restrict__ X, int ldc, const __grid_constant__ FftPlan pl, const float2* tw, int tws,
     const int2* __restrict__ mlim, float* __restrict__ h, double t) {
-  extern __shared__ __align__(16) C2 sm[];
+  extern __shared__ __align__(16) uint8_t smem[];
+  E* sm = reinterpret_cast<E*>(smem);
   if (blockIdx.y == gridDim.y - 1 && h) {   // the heat multipliers
     for (int l = blockIdx.x * blockDim.x + threadIdx.x; l <= lmax; l += gridDim.x * blockDim.x) h[l] = heat_mult(t, l);
     return;
   }
-  C2* b0 = sm;
-  C2* b1 = b0 + G * seq_ld(nlon);
-  const int jh = blockIdx.y, f0 = blockIdx.x * 2 * G;
+  E* b0 = sm;
+  E* b1 = b0 + G * seq_ld(nlon);
+  const int jh = blockIdx.y, f0 = blockIdx.x * E::F * G;
   if (tws) {   // twiddles beside the sequences
     fft_copy_twiddles(reinterpret_cast<float2*>(b1 + G * seq_ld(nlon)), tw, tws);
     tw = reinterpret_cast<const float2*>(b1 + G * seq_ld(nlon));
@@ -175,48 +186,50 @@ __global__ void __launch_bounds__(NT, CTAS) k_dft_fwd(
   load_ring_pairs<G, NT>(in, b0, f0, nf, nlat, nlon, jh, nlat - 1 - jh);
   cp_async_wait_all();
   __syncthreads();
-  const C2* buf = fft_smem_plan<false, PL>(b0, b1, tw, pl, G);
+  const E* buf = fft_smem_plan<false, PL>(b0, b1, tw, pl, G);
   fold_store<G, NT>(buf, f0, nf, nlon, mlim ? mlim[jh].y : lmax, nh, jh, a_ring[jh], ps, scale_which, X, ldc);
 }
 
-template <int G, int NT, int CTAS, class PL>
+template <int G, int NT, int CTAS, class PL, class E>
 __global__ void __launch_bounds__(NT, CTAS) k_idft(
     const float* __restrict__ Y, int ldc, int nf, int nlat, int nlon, int lmax, int nh,
     const float* __restrict__ a_ring, const __grid_constant__ FftPlan pl, const float2* tw, int tws,
     EpiParams ep) {
-  extern __shared__ __align__(16) C2 sm[];
-  __shared__ EpiRed<G, NT> red;
-  __shared__ EpiField fi[2 * G];
+  extern __shared__ __align__(16) uint8_t smem[];
+  E* sm = reinterpret_cast<E*>(smem);
+  constexpr int FG = E::F * G;
+  __shared__ EpiRed<G, NT, E::F> red;
+  __shared__ EpiField fi[FG];
   const int N = nlon, ld = seq_ld(N);
-  C2* buf = sm;
-  C2* b1 = buf + G * ld;
-  const int jh = blockIdx.y, f0 = blockIdx.x * 2 * G;
+  E* buf = sm;
+  E* b1 = buf + G * ld;
+  const int jh = blockIdx.y, f0 = blockIdx.x * FG;
   const int j = jh, J = nlat - 1 - jh;
   const bool two = (J != j);   // false only for the equator ring of an odd grid
   if (tws) {   // twiddles beside the sequences
     fft_copy_twiddles(reinterpret_cast<float2*>(b1 + G * ld), tw, tws);
     tw = reinterpret_cast<const float2*>(b1 + G * ld);
   }
-  float4* stg = reinterpret_cast<float4*>(b1);   // the spectra, before the transform needs b1
+  typename Piece<E>::T* stg = reinterpret_cast<typename Piece<E>::T*>(b1);   // the spectra, before the transform needs b1
   const int2 ml = ep.mlim ? ep.mlim[jh] : make_int2(lmax, lmax);   // orders read, orders written
-  issue_spectra<G, NT>(Y, ldc, nh, ml.x, lmax, jh, f0, nf, stg);
-  const int nfg = min(2 * G, nf - f0);
-  epi_fields_load<2 * G>(ep, f0, nfg, fi);
+  issue_spectra<G, NT, E>(Y, ldc, nh, ml.x, lmax, jh, f0, nf, stg);
+  const int nfg = min(FG, nf - f0);
+  epi_fields_load<FG>(ep, f0, nfg, fi);
   const float aj = a_ring[j];
   cp_async_wait_all();
   __syncthreads();
-  epi_prefetch_marginals<2 * G, true>(ep, fi, nfg, (size_t)j * N, (size_t)J * N, two, N, f0, (size_t)nlat * N);
+  epi_prefetch_marginals<FG, true>(ep, fi, nfg, (size_t)j * N, (size_t)J * N, two, N, f0, (size_t)nlat * N);
   unfold_spectra<G, NT>(stg, buf, N, ml.x, lmax);
   __syncthreads();
-  const C2* z = fft_smem_plan<true, PL>(buf, b1, tw, pl, G);
-  C2* other = (z == buf) ? b1 : buf;   // input of the fused forward transform
+  const E* z = fft_smem_plan<true, PL>(buf, b1, tw, pl, G);
+  E* other = (z == buf) ? b1 : buf;   // input of the fused forward transform
 
   ring_pair_epilogue<G, NT>(z, other, ld, N, nf, f0, (size_t)nlat * N, (size_t)j * N, (size_t)J * N, two, aj, nh,
                                   jh, ep, red, fi);
   if ((ep.mode == EPI_UPDATE || ep.mode == EPI_SYM) && ep.xout) {
     // the new scaling of this ring pair is in `other`: transform it for the next half-step
     __syncthreads();
-    const C2* zf = fft_smem_plan<false, PL>(other, const_cast<C2*>(z), tw, pl, G);
+    const E* zf = fft_smem_plan<false, PL>(other, const_cast<E*>(z), tw, pl, G);
     fold_store<G, NT>(zf, f0, nf, N, ml.y, nh, jh, aj, nullptr, 0, ep.xout, ldc);
   }
 }
@@ -243,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, kCtas) k_idft_p(
     int ngroups) {
   extern __shared__ __align__(16) C2 sm[];
   constexpr int G = 1, NT = kThreads, FG = 2 * G;
-  __shared__ EpiRed<G, NT> red;
+  __shared__ EpiRed<G, NT, 2> red;
   __shared__ EpiField fi[2][2];
   const int N = nlon, ld = seq_ld(N);
   C2* buf = sm;
@@ -257,7 +270,7 @@ __global__ void __launch_bounds__(kThreads, kCtas) k_idft_p(
   int jh = item / ngroups, f0 = (item - jh * ngroups) * FG;
   if (item < nitems) {
     epi_fields_load<FG>(ep, f0, min(FG, nf - f0), fi[0]);
-    issue_spectra<G, NT>(Y, ldc, nh, orders(jh).x, lmax, jh, f0, nf, stg);
+    issue_spectra<G, NT, C2>(Y, ldc, nh, orders(jh).x, lmax, jh, f0, nf, stg);
   }
   __syncthreads();
   if (item < nitems)
@@ -274,7 +287,7 @@ __global__ void __launch_bounds__(kThreads, kCtas) k_idft_p(
     __syncthreads();
     if (next < nitems) {   // the staging area is free again: the next item's state and spectra
       epi_fields_load<FG>(ep, fn, nn, fi[slot ^ 1]);
-      issue_spectra<G, NT>(Y, ldc, nh, orders(jn).x, lmax, jn, fn, nf, stg);
+      issue_spectra<G, NT, C2>(Y, ldc, nh, orders(jn).x, lmax, jn, fn, nf, stg);
     }
     const C2* z = fft_smem_plan<true, PL>(buf, b1, tw, pl, G);
     C2* other = (z == buf) ? b1 : buf;
@@ -311,6 +324,18 @@ int pick_g(const Grid& g, int nf) {
   return G;
 }
 
+template <class E>
+size_t idft_smem(int G, int N) { return (size_t)2 * G * seq_ld(N) * sizeof(E); }
+
+// the runtime plan equals the compile-time one (same N and radices in the same order)
+template <class PL>
+bool plan_is(const FftPlan& p) {
+  return p.N == PL::N && p.nst == 3 && p.R[0] == PL::R0 && p.R[1] == PL::R1 && p.R[2] == PL::R2;
+}
+// plans compiled for the ring lengths of the 720- and 512-ring grids (one pair of fields a CTA)
+using Plan1440 = CtPlan<1440, 15, 8, 12>;
+using Plan1024 = CtPlan<1024, 4, 16, 16>;
+
 // Entries of the twiddle table a CTA copies into shared memory: all for rings of up to 768
 // longitudes (6 KB), where a CTA has few items and would wait for each stage's twiddles from L2 (32
 // rings, one field: 9.4 us an update launch without the copy, 7.3 with it in the scalar form); none
@@ -318,34 +343,34 @@ int pick_g(const Grid& g, int nf) {
 constexpr int kTwMax = 768;
 int twiddles_in_smem(const Grid& g) { return g.nlon <= kTwMax ? fft_tw_len(g.plan) : 0; }
 
-size_t idft_smem(int G, int N) { return (size_t)2 * G * seq_ld(N) * sizeof(C2); }
-
-template <int G, class PL = RuntimePlan, int NT = kThreads, int CTAS = kCtas>
+template <int G, class PL = RuntimePlan, int NT = kThreads, int CTAS = kCtas, class E = C2>
 int launch_fwd_t(const Grid& g, const float* in, int nf, const ProbState* ps, int scale_which, float* X,
                  int ldc, cudaStream_t st, const int2* mlim, const double* heat_t) {
   const int tws = twiddles_in_smem(g);
-  const size_t smem = idft_smem(G, g.nlon) + tws * sizeof(float2);
-  SHOT_CUDA(cudaFuncSetAttribute(k_dft_fwd<G, NT, CTAS, PL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const size_t smem = idft_smem<E>(G, g.nlon) + tws * sizeof(float2);
+  SHOT_CUDA(cudaFuncSetAttribute(k_dft_fwd<G, NT, CTAS, PL, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   // field groups of one ring pair run together
-  dim3 grid((nf + 2 * G - 1) / (2 * G), g.nh + (heat_t ? 1 : 0));
+  dim3 grid((nf + E::F * G - 1) / (E::F * G), g.nh + (heat_t ? 1 : 0));
   ProfScope prof(PK_DFT, st);
   count_launch();
-  k_dft_fwd<G, NT, CTAS, PL><<<grid, NT, smem, st>>>(in, nf, g.nlat, g.nlon, g.lmax, g.nh, g.a_d, ps, scale_which, X,
-                                                 ldc, g.plan, g.tw_d, tws, mlim, heat_t ? g.h_d : nullptr,
-                                                           heat_t ? *heat_t : 0.0);
+  k_dft_fwd<G, NT, CTAS, PL, E><<<grid, NT, smem, st>>>(in, nf, g.nlat, g.nlon, g.lmax, g.nh, g.a_d, ps, scale_which,
+                                                       X, ldc, g.plan, g.tw_d, tws, mlim, heat_t ? g.h_d : nullptr,
+                                                       heat_t ? *heat_t : 0.0);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
 }
 
-template <int G, class PL = RuntimePlan, int NT = kThreads, int CTAS = kCtas>
+template <int G, class PL = RuntimePlan, int NT = kThreads, int CTAS = kCtas, class E = C2>
 int launch_idft_t(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st) {
   const int tws = twiddles_in_smem(g);
-  const size_t smem = idft_smem(G, g.nlon) + tws * sizeof(float2);   // two sequence buffers; the second first stages the spectra
-  SHOT_CUDA(cudaFuncSetAttribute(k_idft<G, NT, CTAS, PL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  dim3 grid((nf + 2 * G - 1) / (2 * G), g.nh);   // field groups of one ring pair run together
+  // two sequence buffers; the second first stages the spectra
+  const size_t smem = idft_smem<E>(G, g.nlon) + tws * sizeof(float2);
+  SHOT_CUDA(cudaFuncSetAttribute(k_idft<G, NT, CTAS, PL, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  dim3 grid((nf + E::F * G - 1) / (E::F * G), g.nh);   // field groups of one ring pair run together
   ProfScope prof(ep.mode == EPI_CHECK || ep.mode == EPI_FINAL ? PK_CHECK : PK_IDFT, st);
   count_launch();
-  k_idft<G, NT, CTAS, PL><<<grid, NT, smem, st>>>(Y, ldc, nf, g.nlat, g.nlon, g.lmax, g.nh, g.a_d, g.plan, g.tw_d, tws, ep);
+  k_idft<G, NT, CTAS, PL, E><<<grid, NT, smem, st>>>(Y, ldc, nf, g.nlat, g.nlon, g.lmax, g.nh, g.a_d, g.plan, g.tw_d,
+                                                    tws, ep);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
 }
@@ -365,18 +390,12 @@ int launch_idft_p_t(const Grid& g, const float* Y, int ldc, int nf, const EpiPar
   return SHOT_OK;
 }
 
-// the runtime plan equals the compile-time one (same N and radices in the same order)
-template <class PL>
-bool plan_is(const FftPlan& p) {
-  return p.N == PL::N && p.nst == 3 && p.R[0] == PL::R0 && p.R[1] == PL::R1 && p.R[2] == PL::R2;
-}
-// plans compiled for the ring lengths of the 720- and 512-ring grids (one pair of fields a CTA)
-using Plan1440 = CtPlan<1440, 15, 8, 12>;
-using Plan1024 = CtPlan<1024, 4, 16, 16>;
-
 }  // namespace
 
-int dft_fields_per_cta(const Grid& g, int nf) { return g.quad == SHOT_QUAD_HEALPIX ? 2 : 2 * pick_g(g, nf); }
+int dft_fields_per_cta(const Grid& g, int nf) {
+  if (g.quad == SHOT_QUAD_HEALPIX) return hp_fields_per_cta(g);
+  return 2 * pick_g(g, nf);
+}
 
 int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, int scale_which,
                    float* X, int ldc, cudaStream_t st, const int2* mlim, const double* heat_t) {

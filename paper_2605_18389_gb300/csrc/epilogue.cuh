@@ -1,8 +1,8 @@
 // The Sinkhorn epilogue of the inverse ring transform, shared by the rectangular grids'
 // FFT kernel and the HEALPix ring kernel.
 //
-// z holds K v on the ring pair of 2 G fields, two fields an element (real parts: ring j,
-// imaginary parts: ring J; G sequences of N longitudes at stride ld); the epilogue applies
+// z holds K v on the ring pair of F G fields, F = 2 (C2) or 1 (C1) fields an element (real parts:
+// ring j, imaginary parts: ring J; G sequences of N longitudes at stride ld); the epilogue applies
 // Algorithm 1's pointwise step of the given mode and reduces the per-field partial sums of the
 // pair into ep.part[f][jh][NPART]:
 //   EPI_PLAIN   out = K v
@@ -98,7 +98,6 @@ __device__ __forceinline__ void epi_prefetch_marginals(const EpiParams& ep, cons
 // update amplifies the rounding of its sum by tau / eps.  Against one plain chain a thread and one sum
 // a warp: 40 iterations of 24 problems at 720 rings 35.9 -> 36.1 ms, four grids of 64 to 180 rings
 // 18.47 -> 18.55.
-__device__ __forceinline__ float add2(float a, float b) { return a + b; }
 template <class V, bool TWO = false>
 struct Chain {
   V a{}, b{};
@@ -119,14 +118,14 @@ struct CompInf {   // the error beside the sum (Knuth's two-sum); an infinite su
   __device__ __forceinline__ double value() const { return fabsf(s) < INFINITY ? (double)s + (double)c : (double)s; }
 };
 
-// Partial sums of a CTA's warps: NT / G threads share a field pair, and each of their GW warps leaves P
-// sums of 32 / P lanes.
-template <int G, int NT>
+// Partial sums of a CTA's warps: NT / G threads share an element's F fields, and each of their GW warps
+// leaves P sums of 32 / P lanes.
+template <int G, int NT, int F>
 struct EpiRed {
   static constexpr int GW = NT / G / 32, P = GW >= 8 ? 1 : GW >= 4 ? 2 : GW >= 2 ? 4 : 8;
   static_assert(GW * P >= 8, "at least eight partial sums");
-  float v[NT / 32][P][2 * NPART];
-  double d[NT / 32][2][2];   // EPI_FINAL: warp sums of m(pi) and the objective
+  float v[NT / 32][P][F * NPART];
+  double d[NT / 32][F][2];   // EPI_FINAL: warp sums of m(pi) and the objective
 };
 
 // The update of one K v value in full generality: u, the terms (t0, t1) of its two sums and the
@@ -245,43 +244,41 @@ __device__ __forceinline__ void epi_update_pair(const float4* zg, float4* og, in
 }
 
 // kFinal = false compiles the EPI_FINAL branch out (kernels never launched with it).
-// The CTA's NT threads form G groups of NT / G (whole warps); group g takes fields f0 + 2 g and
-// f0 + 2 g + 1, a thread longitude k of both rings of the pair, so that one set of sums per
+// The CTA's NT threads form G groups of NT / G (whole warps); group g takes the F fields from
+// f0 + F g on, a thread longitude k of both rings of the pair, so that one set of sums per
 // thread and one warp reduction serve a group whatever G is.
-template <int G, int NT, bool kFinal = true>
-__device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int ld, int N, int nf, int f0,
+template <int G, int NT, bool kFinal = true, class E>
+__device__ __forceinline__ void ring_pair_epilogue(const E* z, E* other, int ld, int N, int nf, int f0,
                                                    size_t fstride, size_t rj, size_t rJ, bool two, float aj,
                                                    int nh, int jh, const EpiParams& ep,
-                                                   EpiRed<G, NT>& red, const EpiField* fi) {
-  constexpr int GT = NT / G, GW = GT / 32, P = EpiRed<G, NT>::P;
+                                                   EpiRed<G, NT, E::F>& red, const EpiField* fi) {
+  constexpr int GT = NT / G, GW = GT / 32, P = EpiRed<G, NT, E::F>::P, F = E::F;
   static_assert(NT % G == 0 && GT % 32 == 0, "a group is whole warps");
   constexpr int kBatchGen = 2;   // the general path of the update
   constexpr int kEpiBatch = 4;   // longitudes per thread whose marginal values are loaded together
   const int g = G == 1 ? 0 : threadIdx.x / GT, t = G == 1 ? threadIdx.x : threadIdx.x - g * GT;
-  const int fa = f0 + 2 * g;                       // first field of the group
-  const int nq = min(2, nf - fa);                  // fields of the group (<= 0: none)
-  const float4* zg = reinterpret_cast<const float4*>(z + g * ld);   // (ring j: 2 fields, ring J: 2 fields)
-  float4* og = reinterpret_cast<float4*>(other + g * ld);
+  const int fa = f0 + F * g;                       // first field of the group
+  const int nq = min(F, nf - fa);                  // fields of the group (<= 0: none)
+  const E* zg = z + g * ld;
+  E* og = other + g * ld;
   if (ep.mode == EPI_PLAIN) {
     float* o = ep.out + (size_t)fa * fstride;
     for (int k = t; k < N; k += GT) {
-      const float4 zz = zg[k];
-      if (nq > 0) {
-        o[rj + k] = zz.x;
-        if (two) o[rJ + k] = zz.z;
-      }
-      if (nq > 1) {
-        o[fstride + rj + k] = zz.y;
-        if (two) o[fstride + rJ + k] = zz.w;
-      }
+      const E zz = zg[k];
+#pragma unroll
+      for (int q = 0; q < F; ++q)
+        if (q < nq) {
+          o[q * fstride + rj + k] = lane_of(zz.re, q);
+          if (two) o[q * fstride + rJ + k] = lane_of(zz.im, q);
+        }
     }
     return;
   }
   // Per-element arithmetic is FP32, and the sums as described at Chain; the final pass, which runs
   // once a solve, compensates its threads' sums instead.
-  float acc[2][NPART];
+  float acc[F][NPART];
 #pragma unroll
-  for (int q = 0; q < 2; ++q)
+  for (int q = 0; q < F; ++q)
 #pragma unroll
     for (int i = 0; i < NPART; ++i) acc[q][i] = 0.f;
   // EPI_FINAL: the dual objective and m(pi) reach the block's FP64 sums through per-thread
@@ -291,110 +288,116 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
   // (and the masses) compensated (Kahan) in FP32 and the offsets applied in FP64; per element
   // the work stays FP32.  m(pi) enters S_dual times eps.
   if (ep.mode == EPI_UPDATE || ep.mode == EPI_SYM) {
-    // both fields of an element in one pass: K v comes and the new scaling leaves as 16 bytes
+    // the fields of an element in one pass: K v comes and the new scaling leaves in one piece
     const bool sym = ep.mode == EPI_SYM;
-    const EpiField* f2 = fi + 2 * g;
-    const bool live0 = nq > 0 && f2[0].live, live1 = nq > 1 && f2[1].live;
-    const bool bal0 = f2[0].balanced, bal1 = f2[1].balanced;
-    if (!sym && two && live0 && live1) {
-      float* out = ep.skip_store ? nullptr : ep.out + (size_t)fa * fstride + rj;
-      const int dJ = (int)(rJ - rj);   // a field has fewer than 2^31 nodes
-      epi_update_pair<GT>(zg, og, t, N, f2, out, fstride, rj, dJ, ep.xout != nullptr, aj, acc);
-    } else {
-    float* outf[2];
-    const float* mg[2];
-    int live[2] = {live0, live1}, bal[2] = {bal0, bal1};
-    float gam[2], rr[2];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      outf[q] = ep.out + (size_t)(fa + q) * fstride;
-      mg[q] = f2[q].marg;
-      gam[q] = f2[q].gamma;
-      rr[q] = f2[q].r;
-    }
-    Chain<f32x2, (GT < 64)> s0, s1;
-    float bad[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-    for (int k0 = t; k0 < N && nq > 0; k0 += kBatchGen * GT) {
-      // the equator ring, an odd last field, frozen problems and self terms: field by field;
-      // the marginal values (self term: and the old scaling's) of all this thread's longitudes
-      // first, then the arithmetic; a frozen problem loads its stored scaling
-      float pv[kBatchGen][2][2], uo[kBatchGen][2][2];
-      f32x2 x0 = 0, x1 = 0;
-#pragma unroll
-      for (int b = 0; b < kBatchGen; ++b) {
-        const int k = k0 + b * GT;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const bool in = k < N && live[q], st = k < N && q < nq && (!live[q] || sym);
-          pv[b][q][0] = in ? __ldg(mg[q] + rj + k) : 0.f;
-          pv[b][q][1] = (in && two) ? __ldg(mg[q] + rJ + k) : 0.f;
-          uo[b][q][0] = st ? outf[q][rj + k] : 0.f;
-          uo[b][q][1] = (st && two) ? outf[q][rJ + k] : 0.f;
-        }
+    const EpiField* f2 = fi + F * g;
+    bool pair = false;   // a pair of live fields on two rings
+    if constexpr (F == 2) {
+      pair = !sym && two && nq > 1 && f2[0].live && f2[1].live;
+      if (pair) {
+        float* out = ep.skip_store ? nullptr : ep.out + (size_t)fa * fstride + rj;
+        const int dJ = (int)(rJ - rj);   // a field has fewer than 2^31 nodes
+        epi_update_pair<GT>(reinterpret_cast<const float4*>(zg), reinterpret_cast<float4*>(og), t, N, f2, out, fstride,
+                            rj, dJ, ep.xout != nullptr, aj, acc);
       }
+    }
+    if (!pair) {
+      float* outf[F];
+      const float* mg[F];
+      bool live[F], bal[F];
+      float gam[F], rr[F], bad[F][2];
 #pragma unroll
-      for (int b = 0; b < kBatchGen; ++b) {
-        const int k = k0 + b * GT;
-        if (k >= N) break;
-        const float4 zz = zg[k];
-        float un[2][2], v0[2] = {0.f, 0.f}, v1[2] = {0.f, 0.f};
+      for (int q = 0; q < F; ++q) {
+        live[q] = q < nq && f2[q].live;
+        bal[q] = f2[q].balanced;
+        outf[q] = ep.out + (size_t)(fa + q) * fstride;
+        mg[q] = f2[q].marg;
+        gam[q] = f2[q].gamma;
+        rr[q] = f2[q].r;
+        bad[q][0] = bad[q][1] = 0.f;
+      }
+      Chain<typename E::V, (GT < 64)> s0, s1;
+      for (int k0 = t; k0 < N && nq > 0; k0 += kBatchGen * GT) {
+        // one field an element, the equator ring, an odd last field, frozen problems and self terms:
+        // field by field; the marginal values (self term: and the old scaling's) of all this thread's
+        // longitudes first, then the arithmetic; a frozen problem loads its stored scaling
+        float pv[kBatchGen][F][2], uo[kBatchGen][F][2];
+        typename E::V x0{}, x1{};
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          un[q][0] = uo[b][q][0];
-          un[q][1] = uo[b][q][1];
-          if (!live[q]) continue;
+        for (int b = 0; b < kBatchGen; ++b) {
+          const int k = k0 + b * GT;
 #pragma unroll
-          for (int r = 0; r < 2; ++r) {
-            if (r == 1 && !two) { un[q][1] = 0.f; break; }
-            const float kv = q ? (r ? zz.w : zz.y) : (r ? zz.z : zz.x);
-            const float pm = pv[b][q][r];
-            float u;
-            if (sym) {
-              const float ratio = __fdividef(pm, kv);
-              const float x = bal[q] ? ratio : exp2f(gam[q] * __log2f(ratio));
-              u = sqrtf(uo[b][q][r] * x);
-              if (!(kv > 0.f && kv < INFINITY && fabsf(u) < INFINITY)) {
-                if (kv <= 0.f) bad[q][0] += 1.f;
-                else bad[q][1] += 1.f;
-              }
-            } else {
-              float t0, t1;
-              u = epi_update_value(pm, kv, rr[q], bal[q], gam[q], aj, t0, t1, bad[q]);
-              v0[q] = r ? v0[q] + t0 : t0;
-              v1[q] = r ? v1[q] + t1 : t1;
-            }
-            if (sym || !ep.skip_store) outf[q][(r ? rJ : rj) + k] = u;
-            un[q][r] = u;
+          for (int q = 0; q < F; ++q) {
+            const bool in = k < N && live[q], st = k < N && q < nq && (!live[q] || sym);
+            pv[b][q][0] = in ? __ldg(mg[q] + rj + k) : 0.f;
+            pv[b][q][1] = (in && two) ? __ldg(mg[q] + rJ + k) : 0.f;
+            uo[b][q][0] = st ? outf[q][rj + k] : 0.f;
+            uo[b][q][1] = (st && two) ? outf[q][rJ + k] : 0.f;
           }
         }
-        x0 = add2(x0, pk2(v0[0], v0[1]));
-        x1 = add2(x1, pk2(v1[0], v1[1]));
-        if (ep.xout) og[k] = make_float4(un[0][0], un[1][0], un[0][1], un[1][1]);
-      }
-      s0.add(x0);
-      s1.add(x1);
-    }
-    const float2 a0 = unpk2(s0.value()), a1 = unpk2(s1.value());
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      acc[q][0] = q ? a0.y : a0.x;
-      acc[q][1] = q ? a1.y : a1.x;
-      acc[q][2] = bad[q][0];
-      acc[q][3] = bad[q][1];
-    }
+        for (int b = 0; b < kBatchGen; ++b) {
+          const int k = k0 + b * GT;
+          if (k >= N) break;
+          const E zz = zg[k];
+          float un[2][F], v0[F], v1[F];   // the new scaling on rings j and J, the terms of its sums
+#pragma unroll
+          for (int q = 0; q < F; ++q) {
+            un[0][q] = uo[b][q][0];
+            un[1][q] = uo[b][q][1];
+            v0[q] = v1[q] = 0.f;
+            if (!live[q]) continue;
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+              if (r == 1 && !two) { un[1][q] = 0.f; break; }
+              const float kv = lane_of(r ? zz.im : zz.re, q);
+              const float pm = pv[b][q][r];
+              float u;
+              if (sym) {
+                const float ratio = __fdividef(pm, kv);
+                const float x = bal[q] ? ratio : exp2f(gam[q] * __log2f(ratio));
+                u = sqrtf(uo[b][q][r] * x);
+                if (!(kv > 0.f && kv < INFINITY && fabsf(u) < INFINITY)) {
+                  if (kv <= 0.f) bad[q][0] += 1.f;
+                  else bad[q][1] += 1.f;
+                }
+              } else {
+                float t0, t1;
+                u = epi_update_value(pm, kv, rr[q], bal[q], gam[q], aj, t0, t1, bad[q]);
+                v0[q] = r ? v0[q] + t0 : t0;
+                v1[q] = r ? v1[q] + t1 : t1;
+              }
+              if (sym || !ep.skip_store) outf[q][(r ? rJ : rj) + k] = u;
+              un[r][q] = u;
+            }
+          }
+          x0 = add2(x0, of_lanes(v0));
+          x1 = add2(x1, of_lanes(v1));
+          if (ep.xout) og[k] = cx(of_lanes(un[0]), of_lanes(un[1]));
+        }
+        s0.add(x0);
+        s1.add(x1);
+      }
+#pragma unroll
+      for (int q = 0; q < F; ++q) {
+        acc[q][0] = lane_of(s0.value(), q);
+        acc[q][1] = lane_of(s1.value(), q);
+        acc[q][2] = bad[q][0];
+        acc[q][3] = bad[q][1];
+      }
     }
   } else {
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < F; ++q) {
       if (q >= nq) break;
       const int f = fa + q;
       const size_t fbase = (size_t)f * fstride;
       float* outf = ep.out + fbase;
       float* othf = ep.other ? ep.other + fbase : nullptr;
-      const EpiField F = fi[2 * g + q];
-      if (!F.live) continue;
+      const EpiField ef = fi[F * g + q];
+      if (!ef.live) continue;
       if (ep.mode == EPI_CHECK) {
-        const float* mg = F.marg;
+        const float* mg = ef.marg;
         const float cuv = ep.ps[f].cuv;
         Chain<float> e0, e1;
         for (int k0 = t; k0 < N; k0 += kEpiBatch * GT) {
@@ -414,11 +417,11 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
             const int k = k0 + b * GT;
             x0[b] = x1[b] = 0.f;
             if (k >= N) continue;
-            const float4 zz = zg[k];
+            const E zz = zg[k];
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
               if (r == 1 && !two) break;
-              const float kv = q ? (r ? zz.w : zz.y) : (r ? zz.z : zz.x);
+              const float kv = lane_of(r ? zz.im : zz.re, q);
               const float pm = pv[b][r];
               const float d = fmaf(cuv * uv[b][r], kv, -pm);
               const float t0 = ep.norm_l1 ? aj * fabsf(d) : d * d, t1 = ep.norm_l1 ? aj * pm : pm * pm;
@@ -455,11 +458,11 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
           s = t;
         };
         for (int k = t; k < N; k += GT) {
-          const float4 zz = zg[k];
+          const E zz = zg[k];
 #pragma unroll
           for (int r = 0; r < 2; ++r) {
             if (r == 1 && !two) break;
-            const float kv = q ? (r ? zz.w : zz.y) : (r ? zz.z : zz.x);
+            const float kv = lane_of(r ? zz.im : zz.re, q);
             const size_t o = (r ? rJ : rj) + k;
             const float pm = __ldg(pp + o), qm = __ldg(qq + o);
             const float ub = othf[o], vb = outf[o];
@@ -513,10 +516,10 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
       }
     }
   }
-  // one block reduction, each group's warps for its own two fields
+  // one block reduction, each group's warps for its own fields
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-  for (int q = 0; q < 2; ++q)
+  for (int q = 0; q < F; ++q)
 #pragma unroll
     for (int i = 0; i < NPART; ++i) {
       float v = acc[q][i];
@@ -526,11 +529,11 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
     }
   __syncthreads();
   if constexpr (kFinal) {
-    if (ep.mode == EPI_FINAL && threadIdx.x < 4 * G) {
+    if (ep.mode == EPI_FINAL && threadIdx.x < 2 * F * G) {
       const int fq = threadIdx.x >> 1, i = threadIdx.x & 1;   // field of the CTA
       if (f0 + fq < nf && fi[fq].live) {
         double s = 0.0;
-        for (int w = 0; w < GW; ++w) s += red.d[(fq >> 1) * GW + w][fq & 1][i];
+        for (int w = 0; w < GW; ++w) s += red.d[fq / F * GW + w][fq % F][i];
         // m(pi) sums a_j times the node values; the balanced objective's sums are of
         // p (la + log u_buf) + q (lb + log v_buf): times eps a_j
         const double sc = (i == 1 && fi[fq].balanced) ? ep.eps * (double)aj : (double)aj;
@@ -539,13 +542,13 @@ __device__ __forceinline__ void ring_pair_epilogue(const C2* z, C2* other, int l
     }
   }
   // four lanes a sum: the FP64 additions of one thread would be a chain that the CTA waits for
-  constexpr int kSums = 2 * G * NPART;
+  constexpr int kSums = F * G * NPART;
   static_assert(4 * kSums <= NT && (4 * kSums < 32 || 4 * kSums % 32 == 0), "whole warps, or one");
   int tid = threadIdx.x;
   asm volatile("" : "+r"(tid));   // keeps a persistent kernel's loop from carrying the indices below
   if (tid < 4 * kSums) {
     const int x = tid >> 2, fq = x / NPART, i = x - fq * NPART;
-    const int w0 = fq / 2 * GW, c = fq % 2 * NPART + i;
+    const int w0 = fq / F * GW, c = fq % F * NPART + i;
     double s = 0.0;
 #pragma unroll
     for (int y = 0; y < (GW * P + 3) / 4; ++y) {

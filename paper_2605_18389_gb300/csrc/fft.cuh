@@ -6,7 +6,8 @@
 // (0 <= j < N/R) reads in[j + r N/R] (r < R), multiplies input r by W_N^{(j mod Ns) r N/(Ns R)},
 // applies an R-point DFT and writes output r to out[(j div Ns) Ns R + (j mod Ns) + r Ns].
 //
-// Two fields travel together.  An element is a C2: the real parts of the two fields' values as
+// Two fields travel together (C2; one field, C1, where a pair would not fit or would leave the
+// chip short of work).  An element is the real parts of the two fields' values as
 // one packed pair of FP32, then the imaginary parts.  Every butterfly and twiddle is packed
 // arithmetic (add / mul / fma.rn.f32x2: two FP32 results an instruction, at half the rate of the
 // scalar ones), every shared-memory access 16 bytes, and the index arithmetic serves both fields.
@@ -67,35 +68,77 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
   return r;
 }
 
-// One complex value of each of two fields.
-struct __align__(16) C2 {
-  f32x2 re, im;
+// the same on one FP32 value
+__device__ __forceinline__ float add2(float a, float b) { return a + b; }
+__device__ __forceinline__ float sub2(float a, float b) { return a - b; }
+__device__ __forceinline__ float mul2(float a, float b) { return a * b; }
+__device__ __forceinline__ float fma2(float a, float b, float c) { return fmaf(a, b, c); }
+// one value for every field: a constant (kc) or a variable (dup)
+template <class V> __device__ __forceinline__ V kc(float c);
+template <> __device__ __forceinline__ float kc<float>(float c) { return c; }
+template <> __device__ __forceinline__ f32x2 kc<f32x2>(float c) { return kc2(c); }
+template <class V> __device__ __forceinline__ V dup(float x);
+template <> __device__ __forceinline__ float dup<float>(float x) { return x; }
+template <> __device__ __forceinline__ f32x2 dup<f32x2>(float x) { return pk2(x, x); }
+// the value of field q, and the values of the fields of an element together
+__device__ __forceinline__ float lane_of(float a, int) { return a; }
+__device__ __forceinline__ float lane_of(f32x2 a, int q) {
+  const float2 v = unpk2(a);
+  return q ? v.y : v.x;
+}
+__device__ __forceinline__ float of_lanes(const float (&x)[1]) { return x[0]; }
+__device__ __forceinline__ f32x2 of_lanes(const float (&x)[2]) { return pk2(x[0], x[1]); }
+
+// One complex value of each of F fields: C2 two fields, C1 one.
+template <class T>
+struct __align__(2 * sizeof(T)) Cx {
+  typedef T V;
+  static constexpr int F = sizeof(T) / sizeof(float);
+  V re, im;
 };
-__device__ __forceinline__ C2 c2(f32x2 re, f32x2 im) {
-  C2 r;
+using C2 = Cx<f32x2>;
+using C1 = Cx<float>;
+template <class V>
+__device__ __forceinline__ Cx<V> cx(V re, V im) {
+  Cx<V> r;
   r.re = re;
   r.im = im;
   return r;
 }
-__device__ __forceinline__ C2 cadd(C2 a, C2 b) { return c2(add2(a.re, b.re), add2(a.im, b.im)); }
-__device__ __forceinline__ C2 csub(C2 a, C2 b) { return c2(sub2(a.re, b.re), sub2(a.im, b.im)); }
-// a * w (CONJ: a * conj w), the same w for both fields
-template <bool CONJ>
-__device__ __forceinline__ C2 cmul(C2 a, float2 w) {
-  const f32x2 c = pk2(w.x, w.x), s = pk2(w.y, w.y), ns = pk2(-w.y, -w.y);
-  return CONJ ? c2(fma2(a.re, c, mul2(a.im, s)), fma2(a.im, c, mul2(a.re, ns)))
-              : c2(fma2(a.re, c, mul2(a.im, ns)), fma2(a.re, s, mul2(a.im, c)));
+template <class E> __device__ __forceinline__ E cadd(E a, E b) { return cx(add2(a.re, b.re), add2(a.im, b.im)); }
+template <class E> __device__ __forceinline__ E csub(E a, E b) { return cx(sub2(a.re, b.re), sub2(a.im, b.im)); }
+__device__ __forceinline__ f32x2 neg2(f32x2 a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ float neg2(float a) { return -a; }
+// a * w (CONJ: a * conj w), the same w for every field
+template <bool CONJ, class E>
+__device__ __forceinline__ E cmul(E a, float2 w) {
+  typedef typename E::V V;
+  const V c = dup<V>(w.x), s = dup<V>(w.y), ns = dup<V>(-w.y);
+  return CONJ ? cx(fma2(a.re, c, mul2(a.im, s)), fma2(a.im, c, mul2(a.re, ns)))
+              : cx(fma2(a.re, c, mul2(a.im, ns)), fma2(a.re, s, mul2(a.im, c)));
 }
 // a -+ i b: a - i b (forward) or a + i b (inverse)
-template <bool INV>
-__device__ __forceinline__ C2 add_mi(C2 a, C2 b) {
-  return INV ? c2(sub2(a.re, b.im), add2(a.im, b.re)) : c2(add2(a.re, b.im), sub2(a.im, b.re));
+template <bool INV, class E>
+__device__ __forceinline__ E add_mi(E a, E b) {
+  return INV ? cx(sub2(a.re, b.im), add2(a.im, b.re)) : cx(add2(a.re, b.im), sub2(a.im, b.re));
 }
 // multiply by -i (forward) or +i (inverse)
-__device__ __forceinline__ f32x2 neg2(f32x2 a) { return a ^ 0x8000000080000000ull; }
-template <bool INV>
-__device__ __forceinline__ C2 mul_mi(C2 a) {
-  return INV ? c2(neg2(a.im), a.re) : c2(a.im, neg2(a.re));
+template <bool INV, class E>
+__device__ __forceinline__ E mul_mi(E a) {
+  return INV ? cx(neg2(a.im), a.re) : cx(a.im, neg2(a.re));
+}
+
+// One row's piece of an element's spectra as it lies in memory, (re, im) of each field.
+template <class E> struct Piece { typedef float4 T; };
+template <> struct Piece<C1> { typedef float2 T; };
+__device__ __forceinline__ C2 piece_value(float4 v) { return cx(pk2(v.x, v.z), pk2(v.y, v.w)); }
+__device__ __forceinline__ C1 piece_value(float2 v) { return cx(v.x, v.y); }
+__device__ __forceinline__ void store_piece(float* p, C2 v) {
+  const float2 re = unpk2(v.re), im = unpk2(v.im);
+  *reinterpret_cast<float4*>(p) = make_float4(re.x, im.x, re.y, im.y);
+}
+__device__ __forceinline__ void store_piece(float* p, C1 v) {
+  *reinterpret_cast<float2*>(p) = make_float2(v.re, v.im);
 }
 
 // ---- compile-time roots of unity ----------------------------------------------------
@@ -126,13 +169,14 @@ __host__ __device__ constexpr double root_angle(int j, int R) {
 }
 
 // a * W_R^J with W_R = exp(-2 pi i / R) (forward) or its conjugate (inverse)
-template <int R, int J, bool INV>
-__device__ __forceinline__ C2 mul_root(C2 a) {
+template <int R, int J, bool INV, class E>
+__device__ __forceinline__ E mul_root(E a) {
+  typedef typename E::V V;
   constexpr int j = ((J % R) + R) % R;
   if constexpr (j == 0) {
     return a;
   } else if constexpr (2 * j == R) {
-    return c2(neg2(a.re), neg2(a.im));
+    return cx(neg2(a.re), neg2(a.im));
   } else if constexpr (4 * j == R) {
     return mul_mi<INV>(a);
   } else if constexpr (4 * j == 3 * R) {
@@ -141,31 +185,31 @@ __device__ __forceinline__ C2 mul_root(C2 a) {
     constexpr float c = (float)taylor_cos(root_angle(j, R));
     constexpr float s = (float)taylor_sin(root_angle(j, R));
     constexpr float sy = INV ? s : -s;   // W^j = (c, -s) forward
-    return c2(fma2(a.re, kc2(c), mul2(a.im, kc2(-sy))), fma2(a.re, kc2(sy), mul2(a.im, kc2(c))));
+    return cx(fma2(a.re, kc<V>(c), mul2(a.im, kc<V>(-sy))), fma2(a.re, kc<V>(sy), mul2(a.im, kc<V>(c))));
   }
 }
 
 // ---- prime-size butterflies (in place on v[0..R-1]) ---------------------------------
-template <bool INV>
-__device__ __forceinline__ void bfly2(C2* v) {
-  const C2 a = v[0], b = v[1];
+template <bool INV, class E>
+__device__ __forceinline__ void bfly2(E* v) {
+  const E a = v[0], b = v[1];
   v[0] = cadd(a, b);
   v[1] = csub(a, b);
 }
 
-template <bool INV>
-__device__ __forceinline__ void bfly4(C2* v) {
-  const C2 a = cadd(v[0], v[2]), b = csub(v[0], v[2]), c = cadd(v[1], v[3]), d = csub(v[1], v[3]);
+template <bool INV, class E>
+__device__ __forceinline__ void bfly4(E* v) {
+  const E a = cadd(v[0], v[2]), b = csub(v[0], v[2]), c = cadd(v[1], v[3]), d = csub(v[1], v[3]);
   v[0] = cadd(a, c);
   v[2] = csub(a, c);
   v[1] = add_mi<INV>(b, d);
   v[3] = add_mi<!INV>(b, d);
 }
 
-template <bool INV>
-__device__ __forceinline__ void bfly8(C2* v) {
-  C2 e[4] = {v[0], v[2], v[4], v[6]};
-  C2 o[4] = {v[1], v[3], v[5], v[7]};
+template <bool INV, class E>
+__device__ __forceinline__ void bfly8(E* v) {
+  E e[4] = {v[0], v[2], v[4], v[6]};
+  E o[4] = {v[1], v[3], v[5], v[7]};
   bfly4<INV>(e);
   bfly4<INV>(o);
   o[1] = mul_root<8, 1, INV>(o[1]);
@@ -180,36 +224,38 @@ __device__ __forceinline__ void bfly8(C2* v) {
   v[7] = csub(e[3], o[3]);
 }
 
-template <bool INV>
-__device__ __forceinline__ void bfly3(C2* v) {
-  const f32x2 s = kc2(0.86602540378443865f);   // sin(2 pi / 3)
-  const f32x2 h = kc2(-0.5f);
-  const C2 t = cadd(v[1], v[2]);
-  const C2 d = csub(v[1], v[2]);
-  const C2 a = c2(fma2(h, t.re, v[0].re), fma2(h, t.im, v[0].im));
-  const f32x2 ns = kc2(-0.86602540378443865f);
+template <bool INV, class E>
+__device__ __forceinline__ void bfly3(E* v) {
+  typedef typename E::V V;
+  const V s = kc<V>(0.86602540378443865f);   // sin(2 pi / 3)
+  const V h = kc<V>(-0.5f);
+  const E t = cadd(v[1], v[2]);
+  const E d = csub(v[1], v[2]);
+  const E a = cx(fma2(h, t.re, v[0].re), fma2(h, t.im, v[0].im));
+  const V ns = kc<V>(-0.86602540378443865f);
   v[0] = cadd(v[0], t);
   // a -+ i s d
-  const C2 m = c2(fma2(s, d.im, a.re), fma2(ns, d.re, a.im));   // a - i s d
-  const C2 p = c2(fma2(ns, d.im, a.re), fma2(s, d.re, a.im));   // a + i s d
+  const E m = cx(fma2(s, d.im, a.re), fma2(ns, d.re, a.im));   // a - i s d
+  const E p = cx(fma2(ns, d.im, a.re), fma2(s, d.re, a.im));   // a + i s d
   v[1] = INV ? p : m;
   v[2] = INV ? m : p;
 }
 
-template <bool INV>
-__device__ __forceinline__ void bfly5(C2* v) {
-  const f32x2 c1 = kc2(0.30901699437494742f);     // cos(2pi/5)
-  const f32x2 k2 = kc2(-0.80901699437494742f);   // cos(4pi/5)
-  const f32x2 s1 = kc2(0.95105651629515357f);     // sin(2pi/5)
-  const f32x2 s2 = kc2(0.58778525229247313f);     // sin(4pi/5)
-  const C2 t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
-  const C2 d1 = csub(v[1], v[4]), d2 = csub(v[2], v[3]);
-  const C2 x0 = v[0];
-  const C2 a1 = c2(fma2(k2, t2.re, fma2(c1, t1.re, x0.re)), fma2(k2, t2.im, fma2(c1, t1.im, x0.im)));
-  const C2 a2 = c2(fma2(c1, t2.re, fma2(k2, t1.re, x0.re)), fma2(c1, t2.im, fma2(k2, t1.im, x0.im)));
-  const f32x2 ns1 = kc2(-0.95105651629515357f);
-  const C2 b1 = c2(fma2(s1, d1.re, mul2(s2, d2.re)), fma2(s1, d1.im, mul2(s2, d2.im)));
-  const C2 b2 = c2(fma2(s2, d1.re, mul2(ns1, d2.re)), fma2(s2, d1.im, mul2(ns1, d2.im)));
+template <bool INV, class E>
+__device__ __forceinline__ void bfly5(E* v) {
+  typedef typename E::V V;
+  const V c1 = kc<V>(0.30901699437494742f);     // cos(2pi/5)
+  const V k2 = kc<V>(-0.80901699437494742f);   // cos(4pi/5)
+  const V s1 = kc<V>(0.95105651629515357f);     // sin(2pi/5)
+  const V s2 = kc<V>(0.58778525229247313f);     // sin(4pi/5)
+  const E t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
+  const E d1 = csub(v[1], v[4]), d2 = csub(v[2], v[3]);
+  const E x0 = v[0];
+  const E a1 = cx(fma2(k2, t2.re, fma2(c1, t1.re, x0.re)), fma2(k2, t2.im, fma2(c1, t1.im, x0.im)));
+  const E a2 = cx(fma2(c1, t2.re, fma2(k2, t1.re, x0.re)), fma2(c1, t2.im, fma2(k2, t1.im, x0.im)));
+  const V ns1 = kc<V>(-0.95105651629515357f);
+  const E b1 = cx(fma2(s1, d1.re, mul2(s2, d2.re)), fma2(s1, d1.im, mul2(s2, d2.im)));
+  const E b2 = cx(fma2(s2, d1.re, mul2(ns1, d2.re)), fma2(s2, d1.im, mul2(ns1, d2.im)));
   v[0] = cadd(x0, cadd(t1, t2));
   v[1] = add_mi<INV>(a1, b1);
   v[4] = add_mi<!INV>(a1, b1);
@@ -217,8 +263,8 @@ __device__ __forceinline__ void bfly5(C2* v) {
   v[3] = add_mi<!INV>(a2, b2);
 }
 
-template <int R, bool INV>
-__device__ __forceinline__ void bfly_prime(C2* v) {
+template <int R, bool INV, class E>
+__device__ __forceinline__ void bfly_prime(E* v) {
   if constexpr (R == 2) bfly2<INV>(v);
   else if constexpr (R == 3) bfly3<INV>(v);
   else if constexpr (R == 4) bfly4<INV>(v);
@@ -227,9 +273,9 @@ __device__ __forceinline__ void bfly_prime(C2* v) {
 }
 
 // R-point DFT of the registers v[O + S i], i < R
-template <int R, int O, int S, bool INV>
-__device__ __forceinline__ void dft_at(C2* v) {
-  C2 t[R];
+template <int R, int O, int S, bool INV, class E>
+__device__ __forceinline__ void dft_at(E* v) {
+  E t[R];
 #pragma unroll
   for (int i = 0; i < R; ++i) t[i] = v[O + S * i];
   bfly_prime<R, INV>(t);
@@ -240,22 +286,22 @@ __device__ __forceinline__ void dft_at(C2* v) {
 // Composite R = R1 R2 with n = R2 n1 + n2, k = k1 + R1 k2:
 //   X[k] = sum_{n2} W_R2^{n2 k2} W_R^{n2 k1} sum_{n1} W_R1^{n1 k1} x[R2 n1 + n2].
 // After the call X[k1 + R1 k2] is in v[R2 k1 + k2].
-template <int R1, int R2, bool INV, int... I>
-__device__ __forceinline__ void composite_level1(C2* v, std::integer_sequence<int, I...>) {
+template <int R1, int R2, bool INV, class E, int... I>
+__device__ __forceinline__ void composite_level1(E* v, std::integer_sequence<int, I...>) {
   (dft_at<R1, I, R2, INV>(v), ...);
 }
-template <int R1, int R2, bool INV, int... I>
-__device__ __forceinline__ void composite_twiddle(C2* v, std::integer_sequence<int, I...>) {
+template <int R1, int R2, bool INV, class E, int... I>
+__device__ __forceinline__ void composite_twiddle(E* v, std::integer_sequence<int, I...>) {
   // element I = R2 k1 + n2 takes W_R^{n2 k1}
   ((v[I] = mul_root<R1 * R2, (I % R2) * (I / R2), INV>(v[I])), ...);
 }
-template <int R1, int R2, bool INV, int... I>
-__device__ __forceinline__ void composite_level2(C2* v, std::integer_sequence<int, I...>) {
+template <int R1, int R2, bool INV, class E, int... I>
+__device__ __forceinline__ void composite_level2(E* v, std::integer_sequence<int, I...>) {
   (dft_at<R2, R2 * I, 1, INV>(v), ...);
 }
 
-template <int R1, int R2, bool INV>
-__device__ __forceinline__ void bfly_composite(C2* v) {
+template <int R1, int R2, bool INV, class E>
+__device__ __forceinline__ void bfly_composite(E* v) {
   composite_level1<R1, R2, INV>(v, std::make_integer_sequence<int, R2>{});
   composite_twiddle<R1, R2, INV>(v, std::make_integer_sequence<int, R1 * R2>{});
   composite_level2<R1, R2, INV>(v, std::make_integer_sequence<int, R1>{});
@@ -273,8 +319,8 @@ template <> struct Radix<12> { static constexpr int R1 = 4, R2 = 3; };
 template <> struct Radix<15> { static constexpr int R1 = 3, R2 = 5; };
 template <> struct Radix<16> { static constexpr int R1 = 4, R2 = 4; };
 
-template <int R, bool INV>
-__device__ __forceinline__ void butterfly(C2* v) {
+template <int R, bool INV, class E>
+__device__ __forceinline__ void butterfly(E* v) {
   if constexpr (Radix<R>::R1 == 1) bfly_prime<R, INV>(v);
   else bfly_composite<Radix<R>::R1, Radix<R>::R2, INV>(v);
 }
@@ -300,8 +346,8 @@ __device__ __forceinline__ int fast_div(int a, uint32_t mul) {
   return mul ? (int)__umulhi((uint32_t)a, mul) : a;
 }
 
-template <int R, bool INV>
-__device__ __forceinline__ void stockham_stage(const C2* __restrict__ src, C2* __restrict__ dst,
+template <int R, bool INV, class E>
+__device__ __forceinline__ void stockham_stage(const E* __restrict__ src, E* __restrict__ dst,
                                                const float2* __restrict__ tws, int N, int Ns, int nseq,
                                                uint32_t ns_mul, uint32_t nr_mul) {
   const int NR = N / R;
@@ -312,8 +358,8 @@ __device__ __forceinline__ void stockham_stage(const C2* __restrict__ src, C2* _
     const int j = idx - q * NR;
     const int jd = fast_div(j, ns_mul);
     const int k = j - jd * Ns;
-    const C2* s = src + q * ld + j;
-    C2 v[R];
+    const E* s = src + q * ld + j;
+    E v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = s[r * NR];
     if (Ns > 1) {   // the first stage's twiddles are all 1
@@ -323,7 +369,7 @@ __device__ __forceinline__ void stockham_stage(const C2* __restrict__ src, C2* _
       }
     }
     butterfly<R, INV>(v);
-    C2* d = dst + q * ld + jd * Ns * R + k;
+    E* d = dst + q * ld + jd * Ns * R + k;
 #pragma unroll
     for (int r = 0; r < R; ++r) d[r * Ns] = v[out_reg<R>(r)];
   }
@@ -335,8 +381,8 @@ __device__ __forceinline__ void stockham_stage(const C2* __restrict__ src, C2* _
 // two outputs, where one output a task took twelve operations for two.  Tasks run r-major over the
 // butterflies, so consecutive threads read consecutive inputs.  A solve of 101 rings of 211 longitudes, one field, 20
 // iterations: 2.6 -> 1.8 ms (2.1 in the scalar form); 97 x 202, 8 fields 2.03 -> 1.60 (2.44).
-template <bool INV>
-__device__ __noinline__ void stockham_stage_generic(const C2* __restrict__ src, C2* __restrict__ dst,
+template <bool INV, class E>
+__device__ __noinline__ void stockham_stage_generic(const E* __restrict__ src, E* __restrict__ dst,
                                                     const float2* __restrict__ tws, const float2* __restrict__ roots,
                                                     int N, int R, int Ns, int nseq, uint32_t ns_mul,
                                                     uint32_t nr_mul) {
@@ -349,21 +395,21 @@ __device__ __noinline__ void stockham_stage_generic(const C2* __restrict__ src, 
     const int q = qr / H, r = qr - q * H;
     const int jd = fast_div(j, ns_mul);
     const int k = j - jd * Ns;
-    const C2* s = src + q * ld + j;
-    C2 A = c2(0ull, 0ull), B = A;
+    const E* s = src + q * ld + j;
+    E A{}, B{};
     int e = 0;   // r t mod R
 #pragma unroll 4
     for (int t = 0; t < R; ++t) {
-      C2 v = s[t * NR];
+      E v = s[t * NR];
       if (Ns > 1 && t > 0) v = cmul<INV>(v, tws[(t - 1) * Ns + k]);
       const float2 w = roots[e];
-      const f32x2 c = pk2(w.x, w.x), sn = pk2(w.y, w.y);
-      A = c2(fma2(v.re, c, A.re), fma2(v.im, c, A.im));
-      B = c2(fma2(v.re, sn, B.re), fma2(v.im, sn, B.im));
+      const typename E::V c = dup<typename E::V>(w.x), sn = dup<typename E::V>(w.y);
+      A = cx(fma2(v.re, c, A.re), fma2(v.im, c, A.im));
+      B = cx(fma2(v.re, sn, B.re), fma2(v.im, sn, B.im));
       e += r;
       if (e >= R) e -= R;
     }
-    C2* d = dst + q * ld + jd * Ns * R + k;
+    E* d = dst + q * ld + jd * Ns * R + k;
     d[r * Ns] = add_mi<!INV>(A, B);   // A + i B (forward), A - i B (inverse)
     if (r) d[(R - r) * Ns] = add_mi<INV>(A, B);
   }
@@ -374,8 +420,8 @@ __device__ __noinline__ void stockham_stage_generic(const C2* __restrict__ src, 
 // the short rings, whose CTAs would wait a global-memory latency in every stage.  Returns
 // the buffer holding the result.  All threads of the block must call it; it
 // synchronises after every stage.
-template <bool INV>
-__device__ C2* fft_smem(C2* a, C2* b, const float2* tw, const FftPlan& pl, int nseq) {
+template <bool INV, class E>
+__device__ E* fft_smem(E* a, E* b, const float2* tw, const FftPlan& pl, int nseq) {
   int Ns = 1;
 #pragma unroll 1
   for (int s = 0; s < pl.nst; ++s) {
@@ -399,7 +445,7 @@ __device__ C2* fft_smem(C2* a, C2* b, const float2* tw, const FftPlan& pl, int n
         break;
     }
     __syncthreads();
-    C2* t = a;
+    E* t = a;
     a = b;
     b = t;
     Ns *= R;
@@ -417,8 +463,8 @@ struct CtPlan {
 };
 using RuntimePlan = CtPlan<0>;
 
-template <int R, bool INV, int N, int NS, int TWOFF>
-__device__ __forceinline__ void stockham_stage_ct(const C2* src, C2* dst, const float2* __restrict__ tw, int nseq) {
+template <int R, bool INV, int N, int NS, int TWOFF, class E>
+__device__ __forceinline__ void stockham_stage_ct(const E* src, E* dst, const float2* __restrict__ tw, int nseq) {
   constexpr int NR = N / R, LD = seq_ld(N);
   const int total = nseq * NR;
   // opaque to the compiler, which would otherwise hoist a persistent kernel's index arithmetic and
@@ -430,8 +476,8 @@ __device__ __forceinline__ void stockham_stage_ct(const C2* src, C2* dst, const 
     const int j = idx - q * NR;
     const int jd = j / NS;
     const int k = j - jd * NS;
-    const C2* s = src + q * LD + j;
-    C2 v[R];
+    const E* s = src + q * LD + j;
+    E v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = s[r * NR];
     if constexpr (NS > 1) {
@@ -440,7 +486,7 @@ __device__ __forceinline__ void stockham_stage_ct(const C2* src, C2* dst, const 
       for (int r = 1; r < R; ++r) v[r] = cmul<INV>(v[r], __ldg(tws + (r - 1) * NS));
     }
     butterfly<R, INV>(v);
-    C2* d = dst + q * LD + jd * NS * R + k;
+    E* d = dst + q * LD + jd * NS * R + k;
 #pragma unroll
     for (int r = 0; r < R; ++r) d[r * NS] = v[out_reg<R>(r)];
   }
@@ -449,8 +495,8 @@ __device__ __forceinline__ void stockham_stage_ct(const C2* src, C2* dst, const 
 
 // three-stage compile-time plan; the twiddle table layout is the runtime plan's (stage s at
 // sum over earlier stages s' >= 1 of (R_s' - 1) Ns_s')
-template <bool INV, class PL>
-__device__ C2* fft_smem_ct(C2* a, C2* b, const float2* tw, int nseq) {
+template <bool INV, class PL, class E>
+__device__ E* fft_smem_ct(E* a, E* b, const float2* tw, int nseq) {
   constexpr int N = PL::N, R0 = PL::R0, R1 = PL::R1, R2 = PL::R2;
   static_assert(R0 * R1 * R2 == N, "plan radices must multiply to N");
   stockham_stage_ct<R0, INV, N, 1, 0>(a, b, tw, nseq);
@@ -459,8 +505,8 @@ __device__ C2* fft_smem_ct(C2* a, C2* b, const float2* tw, int nseq) {
   return b;
 }
 
-template <bool INV, class PL>
-__device__ __forceinline__ C2* fft_smem_plan(C2* a, C2* b, const float2* tw, const FftPlan& pl,
+template <bool INV, class PL, class E>
+__device__ __forceinline__ E* fft_smem_plan(E* a, E* b, const float2* tw, const FftPlan& pl,
                                                  int nseq) {
   if constexpr (PL::N == 0) return fft_smem<INV>(a, b, tw, pl, nseq);
   else return fft_smem_ct<INV, PL>(a, b, tw, nseq);

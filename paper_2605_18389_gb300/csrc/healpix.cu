@@ -16,7 +16,8 @@
 //   inverse  f_j = sum_k Z_k e^{2 pi i k j / n},
 //            Z_k = sum_{m = -lmax..lmax, m = k mod n} e^{i m phi0} G_m,   G_{-m} = conj G_m.
 // Two rings (j north, J south) travel as one complex sequence and two fields as one packed
-// element, as on the other grids.
+// element, as on the other grids; one field where two sequences of pairs exceed an SM's shared
+// memory (from nside 1800 on).
 #include <cmath>
 #include <vector>
 
@@ -26,7 +27,7 @@
 namespace shot {
 namespace {
 
-// One ring pair of two fields a CTA.  The chain of one CTA bounds these kernels (a solve's rings
+// One ring pair of one element's fields a CTA.  The chain of one CTA bounds these kernels (a solve's rings
 // are short, and all CTAs of nside 64 and 8 fields are resident at once): 128 threads take most
 // stages in one step, the generic stage of a prime factor p in p steps.
 constexpr int kHpThreads = 128;
@@ -34,7 +35,10 @@ constexpr int kHpThreads = 128;
 // most 2 n entries: n, and the roots of its generic stages)
 constexpr int kHpTwMax = 1024;
 // two sequences of the longest ring n and room for its twiddles
-size_t hp_smem(int n, int tws) { return (size_t)2 * seq_ld(n) * sizeof(C2) + (tws ? 2 * n * sizeof(float2) : 0); }
+template <class E>
+size_t hp_smem(int n) { return (size_t)2 * seq_ld(n) * sizeof(E) + (n <= kHpTwMax ? 2 * n * sizeof(float2) : 0); }
+// what a block may have, less the kernels' own static shared memory (under 2 KB)
+constexpr size_t kHpSmemMax = 225 * 1024;
 
 // e^{i pi r / d} for an integer r reduced modulo 2d (exact argument reduction)
 __device__ __forceinline__ float2 half_turns(int r, int d) {
@@ -59,24 +63,25 @@ __device__ __forceinline__ const float2* load_plan(FftPlan* pl, const FftPlan* _
 
 // from the transformed ring pair D: S = a (F_N + F_S), D = a (F_N - F_S) for m <= mmax into X
 // (sc = a / 2 per field, with the field's factor), each order turned by e^{-i m phi0}
-__device__ __forceinline__ void hp_fold_store(const C2* D, int n, int2 phase, int f0, int mmax, int nh, int jh, f32x2 sc,
+template <class E>
+__device__ __forceinline__ void hp_fold_store(const E* D, int n, int2 phase, int f0, int mmax, int nh, int jh, typename E::V sc,
                                               float* __restrict__ X, int ldc) {
+  typedef typename E::V V;
   float* x = X + (size_t)jh * ldc + 2 * f0;
   const size_t row = (size_t)nh * ldc;
   for (int m = threadIdx.x; m <= mmax; m += kHpThreads) {
     const int k = m % n;
-    const C2 zm = D[k], zn = D[k ? n - k : 0];
+    const E zm = D[k], zn = D[k ? n - k : 0];
     const float2 e = half_turns(m * phase.x, phase.y);
     // 2 F_N = z_k + conj z_{n-k}, 2 F_S = (z_k - conj z_{n-k}) / i, both times e^{-i m phi0}
-    const C2 FN = cmul<true>(c2(add2(zm.re, zn.re), sub2(zm.im, zn.im)), e);
-    const C2 FS = cmul<true>(c2(add2(zm.im, zn.im), sub2(zn.re, zm.re)), e);
-    const float2 Sr = unpk2(mul2(sc, add2(FN.re, FS.re))), Si = unpk2(mul2(sc, add2(FN.im, FS.im)));
-    const float2 Dr = unpk2(mul2(sc, sub2(FN.re, FS.re))), Di = unpk2(mul2(sc, sub2(FN.im, FS.im)));
-    *reinterpret_cast<float4*>(x + (size_t)(2 * m) * row) = make_float4(Sr.x, Si.x, Sr.y, Si.y);
-    *reinterpret_cast<float4*>(x + (size_t)(2 * m + 1) * row) = make_float4(Dr.x, Di.x, Dr.y, Di.y);
+    const E FN = cmul<true>(cx(add2(zm.re, zn.re), sub2(zm.im, zn.im)), e);
+    const E FS = cmul<true>(cx(add2(zm.im, zn.im), sub2(zn.re, zm.re)), e);
+    store_piece(x + (size_t)(2 * m) * row, cx(mul2(sc, add2(FN.re, FS.re)), mul2(sc, add2(FN.im, FS.im))));
+    store_piece(x + (size_t)(2 * m + 1) * row, cx(mul2(sc, sub2(FN.re, FS.re)), mul2(sc, sub2(FN.im, FS.im))));
   }
 }
 
+template <class E>
 __global__ void __launch_bounds__(kHpThreads, 4) k_hp_fwd(const float* __restrict__ in, int nf, size_t npix,
                                                        const int* __restrict__ rlen,
                                                        const long long* __restrict__ roff,
@@ -88,33 +93,41 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_fwd(const float* __restric
                                                        const ProbState* __restrict__ ps,
                                                        const int2* __restrict__ mlim, float* __restrict__ h,
                                                        double t) {
-  extern __shared__ __align__(16) C2 sm[];
+  constexpr int F = E::F;
+  extern __shared__ __align__(16) uint8_t smem[];
   __shared__ FftPlan pl;
   if (blockIdx.y == gridDim.y - 1 && h) {   // the heat multipliers
     for (int l = blockIdx.x * blockDim.x + threadIdx.x; l <= lmax; l += gridDim.x * blockDim.x) h[l] = heat_mult(t, l);
     return;
   }
-  const int jh = blockIdx.y, f0 = blockIdx.x * 2;
+  const int jh = blockIdx.y, f0 = blockIdx.x * F;
   const int j = jh, J = nrings - 1 - jh;
-  const bool second = f0 + 1 < nf, two = J != j;
+  const bool two = J != j;
   const int n = rlen[j], pi = rplan[j];
-  C2* zb = sm;
-  C2* db = zb + seq_ld(n);
+  E* zb = reinterpret_cast<E*>(smem);
+  E* db = zb + seq_ld(n);
   const float2* tw = load_plan(&pl, plans, pi, tw_all, tw_base, reinterpret_cast<float2*>(db + seq_ld(n)), tws);
   const float* fj = in + (size_t)f0 * npix + roff[j];
   const float* fJ = in + (size_t)f0 * npix + roff[J];
-  for (int k = threadIdx.x; k < n; k += kHpThreads)
-    reinterpret_cast<float4*>(zb)[k] =
-        make_float4(fj[k], second ? fj[npix + k] : 0.f, two ? fJ[k] : 0.f, (two && second) ? fJ[npix + k] : 0.f);
-  // per-field factor (gradient sweeps)
-  const float s0 = 0.5f * area * (ps ? (float)ps[f0].beta : 1.f);
-  const float s1 = 0.5f * area * (ps && second ? (float)ps[f0 + 1].beta : 1.f);
+  float sc[F];   // per-field factor (gradient sweeps)
+#pragma unroll
+  for (int q = 0; q < F; ++q) sc[q] = 0.5f * area * (ps && f0 + q < nf ? (float)ps[f0 + q].beta : 1.f);
+  for (int k = threadIdx.x; k < n; k += kHpThreads) {
+    float a[F], b[F];
+#pragma unroll
+    for (int q = 0; q < F; ++q) {
+      a[q] = f0 + q < nf ? fj[q * npix + k] : 0.f;
+      b[q] = two && f0 + q < nf ? fJ[q * npix + k] : 0.f;
+    }
+    zb[k] = cx(of_lanes(a), of_lanes(b));
+  }
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  const C2* D = fft_smem<false>(zb, db, tw, pl, 1);
-  hp_fold_store(D, n, rphase[j], f0, mlim ? mlim[jh].y : lmax, nh, jh, pk2(s0, s1), X, ldc);
+  const E* D = fft_smem<false>(zb, db, tw, pl, 1);
+  hp_fold_store(D, n, rphase[j], f0, mlim ? mlim[jh].y : lmax, nh, jh, of_lanes(sc), X, ldc);
 }
 
+template <class E>
 __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restrict__ Y, int ldc, int nf, size_t npix,
                                                         const int* __restrict__ rlen,
                                                         const long long* __restrict__ roff,
@@ -124,22 +137,24 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
                                                         const FftPlan* __restrict__ plans,
                                                         const float2* __restrict__ tw_all,
                                                         const int* __restrict__ tw_base, int tws) {
-  extern __shared__ __align__(16) C2 sm[];
+  constexpr int F = E::F;
+  typedef typename Piece<E>::T Pc;
+  extern __shared__ __align__(16) uint8_t smem[];
   __shared__ FftPlan pl;
-  __shared__ EpiRed<1, kHpThreads> red;
-  __shared__ EpiField fi[2];
-  const int jh = blockIdx.y, f0 = blockIdx.x * 2;
-  const int nfg = min(2, nf - f0);
+  __shared__ EpiRed<1, kHpThreads, F> red;
+  __shared__ EpiField fi[F];
+  const int jh = blockIdx.y, f0 = blockIdx.x * F;
+  const int nfg = min(F, nf - f0);
   const int j = jh, J = nrings - 1 - jh;
   const bool two = (J != j);
   const int n = rlen[j], ld = seq_ld(n), pi = rplan[j];
   const size_t rj = (size_t)roff[j], rJ = (size_t)roff[J];
   const int2 phase = rphase[j];
   const int2 ml = ep.mlim ? ep.mlim[jh] : make_int2(lmax, lmax);   // orders read, orders written
-  C2* za = sm;          // spectra Z
-  C2* zb = za + ld;
+  E* za = reinterpret_cast<E*>(smem);   // spectra Z
+  E* zb = za + ld;
   const float2* tw = load_plan(&pl, plans, pi, tw_all, tw_base, reinterpret_cast<float2*>(zb + ld), tws);
-  epi_fields_load<2>(ep, f0, nfg, fi);
+  epi_fields_load<F>(ep, f0, nfg, fi);
   // Z_k = A_k + B_{n-k}: A_r sums e^{i m phi0} (G_N + i G_S) over the orders m >= 0 of residue r
   // modulo n, B_r sums e^{-i m phi0} (conj G_N + i conj G_S) over the orders m >= 1.  A thread owns
   // a residue, so every spectra row is read once, straight from global memory.
@@ -147,17 +162,15 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
     const float* y = Y + (size_t)jh * ldc + 2 * f0;
     const size_t row = (size_t)nh * ldc;
     for (int r = threadIdx.x; r < n; r += kHpThreads) {
-      C2 A = c2(0ull, 0ull), B = A;
+      E A{}, B{};
 #pragma unroll 4
       for (int m = r; m <= ml.x; m += n) {
-        const float4 e = *reinterpret_cast<const float4*>(y + (size_t)(2 * m) * row);
-        const float4 o = m < lmax ? *reinterpret_cast<const float4*>(y + (size_t)(2 * m + 1) * row)
-                                  : make_float4(0.f, 0.f, 0.f, 0.f);
-        const C2 E = c2(pk2(e.x, e.z), pk2(e.y, e.w)), O = c2(pk2(o.x, o.z), pk2(o.y, o.w));
-        const C2 GN = cadd(E, O), GS = csub(E, O);
+        const E e = piece_value(*reinterpret_cast<const Pc*>(y + (size_t)(2 * m) * row));
+        const E o = m < lmax ? piece_value(*reinterpret_cast<const Pc*>(y + (size_t)(2 * m + 1) * row)) : E{};
+        const E GN = cadd(e, o), GS = csub(e, o);
         const float2 w = half_turns(m * phase.x, phase.y);
-        A = cadd(A, cmul<false>(c2(sub2(GN.re, GS.im), add2(GN.im, GS.re)), w));
-        if (m > 0) B = cadd(B, cmul<true>(c2(add2(GN.re, GS.im), sub2(GS.re, GN.im)), w));
+        A = cadd(A, cmul<false>(cx(sub2(GN.re, GS.im), add2(GN.im, GS.re)), w));
+        if (m > 0) B = cadd(B, cmul<true>(cx(add2(GN.re, GS.im), sub2(GS.re, GN.im)), w));
       }
       za[r] = A;
       zb[r] = B;
@@ -165,47 +178,67 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  epi_prefetch_marginals<2, true>(ep, fi, nfg, rj, rJ, two, n, f0, npix);
+  epi_prefetch_marginals<F, true>(ep, fi, nfg, rj, rJ, two, n, f0, npix);
   for (int k = threadIdx.x; k < n; k += kHpThreads) za[k] = cadd(za[k], zb[k ? n - k : 0]);
   __syncthreads();
-  C2* z = fft_smem<true>(za, zb, tw, pl, 1);   // K v on the ring pair
-  C2* other = (z == za) ? zb : za;   // receives the new scaling
+  E* z = fft_smem<true>(za, zb, tw, pl, 1);   // K v on the ring pair
+  E* other = (z == za) ? zb : za;   // receives the new scaling
   ring_pair_epilogue<1, kHpThreads>(z, other, ld, n, nf, f0, npix, rj, rJ, two, area, nh, jh, ep, red, fi);
   if ((ep.mode == EPI_UPDATE || ep.mode == EPI_SYM) && ep.xout) {   // transform the new scaling
     __syncthreads();
-    const C2* D = fft_smem<false>(other, z, tw, pl, 1);
-    hp_fold_store(D, n, phase, f0, ml.y, nh, jh, pk2(0.5f * area, 0.5f * area), ep.xout, ldc);
+    const E* D = fft_smem<false>(other, z, tw, pl, 1);
+    hp_fold_store(D, n, phase, f0, ml.y, nh, jh, dup<typename E::V>(0.5f * area), ep.xout, ldc);
   }
 }
 
-}  // namespace
-
-int launch_hp_dft_fwd(const Grid& g, const float* in, int nf, float* X, int ldc, cudaStream_t st,
-                      const ProbState* ps, const int2* mlim, const double* heat_t) {
-  const int tws = g.nlon <= kHpTwMax;
-  const size_t smem = hp_smem(g.nlon, tws);
-  SHOT_CUDA(cudaFuncSetAttribute(k_hp_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+template <class E>
+int hp_fwd_t(const Grid& g, const float* in, int nf, float* X, int ldc, cudaStream_t st, const ProbState* ps,
+             const int2* mlim, const double* heat_t) {
+  const size_t smem = hp_smem<E>(g.nlon);
+  SHOT_CUDA(cudaFuncSetAttribute(k_hp_fwd<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   ProfScope prof(PK_DFT, st);
   count_launch();
-  k_hp_fwd<<<dim3((nf + 1) / 2, g.nh + (heat_t ? 1 : 0)), kHpThreads, smem, st>>>(
+  k_hp_fwd<E><<<dim3((nf + E::F - 1) / E::F, g.nh + (heat_t ? 1 : 0)), kHpThreads, smem, st>>>(
       in, nf, g.npix, g.ring_len_d, g.ring_off_d, g.ring_phase_d, g.nlat, g.lmax, g.nh, (float)g.a_ring[0], X, ldc,
-      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d, tws, ps, mlim, heat_t ? g.h_d : nullptr,
+      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d, g.nlon <= kHpTwMax, ps, mlim, heat_t ? g.h_d : nullptr,
       heat_t ? *heat_t : 0.0);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
 }
 
-int launch_hp_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st) {
-  const int tws = g.nlon <= kHpTwMax;
-  const size_t smem = hp_smem(g.nlon, tws);
-  SHOT_CUDA(cudaFuncSetAttribute(k_hp_idft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+template <class E>
+int hp_idft_t(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st) {
+  const size_t smem = hp_smem<E>(g.nlon);
+  SHOT_CUDA(cudaFuncSetAttribute(k_hp_idft<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   ProfScope prof(ep.mode == EPI_CHECK || ep.mode == EPI_FINAL ? PK_CHECK : PK_IDFT, st);
   count_launch();
-  k_hp_idft<<<dim3((nf + 1) / 2, g.nh), kHpThreads, smem, st>>>(
+  k_hp_idft<E><<<dim3((nf + E::F - 1) / E::F, g.nh), kHpThreads, smem, st>>>(
       Y, ldc, nf, g.npix, g.ring_len_d, g.ring_off_d, g.ring_phase_d, g.nlat, g.lmax, g.nh, (float)g.a_ring[0], ep,
-      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d, tws);
+      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d, g.nlon <= kHpTwMax);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
+}
+
+int hp_too_long() {
+  set_error("nside too large for the shared-memory ring FFT");
+  return SHOT_ERR_UNSUPPORTED;
+}
+
+}  // namespace
+
+int hp_fields_per_cta(const Grid& g) { return hp_smem<C2>(g.nlon) <= kHpSmemMax ? 2 : 1; }
+
+int launch_hp_dft_fwd(const Grid& g, const float* in, int nf, float* X, int ldc, cudaStream_t st,
+                      const ProbState* ps, const int2* mlim, const double* heat_t) {
+  if (hp_smem<C2>(g.nlon) <= kHpSmemMax) return hp_fwd_t<C2>(g, in, nf, X, ldc, st, ps, mlim, heat_t);
+  if (hp_smem<C1>(g.nlon) <= kHpSmemMax) return hp_fwd_t<C1>(g, in, nf, X, ldc, st, ps, mlim, heat_t);
+  return hp_too_long();
+}
+
+int launch_hp_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st) {
+  if (hp_smem<C2>(g.nlon) <= kHpSmemMax) return hp_idft_t<C2>(g, Y, ldc, nf, ep, st);
+  if (hp_smem<C1>(g.nlon) <= kHpSmemMax) return hp_idft_t<C1>(g, Y, ldc, nf, ep, st);
+  return hp_too_long();
 }
 
 // Ring geometry of a HEALPix grid of resolution nside (host, FP64), into the Grid: node

@@ -280,6 +280,7 @@ int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, 
                    float* X, int ldc, cudaStream_t st, const int2* mlim = nullptr, const double* heat_t = nullptr);
 int launch_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st);
 int dft_fields_per_cta(const Grid& g, int nf);   // fields a ring-transform CTA takes
+int hp_fields_per_cta(const Grid& g);            // the same on a HEALPix grid
 // Grids whose Legendre contractions run the TF32x3 tensor-core kernels: TF32X3 grids, and BF16X3
 // grids in recurrence mode (the recurrence kernels are bound by generating the A operand, not by
 // the MMA's operand width, so a bf16 split of the generated values would gain nothing; TF32x3

@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
                                                         const int* __restrict__ rplan,
                                                         const FftPlan* __restrict__ plans,
                                                         const float2* __restrict__ tw_all,
-                                                        const int* __restrict__ tw_base, int tws) {
+                                                        const int* __restrict__ tw_base, int tws, int nmax) {
   constexpr int F = E::F;
   typedef typename Piece<E>::T Pc;
   extern __shared__ __align__(16) uint8_t smem[];
@@ -151,20 +151,24 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
   const size_t rj = (size_t)roff[j], rJ = (size_t)roff[J];
   const int2 phase = rphase[j];
   const int2 ml = ep.mlim ? ep.mlim[jh] : make_int2(lmax, lmax);   // orders read, orders written
-  E* za = reinterpret_cast<E*>(smem);   // spectra Z
-  E* zb = za + ld;
-  const float2* tw = load_plan(&pl, plans, pi, tw_all, tw_base, reinterpret_cast<float2*>(zb + ld), tws);
+  E* za = reinterpret_cast<E*>(smem);   // spectra Z; the buffers are of the longest ring's size
+  E* zb = za + seq_ld(nmax);
+  const float2* tw = load_plan(&pl, plans, pi, tw_all, tw_base, reinterpret_cast<float2*>(zb + seq_ld(nmax)), tws);
   epi_fields_load<F>(ep, f0, nfg, fi);
   // Z_k = A_k + B_{n-k}: A_r sums e^{i m phi0} (G_N + i G_S) over the orders m >= 0 of residue r
-  // modulo n, B_r sums e^{-i m phi0} (conj G_N + i conj G_S) over the orders m >= 1.  A thread owns
-  // a residue, so every spectra row is read once, straight from global memory.
+  // modulo n, B_r sums e^{-i m phi0} (conj G_N + i conj G_S) over the orders m >= 1.  The orders of a
+  // residue are shared by S threads (short rings near the poles have many orders of each residue,
+  // whose rows are one latency after the other in one thread: nside 64, one field, plain synthesis
+  // 25.8 us with the rows gathered through shared memory,
+  // 33.0 with one thread a residue, 20.7 so), each spectra row is read once, straight from global memory.
+  const int S = max(1, min((int)kHpThreads, nmax) / n);
   {
     const float* y = Y + (size_t)jh * ldc + 2 * f0;
     const size_t row = (size_t)nh * ldc;
-    for (int r = threadIdx.x; r < n; r += kHpThreads) {
+    for (int i = threadIdx.x; i < S * n; i += kHpThreads) {
       E A{}, B{};
 #pragma unroll 4
-      for (int m = r; m <= ml.x; m += n) {
+      for (int m = i; m <= ml.x; m += S * n) {
         const E e = piece_value(*reinterpret_cast<const Pc*>(y + (size_t)(2 * m) * row));
         const E o = m < lmax ? piece_value(*reinterpret_cast<const Pc*>(y + (size_t)(2 * m + 1) * row)) : E{};
         const E GN = cadd(e, o), GS = csub(e, o);
@@ -172,14 +176,19 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
         A = cadd(A, cmul<false>(cx(sub2(GN.re, GS.im), add2(GN.im, GS.re)), w));
         if (m > 0) B = cadd(B, cmul<true>(cx(add2(GN.re, GS.im), sub2(GS.re, GN.im)), w));
       }
-      za[r] = A;
-      zb[r] = B;
+      za[i] = A;   // part i / n of residue i % n
+      zb[i] = B;
     }
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   epi_prefetch_marginals<F, true>(ep, fi, nfg, rj, rJ, two, n, f0, npix);
-  for (int k = threadIdx.x; k < n; k += kHpThreads) za[k] = cadd(za[k], zb[k ? n - k : 0]);
+  for (int k = threadIdx.x; k < n; k += kHpThreads) {
+    const int kb = k ? n - k : 0;
+    E z = cadd(za[k], zb[kb]);
+    for (int s = 1; s < S; ++s) z = cadd(z, cadd(za[s * n + k], zb[s * n + kb]));
+    za[k] = z;
+  }
   __syncthreads();
   E* z = fft_smem<true>(za, zb, tw, pl, 1);   // K v on the ring pair
   E* other = (z == za) ? zb : za;   // receives the new scaling
@@ -214,7 +223,7 @@ int hp_idft_t(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& e
   count_launch();
   k_hp_idft<E><<<dim3((nf + E::F - 1) / E::F, g.nh), kHpThreads, smem, st>>>(
       Y, ldc, nf, g.npix, g.ring_len_d, g.ring_off_d, g.ring_phase_d, g.nlat, g.lmax, g.nh, (float)g.a_ring[0], ep,
-      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d, g.nlon <= kHpTwMax);
+      g.ring_plan_d, g.hp_plan_d, g.hp_tw_d, g.hp_tw_base_d, g.nlon <= kHpTwMax, g.nlon);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
 }

@@ -336,6 +336,24 @@ bool plan_is(const FftPlan& p) {
 using Plan1440 = CtPlan<1440, 15, 8, 12>;
 using Plan1024 = CtPlan<1024, 4, 16, 16>;
 
+// Whether a CTA takes one field (C1, kThreads1 threads as one FFT butterfly needs half the registers)
+// instead of a pair: a single field, which leaves half of every pair idle; where one field each gives CTAs
+// that are all resident at once, so that pairs would halve the work in flight; and on rings so long that
+// one CTA of pairs fills an SM.  Measured, pairs -> one field: a solve of one problem, 60 iterations, 64
+// rings (TF32x3) 3.00 -> 2.85 ms, 256 rings 5.07 -> 4.77; of five problems on 64 rings 2.99 -> 2.90; of three on
+// 200 rings of 1000 longitudes, 20 iterations (pairs in the persistent form) 1.51 -> 1.38; of three on rings
+// of 4096 longitudes 22.7 -> 15.2; a heat application, one field, rings of 2000 longitudes 93 -> 84 us.
+// Elsewhere pairs are as fast or faster: eight problems on 128 rings 3.52 against 3.53 ms, on rings of 3000
+// longitudes 14.5 against 16.4.  Rings with a compiled plan keep the pairs (1024 longitudes, one field: 50
+// against 55 us).
+constexpr int kThreads1 = 256;
+bool one_field(const Grid& g, int nf) {
+  const bool fills_sm = 2 * (idft_smem<C2>(1, g.nlon) + 2048) > 228 * 1024;   // 2 KB: static and reserved
+  if (fills_sm) return true;
+  if (plan_is<Plan1440>(g.plan) || plan_is<Plan1024>(g.plan)) return false;
+  return nf == 1 || (long long)g.nh * nf <= kCtas * g.num_sms;
+}
+
 // Entries of the twiddle table a CTA copies into shared memory: all for rings of up to 768
 // longitudes (6 KB), where a CTA has few items and would wait for each stage's twiddles from L2 (32
 // rings, one field: 9.4 us an update launch without the copy, 7.3 with it in the scalar form); none
@@ -394,7 +412,7 @@ int launch_idft_p_t(const Grid& g, const float* Y, int ldc, int nf, const EpiPar
 
 int dft_fields_per_cta(const Grid& g, int nf) {
   if (g.quad == SHOT_QUAD_HEALPIX) return hp_fields_per_cta(g);
-  return 2 * pick_g(g, nf);
+  return one_field(g, nf) ? 1 : 2 * pick_g(g, nf);
 }
 
 int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, int scale_which,
@@ -410,6 +428,8 @@ int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, 
     set_error("nlon too large for the shared-memory ring FFT");
     return SHOT_ERR_UNSUPPORTED;
   }
+  if (one_field(g, nf))
+    return launch_fwd_t<1, RuntimePlan, kThreads1, kCtas, C1>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
   switch (pick_g(g, nf)) {
     case 6: return launch_fwd_t<6>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
     case 3: return launch_fwd_t<3>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
@@ -428,7 +448,7 @@ int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, 
 // to 180 rings, 72 fields each, in one solve: 19.7 against 20.9 ms).
 static bool idft_is_persistent(const Grid& g, int nf, const EpiParams& ep) {
   return (((ep.mode == EPI_UPDATE || ep.mode == EPI_SYM) && ep.xout) || ep.mode == EPI_CHECK) &&
-         !g.idft_nonpersistent && nf >= 2 && g.nlon > kTwMax && pick_g(g, nf) == 1 &&
+         !g.idft_nonpersistent && nf >= 2 && g.nlon > kTwMax && !one_field(g, nf) && pick_g(g, nf) == 1 &&
          idft_p_layout(g.nlon, g.lmax) <= 74 * 1024;
 }
 
@@ -446,6 +466,7 @@ int launch_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams&
     if (plan_is<Plan1024>(g.plan)) return launch_idft_p_t<Plan1024>(g, Y, ldc, nf, ep, st);
     return launch_idft_p_t<RuntimePlan>(g, Y, ldc, nf, ep, st);
   }
+  if (one_field(g, nf)) return launch_idft_t<1, RuntimePlan, kThreads1, kCtas, C1>(g, Y, ldc, nf, ep, st);
   switch (G) {
     case 6: return launch_idft_t<6>(g, Y, ldc, nf, ep, st);
     case 3: return launch_idft_t<3>(g, Y, ldc, nf, ep, st);

@@ -332,9 +332,15 @@ template <class PL>
 bool plan_is(const FftPlan& p) {
   return p.N == PL::N && p.nst == 3 && p.R[0] == PL::R0 && p.R[1] == PL::R1 && p.R[2] == PL::R2;
 }
-// plans compiled for the ring lengths of the 720- and 512-ring grids (one pair of fields a CTA)
+// Plans compiled for the ring lengths of the 720- and 512-ring grids (one pair of fields a CTA).  Constant
+// strides and divisions leave their kernels 80 registers without a spill that matters, so that four CTAs
+// of 192 threads share an SM (kCtasCt; the shared memory allows it up to 1750 longitudes); the persistent
+// form's staging area leaves room for three.  Heat applications, 24 fields, band limit 255, three -> four
+// CTAs: 1440 longitudes 197 -> 187 us, 1024 145 -> 140.  Any other length runs the runtime plan, which these two
+// would on 218 and 162 us (a solve of 24 problems, 20 iterations: 11.7 instead of 9.4 ms, 8.2 instead of 7.1).
 using Plan1440 = CtPlan<1440, 15, 8, 12>;
 using Plan1024 = CtPlan<1024, 4, 16, 16>;
+constexpr int kCtasCt = 4;
 
 // Whether a CTA takes one field (C1, kThreads1 threads as one FFT butterfly needs half the registers)
 // instead of a pair: a single field, which leaves half of every pair idle; where one field each gives CTAs
@@ -435,8 +441,10 @@ int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, 
     case 3: return launch_fwd_t<3>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
     case 2: return launch_fwd_t<2>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
     default:
-      if (plan_is<Plan1440>(g.plan)) return launch_fwd_t<1, Plan1440, 192, 4>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
-      if (plan_is<Plan1024>(g.plan)) return launch_fwd_t<1, Plan1024>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
+      if (plan_is<Plan1440>(g.plan))
+        return launch_fwd_t<1, Plan1440, kThreads, kCtasCt>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
+      if (plan_is<Plan1024>(g.plan))
+        return launch_fwd_t<1, Plan1024, kThreads, kCtasCt>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
       return launch_fwd_t<1>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
   }
 }
@@ -472,8 +480,8 @@ int launch_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams&
     case 3: return launch_idft_t<3>(g, Y, ldc, nf, ep, st);
     case 2: return launch_idft_t<2>(g, Y, ldc, nf, ep, st);
     default:
-      if (plan_is<Plan1440>(g.plan)) return launch_idft_t<1, Plan1440, 192, 4>(g, Y, ldc, nf, ep, st);
-      if (plan_is<Plan1024>(g.plan)) return launch_idft_t<1, Plan1024>(g, Y, ldc, nf, ep, st);
+      if (plan_is<Plan1440>(g.plan)) return launch_idft_t<1, Plan1440, kThreads, kCtasCt>(g, Y, ldc, nf, ep, st);
+      if (plan_is<Plan1024>(g.plan)) return launch_idft_t<1, Plan1024, kThreads, kCtasCt>(g, Y, ldc, nf, ep, st);
       return launch_idft_t<1>(g, Y, ldc, nf, ep, st);
   }
 }

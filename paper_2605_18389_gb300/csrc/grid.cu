@@ -404,19 +404,22 @@ int build_grid_tables(Grid& g, cudaStream_t st) {
   float* tab = nullptr;
   __nv_bfloat16 *hi = nullptr, *lo = nullptr;
   g.ldi = (g.M[0] + 7) / 8 * 8;
-  // first degrees above the cut, after the order limits in one allocation.  None in the FP32
+  // first degrees above the cut, on the device only until the host has them.  None in the FP32
   // recurrence mode, which has its own seeds, and none below degree 64: no chunk of 16 terms of any
   // tile would go (128 rings: 4 % of the analysis' terms; 256: 6 %; 720: 17 %).
   std::vector<int> lfirst;
-  int* lfirst_d = nullptr;
+  struct DeviceInts {
+    int* p = nullptr;
+    ~DeviceInts() { cudaFree(p); }
+  } lfirst_d;
   const bool polar = g.lmax >= 64 && (g.mode != SHOT_RECURRENCE || tf32_kernels(g));
   if (polar) {
     lfirst.resize((size_t)L * nh);
-    SHOT_CUDA(cudaMalloc(&g.mlim_d, nh * sizeof(int2) + lfirst.size() * sizeof(int)));
-    lfirst_d = reinterpret_cast<int*>(g.mlim_d + nh);
+    SHOT_CUDA(cudaMalloc(&g.mlim_d, nh * sizeof(int2)));
+    SHOT_CUDA(cudaMalloc(&lfirst_d.p, lfirst.size() * sizeof(int)));
   }
   if (g.mode == SHOT_RECURRENCE) {
-    int rc = tf32_kernels(g) ? build_tf32_recurrence(g, lfirst_d, st) : build_recurrence(g, st);
+    int rc = tf32_kernels(g) ? build_tf32_recurrence(g, lfirst_d.p, st) : build_recurrence(g, st);
     if (rc) return rc;
   } else {
   float* tabT = nullptr;
@@ -440,12 +443,12 @@ int build_grid_tables(Grid& g, cudaStream_t st) {
   }
   dim3 gp((nh + 127) / 128, L);
   count_launch();
-  k_pbar<<<gp, 128, 0, st>>>(g.lmax, nh, g.x_d, g.row_off_d, g.ldt, tab, hi, lo, tabT, g.ldi, lfirst_d);
+  k_pbar<<<gp, 128, 0, st>>>(g.lmax, nh, g.x_d, g.row_off_d, g.ldt, tab, hi, lo, tabT, g.ldi, lfirst_d.p);
   SHOT_CUDA(cudaGetLastError());
   }
 
   if (polar) {
-    SHOT_CUDA(cudaMemcpyAsync(lfirst.data(), lfirst_d, lfirst.size() * sizeof(int), cudaMemcpyDeviceToHost, st));
+    SHOT_CUDA(cudaMemcpyAsync(lfirst.data(), lfirst_d.p, lfirst.size() * sizeof(int), cudaMemcpyDeviceToHost, st));
     SHOT_CUDA(cudaStreamSynchronize(st));
   }
   // first terms of a tile's sums: analysis, rows up to i_last of block (m, p): the first node whose

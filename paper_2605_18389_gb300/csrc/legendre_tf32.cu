@@ -676,7 +676,7 @@ __global__ void k_ck_build(int lmax, int nh, const double* __restrict__ x, const
       p2 = p1;
       p1 = pl;
     }
-    if (first > lmax && fabs(pl) >= kPolarCut) first = l;
+    if (first > lmax && above_polar_cut(pl)) first = l;
     const int d = l - m, r = d % kSeg;
     if (r < 4) {   // offsets 0, 2 -> plane 0; 1, 3 -> plane 1; first or second value by r / 2
       const int par = r & 1;

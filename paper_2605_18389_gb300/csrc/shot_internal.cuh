@@ -103,6 +103,9 @@ struct Tile {
 // 181 -> 187 / 173 us; the ring transforms skip the orders that no tile reads or writes: forward 87 -> 72,
 // inverse 66 -> 58, update 152 -> 144 us.
 constexpr double kPolarCut = 0x1p-100;
+// |v| >= kPolarCut from the high word: an integer comparison beside the recurrence's FP64
+constexpr int kPolarCutHi = (1023 - 100) << 20;
+__device__ __forceinline__ bool above_polar_cut(double v) { return (__double2hiint(v) & 0x7fffffff) >= kPolarCutHi; }
 constexpr int kPolarAlign = 64;   // the Legendre kernels' longest chunk of terms
 
 struct Workspace {
@@ -185,7 +188,7 @@ struct Grid {
   int* M_d = nullptr;
   long long* row_off_d = nullptr;
   // heat convolutions: per north ring the highest order whose synthesis rows are nonzero (.x) and
-  // whose spectra the analysis reads (.y); null (FP32 recurrence mode): lmax
+  // whose spectra the analysis reads (.y), behind M_d; null (no cut): lmax
   int2* mlim_d = nullptr;
   Tile* tiles_ana = nullptr;
   Tile* tiles_syn = nullptr;

@@ -156,12 +156,11 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
   const float2* tw = load_plan(&pl, plans, pi, tw_all, tw_base, reinterpret_cast<float2*>(zb + seq_ld(nmax)), tws);
   epi_fields_load<F>(ep, f0, nfg, fi);
   // Z_k = A_k + B_{n-k}: A_r sums e^{i m phi0} (G_N + i G_S) over the orders m >= 0 of residue r
-  // modulo n, B_r sums e^{-i m phi0} (conj G_N + i conj G_S) over the orders m >= 1.  The orders of a
-  // residue are shared by S threads (short rings near the poles have many orders of each residue,
-  // whose rows are one latency after the other in one thread: nside 64, one field, plain synthesis
-  // 25.8 us with the rows gathered through shared memory,
-  // 33.0 with one thread a residue, 20.7 so), each spectra row is read once, straight from global memory.
-  const int S = max(1, min((int)kHpThreads, nmax) / n);
+  // modulo n, B_r sums e^{-i m phi0} (conj G_N + i conj G_S) over the orders m >= 1; each spectra row is
+  // read once, straight from global memory.  On the short rings near the poles a residue has many orders,
+  // and S threads share them, four rows in flight each (nside 64, one field, plain synthesis: 25.8 us with
+  // the rows gathered through shared memory, 33.0 with one thread a residue, 20.7 with all threads).
+  const int S = ml.x < 4 * n ? 1 : max(1, min(min(kHpThreads, nmax) / n, (ml.x + 4 * n) / (4 * n)));
   {
     const float* y = Y + (size_t)jh * ldc + 2 * f0;
     const size_t row = (size_t)nh * ldc;

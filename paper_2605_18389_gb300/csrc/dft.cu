@@ -61,28 +61,28 @@ __device__ __forceinline__ void load_ring_pairs(const float* __restrict__ in, E*
   const Group<G, NT> gr;
   const int fa = f0 + F * gr.g;
   if (fa >= nf) return;
-  const bool two = J != j;
+  const bool second = fa + 1 < nf, two = J != j;   // (of a pair)
   const size_t fs = (size_t)nlat * N;
   const float* aj = in + (size_t)fa * fs + (size_t)j * N;
   const float* aJ = in + (size_t)fa * fs + (size_t)J * N;
   E* b = buf + gr.g * seq_ld(N);
   constexpr int kBatch = 4;
   for (int k0 = gr.t; k0 < N; k0 += kBatch * gr.T) {
-    float v[kBatch][2][F];
+    float4 v[kBatch];
 #pragma unroll
     for (int i = 0; i < kBatch; ++i) {
       const int k = k0 + i * gr.T;
-#pragma unroll
-      for (int q = 0; q < F; ++q) {
-        const bool on = k < N && fa + q < nf;
-        v[i][0][q] = on ? __ldg(aj + q * fs + k) : 0.f;
-        v[i][1][q] = (on && two) ? __ldg(aJ + q * fs + k) : 0.f;
-      }
+      v[i].x = k < N ? __ldg(aj + k) : 0.f;
+      v[i].y = (k < N && second && F == 2) ? __ldg(aj + fs + k) : 0.f;
+      v[i].z = (k < N && two) ? __ldg(aJ + k) : 0.f;
+      v[i].w = (k < N && two && second && F == 2) ? __ldg(aJ + fs + k) : 0.f;
     }
 #pragma unroll
     for (int i = 0; i < kBatch; ++i) {
       const int k = k0 + i * gr.T;
-      if (k < N) b[k] = cx(of_lanes(v[i][0]), of_lanes(v[i][1]));
+      if (k >= N) continue;
+      if constexpr (F == 2) reinterpret_cast<float4*>(b)[k] = v[i];
+      else b[k] = cx(v[i].x, v[i].z);
     }
   }
 }

@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_dft_fwd(
   fold_store<G, NT>(buf, f0, nf, nlon, mlim ? mlim[jh].y : lmax, nh, jh, a_ring[jh], ps, scale_which, X, ldc);
 }
 
-template <int G, int NT, int CTAS, class PL, class E>
+template <int G, int NT, int CTAS, class PL, class E, bool LONG>
 __global__ void __launch_bounds__(NT, CTAS) k_idft(
     const float* __restrict__ Y, int ldc, int nf, int nlat, int nlon, int lmax, int nh,
     const float* __restrict__ a_ring, const __grid_constant__ FftPlan pl, const float2* tw, int tws,
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_idft(
   extern __shared__ __align__(16) uint8_t smem[];
   E* sm = reinterpret_cast<E*>(smem);
   constexpr int FG = E::F * G;
-  __shared__ EpiRed<G, NT, E::F> red;
+  __shared__ EpiRed<G, NT, E::F, LONG> red;
   __shared__ EpiField fi[FG];
   const int N = nlon, ld = seq_ld(N);
   E* buf = sm;
@@ -224,8 +224,8 @@ __global__ void __launch_bounds__(NT, CTAS) k_idft(
   const E* z = fft_smem_plan<true, PL>(buf, b1, tw, pl, G);
   E* other = (z == buf) ? b1 : buf;   // input of the fused forward transform
 
-  ring_pair_epilogue<G, NT>(z, other, ld, N, nf, f0, (size_t)nlat * N, (size_t)j * N, (size_t)J * N, two, aj, nh,
-                                  jh, ep, red, fi);
+  ring_pair_epilogue<G, NT, LONG>(z, other, ld, N, nf, f0, (size_t)nlat * N, (size_t)j * N, (size_t)J * N, two, aj,
+                                  nh, jh, ep, red, fi);
   if ((ep.mode == EPI_UPDATE || ep.mode == EPI_SYM) && ep.xout) {
     // the new scaling of this ring pair is in `other`: transform it for the next half-step
     __syncthreads();
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, kCtas) k_idft_p(
     int ngroups) {
   extern __shared__ __align__(16) C2 sm[];
   constexpr int G = 1, NT = kThreads, FG = 2 * G;
-  __shared__ EpiRed<G, NT, 2> red;
+  __shared__ EpiRed<G, NT, 2, true> red;
   __shared__ EpiField fi[2][2];
   const int N = nlon, ld = seq_ld(N);
   C2* buf = sm;
@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(kThreads, kCtas) k_idft_p(
                                  nlat - 1 - jn != jn, N, fn, fs);
     const float aj = a_ring[j];
     // the persistent kernel runs updates and checks only: no final-objective branch
-    ring_pair_epilogue<G, NT, false>(z, other, ld, N, nf, f0, fs, (size_t)j * N, (size_t)J * N, J != j, aj, nh,
+    ring_pair_epilogue<G, NT, true, false>(z, other, ld, N, nf, f0, fs, (size_t)j * N, (size_t)J * N, J != j, aj, nh,
                                            jh, ep, red, fi[slot]);
     if (ep.xout) {   // the update's new scaling: its spectra for the next half-step
       __syncthreads();
@@ -342,6 +342,13 @@ using Plan1440 = CtPlan<1440, 15, 8, 12>;
 using Plan1024 = CtPlan<1024, 4, 16, 16>;
 constexpr int kCtasCt = 4;
 
+// Entries of the twiddle table a CTA copies into shared memory: all for rings of up to 768
+// longitudes (6 KB), where a CTA has few items and would wait for each stage's twiddles from L2 (32
+// rings, one field: 9.4 us an update launch without the copy, 7.3 with it in the scalar form); none
+// beyond, where many items read them through L1.
+constexpr int kTwMax = 768;
+int twiddles_in_smem(const Grid& g) { return g.nlon <= kTwMax ? fft_tw_len(g.plan) : 0; }
+
 // Whether a CTA takes one field (C1, kThreads1 threads as one FFT butterfly needs half the registers)
 // instead of a pair: a single field, which leaves half of every pair idle; where one field each gives CTAs
 // that are all resident at once, so that pairs would halve the work in flight; and on rings so long that
@@ -360,13 +367,6 @@ bool one_field(const Grid& g, int nf) {
   return nf == 1 || (long long)g.nh * nf <= kCtas * g.num_sms;
 }
 
-// Entries of the twiddle table a CTA copies into shared memory: all for rings of up to 768
-// longitudes (6 KB), where a CTA has few items and would wait for each stage's twiddles from L2 (32
-// rings, one field: 9.4 us an update launch without the copy, 7.3 with it in the scalar form); none
-// beyond, where many items read them through L1.
-constexpr int kTwMax = 768;
-int twiddles_in_smem(const Grid& g) { return g.nlon <= kTwMax ? fft_tw_len(g.plan) : 0; }
-
 template <int G, class PL = RuntimePlan, int NT = kThreads, int CTAS = kCtas, class E = C2>
 int launch_fwd_t(const Grid& g, const float* in, int nf, const ProbState* ps, int scale_which, float* X,
                  int ldc, cudaStream_t st, const int2* mlim, const double* heat_t) {
@@ -384,17 +384,17 @@ int launch_fwd_t(const Grid& g, const float* in, int nf, const ProbState* ps, in
   return SHOT_OK;
 }
 
-template <int G, class PL = RuntimePlan, int NT = kThreads, int CTAS = kCtas, class E = C2>
+template <int G, class PL = RuntimePlan, int NT = kThreads, int CTAS = kCtas, class E = C2, bool LONG = (PL::N > kTwMax)>
 int launch_idft_t(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st) {
   const int tws = twiddles_in_smem(g);
   // two sequence buffers; the second first stages the spectra
   const size_t smem = idft_smem<E>(G, g.nlon) + tws * sizeof(float2);
-  SHOT_CUDA(cudaFuncSetAttribute(k_idft<G, NT, CTAS, PL, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  SHOT_CUDA(cudaFuncSetAttribute(k_idft<G, NT, CTAS, PL, E, LONG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   dim3 grid((nf + E::F * G - 1) / (E::F * G), g.nh);   // field groups of one ring pair run together
   ProfScope prof(ep.mode == EPI_CHECK || ep.mode == EPI_FINAL ? PK_CHECK : PK_IDFT, st);
   count_launch();
-  k_idft<G, NT, CTAS, PL, E><<<grid, NT, smem, st>>>(Y, ldc, nf, g.nlat, g.nlon, g.lmax, g.nh, g.a_d, g.plan, g.tw_d,
-                                                    tws, ep);
+  k_idft<G, NT, CTAS, PL, E, LONG><<<grid, NT, smem, st>>>(Y, ldc, nf, g.nlat, g.nlon, g.lmax, g.nh, g.a_d, g.plan,
+                                                          g.tw_d, tws, ep);
   SHOT_CUDA(cudaGetLastError());
   return SHOT_OK;
 }
@@ -474,7 +474,8 @@ int launch_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams&
     if (plan_is<Plan1024>(g.plan)) return launch_idft_p_t<Plan1024>(g, Y, ldc, nf, ep, st);
     return launch_idft_p_t<RuntimePlan>(g, Y, ldc, nf, ep, st);
   }
-  if (one_field(g, nf)) return launch_idft_t<1, RuntimePlan, kThreads1, kCtas, C1>(g, Y, ldc, nf, ep, st);
+  if (one_field(g, nf))
+    return launch_idft_t<1, RuntimePlan, kThreads1, kCtas, C1>(g, Y, ldc, nf, ep, st);
   switch (G) {
     case 6: return launch_idft_t<6>(g, Y, ldc, nf, ep, st);
     case 3: return launch_idft_t<3>(g, Y, ldc, nf, ep, st);
@@ -482,6 +483,7 @@ int launch_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams&
     default:
       if (plan_is<Plan1440>(g.plan)) return launch_idft_t<1, Plan1440, kThreads, kCtasCt>(g, Y, ldc, nf, ep, st);
       if (plan_is<Plan1024>(g.plan)) return launch_idft_t<1, Plan1024, kThreads, kCtasCt>(g, Y, ldc, nf, ep, st);
+      if (g.nlon > kTwMax) return launch_idft_t<1, RuntimePlan, kThreads, kCtas, C2, true>(g, Y, ldc, nf, ep, st);
       return launch_idft_t<1>(g, Y, ldc, nf, ep, st);
   }
 }

@@ -95,9 +95,11 @@ __device__ __forceinline__ void epi_prefetch_marginals(const EpiParams& ep, cons
 // field whatever number of threads share it.  No term passes more FP32 additions than with 256 threads
 // and eight warps per field (4 + 2 ceil(N / 256): a chain of both rings' terms and five lane steps),
 // which the short rings of G = 6 would otherwise exceed: 32 threads, 16 terms each.  The unbalanced
-// update amplifies the rounding of its sum by tau / eps.  Against one plain chain a thread and one sum
-// a warp: 40 iterations of 24 problems at 720 rings 35.9 -> 36.1 ms, four grids of 64 to 180 rings
-// 18.47 -> 18.55.
+// update amplifies the rounding of its sum by tau / eps.  LONG (one pair of fields a CTA on rings of more
+// than 768 longitudes): ceil(N / 192) + 5 additions are within that without batches and with whole-warp
+// sums, and the shorter code keeps registers.  An update in the persistent kernel, plain chain -> batches ->
+// LONG: 420 x 864, 12 problems 48.5 -> 51.8 -> 49.6 us; 720 x 1440, 24 problems, band limit 255 113.8 ->
+// 117.3 -> 116.3.  Four grids of 64 to 180 rings, 40 iterations, against the plain chain: 18.47 -> 18.55 ms.
 template <class V, bool TWO = false>
 struct Chain {
   V a{}, b{};
@@ -120,10 +122,10 @@ struct CompInf {   // the error beside the sum (Knuth's two-sum); an infinite su
 
 // Partial sums of a CTA's warps: NT / G threads share an element's F fields, and each of their GW warps
 // leaves P sums of 32 / P lanes.
-template <int G, int NT, int F>
+template <int G, int NT, int F, bool LONG = false>
 struct EpiRed {
-  static constexpr int GW = NT / G / 32, P = GW >= 8 ? 1 : GW >= 4 ? 2 : GW >= 2 ? 4 : 8;
-  static_assert(GW * P >= 8, "at least eight partial sums");
+  static constexpr int GW = NT / G / 32, P = LONG || GW >= 8 ? 1 : GW >= 4 ? 2 : GW >= 2 ? 4 : 8;
+  static_assert(LONG || GW * P >= 8, "at least eight partial sums");
   float v[NT / 32][P][F * NPART];
   double d[NT / 32][F][2];   // EPI_FINAL: warp sums of m(pi) and the objective
 };
@@ -158,7 +160,7 @@ __device__ __forceinline__ float epi_update_value(float pm, float kv, float rr, 
 // on the thread's sum: it is finite exactly if every u is (or the sum has overflowed, which stops
 // the problem too).  The pointwise part is instruction issue: with a check and a scaled divide per
 // value it took 38 of the update kernel's 79 million warp instructions (720 rings, 24 fields).
-template <int GT>
+template <int GT, bool LONG>
 __device__ __forceinline__ void epi_update_pair(const float4* zg, float4* og, int t, int N, const EpiField* fi,
                                                 float* out, size_t fstride, size_t rj, int dJ, bool xout, float aj,
                                                 float (&acc)[2][NPART]) {
@@ -216,8 +218,14 @@ __device__ __forceinline__ void epi_update_pair(const float4* zg, float4* og, in
         u.z = epi_update_value(pv[b].z, z.z, rr[0], bal0, gam[0], aj, v0.z, v1.z, bad[0]);
         u.w = epi_update_value(pv[b].w, z.w, rr[1], bal1, gam[1], aj, v0.w, v1.w, bad[1]);
       }
-      x0 = add2(x0, add2(pk2(v0.x, v0.y), pk2(v0.z, v0.w)));
-      if (!(bal0 && bal1)) x1 = add2(x1, add2(pk2(v1.x, v1.y), pk2(v1.z, v1.w)));
+      const f32x2 y0 = add2(pk2(v0.x, v0.y), pk2(v0.z, v0.w));
+      if constexpr (LONG) s0.add(y0);
+      else x0 = add2(x0, y0);
+      if (!(bal0 && bal1)) {
+        const f32x2 y1 = add2(pk2(v1.x, v1.y), pk2(v1.z, v1.w));
+        if constexpr (LONG) s1.add(y1);
+        else x1 = add2(x1, y1);
+      }
       if (out) {
         float* o = out + k;
         o[0] = u.x;
@@ -227,8 +235,10 @@ __device__ __forceinline__ void epi_update_pair(const float4* zg, float4* og, in
       }
       if (xout) og[k] = u;
     }
-    s0.add(x0);
-    s1.add(x1);
+    if constexpr (!LONG) {
+      s0.add(x0);
+      s1.add(x1);
+    }
   }
   const float2 a0 = unpk2(s0.value()), a1 = unpk2(s1.value());
   acc[0][0] = a0.x;
@@ -243,16 +253,17 @@ __device__ __forceinline__ void epi_update_pair(const float4* zg, float4* og, in
   }
 }
 
-// kFinal = false compiles the EPI_FINAL branch out (kernels never launched with it).
+// LONG: the sums' form for rings of more than 768 longitudes.  kFinal = false compiles the EPI_FINAL
+// branch out (kernels never launched with it).
 // The CTA's NT threads form G groups of NT / G (whole warps); group g takes the F fields from
 // f0 + F g on, a thread longitude k of both rings of the pair, so that one set of sums per
 // thread and one warp reduction serve a group whatever G is.
-template <int G, int NT, bool kFinal = true, class E>
+template <int G, int NT, bool LONG = false, bool kFinal = true, class E>
 __device__ __forceinline__ void ring_pair_epilogue(const E* z, E* other, int ld, int N, int nf, int f0,
                                                    size_t fstride, size_t rj, size_t rJ, bool two, float aj,
                                                    int nh, int jh, const EpiParams& ep,
-                                                   EpiRed<G, NT, E::F>& red, const EpiField* fi) {
-  constexpr int GT = NT / G, GW = GT / 32, P = EpiRed<G, NT, E::F>::P, F = E::F;
+                                                   EpiRed<G, NT, E::F, LONG>& red, const EpiField* fi) {
+  constexpr int GT = NT / G, GW = GT / 32, P = EpiRed<G, NT, E::F, LONG>::P, F = E::F;
   static_assert(NT % G == 0 && GT % 32 == 0, "a group is whole warps");
   constexpr int kBatchGen = 2;   // the general path of the update
   constexpr int kEpiBatch = 4;   // longitudes per thread whose marginal values are loaded together
@@ -297,7 +308,7 @@ __device__ __forceinline__ void ring_pair_epilogue(const E* z, E* other, int ld,
       if (pair) {
         float* out = ep.skip_store ? nullptr : ep.out + (size_t)fa * fstride + rj;
         const int dJ = (int)(rJ - rj);   // a field has fewer than 2^31 nodes
-        epi_update_pair<GT>(reinterpret_cast<const float4*>(zg), reinterpret_cast<float4*>(og), t, N, f2, out, fstride,
+        epi_update_pair<GT, LONG>(reinterpret_cast<const float4*>(zg), reinterpret_cast<float4*>(og), t, N, f2, out, fstride,
                             rj, dJ, ep.xout != nullptr, aj, acc);
       }
     }
@@ -371,12 +382,19 @@ __device__ __forceinline__ void ring_pair_epilogue(const E* z, E* other, int ld,
               un[r][q] = u;
             }
           }
-          x0 = add2(x0, of_lanes(v0));
-          x1 = add2(x1, of_lanes(v1));
+          if constexpr (LONG) {
+            s0.add(of_lanes(v0));
+            s1.add(of_lanes(v1));
+          } else {
+            x0 = add2(x0, of_lanes(v0));
+            x1 = add2(x1, of_lanes(v1));
+          }
           if (ep.xout) og[k] = cx(of_lanes(un[0]), of_lanes(un[1]));
         }
-        s0.add(x0);
-        s1.add(x1);
+        if constexpr (!LONG) {
+          s0.add(x0);
+          s1.add(x1);
+        }
       }
 #pragma unroll
       for (int q = 0; q < F; ++q) {
@@ -541,25 +559,36 @@ __device__ __forceinline__ void ring_pair_epilogue(const E* z, E* other, int ld,
       }
     }
   }
-  // four lanes a sum: the FP64 additions of one thread would be a chain that the CTA waits for
-  constexpr int kSums = F * G * NPART;
-  static_assert(4 * kSums <= NT && (4 * kSums < 32 || 4 * kSums % 32 == 0), "whole warps, or one");
-  int tid = threadIdx.x;
-  asm volatile("" : "+r"(tid));   // keeps a persistent kernel's loop from carrying the indices below
-  if (tid < 4 * kSums) {
-    const int x = tid >> 2, fq = x / NPART, i = x - fq * NPART;
-    const int w0 = fq / F * GW, c = fq % F * NPART + i;
-    double s = 0.0;
-#pragma unroll
-    for (int y = 0; y < (GW * P + 3) / 4; ++y) {
-      const int e = 4 * y + (tid & 3);
-      if (e < GW * P) s += (double)red.v[w0 + e / P][e % P][c];
+  if constexpr (LONG) {
+    if (threadIdx.x < F * G * NPART) {
+      const int fq = threadIdx.x / NPART, i = threadIdx.x - fq * NPART;
+      if (f0 + fq < nf && fi[fq].live && !(ep.mode == EPI_FINAL && i >= 2)) {
+        double s = 0.0;
+        for (int w = 0; w < GW; ++w) s += (double)red.v[fq / F * GW + w][0][fq % F * NPART + i];
+        ep.part[((size_t)(f0 + fq) * nh + jh) * NPART + i] = s;
+      }
     }
-    constexpr unsigned kMask = 4 * kSums >= 32 ? 0xffffffffu : (1u << (4 * kSums % 32)) - 1;
-    s += __shfl_xor_sync(kMask, s, 1);
-    s += __shfl_xor_sync(kMask, s, 2);
-    if ((tid & 3) == 0 && f0 + fq < nf && fi[fq].live && !(ep.mode == EPI_FINAL && i >= 2))
-      ep.part[((size_t)(f0 + fq) * nh + jh) * NPART + i] = s;
+  } else {
+    // four lanes a sum: the FP64 additions of one thread would be a chain that the CTA waits for
+    constexpr int kSums = F * G * NPART;
+    static_assert(4 * kSums <= NT && (4 * kSums < 32 || 4 * kSums % 32 == 0), "whole warps, or one");
+    int tid = threadIdx.x;
+    asm volatile("" : "+r"(tid));   // keeps a persistent kernel's loop from carrying the indices below
+    if (tid < 4 * kSums) {
+      const int x = tid >> 2, fq = x / NPART, i = x - fq * NPART;
+      const int w0 = fq / F * GW, c = fq % F * NPART + i;
+      double s = 0.0;
+#pragma unroll
+      for (int y = 0; y < (GW * P + 3) / 4; ++y) {
+        const int e = 4 * y + (tid & 3);
+        if (e < GW * P) s += (double)red.v[w0 + e / P][e % P][c];
+      }
+      constexpr unsigned kMask = 4 * kSums >= 32 ? 0xffffffffu : (1u << (4 * kSums % 32)) - 1;
+      s += __shfl_xor_sync(kMask, s, 1);
+      s += __shfl_xor_sync(kMask, s, 2);
+      if ((tid & 3) == 0 && f0 + fq < nf && fi[fq].live && !(ep.mode == EPI_FINAL && i >= 2))
+        ep.part[((size_t)(f0 + fq) * nh + jh) * NPART + i] = s;
+    }
   }
 }
 

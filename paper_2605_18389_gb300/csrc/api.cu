@@ -768,6 +768,7 @@ int shot_grid_init_quad(shot_grid* out, int quadrature, int nlat, int nlon, int 
     g->t32_in_override = (e && e[0] >= '1' && e[0] <= '8') ? e[0] - '0' : 0;
   }
   g->plan = plan;
+  g->generic_radix = fft_generic_radix(plan);
   cudaGetDevice(&g->dev);
   cudaDeviceGetAttribute(&g->num_sms, cudaDevAttrMultiProcessorCount, g->dev);
   int rc = build_grid_tables(*g, as_stream(stream));

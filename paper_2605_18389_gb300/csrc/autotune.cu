@@ -96,7 +96,8 @@ extern "C" int shot_grid_autotune(shot_grid gh, int nfields, int* choice, void* 
   if ((rc = launch_heat_mult(*g, 0.0, st))) return rc;
   if ((rc = autotune(*g, nfields, st))) return rc;
   if (choice) {
-    choice[0] = choice[1] = dft_fields_per_cta(*g, nfields);   // a rule on sizes, not timed
+    choice[0] = dft_fields_per_cta(*g, nfields, false);   // rules on sizes, not timed
+    choice[1] = dft_fields_per_cta(*g, nfields, true);    // (the solver's half-steps)
     choice[2] = g->active.simt_bn;
     choice[3] = g->active.tc_stages;
   }

@@ -350,21 +350,26 @@ constexpr int kTwMax = 768;
 int twiddles_in_smem(const Grid& g) { return g.nlon <= kTwMax ? fft_tw_len(g.plan) : 0; }
 
 // Whether a CTA takes one field (C1, kThreads1 threads as one FFT butterfly needs half the registers)
-// instead of a pair: a single field, which leaves half of every pair idle; where one field each gives CTAs
-// that are all resident at once, so that pairs would halve the work in flight; and on rings so long that
-// one CTA of pairs fills an SM.  Measured, pairs -> one field: a solve of one problem, 60 iterations, 64
-// rings (TF32x3) 3.00 -> 2.85 ms, 256 rings 5.07 -> 4.77; of five problems on 64 rings 2.99 -> 2.90; of three on
-// 200 rings of 1000 longitudes, 20 iterations (pairs in the persistent form) 1.51 -> 1.38; of three on rings
-// of 4096 longitudes 22.7 -> 15.2; a heat application, one field, rings of 2000 longitudes 93 -> 84 us.
-// Elsewhere pairs are as fast or faster: eight problems on 128 rings 3.52 against 3.53 ms, on rings of 3000
-// longitudes 14.5 against 16.4.  Rings with a compiled plan keep the pairs (1024 longitudes, one field: 50
-// against 55 us).
+// instead of a pair:
+// - a single field, which leaves half of every pair idle.  A solve of one problem, 60 iterations, pairs -> one
+//   field: 64 rings (TF32x3) 3.00 -> 2.85 ms, 256 rings 5.07 -> 4.77; a heat application on rings of 2000
+//   longitudes 93 -> 84 us;
+// - the solver's half-steps where one field each gives CTAs that are all resident at once, so that pairs
+//   would halve the work in flight: five problems on 64 rings 2.99 -> 2.90 ms, three on 200 rings of 1000
+//   longitudes (pairs in the persistent form) 1.51 -> 1.38.  Beyond it pairs are as fast or faster (eight
+//   problems on 128 rings 3.52 against 3.53).  Not the plain transforms, whose CTAs have less to do (five
+//   fields on 128 rings 25.9 -> 27.1 us a heat application), and not rings with a generic stage, whose pairs share
+//   the roots' loads (eight problems on 97 x 202 4.12 -> 4.22 ms);
+// - rings so long that one CTA of pairs fills an SM: three problems on rings of 4096 longitudes, 20 iterations
+//   22.7 -> 15.2 ms (3000 longitudes, eight problems: 14.5 -> 16.4).
+// Pairs stay on rings with a compiled plan (1024 longitudes, one field: 50 against 55 us) and on long rings
+// with a generic radix above 16, whose roots come through L1 (4099 longitudes: 3.4 against 5.7 ms).
 constexpr int kThreads1 = 256;
-bool one_field(const Grid& g, int nf) {
+bool one_field(const Grid& g, int nf, bool solver) {
+  const int generic = g.generic_radix;
+  if (plan_is<Plan1440>(g.plan) || plan_is<Plan1024>(g.plan) || (generic > 16 && g.nlon > kTwMax)) return false;
   const bool fills_sm = 2 * (idft_smem<C2>(1, g.nlon) + 2048) > 228 * 1024;   // 2 KB: static and reserved
-  if (fills_sm) return true;
-  if (plan_is<Plan1440>(g.plan) || plan_is<Plan1024>(g.plan)) return false;
-  return nf == 1 || (long long)g.nh * nf <= kCtas * g.num_sms;
+  return fills_sm || nf == 1 || (solver && generic == 1 && (long long)g.nh * nf <= kCtas * g.num_sms);
 }
 
 template <int G, class PL = RuntimePlan, int NT = kThreads, int CTAS = kCtas, class E = C2>
@@ -416,9 +421,9 @@ int launch_idft_p_t(const Grid& g, const float* Y, int ldc, int nf, const EpiPar
 
 }  // namespace
 
-int dft_fields_per_cta(const Grid& g, int nf) {
+int dft_fields_per_cta(const Grid& g, int nf, bool solver) {
   if (g.quad == SHOT_QUAD_HEALPIX) return hp_fields_per_cta(g);
-  return one_field(g, nf) ? 1 : 2 * pick_g(g, nf);
+  return one_field(g, nf, solver) ? 1 : 2 * pick_g(g, nf);
 }
 
 int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, int scale_which,
@@ -434,7 +439,7 @@ int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, 
     set_error("nlon too large for the shared-memory ring FFT");
     return SHOT_ERR_UNSUPPORTED;
   }
-  if (one_field(g, nf))
+  if (one_field(g, nf, false))
     return launch_fwd_t<1, RuntimePlan, kThreads1, kCtas, C1>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
   switch (pick_g(g, nf)) {
     case 6: return launch_fwd_t<6>(g, in, nf, ps, scale_which, X, ldc, st, mlim, heat_t);
@@ -456,7 +461,7 @@ int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, 
 // to 180 rings, 72 fields each, in one solve: 19.7 against 20.9 ms).
 static bool idft_is_persistent(const Grid& g, int nf, const EpiParams& ep) {
   return (((ep.mode == EPI_UPDATE || ep.mode == EPI_SYM) && ep.xout) || ep.mode == EPI_CHECK) &&
-         !g.idft_nonpersistent && nf >= 2 && g.nlon > kTwMax && !one_field(g, nf) && pick_g(g, nf) == 1 &&
+         !g.idft_nonpersistent && nf >= 2 && g.nlon > kTwMax && !one_field(g, nf, true) && pick_g(g, nf) == 1 &&
          idft_p_layout(g.nlon, g.lmax) <= 74 * 1024;
 }
 
@@ -474,7 +479,7 @@ int launch_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams&
     if (plan_is<Plan1024>(g.plan)) return launch_idft_p_t<Plan1024>(g, Y, ldc, nf, ep, st);
     return launch_idft_p_t<RuntimePlan>(g, Y, ldc, nf, ep, st);
   }
-  if (one_field(g, nf))
+  if (one_field(g, nf, ep.mode != EPI_PLAIN))
     return launch_idft_t<1, RuntimePlan, kThreads1, kCtas, C1>(g, Y, ldc, nf, ep, st);
   switch (G) {
     case 6: return launch_idft_t<6>(g, Y, ldc, nf, ep, st);

@@ -289,6 +289,17 @@ bool make_fft_plan(int N, FftPlan* pl) {
   return true;
 }
 
+int fft_generic_radix(const FftPlan& pl) {
+  int r = 1;
+  for (int s = 0; s < pl.nst; ++s) {
+    int n = pl.R[s];
+    for (int f : {2, 3, 5})
+      while (n % f == 0) n /= f;
+    r = std::max(r, n);
+  }
+  return r;
+}
+
 void fft_plan_twiddles(const FftPlan& pl, std::vector<float2>& tw) {
   const int N = pl.N;
   size_t total = N;

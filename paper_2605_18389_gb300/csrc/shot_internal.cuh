@@ -73,6 +73,8 @@ bool make_fft_plan(int N, FftPlan* plan);
 // the plan's stage twiddles W_N^{k r N/(Ns R)} (forward sign), then the roots of its generic
 // stages: N + (sum of their radices) complex values
 void fft_plan_twiddles(const FftPlan& plan, std::vector<float2>& tw);
+// largest radix of the plan without a compiled butterfly (a prime factor above 5; 1: none)
+int fft_generic_radix(const FftPlan& plan);
 
 // ---------------------------------------------------------------------------------
 // Spectral layout.  For order m and parity p (p = (l - m) mod 2) the block (m,p)
@@ -151,6 +153,7 @@ struct Grid {
   int dev = 0;
   int num_sms = 148;
   FftPlan plan{};
+  int generic_radix = 1;        // fft_generic_radix(plan)
   // host copies (FP64)
   std::vector<double> x, w, a_ring;
   // blocks
@@ -282,7 +285,7 @@ bool profiling_on();
 int launch_dft_fwd(const Grid& g, const float* in, int nf, const ProbState* ps, int scale_which,
                    float* X, int ldc, cudaStream_t st, const int2* mlim = nullptr, const double* heat_t = nullptr);
 int launch_idft(const Grid& g, const float* Y, int ldc, int nf, const EpiParams& ep, cudaStream_t st);
-int dft_fields_per_cta(const Grid& g, int nf);   // fields a ring-transform CTA takes
+int dft_fields_per_cta(const Grid& g, int nf, bool solver);   // fields a ring-transform CTA takes
 int hp_fields_per_cta(const Grid& g);            // the same on a HEALPix grid
 // Grids whose Legendre contractions run the TF32x3 tensor-core kernels: TF32X3 grids, and BF16X3
 // grids in recurrence mode (the recurrence kernels are bound by generating the A operand, not by

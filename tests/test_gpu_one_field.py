@@ -1,7 +1,8 @@
 """Solves around the line between one field and two fields an element of the ring transforms, against the
-oracle: one problem, the last count whose CTAs of one field are all resident (33 ring pairs, 13 problems)
-and the first beyond it, and rings on both sides of 3583 longitudes, the longest of which two CTAs of pairs share an SM.  Balanced
-and unbalanced, an equator ring, a marginal check."""
+oracle: one problem, the last count whose CTAs of one field are all resident (33 ring pairs, 13 problems) and the
+first beyond it, rings on both sides of 3583 longitudes, the longest of which two CTAs of pairs share an SM,
+and rings with a prime factor that a generic stage takes.  Balanced and unbalanced, an equator ring, a
+marginal check."""
 import math
 
 import numpy as np
@@ -21,8 +22,9 @@ TOL = 1e-5   # potentials, transport cost and mass of an FP32 solve against the 
 
 
 @pytest.mark.parametrize("nlat,nlon,lmax,n,eps,fields", [
-    (65, 130, 64, 1, 0.05, 1), (65, 130, 64, 13, 0.05, 1), (65, 130, 64, 14, 0.05, 2),
-    (305, 3582, 20, 3, 0.5, 2), (305, 3584, 20, 3, 0.5, 1), (12, 6400, 11, 2, 0.5, 1),
+    (65, 135, 64, 1, 0.05, 1), (65, 135, 64, 13, 0.05, 1), (65, 135, 64, 14, 0.05, 2),
+    (65, 130, 64, 1, 0.05, 1), (65, 130, 64, 13, 0.05, 2), (20, 802, 19, 1, 0.2, 2),
+    (305, 3575, 20, 3, 0.5, 2), (305, 3584, 20, 3, 0.5, 1), (12, 6400, 11, 2, 0.5, 1),
 ])
 @pytest.mark.parametrize("tau", [math.inf, 1.0])
 def test_solve_matches_oracle(nlat, nlon, lmax, n, eps, fields, tau):
@@ -32,7 +34,7 @@ def test_solve_matches_oracle(nlat, nlon, lmax, n, eps, fields, tau):
     (p32, p64), (q32, q64) = f32(p), f32(q)
     g = shot.shot_grid_init(nlat, nlon, lmax)
     try:
-        assert shot.shot_grid_autotune(g, n)["dft_fg"] == fields
+        assert shot.shot_grid_autotune(g, n)["idft_fg"] == fields
         rc, r = shot.shot_sinkhorn(g, torch.from_numpy(p32).cuda(), torch.from_numpy(q32).cuda(), eps, tau,
                                    max_iter=T, tol=0.0, check_every=10)
         assert rc == 0 and np.all(r["status"] == 0)

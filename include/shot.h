@@ -317,8 +317,8 @@ int shot_heat_apply_noalloc(shot_grid g, double t, const float* in, float* out, 
 /* Autotune the launch shapes used for calls on `nfields` fields (FP32 Legendre tile width, BF16x3
  * analysis pipeline depth) by timing the candidates with CUDA events; the solvers do this
  * automatically on their first call for a field count.  choice: host int[4] or NULL, receives the
- * fields per ring-DFT and inverse-DFT CTA (a rule on sizes, not timed) and the two selections (0 =
- * the default).  The choices change no summation order (results are bit-identical).
+ * fields per CTA of the ring transforms and of the solver's inverse ring transforms (rules on
+ * sizes, not timed) and the two selections (0 = the default).  The choices change no summation order (results are bit-identical).
  * Synchronises `stream`. */
 int shot_grid_autotune(shot_grid g, int nfields, int* choice, void* stream);
 

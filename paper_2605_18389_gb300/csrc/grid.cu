@@ -207,7 +207,10 @@ __global__ void k_coeff_scatter(int lmax, int nf, const long long* __restrict__ 
 // conflicts of the first stage's stores (lanes at a stride of R elements: conflict-free for odd R,
 // gcd(2R, 32)/2-way otherwise), which puts an odd radix first when there is one and otherwise the
 // smallest; then the smallest largest radix (registers, and for a short ring the time of a stage: a
-// few threads, each with one butterfly; 64 points as 8 * 8 instead of 4 * 16).
+// few threads, each with one butterfly; 64 points as 8 * 8 instead of 4 * 16).  Solves of 2 to 24 problems:
+// with the conflicts counted on the short rings too, 24 to 96 points take 3-9 % longer; with no such count on
+// the longer ones, 120 to 288 points 2-5 % less, but the plans of the grids that the accuracy tests were
+// set on would change with it.
 bool make_fft_plan(int N, FftPlan* pl) {
   if (N < 1 || N >= (1 << 16)) return false;
   // prime factors above 5 become generic stages, placed first (their stage twiddles are 1)

@@ -401,7 +401,9 @@ def shot_divergence_multi(sets, max_iter=200, tol=0.0, check_every=10, flags=0, 
 
 
 def shot_grid_autotune(g, nfields, stream=None):
-    """Tune (or look up) the launch shapes for nfields; returns dict of the four choices."""
+    """Tune (or look up) the launch shapes for nfields; returns a dict: the fields per CTA of the ring transforms
+    (dft_fg) and of the solver's inverse transforms (idft_fg), which are rules on sizes, and the two tuned
+    choices (0 = the default)."""
     ch = np.zeros(4, np.int32)
     _check(lib().shot_grid_autotune(g, int(nfields), _np_ptr(ch, ctypes.c_int), _stream(stream)))
     return dict(zip(("dft_fg", "idft_fg", "simt_bn", "tc_stages"), [int(x) for x in ch]))

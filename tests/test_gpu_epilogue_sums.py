@@ -5,9 +5,9 @@ whatever the number of threads that share a field.
 The gauge makes the returned u sum to 1 over the nodes, so the FP64 sum of u shows the rounding of the
 device's own sum.  The marginal below is 1.01 on the longitudes a thread meets first and 0.99 * 2^-23 on
 the others: one plain FP32 chain a thread loses every later term (each is below half a unit in the last
-place of 2.02), 8e-7 of the sum for eight longitudes a thread.  The bar is the worst case of the roundings
-of 2^-24 each: the factor of u, its product with the buffer, and the eight additions that a term passes
-at most at these sizes."""
+place of 2.02), 8e-7 of the sum for eight longitudes a thread.  The bar is ten roundings of 2^-24: the factor
+of u, its product with the buffer, and eight additions, the most that a term passes on rings of up to 768
+longitudes and on HEALPix rings of 1024 points (13 on rings of 1440)."""
 import numpy as np
 import pytest
 

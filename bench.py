@@ -232,10 +232,13 @@ def algorithmic_work(kind, nlat, npix, lmax, nfields, legendre="table"):
     return 0.0, 0.0
 
 
-# DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) from ncu captures of this
-# file's 720 x 1440, 24-field runs, by (kind, precision, legendre); empty where the kernels have
-# changed since their last capture (the packed ring transforms and the polar cut): null in the line.
-NCU_TRAFFIC = {}
+# DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) from ncu captures of the headline
+# workload's launches (720 x 1440, 24 fields; profiles/ncu_ring_fft_packed_720x1440.md), by (kind,
+# precision, legendre); the forms without an entry report null.  The update kernel is the same in every
+# precision and stores the scaling in 2 of a block's 20 half-steps.
+NCU_TRAFFIC = {("inverse_dft_epilogue", "*", "*"): (18 * 180.0e6 + 2 * 268.1e6) / 20,
+               ("legendre_analysis", "tf32x3", "table"): 479.0e6, ("legendre_synthesis", "tf32x3", "table"): 586.2e6,
+               ("legendre_analysis", "bf16x3", "table"): 507.9e6, ("legendre_synthesis", "bf16x3", "table"): 514.1e6}
 
 
 def roofline(kind, avg_ms, nlat, npix, lmax, nfields, prec, legendre="table"):

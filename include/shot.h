@@ -318,8 +318,8 @@ int shot_heat_apply_noalloc(shot_grid g, double t, const float* in, float* out, 
  * analysis pipeline depth) by timing the candidates with CUDA events; the solvers do this
  * automatically on their first call for a field count.  choice: host int[4] or NULL, receives the
  * fields per CTA of the ring transforms and of the solver's inverse ring transforms (rules on
- * sizes, not timed) and the two selections (0 = the default).  The choices change no summation order (results are bit-identical).
- * Synchronises `stream`. */
+ * sizes, not timed) and the two selections (0 = the default).  The selections change no summation
+ * order (results are bit-identical).  Synchronises `stream`. */
 int shot_grid_autotune(shot_grid g, int nfields, int* choice, void* stream);
 
 /* ---- heat convolution vs explicit matrix convolution -----------------------

@@ -157,10 +157,11 @@ __global__ void __launch_bounds__(kHpThreads, 4) k_hp_idft(const float* __restri
   epi_fields_load<F>(ep, f0, nfg, fi);
   // Z_k = A_k + B_{n-k}: A_r sums e^{i m phi0} (G_N + i G_S) over the orders m >= 0 of residue r
   // modulo n, B_r sums e^{-i m phi0} (conj G_N + i conj G_S) over the orders m >= 1; each spectra row is
-  // read once, straight from global memory.  On the short rings near the poles a residue has many orders,
-  // and S threads share them, four rows in flight each (nside 64, one field, plain synthesis: 25.8 us with
-  // the rows gathered through shared memory, 33.0 with one thread a residue, 20.7 with all threads).
-  const int S = ml.x < 4 * n ? 1 : max(1, min(min(kHpThreads, nmax) / n, (ml.x + 4 * n) / (4 * n)));
+  // read once, straight from global memory.  Where a thread would have 16 rows or more (the short rings
+  // near the poles without a polar cut: plain synthesis, FP32 recurrence), S threads share a residue, four
+  // rows in flight each (nside 64, one field, plain synthesis: 25.8 us with the rows gathered through shared
+  // memory, 33.0 with one thread a residue, 23.0 so).  With the cut a residue of such a ring has a few orders.
+  const int S = ml.x < 16 * n ? 1 : max(1, min(min(kHpThreads, nmax) / n, (ml.x + 4 * n) / (4 * n)));
   {
     const float* y = Y + (size_t)jh * ldc + 2 * f0;
     const size_t row = (size_t)nh * ldc;
